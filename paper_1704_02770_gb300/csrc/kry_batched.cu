@@ -410,42 +410,46 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
 // ---------------------------------------------------------------- per-realisation reductions
 
 // mode: 0 pass A, 1 pass B, 3 pass C1 (dots of w), 2 pass C2 (correction), 4 combine,
-// 5 load of a general psi0.
-__global__ void __launch_bounds__(128) k_reduce_b(KryCtlB *ctl, const double2 *__restrict__ part,
+// 5 load of a general psi0.  One CTA per realisation.  A warp takes a whole slot (lanes over the
+// CTAs' partials, then a shuffle tree) and lane i of warp 0 the scalars of vector i: GB300 issues
+// one FP64 warp instruction per about 77 cycles and SM sub-partition whatever its active lanes, so
+// block-wide trees slot by slot and loops over the vectors in one thread cost tens of us at j = 30.
+__global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *__restrict__ part,
                                                   int grid, int Kp, int mode, int jj, int general)
 {
     KryHdrB &H = ctl->hd;
     if (H.done) return;
     if (mode <= 3 && jj >= H.m_run) return;
-    const int k = blockIdx.x, tid = threadIdx.x;
+    const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (mode == 2 && !H.corr_any) return;   // pass C2 did not run
     if (mode == 3 && !H.dots_any) return;   // pass C1 did not run
-    __shared__ double2 red[128];
     __shared__ double2 fin[PSB];
     const int nd = (mode == 0 || mode == 3) ? jj + 1 : 0;
-    auto reduce_slot = [&](int slot) {
+    const int ns = nd + (mode != 3 ? 1 : 0) + (general && mode != 0 && mode != 3 ? 1 : 0);
+    for (int q = warp; q < ns; q += 8) {
+        const int slot = q < nd ? q : q == nd ? SLOT_NRM : SLOT_G;
         double2 s = make_double2(0.0, 0.0);
-        for (int c = tid; c < grid; c += 128) {
+#pragma unroll 4
+        for (int c = lane; c < grid; c += 32) {
             const double2 v = __ldg(part + ((size_t)c * PSB + slot) * Kp + k);
             s.x += v.x;
             s.y += v.y;
         }
-        red[tid] = s;
-        __syncthreads();
-        for (int o = 64; o > 0; o >>= 1) {
-            if (tid < o) { red[tid].x += red[tid + o].x; red[tid].y += red[tid + o].y; }
-            __syncthreads();
-        }
-        if (tid == 0) fin[slot] = red[0];
-        __syncthreads();
-    };
-    for (int i = 0; i < nd; ++i) reduce_slot(i);
-    if (mode != 3) reduce_slot(SLOT_NRM);
-    if (general && mode != 0 && mode != 3) reduce_slot(SLOT_G);
-    if (tid != 0) return;
+        s = warp_sum(s);
+        if (lane == 0) fin[slot] = s;
+    }
+    __syncthreads();
+    if (tid >= 32) return;
     const double nw2 = (mode == 3) ? ctl->wnorm2[k] : fin[SLOT_NRM].x;
     const double2 gdot = (mode == 3) ? ctl->wg[k]
                                      : ((general && mode != 0) ? fin[SLOT_G] : make_double2(0.0, 0.0));
+    // lane i: <v_i, y> = c, c sigma_i (modes 0 and 3)
+    double2 c = make_double2(0.0, 0.0), cs = c;
+    if (lane < nd) {
+        const double s = ctl->sigma[lane][k];
+        c = make_double2(fin[lane].x * s, fin[lane].y * s);
+        cs = make_double2(c.x * s, c.y * s);
+    }
     auto finalize = [&](double w2, double2 gd) {
         const double bt = sqrt(w2);
         ctl->beta[jj][k] = bt;
@@ -460,34 +464,28 @@ __global__ void __launch_bounds__(128) k_reduce_b(KryCtlB *ctl, const double2 *_
         }
     };
     if (mode == 0) {
-        if (k == 0) {
+        if (k == 0 && lane == 0) {
             H.n_hv += 1;
-            H.vec_passes += (double)(jj + 4);
-            H.vp_kind[KIND_PASSA] += (double)(jj + 2);   // u and v_0 .. v_j
-            H.vp_kind[KIND_HV] += 2.0;                  // the H.v: v_j read, u written
+            H.vec_passes += jj + 4;
+            H.vp_kind[KIND_PASSA] += jj + 2;   // u and v_0 .. v_j
+            H.vp_kind[KIND_HV] += 2;                  // the H.v: v_j read, u written
             H.corr_any = 0;
             H.dots_any = 0;
         }
-        if (jj >= ctl->m_eff[k]) {
-            // invariant subspace already reached: this realisation's next vectors stay zero
-            for (int i = 0; i <= jj; ++i) ctl->coefA[i][k] = make_double2(0.0, 0.0);
-            return;
-        }
-        for (int i = 0; i <= jj; ++i) {
-            const double s = ctl->sigma[i][k];
-            const double2 c = make_double2(fin[i].x * s, fin[i].y * s);
-            ctl->coefA[i][k] = make_double2(c.x * s, c.y * s);
-            if (i == jj) ctl->alpha[jj][k] = c.x;
-        }
-        ctl->normu2[k] = nw2;
+        // (invariant subspace already reached: this realisation's next vectors stay zero)
+        const bool run = jj < ctl->m_eff[k];
+        if (lane <= jj) ctl->coefA[lane][k] = run ? cs : make_double2(0.0, 0.0);
+        if (run && lane == jj) ctl->alpha[jj][k] = c.x;
+        if (run && lane == 0) ctl->normu2[k] = nw2;
     } else if (mode == 1) {
-        if (k == 0) {
-            H.vec_passes += (double)(jj + 3) + (general ? 1.0 : 0.0);
-            H.vp_kind[KIND_PASSB] += (double)(jj + 3) + (general ? 1.0 : 0.0);
+        if (k == 0 && lane == 0) {
+            H.vec_passes += jj + 3 + (general ? 1 : 0);
+            H.vp_kind[KIND_PASSB] += jj + 3 + (general ? 1 : 0);
         }
+        if (lane <= jj) ctl->coefC[lane][k] = make_double2(0.0, 0.0);
+        if (lane != 0) return;
         ctl->corr[k] = 0;
         ctl->dots[k] = 0;
-        for (int i = 0; i <= jj; ++i) ctl->coefC[i][k] = make_double2(0.0, 0.0);
         if (jj >= ctl->m_eff[k]) return;
         // One classical Gram-Schmidt pass is enough unless the projection cancelled most of
         // u (||w|| < eta ||u||, the Daniel-Gragg-Kaufman-Stewart test); then this
@@ -501,32 +499,29 @@ __global__ void __launch_bounds__(128) k_reduce_b(KryCtlB *ctl, const double2 *_
             finalize(nw2, gdot);
         }
     } else if (mode == 3) {
-        if (k == 0) {
-            H.vec_passes += (double)(jj + 2);
-            H.vp_kind[KIND_PASSC] += (double)(jj + 2);
+        if (k == 0 && lane == 0) {
+            H.vec_passes += jj + 2;
+            H.vp_kind[KIND_PASSC] += jj + 2;
         }
         if (!ctl->dots[k] || jj >= ctl->m_eff[k]) return;
-        double nd2 = 0.0;
-        for (int i = 0; i <= jj; ++i) {
-            const double s = ctl->sigma[i][k];
-            nd2 += (fin[i].x * fin[i].x + fin[i].y * fin[i].y) * s * s;
-        }
+        const double nd2 = warp_sum(c.x * c.x + c.y * c.y);
+        const bool sub = nw2 > 0.0 && sqrt(nd2) > H.eta_corr * sqrt(nw2);
+        if (sub && lane <= jj) ctl->coefC[lane][k] = cs;
+        if (sub && lane == jj) ctl->alpha[jj][k] += c.x;
+        if (lane != 0) return;
         if (nw2 > 0.0) ctl->orth[k] = fmax(ctl->orth[k], sqrt(nd2 / nw2));
-        if (nw2 > 0.0 && sqrt(nd2) > H.eta_corr * sqrt(nw2)) {
+        if (sub) {
             ctl->corr[k] = 1;
             H.corr_any = 1;
-            for (int i = 0; i <= jj; ++i) {
-                const double s = ctl->sigma[i][k];
-                ctl->coefC[i][k] = make_double2(fin[i].x * s * s, fin[i].y * s * s);
-            }
-            ctl->alpha[jj][k] += fin[jj].x * ctl->sigma[jj][k];
         } else {
             finalize(nw2, gdot);
         }
+    } else if (lane != 0) {
+        return;
     } else if (mode == 2) {
-        if (k == 0) {
-            H.vec_passes += (double)(jj + 3) + (general ? 1.0 : 0.0);
-            H.vp_kind[KIND_PASSC] += (double)(jj + 3) + (general ? 1.0 : 0.0);
+        if (k == 0 && lane == 0) {
+            H.vec_passes += jj + 3 + (general ? 1 : 0);
+            H.vp_kind[KIND_PASSC] += jj + 3 + (general ? 1 : 0);
         }
         if (jj < ctl->m_eff[k] && ctl->corr[k]) {
             atomicAdd(&H.n_corr, 1ull);
@@ -556,8 +551,8 @@ __global__ void k_step_done_b(KryCtlB *ctl, int general)
     for (int k = 0; k < H.K; ++k) e = fmax(e, ctl->err_k[k]);
     H.err_sum += e;
     H.n_steps += 1;
-    H.vec_passes += (double)(H.m_run + 1) + (general ? 1.0 : 0.0);
-    H.vp_kind[KIND_COMBINE] += (double)(H.m_run + 1) + (general ? 1.0 : 0.0);
+    H.vec_passes += H.m_run + 1 + (general ? 1 : 0);
+    H.vp_kind[KIND_COMBINE] += H.m_run + 1 + (general ? 1 : 0);
     H.t_now = H.t_next;
     H.next_out = H.next_out_new;
     H.m_run = H.m;
@@ -709,7 +704,7 @@ int launch_lincomb_b(const EvArgsB<V> &a, int mode, int jj, int grid, cudaStream
 int launch_reduce_b(KryCtlB *ctl, const double2 *part, int grid, int K, int Kp, int mode, int jj,
                     int general, double, cudaStream_t s)
 {
-    k_reduce_b<<<K, 128, 0, s>>>(ctl, part, grid, Kp, mode, jj, general);
+    k_reduce_b<<<K, 256, 0, s>>>(ctl, part, grid, Kp, mode, jj, general);
     KRY_CU(cudaGetLastError());
     if (mode == 2) {
         k_mrun_b<<<1, 1, 0, s>>>(ctl);

@@ -439,6 +439,13 @@ __device__ __forceinline__ double2 warp_sum(double2 v)
     return v;
 }
 
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // ---------------------------------------------------------------- rank tables
 
 // Locate rank r0 + t (< D) as (block hi, offset in block, particles in the lower part):

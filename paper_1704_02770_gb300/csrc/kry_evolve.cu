@@ -400,7 +400,6 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
     const long long max_launch = 500000;   // Krylov steps before KRY_ETIMEOUT
     int batch = 1;
     const int nk = 3 * m + 2;   // kernels of the step graph (pass C not counted)
-    const double vp0[NKIND] = {0, 0, 0, 0, 0, 0};
     for (;;) {
         if (H->prof_on) batch = 1;   // events are read after every step
         for (int i = 0; i < batch; ++i) KRY_CU(cudaGraphLaunch(H->gexec, s));
@@ -428,7 +427,7 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
     KRY_CU(cudaEventRecord(ev1, s));
     if (H->prof_on)
         for (int q = 0; q < NKIND; ++q)
-            H->prof_bytes[q] += (hp->vp_kind[q] - vp0[q]) * (double)nvec * (double)es;
+            H->prof_bytes[q] += (double)hp->vp_kind[q] * (double)nvec * (double)es;
     if (hp->err) {
         if (hp->err == KRY_ETOL) set_error("kry_evolve: no step size meets tol=%g at t=%g", tol, hp->t_now);
         else set_error("kry_evolve: initial vector has zero norm");
@@ -452,7 +451,7 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
         st->err_estimate = hp->err_sum;
         st->max_orth_loss = hp->max_orth;
         st->time_ms = ms;
-        st->algo_bytes = hp->vec_passes * (double)nvec * (double)es;
+        st->algo_bytes = (double)hp->vec_passes * (double)nvec * (double)es;
         const bool plain = plain_step_graph(H);
         st->n_launches = launched * (nk + (plain ? 2 * m : 0) + (ea.Yout ? 1 : 0) + ((opt && opt->ckpt) ? 1 : 0)) +
                          (plain ? 0 : 2 * hp->n_c1) + 1 + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
@@ -712,7 +711,7 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
     }
     KRY_CU(cudaEventRecord(ev1, s));
     if (H->prof_on)
-        for (int q = 0; q < NKIND; ++q) H->prof_bytes[q] += hp->vp_kind[q] * (double)nvec * (double)es;
+        for (int q = 0; q < NKIND; ++q) H->prof_bytes[q] += (double)hp->vp_kind[q] * (double)nvec * (double)es;
     if (hp->err) {
         if (hp->err == KRY_ETOL) set_error("kry_evolve: no step size meets tol=%g at t=%g", tol, hp->t_now);
         else set_error("kry_evolve: an initial vector has zero norm");
@@ -738,7 +737,7 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
         st->err_estimate = hp->err_sum;
         st->max_orth_loss = *std::max_element(orth.begin(), orth.end());
         st->time_ms = ms;
-        st->algo_bytes = hp->vec_passes * (double)nvec * (double)es;
+        st->algo_bytes = (double)hp->vec_passes * (double)nvec * (double)es;
         st->n_launches = launched * (10 * m + 5) + (general ? 2 : 1) + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
         st->n_second_dots = 0;
     }

@@ -142,7 +142,7 @@ __device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, d
 {
     const double bt = sqrt(nw2);
     ctl->beta[jj] = bt;
-    if (!(bt > ctl->eta_bd * sqrt(ctl->normu2))) {   // invariant subspace (or zero vector)
+    if (!(nw2 > ctl->eta_bd * ctl->eta_bd * ctl->normu2)) {   // invariant subspace (or zero vector)
         ctl->m_eff = jj + 1;
         ctl->n_bd += 1;
     } else {
@@ -342,44 +342,40 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
     __syncthreads();
     double2 *fin = red;
     if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, nv, MODE == 0)) return;
-    if (tid != 0) return;
+    // Scalar epilogue, one lane of warp 0 per vector.  GB300 issues one FP64 warp instruction per
+    // about 77 cycles and SM sub-partition whatever its active lanes, so a loop over the vectors
+    // in one thread cost 4 us at j = 30.
+    if (tid >= 32) return;
+    const bool in = tid <= jj;
+    const double s = in ? ctl->sigma[tid] : 0.0;
+    const double2 c = make_double2(fin[tid].x * s, fin[tid].y * s);   // <v_i, y>
+    const double2 cs = make_double2(c.x * s, c.y * s);
+    const double c2 = warp_sum(c.x * c.x + c.y * c.y);
     if (MODE == 0) {
-        for (int i = 0; i <= jj; ++i) {
-            const double s = ctl->sigma[i];
-            const double2 c = make_double2(fin[i].x * s, fin[i].y * s);   // <v_i, u>
-            ctl->coefA[i] = make_double2(c.x * s, c.y * s);
-            if (i == jj) ctl->alpha[jj] = c.x;
-        }
+        if (in) ctl->coefA[tid] = cs;
+        if (tid == jj) ctl->alpha[jj] = c.x;
+        if (tid != 0) return;
+        ctl->c2 = c2;
         ctl->normu2 = fin[SLOT_NRM].x;
         ctl->n_hv += 1;
-        ctl->vec_passes += (double)(jj + 4);
-        ctl->vp_kind[KIND_PASSA] += (double)(jj + 2);   // u and v_0 .. v_j
-        ctl->vp_kind[KIND_HV] += 2.0;                  // the H.v: v_j read, u written
+        ctl->vec_passes += jj + 4;
+        ctl->vp_kind[KIND_PASSA] += jj + 2;   // u and v_0 .. v_j
+        ctl->vp_kind[KIND_HV] += 2;          // the H.v: v_j read, u written
         ctl->counter = 0;
         return;
     }
     const double nw2 = ctl->wnorm2;
-    double nd2 = 0.0;
-    for (int i = 0; i <= jj; ++i) {
-        const double s = ctl->sigma[i];
-        nd2 += (fin[i].x * fin[i].x + fin[i].y * fin[i].y) * s * s;
-    }
-    if (nw2 > 0.0) ctl->max_orth = fmax(ctl->max_orth, sqrt(nd2 / nw2));
+    const bool sub = nw2 > 0.0 && sqrt(c2) > ctl->eta_corr * sqrt(nw2);
+    if (sub && in) ctl->coefC[tid] = cs;
+    if (sub && tid == jj) ctl->alpha[jj] += c.x;
+    if (tid != 0) return;
+    if (nw2 > 0.0) ctl->max_orth = fmax(ctl->max_orth, sqrt(c2 / nw2));
     ctl->n_c1 += 1;
-    ctl->vec_passes += (double)(jj + 2);
-    ctl->vp_kind[KIND_PASSC] += (double)(jj + 2);
+    ctl->vec_passes += jj + 2;
+    ctl->vp_kind[KIND_PASSC] += jj + 2;
     ctl->corr = 0;
-    if (nw2 > 0.0 && sqrt(nd2) > ctl->eta_corr * sqrt(nw2)) {
-        ctl->corr2 = 1;
-        for (int i = 0; i <= jj; ++i) {
-            const double s = ctl->sigma[i];
-            ctl->coefC[i] = make_double2(fin[i].x * s * s, fin[i].y * s * s);
-        }
-        ctl->alpha[jj] += fin[jj].x * ctl->sigma[jj];
-    } else {
-        ctl->corr2 = 0;
-        finalize_beta(ctl, jj, nw2, ctl->wg);
-    }
+    ctl->corr2 = sub ? 1 : 0;
+    if (!sub) finalize_beta(ctl, jj, nw2, ctl->wg);
     ctl->counter = 0;
 }
 
@@ -468,8 +464,8 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     const double nw2 = fin[SLOT_NRM].x;
     const double2 gdot = fin[SLOT_G];
     if (MODE == 0) {
-        ctl->vec_passes += (double)(jj + 3) + (a.G ? 1.0 : 0.0);
-        ctl->vp_kind[KIND_PASSB] += (double)(jj + 3) + (a.G ? 1.0 : 0.0);
+        ctl->vec_passes += jj + 3 + (a.G ? 1 : 0);
+        ctl->vp_kind[KIND_PASSB] += jj + 3 + (a.G ? 1 : 0);
         // One classical Gram-Schmidt pass is enough unless the projection cancelled most of
         // u (||w|| < eta ||u||, the Daniel-Gragg-Kaufman-Stewart test), or the lengths show a
         // loss of orthogonality: with c = V^H u and G = V^H V = I + E, ||w||^2 = ||u||^2 -
@@ -477,14 +473,11 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
         // ||E c|| / ||w|| = ||V^H w|| / ||w|| (Pythagoras test).  Either way the dots of w
         // with every previous vector are taken (pass C1) and subtracted if needed (C2).
         // With orth_check set the dots are taken after every update.
-        double c2 = 0.0;
-        for (int i = 0; i <= jj; ++i) {
-            const double s = ctl->sigma[i];
-            c2 += (ctl->coefA[i].x * ctl->coefA[i].x + ctl->coefA[i].y * ctl->coefA[i].y) / (s * s);
-        }
-        // (the second term is the noise floor of the lengths of vectors in storage precision)
-        const double pyth = fabs(nw2 - (ctl->normu2 - c2));
-        const bool lost = pyth > ctl->eta_corr * sqrt(c2 * nw2) + 0.1 * ctl->eta_bd * ctl->normu2;
+        const double c2 = ctl->c2;
+        // (floor: the noise of the lengths of vectors in storage precision; the square root is
+        // taken only above it)
+        const double pyth = fabs(nw2 - (ctl->normu2 - c2)), floor = 0.1 * ctl->eta_bd * ctl->normu2;
+        const bool lost = pyth > floor && pyth > ctl->eta_corr * sqrt(c2 * nw2) + floor;
         if (ctl->verify || nw2 < ctl->eta_cancel * ctl->eta_cancel * ctl->normu2 || lost) {
             ctl->corr = 1;
             ctl->wnorm2 = nw2;
@@ -498,8 +491,8 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
         if (COND && a.use_cond) cudaGraphSetConditional(a.cond, ctl->corr ? 1u : 0u);
     } else if (MODE == 1) {
         ctl->n_corr += 1;
-        ctl->vec_passes += (double)(jj + 3) + (a.G ? 1.0 : 0.0);
-        ctl->vp_kind[KIND_PASSC] += (double)(jj + 3) + (a.G ? 1.0 : 0.0);
+        ctl->vec_passes += jj + 3 + (a.G ? 1 : 0);
+        ctl->vp_kind[KIND_PASSC] += jj + 3 + (a.G ? 1 : 0);
         ctl->corr2 = 0;
         finalize_beta(ctl, jj, nw2, gdot);
     } else {
@@ -513,8 +506,8 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
             ctl->g[0] = (MODE == 3) ? make_double2(b0, 0.0)
                                     : make_double2(gdot.x / b0, gdot.y / b0);
         }
-        ctl->vec_passes += (double)(nvec + 1) + ((a.G && MODE == 2) ? 1.0 : 0.0);
-        if (MODE == 2) ctl->vp_kind[KIND_COMBINE] += (double)(nvec + 1) + (a.G ? 1.0 : 0.0);
+        ctl->vec_passes += nvec + 1 + ((a.G && MODE == 2) ? 1 : 0);
+        if (MODE == 2) ctl->vp_kind[KIND_COMBINE] += nvec + 1 + (a.G ? 1 : 0);
         ctl->m_eff = ctl->m;
         ctl->corr = 0;
         ctl->corr2 = 0;

@@ -128,8 +128,8 @@ enum { KIND_PASSA = 0, KIND_PASSB = 1, KIND_PASSC = 2, KIND_EXP = 3, KIND_COMBIN
 struct KryHdrB {   // shared scalars (copied to the host when polling)
     double t_now, t_end, tol, t_next;
     double eta_corr, eta_bd;
-    double err_sum, max_orth, vec_passes;
-    double vp_kind[NKIND];
+    double err_sum, max_orth;
+    long long vec_passes, vp_kind[NKIND];   // vector passes, in all and by kernel kind
     unsigned long long n_hv, n_steps, n_corr, n_bd;
     int K, m, m_run, corr_any, finishing, done, err;
     int n_times, next_out, next_out_new, r0;
@@ -199,11 +199,13 @@ struct KryCtl {
     double2 coefY[MMAX + 1];   // combine coefficients -beta0 y_i sigma_i
     double2 g[MMAX + 2];       // readout <psi0, v_i>
     double normu2;             // ||H v_j||^2 of the last pass A
+    double c2;                 // ||V^H H v_j||^2 of the last pass A (Pythagoras test of pass B)
     double beta0;              // ||psi|| at the start of the Krylov step
     double t_now, t_end, tol, tau_prev;
     double eta_corr, eta_bd;   // second-pass and breakdown thresholds (relative)
-    double err_sum, max_orth, vec_passes;
-    double vp_kind[NKIND];     // vector passes by kernel kind (KIND_*)
+    double err_sum, max_orth;
+    long long vec_passes;      // vector passes (counters are integers: an FP64 add costs the
+    long long vp_kind[NKIND];  // epilogues as much as 77 issue slots); by kernel kind (KIND_*)
     long long n_hv, n_steps, n_corr, n_bd;
     int m, m_eff, corr, finishing, done, err;
     int n_times, next_out, r0;

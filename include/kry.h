@@ -267,6 +267,9 @@ int kry_autotune(kry_ham H, int dtype, int m, uint64_t probe_state, double t_pro
  * Lanczos vector is orthogonalised against all previous ones by one classical Gram-Schmidt
  * pass (Sec. 2: Arnoldi orthogonalises each new vector against the whole basis); a second
  * pass is made only when that pass cancelled most of the vector (||w|| < 0.1 ||H v_j||).
+ * H is real and symmetric, so the process runs in the real inner product Re <a, b> of the
+ * vectors' real and imaginary parts: the same alpha_j and beta_j, and Im <v_i, v_j> = 0 holds
+ * by itself in exact arithmetic and does not enter the results' errors; <.,.> below means it.
  * With on = 1 the dots of every new vector with all previous ones are measured after each
  * pass (kry_stats.max_orth_loss) and subtracted when they exceed eta ||w||, with eta about
  * 1e4 units of roundoff of the vector storage: 1e-12 (KRY_C128), 3e-11 (KRY_C128E), 1e-5

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(NTHR) k_hv_bc(EvArgsB<V> a, int jj)
     }
 }
 
-// Part 2: the dots <W_i[:, k], U[:, k]>, i <= j, and ||U[:, k]||^2 of every realisation.
+// Part 2: the dots Re <W_i[:, k], U[:, k]>, i <= j, and ||U[:, k]||^2 of every realisation.
 // Thread (k, g) takes column k and the vectors i = g, g + NG, ...; the rows of U of a tile
 // are loaded once and serve all of them.
 template <class V, int KQ>
@@ -225,24 +225,21 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots_b(EvArgsB<V> a, int jj)
 {
     KryCtlB *ctl = a.ctl;
     if (ctl->hd.done || jj >= ctl->hd.m_run) return;
-    // vectors i = g + NG q < MMAX (j <= MMAX - 1); complex64 accumulates with the packed
-    // float-float pairs while they fit the registers (K <= 64), else with the scalar pairs;
-    // complex128 in FP64
+    // vectors i = g + NG q < MMAX (j <= MMAX - 1)
     constexpr int Kp = 32 * KQ, NG = NTHR / Kp, QD = (MMAX + NG - 1) / NG;
-    using Acc = typename std::conditional<sizeof(V) == sizeof(float2) && KQ <= 2, DotAccF2, DotAcc<V>>::type;
-    constexpr int RH = TROWS / 2;   // rows per half tile
+    // rows in registers at a time (16-byte elements with the 16 accumulators of K > 64: four)
+    constexpr int RH = sizeof(V) == 16 && KQ == 4 ? TROWS / 4 : TROWS / 2;
     const int tid = threadIdx.x, K = a.K;
     const int k = tid % Kp, g = tid / Kp;
     const uint32_t D = a.b.D, ntiles = (D + TROWS - 1) / TROWS;
-    Acc acc[QD];
-    DotAcc<V> nrm;
+    RealAcc<V> acc[QD], nrm;
     if (k < K) {
         for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
             const uint32_t r0 = tile * TROWS;
-            // rows past D are skipped by one test per half tile, not per element
+            // rows past D are skipped by one test per RH rows, not per element
             // (a select of FP64 values occupies the FP64 pipe)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < TROWS / RH; ++h) {
                 const uint32_t rh = r0 + h * RH;
                 const int nr = rh >= D ? 0 : (int)min((uint32_t)RH, D - rh);
                 V uu[RH];
@@ -256,9 +253,12 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots_b(EvArgsB<V> a, int jj)
                     for (int rr = 0; rr < RH; ++rr)
                         if (rr < nr) uu[rr] = ldg(a.U + (size_t)(rh + rr) * K + k);
                 }
+                typename RealAcc<V>::Pre up[RH];
+#pragma unroll
+                for (int rr = 0; rr < RH; ++rr) up[rr] = RealAcc<V>::pre(uu[rr]);
                 if (g == 0) {
 #pragma unroll
-                    for (int rr = 0; rr < RH; ++rr) nrm.add_norm(uu[rr]);
+                    for (int rr = 0; rr < RH; ++rr) nrm.add(uu[rr], up[rr]);
                 }
                 // rows rh .. rh + RH of vector iv, column k (zero past D)
                 auto load = [&](int iv, V *dst) {
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots_b(EvArgsB<V> a, int jj)
                         V vv[RH];
                         load(iv, vv);
 #pragma unroll
-                        for (int rr = 0; rr < RH; ++rr) acc[q].add(vv[rr], uu[rr]);
+                        for (int rr = 0; rr < RH; ++rr) acc[q].add(vv[rr], up[rr]);
                     }
                 }
             }
@@ -295,9 +295,9 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots_b(EvArgsB<V> a, int jj)
 #pragma unroll
     for (int q = 0; q < QD; ++q) {
         const int iv = g + NG * q;
-        if (iv <= jj) pc[(size_t)iv * Kp + k] = acc[q].value();
+        if (iv <= jj) pc[(size_t)iv * Kp + k] = make_double2(to_double(acc[q].sum()), 0.0);
     }
-    if (g == 0) pc[(size_t)SLOT_NRM * Kp + k] = make_double2(nrm.value().x, 0.0);
+    if (g == 0) pc[(size_t)SLOT_NRM * Kp + k] = make_double2(to_double(nrm.sum()), 0.0);
 }
 
 
@@ -317,25 +317,27 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
     constexpr int Kp = 32 * KQ, NG = NTHR / Kp, QD = (MMAX + NG) / NG;
     const int nvec = (MODE == 2) ? ctl->hd.m_run : ((MODE == 3 || MODE == 4) ? 0 : jj + 1);
     extern __shared__ __align__(16) unsigned char smem[];
-    using Coef = typename Arith<V>::Coef;
-    static_assert(sizeof(Coef) == sizeof(V), "coefficient slots have the element size");
+    // modes 0 and 1 subtract real multiples (RealAcc), the combine takes complex ones
+    constexpr bool RE = MODE <= 1;
+    using Lin = typename std::conditional<RE, RealLin<V>, CplxLin<V>>::type;
+    using Coef = typename Lin::RCoef;
+    static_assert(sizeof(Coef) <= sizeof(V), "coefficient slots have the element size");
     Coef *coef = (Coef *)smem;                    // [MMAX+1][Kp]
-    V *wtile = (V *)(coef + (MMAX + 1) * Kp);     // [TROWS][Kp]
+    V *wtile = (V *)smem + (MMAX + 1) * Kp;       // [TROWS][Kp]
     double2 *nred = (double2 *)(wtile + TROWS * Kp);   // [NG][Kp] (norm), then [NG][Kp] (G)
     const int tid = threadIdx.x, K = a.K;
     for (int e = tid; e < nvec * Kp; e += NTHR) {
         const int i = e / Kp, k = e % Kp;
-        double2 c = make_double2(0.0, 0.0);
-        if (k < K) c = (MODE == 0) ? ctl->coefA[i][k] : (MODE == 1) ? ctl->coefC[i][k] : ctl->coefY[i][k];
-        coef[i * Kp + k] = coef_from<V>(c);
+        if constexpr (RE) coef[i * Kp + k] = Lin::coef(k >= K ? 0.0 : MODE == 0 ? ctl->coefA[i][k] : ctl->coefC[i][k]);
+        else coef[i * Kp + k] = Lin::coef(k < K ? ctl->coefY[i][k] : make_double2(0.0, 0.0));
     }
     __syncthreads();
     V *out = (MODE == 2 || MODE == 3) ? a.W : a.W + (size_t)(jj + 1) * a.ldW;
     const V *src = (MODE == 0) ? a.U : (MODE == 1 || MODE == 4) ? out : (MODE == 3) ? a.G : nullptr;
     const uint32_t D = a.b.D, ntiles = (D + TROWS - 1) / TROWS;
     const int k = tid % Kp, g = tid / Kp;
-    DotAcc<V> acc[QD];
-    DotAcc<V> nrm, gacc;
+    RealAcc<V> acc[QD], nrm;
+    DotAcc<V> gacc;
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const uint32_t r0 = tile * TROWS;
         for (int rr = g; rr < TROWS; rr += NG) {
@@ -344,17 +346,17 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
                 const size_t idx = (size_t)(r0 + rr) * K + k;
                 if (src) w = src[idx];
                 if (MODE != 4) {
-                    typename Arith<V>::Lin wl = lin_init(w);
+                    Lin wl(w);
                     if (MODE == 2) {
 #pragma unroll 8
-                        for (int i = 0; i < nvec; ++i) lin_fms(wl, coef[i * Kp + k], a.W[(size_t)i * a.ldW + idx]);
+                        for (int i = 0; i < nvec; ++i) wl.fms(coef[i * Kp + k], a.W[(size_t)i * a.ldW + idx]);
                     } else {
 #pragma unroll 8
-                        for (int i = 0; i < nvec; ++i) lin_fms(wl, coef[i * Kp + k], ldg(a.W + (size_t)i * a.ldW + idx));
+                        for (int i = 0; i < nvec; ++i) wl.fms(coef[i * Kp + k], ldg(a.W + (size_t)i * a.ldW + idx));
                     }
-                    w = (MODE == 3) ? w : lin_out(wl);
+                    w = (MODE == 3) ? w : wl.out();
                     out[idx] = w;
-                    nrm.add_norm(w);
+                    nrm.add(w, RealAcc<V>::pre(w));
                     if (a.G && MODE != 3) gacc.add(ldg(a.G + idx), w);
                 }
             }
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
                         for (int rr = 0; rr < TROWS; ++rr)
                             vv[rr] = (r0 + rr < D) ? ldg(wi + (size_t)rr * K) : VT<V>::zero();
 #pragma unroll
-                        for (int rr = 0; rr < TROWS; ++rr) acc[q].add(vv[rr], wtile[rr * Kp + k]);
+                        for (int rr = 0; rr < TROWS; ++rr) acc[q].add(vv[rr], RealAcc<V>::pre(wtile[rr * Kp + k]));
                         acc[q].renorm();
                     }
                 }
@@ -388,11 +390,11 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
 #pragma unroll
         for (int q = 0; q < QD; ++q) {
             const int iv = g + NG * q;
-            if (iv <= jj) pc[(size_t)iv * Kp + k] = acc[q].value();
+            if (iv <= jj) pc[(size_t)iv * Kp + k] = make_double2(to_double(acc[q].sum()), 0.0);
         }
         return;
     }
-    nred[g * Kp + k] = nrm.value();
+    nred[g * Kp + k] = make_double2(to_double(nrm.sum()), 0.0);
     nred[(NG + g) * Kp + k] = gacc.value();
     __syncthreads();
     for (int kk = tid; kk < Kp; kk += NTHR) {
@@ -429,13 +431,14 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
     for (int q = warp; q < ns; q += 8) {
         const int slot = q < nd ? q : q == nd ? SLOT_NRM : SLOT_G;
         double2 s = make_double2(0.0, 0.0);
+        const bool cplx = slot == SLOT_G;   // the others are real
 #pragma unroll 4
         for (int c = lane; c < grid; c += 32) {
             const double2 v = __ldg(part + ((size_t)c * PSB + slot) * Kp + k);
             s.x += v.x;
-            s.y += v.y;
+            if (cplx) s.y += v.y;
         }
-        s = warp_sum(s);
+        s = cplx ? warp_sum(s) : make_double2(warp_sum(s.x), 0.0);
         if (lane == 0) fin[slot] = s;
     }
     __syncthreads();
@@ -443,12 +446,12 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
     const double nw2 = (mode == 3) ? ctl->wnorm2[k] : fin[SLOT_NRM].x;
     const double2 gdot = (mode == 3) ? ctl->wg[k]
                                      : ((general && mode != 0) ? fin[SLOT_G] : make_double2(0.0, 0.0));
-    // lane i: <v_i, y> = c, c sigma_i (modes 0 and 3)
-    double2 c = make_double2(0.0, 0.0), cs = c;
+    // lane i: Re <v_i, y> = c, c sigma_i (modes 0 and 3)
+    double c = 0.0, cs = 0.0;
     if (lane < nd) {
         const double s = ctl->sigma[lane][k];
-        c = make_double2(fin[lane].x * s, fin[lane].y * s);
-        cs = make_double2(c.x * s, c.y * s);
+        c = fin[lane].x * s;
+        cs = c * s;
     }
     auto finalize = [&](double w2, double2 gd) {
         const double bt = sqrt(w2);
@@ -474,15 +477,15 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         }
         // (invariant subspace already reached: this realisation's next vectors stay zero)
         const bool run = jj < ctl->m_eff[k];
-        if (lane <= jj) ctl->coefA[lane][k] = run ? cs : make_double2(0.0, 0.0);
-        if (run && lane == jj) ctl->alpha[jj][k] = c.x;
+        if (lane <= jj) ctl->coefA[lane][k] = run ? cs : 0.0;
+        if (run && lane == jj) ctl->alpha[jj][k] = c;
         if (run && lane == 0) ctl->normu2[k] = nw2;
     } else if (mode == 1) {
         if (k == 0 && lane == 0) {
             H.vec_passes += jj + 3 + (general ? 1 : 0);
             H.vp_kind[KIND_PASSB] += jj + 3 + (general ? 1 : 0);
         }
-        if (lane <= jj) ctl->coefC[lane][k] = make_double2(0.0, 0.0);
+        if (lane <= jj) ctl->coefC[lane][k] = 0.0;
         if (lane != 0) return;
         ctl->corr[k] = 0;
         ctl->dots[k] = 0;
@@ -504,10 +507,10 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
             H.vp_kind[KIND_PASSC] += jj + 2;
         }
         if (!ctl->dots[k] || jj >= ctl->m_eff[k]) return;
-        const double nd2 = warp_sum(c.x * c.x + c.y * c.y);
+        const double nd2 = warp_sum(c * c);
         const bool sub = nw2 > 0.0 && sqrt(nd2) > H.eta_corr * sqrt(nw2);
         if (sub && lane <= jj) ctl->coefC[lane][k] = cs;
-        if (sub && lane == jj) ctl->alpha[jj][k] += c.x;
+        if (sub && lane == jj) ctl->alpha[jj][k] += c;
         if (lane != 0) return;
         if (nw2 > 0.0) ctl->orth[k] = fmax(ctl->orth[k], sqrt(nd2 / nw2));
         if (sub) {

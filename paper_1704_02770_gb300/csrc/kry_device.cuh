@@ -95,34 +95,27 @@ template <> struct VT<ffc> {
     __device__ __forceinline__ static ffc from(double2 c)
     {
         const float2 a = dsplit(c.x), b = dsplit(c.y);
-        return ffc{a.x, a.y, b.x, b.y};
+        return ffc{a.x, b.x, a.y, b.y};
     }
 };
 __device__ __forceinline__ ffc ldg(const ffc *p)
 {
     const float4 v = __ldg((const float4 *)p);
-    return ffc{v.x, v.y, v.z, v.w};
+    return ffc{v.x, v.y, v.z, v.w};   // (xh, yh, xl, yl)
 }
 __device__ __forceinline__ float2 ldg(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ double2 ldg(const double2 *p) { return __ldg(p); }
 
-// Per element type: the accumulator of a neighbour sum (HvSum), of a linear combination (Lin),
-// a coefficient as kept in shared memory (Coef), a right-hand vector element prepared for
-// several dot products (Pre).  For complex64 and complex128 these are the element itself.
+// Per element type, the accumulator of a neighbour sum: the element itself, or two float-float
+// numbers.
 struct FF4 {   // two float-float numbers (real, imaginary)
     float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
 };
 template <class V> struct Arith {
     using HvSum = V;
-    using Lin = V;
-    using Coef = V;
-    using Pre = V;
 };
 template <> struct Arith<ffc> {
     using HvSum = FF4;
-    using Lin = FF4;
-    using Coef = float4;   // (re hi, re lo, im hi, im lo)
-    using Pre = ffc;
 };
 
 __device__ __forceinline__ double2 operator+(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
@@ -167,43 +160,8 @@ __device__ __forceinline__ ffc hv_finish(double sd, ffc x, double shj, const FF4
     ff_mac(h.x, h.y, acc.si, acc.ci, si, ci);
     ff_renorm(sr, cr);
     ff_renorm(si, ci);
-    return ffc{sr, cr, si, ci};
+    return ffc{sr, si, cr, ci};
 }
-// linear combinations: w = src - sum_i c_i x_i
-template <class V> __device__ __forceinline__ V lin_init(V src) { return src; }
-template <class V> __device__ __forceinline__ V lin_out(V w) { return w; }
-template <class V> __device__ __forceinline__ typename Arith<V>::Coef coef_from(double2 c) { return VT<V>::from(c); }
-__device__ __forceinline__ FF4 lin_init(ffc src)
-{
-    FF4 w;
-    w.sr = src.xh; w.cr = src.xl; w.si = src.yh; w.ci = src.yl;
-    return w;
-}
-__device__ __forceinline__ ffc lin_out(FF4 w)
-{
-    ff_renorm(w.sr, w.cr);
-    ff_renorm(w.si, w.ci);
-    return ffc{w.sr, w.cr, w.si, w.ci};
-}
-template <> __device__ __forceinline__ float4 coef_from<ffc>(double2 c)
-{
-    const float2 a = dsplit(c.x), b = dsplit(c.y);
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ double2 cfms(double2 c, double2 v, double2 w);
-__device__ __forceinline__ float2 cfms(float2 c, float2 v, float2 w);
-template <class V> __device__ __forceinline__ void lin_fms(V &w, V c, V x) { w = cfms(c, x, w); }
-__device__ __forceinline__ void lin_fms(FF4 &w, float4 c, ffc x)
-{
-    // w -= c x: re -= cr xr - ci xi, im -= cr xi + ci xr
-    ff_mac(-c.x, -c.y, x.xh, x.xl, w.sr, w.cr);
-    ff_mac(c.z, c.w, x.yh, x.yl, w.sr, w.cr);
-    ff_mac(-c.x, -c.y, x.yh, x.yl, w.si, w.ci);
-    ff_mac(-c.z, -c.w, x.xh, x.xl, w.si, w.ci);
-}
-// a right-hand vector element prepared for several dot products
-template <class V> __device__ __forceinline__ V pre(V u) { return u; }
-
 __device__ __forceinline__ double2 scale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 // s a for a float-float element: the product of the split scale with each component
 __device__ __forceinline__ ffc scale(ffc a, double s)
@@ -214,7 +172,7 @@ __device__ __forceinline__ ffc scale(ffc a, double s)
     ff_mac(f.x, f.y, a.yh, a.yl, si, ci);
     ff_renorm(sr, cr);
     ff_renorm(si, ci);
-    return ffc{sr, cr, si, ci};
+    return ffc{sr, si, cr, ci};
 }
 __device__ __forceinline__ float2 scale(float2 a, double s) { return make_float2(a.x * (float)s, a.y * (float)s); }
 __device__ __forceinline__ float2 scale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
@@ -232,7 +190,7 @@ __device__ __forceinline__ void pdl_begin()
 }
 
 // ---------------------------------------------------------------- dot accumulators
-// sum conj(a) b.  complex128: FP64 fused multiply-adds.  complex64 and float-float: every
+// sum conj(a) b, complex (the readout <psi0, w>).  complex128: FP64 fused multiply-adds.  complex64 and float-float: every
 // product is split exactly (p = a*b rounded, e = fma(a, b, -p)) and summed with Knuth's
 // TwoSum into a float pair (s, c): the rounding errors of s are kept exactly, and c gathers
 // them in plain float.  c is folded back into s (renorm, a TwoSum) after every few terms --
@@ -249,7 +207,6 @@ struct DotAccD {
         re = fma(a.x, b.x, re); re = fma(a.y, b.y, re);
         im = fma(a.x, b.y, im); im = fma(-a.y, b.x, im);
     }
-    __device__ __forceinline__ void add_norm(double2 a) { re = fma(a.x, a.x, re); re = fma(a.y, a.y, re); }
     __device__ __forceinline__ void renorm() {}
     __device__ __forceinline__ double2 value() const { return make_double2(re, im); }
     // the sum over the warp (valid in every lane)
@@ -301,8 +258,6 @@ struct DotAccF {
         exact_fma(a.x, b.x, sr, cr); exact_fma(a.y, b.y, sr, cr);
         exact_fma(a.x, b.y, si, ci); exact_fma(-a.y, b.x, si, ci);
     }
-    // |a|^2 (the imaginary part of conj(a) a is zero and is not accumulated)
-    __device__ __forceinline__ void add_norm(float2 a) { exact_fma(a.x, a.x, sr, cr); exact_fma(a.y, a.y, sr, cr); }
     __device__ __forceinline__ void renorm()
     {
         ff_renorm(sr, cr);
@@ -320,80 +275,6 @@ struct DotAccF {
         return make_double2((double)a + (double)b, (double)c + (double)d);
     }
 };
-// complex64 dots with packed FP32x2 arithmetic (sm_100 and later): the same error-free
-// products and TwoSum as DotAccF, two components per instruction.  With b_x2 = (bx, bx)
-// and b_y2 = (by, by), the pair products a*b_x2 = (ax bx, ay bx) and a*b_y2 = (ax by, ay by)
-// are summed into two float-float pairs; conj(a) b = (ax bx + ay by, ax by - ay bx) is formed
-// in FP64 at the end.
-__device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ void ff_pair_add(float2 &s, float2 &c, float2 a, float2 b)
-{
-    const float2 p = __fmul2_rn(a, b);
-    const float2 e = __ffma2_rn(a, b, make_float2(-p.x, -p.y));   // a*b - p, exact
-    const float2 t = __fadd2_rn(s, p);
-    const float2 z = fsub2(t, s);
-    const float2 err = __fadd2_rn(fsub2(s, fsub2(t, z)), fsub2(p, z));
-    s = t;
-    c = __fadd2_rn(c, __fadd2_rn(err, e));
-}
-// (s, c) renormalised by TwoSum, two float-float lanes per instruction
-__device__ __forceinline__ void ff_renorm2(float2 &s, float2 &c)
-{
-    const float2 t = __fadd2_rn(s, c);
-    const float2 z = fsub2(t, s);
-    c = __fadd2_rn(fsub2(s, fsub2(t, z)), fsub2(c, z));
-    s = t;
-}
-struct DotAccF2 {
-    float2 s1 = make_float2(0.f, 0.f), c1 = make_float2(0.f, 0.f);
-    float2 s2 = make_float2(0.f, 0.f), c2 = make_float2(0.f, 0.f);
-    // b4 = (bx, bx, by, by)
-    __device__ __forceinline__ void add(float2 a, float4 b4)
-    {
-        ff_pair_add(s1, c1, a, make_float2(b4.x, b4.y));
-        ff_pair_add(s2, c2, a, make_float2(b4.z, b4.w));
-    }
-    __device__ __forceinline__ void add2(float2 a0, float4 b0, float2 a1, float4 b1)
-    {
-        add(a0, b0);
-        add(a1, b1);
-    }
-    // b = (bx, by), broadcast per use
-    __device__ __forceinline__ void add(float2 a, float2 b)
-    {
-        ff_pair_add(s1, c1, a, make_float2(b.x, b.x));
-        ff_pair_add(s2, c2, a, make_float2(b.y, b.y));
-    }
-    __device__ __forceinline__ void add2(float2 a0, float2 b0, float2 a1, float2 b1)
-    {
-        add(a0, b0);
-        add(a1, b1);
-    }
-    __device__ __forceinline__ void renorm()
-    {
-        ff_renorm2(s1, c1);
-        ff_renorm2(s2, c2);
-    }
-    __device__ __forceinline__ double2 value() const
-    {
-        const double axbx = (double)s1.x + (double)c1.x, aybx = (double)s1.y + (double)c1.y;
-        const double axby = (double)s2.x + (double)c2.x, ayby = (double)s2.y + (double)c2.y;
-        return make_double2(axbx + ayby, axby - aybx);
-    }
-    // the sum over the warp, reduced in FP32 float-float arithmetic; converted to FP64 once
-    __device__ __forceinline__ double2 warp_value() const
-    {
-        float a = s1.x, b = c1.x, c = s1.y, d = c1.y, e = s2.x, f = c2.x, g = s2.y, h = c2.y;
-        ff_warp_sum(a, b);
-        ff_warp_sum(c, d);
-        ff_warp_sum(e, f);
-        ff_warp_sum(g, h);
-        const double axbx = (double)a + (double)b, aybx = (double)c + (double)d;
-        const double axby = (double)e + (double)f, ayby = (double)g + (double)h;
-        return make_double2(axbx + ayby, axby - aybx);
-    }
-};
-
 // sum conj(a) b for float-float vectors (ffc)
 struct DotAccFF {
     float sr = 0.f, cr = 0.f, si = 0.f, ci = 0.f;
@@ -403,11 +284,6 @@ struct DotAccFF {
         ff_mac(a.yh, a.yl, b.yh, b.yl, sr, cr);
         ff_mac(a.xh, a.xl, b.yh, b.yl, si, ci);
         ff_mac(-a.yh, -a.yl, b.xh, b.xl, si, ci);
-    }
-    __device__ __forceinline__ void add_norm(ffc a)
-    {
-        ff_mac(a.xh, a.xl, a.xh, a.xl, sr, cr);
-        ff_mac(a.yh, a.yl, a.yh, a.yl, sr, cr);
     }
     __device__ __forceinline__ void renorm()
     {
@@ -445,6 +321,208 @@ __device__ __forceinline__ double warp_sum(double v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+
+// ---------------------------------------------------------------- real inner products
+// The Hamiltonian is real and symmetric, so the Lanczos process of a complex vector is that of
+// H (+) H on its real and imaginary parts: a vector of 2D reals with the inner product
+// Re <a, b>.  Its coefficients alpha_j and beta_j are the same, Re <v_i, v_j> = delta_ij is the
+// orthogonality it needs, and Im <v_i, v_j> = Im <psi, p_i(H) p_j(H) psi> = 0 by itself, since
+// p_i p_j (H) is Hermitian.  Every v_j is a real polynomial of H applied to psi, the Krylov
+// approximation of exp(-i tau (H (+) H)) maps to that of exp(-i tau H) by (x, y) -> x + i y,
+// and an error of the former grows by at most sqrt(2) under that map.  Full reorthogonalisation
+// in this inner product takes half the multiply-adds of the complex one in the dots and in the
+// updates, where GB300 is bound by them (FP64 by its 1/64 rate, float-float by its 10 to 12
+// instructions per product).  The loss of Re-orthogonality and the errors of psi are those of the
+// complex form (tests/test_real_lanczos.py emulates both on the CPU).
+
+struct FF {   // a float-float number
+    float s, c;
+};
+__device__ __forceinline__ double add2(double a, double b) { return a + b; }
+__device__ __forceinline__ FF add2(FF a, FF b)
+{
+    ff_combine(a.s, a.c, b.s, b.c);
+    return a;
+}
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ FF shfl_xor(FF v, int o)
+{
+    return FF{__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o)};
+}
+__device__ __forceinline__ double pick(bool p, double a, double b)
+{
+    // (as integers: a select of doubles occupies the FP64 pipe)
+    return __longlong_as_double(p ? __double_as_longlong(a) : __double_as_longlong(b));
+}
+__device__ __forceinline__ FF pick(bool p, FF a, FF b) { return FF{p ? a.s : b.s, p ? a.c : b.c}; }
+
+// Totals over the warp of N values per lane (N a power of two up to 32), N - 1 + log2(32 / N) adds
+// per lane instead of 5 N: lane l returns the total of value l / (32 / N).
+template <int N, class T>
+__device__ __forceinline__ T warp_totals(T *v)
+{
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const T send = pick(up, v[i], v[i + n]), keep = pick(up, v[i + n], v[i]);
+            v[i] = add2(keep, shfl_xor(send, o));
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) v[0] = add2(v[0], shfl_xor(v[0], o));
+    return v[0];
+}
+__device__ __forceinline__ double to_double(double v) { return v; }
+__device__ __forceinline__ double to_double(FF v) { return (double)v.s + (double)v.c; }
+
+// Accumulators of sum Re(conj(a) b), with b prepared once for several vectors (Pre).
+// complex128: two FP64 multiply-adds per element.
+template <class V> struct RealAcc;
+template <> struct RealAcc<double2> {
+    using Pre = double2;
+    using Sum = double;
+    double s = 0.0;
+    __device__ __forceinline__ static Pre pre(double2 b) { return b; }
+    __device__ __forceinline__ void add(double2 a, Pre b) { s = fma(a.x, b.x, s); s = fma(a.y, b.y, s); }
+    __device__ __forceinline__ void renorm() {}
+    __device__ __forceinline__ Sum sum() const { return s; }
+};
+__device__ __forceinline__ float2 fsub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+// s + c += -n + e with n = -(a product rounded) and e its exact remainder: TwoSum into s, the
+// errors into c, two float-float lanes per packed FP32x2 instruction
+__device__ __forceinline__ void ff2_add_neg(float2 &s, float2 &c, float2 n, float2 e)
+{
+    const float2 t = fsub2(s, n);
+    const float2 z = fsub2(t, s);
+    const float2 err = fsub2(fsub2(s, fsub2(t, z)), __fadd2_rn(n, z));
+    s = t;
+    c = __fadd2_rn(c, __fadd2_rn(err, e));
+}
+// (s, c) renormalised by TwoSum, two float-float lanes per instruction
+__device__ __forceinline__ void ff_renorm2(float2 &s, float2 &c)
+{
+    const float2 t = __fadd2_rn(s, c);
+    const float2 z = fsub2(t, s);
+    c = __fadd2_rn(fsub2(s, fsub2(t, z)), fsub2(c, z));
+    s = t;
+}
+// complex64 and float-float: the lanes of a packed pair sum the products of the real and of the
+// imaginary parts, error-free products and TwoSum as in DotAccF; Pre keeps -b too, so that no
+// instruction is spent on a sign.
+struct RealAccPair {
+    using Sum = FF;
+    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
+    __device__ __forceinline__ void renorm() { ff_renorm2(s, c); }
+    __device__ __forceinline__ Sum sum() const { return add2(FF{s.x, c.x}, FF{s.y, c.y}); }
+};
+template <> struct RealAcc<float2> : RealAccPair {
+    using Pre = float4;   // (b, -b)
+    __device__ __forceinline__ static Pre pre(float2 b) { return make_float4(b.x, b.y, -b.x, -b.y); }
+    __device__ __forceinline__ void add(float2 a, const Pre &b)
+    {
+        const float2 n = __fmul2_rn(a, make_float2(b.z, b.w));
+        ff2_add_neg(s, c, n, __ffma2_rn(a, make_float2(b.x, b.y), n));
+    }
+};
+struct FFPre {
+    float2 h, l, n;   // hi, lo, -hi
+};
+template <> struct RealAcc<ffc> : RealAccPair {
+    using Pre = FFPre;
+    __device__ __forceinline__ static Pre pre(ffc b)
+    {
+        return FFPre{make_float2(b.xh, b.yh), make_float2(b.xl, b.yl), make_float2(-b.xh, -b.yh)};
+    }
+    __device__ __forceinline__ void add(ffc a, const Pre &b)
+    {
+        const float2 h = make_float2(a.xh, a.yh), l = make_float2(a.xl, a.yl);
+        const float2 n = __fmul2_rn(h, b.n);
+        float2 e = __ffma2_rn(h, b.h, n);
+        e = __ffma2_rn(h, b.l, e);
+        e = __ffma2_rn(l, b.h, e);
+        ff2_add_neg(s, c, n, e);
+    }
+};
+
+// Linear combinations with real coefficients: w -= c x, with -c kept (RCoef).
+template <class V> struct RealLin;
+template <> struct RealLin<double2> {
+    using RCoef = double;
+    double2 w;
+    __device__ __forceinline__ static RCoef coef(double c) { return -c; }
+    RealLin() = default;
+    __device__ __forceinline__ RealLin(double2 src) : w(src) {}
+    __device__ __forceinline__ void fms(RCoef nc, double2 x) { w.x = fma(nc, x.x, w.x); w.y = fma(nc, x.y, w.y); }
+    __device__ __forceinline__ double2 out() const { return w; }
+};
+template <> struct RealLin<float2> {
+    using RCoef = float;
+    float2 w;
+    __device__ __forceinline__ static RCoef coef(double c) { return -(float)c; }
+    RealLin() = default;
+    __device__ __forceinline__ RealLin(float2 src) : w(src) {}
+    __device__ __forceinline__ void fms(RCoef nc, float2 x) { w = __ffma2_rn(make_float2(nc, nc), x, w); }
+    __device__ __forceinline__ float2 out() const { return w; }
+};
+template <> struct RealLin<ffc> {
+    using RCoef = float2;   // -c as hi, lo
+    float2 s, c;
+    __device__ __forceinline__ static RCoef coef(double v)
+    {
+        const float2 a = dsplit(v);
+        return neg2(a);
+    }
+    RealLin() = default;
+    __device__ __forceinline__ RealLin(ffc src) : s(make_float2(src.xh, src.yh)), c(make_float2(src.xl, src.yl)) {}
+    __device__ __forceinline__ void fms(RCoef nc, ffc x)
+    {
+        const float2 h = make_float2(x.xh, x.yh), l = make_float2(x.xl, x.yl);
+        const float2 n = __fmul2_rn(make_float2(-nc.x, -nc.x), h);
+        float2 e = __ffma2_rn(make_float2(nc.x, nc.x), h, n);
+        e = __ffma2_rn(make_float2(nc.x, nc.x), l, e);
+        e = __ffma2_rn(make_float2(nc.y, nc.y), h, e);
+        ff2_add_neg(s, c, n, e);
+    }
+    __device__ __forceinline__ ffc out()
+    {
+        ff_renorm2(s, c);
+        return ffc{s.x, s.y, c.x, c.y};
+    }
+};
+
+// Linear combinations with complex coefficients (the combine psi = beta V y): w -= c x.
+template <class V> struct CplxLin {
+    using RCoef = V;
+    V w;
+    __device__ __forceinline__ static RCoef coef(double2 c) { return VT<V>::from(c); }
+    CplxLin() = default;
+    __device__ __forceinline__ CplxLin(V src) : w(src) {}
+    __device__ __forceinline__ void fms(RCoef c, V x) { w = cfms(c, x, w); }
+    __device__ __forceinline__ V out() const { return w; }
+};
+template <> struct CplxLin<ffc> {
+    using RCoef = float4;   // -(re hi, re lo, im hi, im lo)
+    RealLin<ffc> w;
+    __device__ __forceinline__ static RCoef coef(double2 c)
+    {
+        const float2 a = dsplit(c.x), b = dsplit(c.y);
+        return make_float4(-a.x, -a.y, -b.x, -b.y);
+    }
+    CplxLin() = default;
+    __device__ __forceinline__ CplxLin(ffc src) : w(src) {}
+    // re -= cr xr - ci xi, im -= cr xi + ci xr: a real multiple of x, then one of i x
+    __device__ __forceinline__ void fms(RCoef c, ffc x)
+    {
+        w.fms(make_float2(c.x, c.y), x);
+        w.fms(make_float2(c.z, c.w), ffc{-x.yh, x.xh, -x.yl, x.xl});
+    }
+    __device__ __forceinline__ ffc out() { return w.out(); }
+};
 
 // ---------------------------------------------------------------- rank tables
 

@@ -55,10 +55,11 @@ __global__ void __launch_bounds__(NTHR) k_apply(DevBasis b, DevHam hm, const V *
 // (rounded down to a power of two), thread t of a slot adds the partials of CTAs t, t + TPS,
 // ..., and the TPS sums are added by a pairwise tree.  With few slots (the updates need two)
 // this keeps the serial tail of the last CTA to a few loads per thread.  The summation order
-// depends only on the grid and the slot count, so results are bitwise reproducible.
+// depends only on the grid and the slot count, so results are bitwise reproducible.  With cplx
+// unset the imaginary parts are zero and not summed.
 __device__ __forceinline__ bool finish_partials(const double2 *red, double2 *part, KryCtl *ctl,
                                                 double2 *fin, int *flag, unsigned *counter = nullptr,
-                                                int nlead = PSTRIDE, bool tail = true)
+                                                int nlead = PSTRIDE, bool tail = true, bool cplx = true)
 {
     __shared__ double2 tsum[NTHR];
     __shared__ int slots[PSTRIDE];
@@ -89,7 +90,7 @@ __device__ __forceinline__ bool finish_partials(const double2 *red, double2 *par
         for (unsigned c = t; c < gridDim.x; c += tps) {
             const double2 v = __ldcg(part + (size_t)c * PSTRIDE + slot);
             sum.x += v.x;
-            sum.y += v.y;
+            if (cplx) sum.y += v.y;
         }
         tsum[tid] = sum;
     }
@@ -97,7 +98,7 @@ __device__ __forceinline__ bool finish_partials(const double2 *red, double2 *par
     for (int w = tps / 2; w > 0; w >>= 1) {
         if (si < ns && t < w) {
             tsum[tid].x += tsum[tid + w].x;
-            tsum[tid].y += tsum[tid + w].y;
+            if (cplx) tsum[tid].y += tsum[tid + w].y;
         }
         __syncthreads();
     }
@@ -121,12 +122,21 @@ __device__ __forceinline__ void cta_sum_into(double2 v, double2 *red, int slot, 
     __syncthreads();
 }
 
-// The same for per-thread dot accumulators (float-float warp sums for complex64).
+// The same for per-thread dot accumulators (float-float warp sums for complex64): complex ones
+// (warp_value) and real ones.
+template <class Acc>
+__device__ __forceinline__ double2 acc_warp_value(const Acc &acc) { return acc.warp_value(); }
+template <class V>
+__device__ __forceinline__ double2 acc_warp_value(const RealAcc<V> &acc)
+{
+    typename RealAcc<V>::Sum v[1] = {acc.sum()};
+    return make_double2(to_double(warp_totals<1>(v)), 0.0);
+}
 template <class Acc>
 __device__ __forceinline__ void cta_sum_into(const Acc &acc, double2 *red, int slot, double2 *wtmp)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double2 v = acc.warp_value();
+    const double2 v = acc_warp_value(acc);
     if (lane == 0) wtmp[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -191,7 +201,7 @@ __global__ void __launch_bounds__(NTHR) k_hv(EvArgs<V> a, int jj)
     }
 }
 
-// Dots <W_i, y>, i <= j, of a right-hand vector y with the Krylov vectors: a tall-skinny
+// Dots Re <W_i, y>, i <= j, of a right-hand vector y with the Krylov vectors: a tall-skinny
 // GEMV with plain loads.  The vectors are read as KC interleaved columns of rows (thread k
 // takes rows r0 + k + KC e, so a warp loads 32 consecutive rows), and thread (k, g) takes
 // the vectors i = g, g + NG, ... with one accumulator per vector, so the accumulations of
@@ -220,9 +230,8 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
     constexpr int RT = DD ? 4 : 8;                      // rows per column and tile
     constexpr int NG = NTHR / KC, QD = (MMAX + NG - 1) / NG, TR = KC * RT;
     constexpr bool PF = PFT && (F32 || DD);   // prefetch (complex128 is FP64-bound: no gain)
-    using Acc = typename std::conditional<F32, DotAccF2, DotAcc<V>>::type;
     __shared__ double2 red[PSTRIDE];
-    __shared__ double2 wred[NTHR / 32][QD + 1];
+    __shared__ double wred[NTHR / 32][QD + 1];
     __shared__ int flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k = tid % KC, g = tid / KC;
@@ -240,8 +249,7 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
     const bool hasx = Bn > 0 && g < Bn * RX;
     const int xv = NG * A + (Bn > 0 ? g % Bn : 0), xs = Bn > 0 ? g / Bn : 0;
     const int nslot = A + (hasx ? 1 : 0);   // accumulators this group uses
-    Acc acc[QD];
-    DotAcc<V> nrm;
+    RealAcc<V> acc[QD], nrm;
     // the norm of y: group 0 over all tiles when A > 0, else the groups of vector 0
     const bool own_norm = MODE == 0 && (A > 0 ? g == 0 : (hasx && xv == 0));
     uint32_t tl = 0;   // local index of the tile within this CTA
@@ -264,13 +272,13 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
         auto vec = [&](int q) { return a.W + (size_t)(q < A ? g + NG * q : xv) * a.ldW; };
         V uu[RT], cur[RT];
         load(y, uu);
+        typename RealAcc<V>::Pre up[RT];   // y's rows prepared once for every vector of the tile
+#pragma unroll
+        for (int e = 0; e < RT; ++e) up[e] = RealAcc<V>::pre(uu[e]);
         if (own_norm && (A > 0 || xt)) {
 #pragma unroll
-            for (int e = 0; e < RT; ++e) nrm.add_norm(uu[e]);
+            for (int e = 0; e < RT; ++e) nrm.add(uu[e], up[e]);
         }
-        typename Arith<V>::Pre up[RT];   // y's rows prepared once for every vector of the tile
-#pragma unroll
-        for (int e = 0; e < RT; ++e) up[e] = pre(uu[e]);
         if (PF) {
             V nxt[RT];
             load(vec(0), cur);
@@ -301,59 +309,55 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
         nrm.renorm();
     }
     // per warp: the sum over its 32 columns; then the warps of a vector's groups, in order
+    // (accumulators that were not used are zero)
+    {
+        typename RealAcc<V>::Sum v[QD];
 #pragma unroll
-    for (int q = 0; q < QD; ++q) {
-        if (q < nslot) {   // (warp-uniform)
-            const double2 v = acc[q].warp_value();
-            if (lane == 0) wred[warp][q] = v;
-        } else if (lane == 0) {
-            wred[warp][q] = make_double2(0.0, 0.0);
-        }
+        for (int q = 0; q < QD; ++q) v[q] = acc[q].sum();
+        const double t = to_double(warp_totals<QD>(v));
+        if (lane % (32 / QD) == 0) wred[warp][lane / (32 / QD)] = t;
     }
     if (MODE == 0) {
-        const double2 v = nrm.warp_value();
-        if (lane == 0) wred[warp][QD] = v;
+        typename RealAcc<V>::Sum v[1] = {nrm.sum()};
+        const double t = to_double(warp_totals<1>(v));
+        if (lane == 0) wred[warp][QD] = t;
     }
     __syncthreads();
     constexpr int WG = KC / 32;   // warps per group
     if (tid < nv) {
         // vector tid: group tid mod NG at slot tid / NG, or the RX groups sharing it at slot A
-        double2 t = make_double2(0.0, 0.0);
+        double t = 0.0;
         const bool whole = tid < NG * A;
         for (int sv = 0; sv < (whole ? 1 : RX); ++sv) {
             const int gg = whole ? tid % NG : (tid - NG * A) + Bn * sv, q = whole ? tid / NG : A;
 #pragma unroll
-            for (int w = 0; w < WG; ++w) {
-                t.x += wred[WG * gg + w][q].x;
-                t.y += wred[WG * gg + w][q].y;
-            }
+            for (int w = 0; w < WG; ++w) t += wred[WG * gg + w][q];
         }
-        red[tid] = t;
+        red[tid] = make_double2(t, 0.0);
     }
     if (MODE == 0 && tid == 0) {
         double t = 0.0;
         for (int sv = 0; sv < (A > 0 ? 1 : RX); ++sv) {
             const int gg = A > 0 ? 0 : Bn * sv;
 #pragma unroll
-            for (int w = 0; w < WG; ++w) t += wred[WG * gg + w][QD].x;
+            for (int w = 0; w < WG; ++w) t += wred[WG * gg + w][QD];
         }
         red[SLOT_NRM] = make_double2(t, 0.0);
     }
     __syncthreads();
     double2 *fin = red;
-    if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, nv, MODE == 0)) return;
+    if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, nv, MODE == 0, false)) return;
     // Scalar epilogue, one lane of warp 0 per vector.  GB300 issues one FP64 warp instruction per
     // about 77 cycles and SM sub-partition whatever its active lanes, so a loop over the vectors
     // in one thread cost 4 us at j = 30.
     if (tid >= 32) return;
     const bool in = tid <= jj;
     const double s = in ? ctl->sigma[tid] : 0.0;
-    const double2 c = make_double2(fin[tid].x * s, fin[tid].y * s);   // <v_i, y>
-    const double2 cs = make_double2(c.x * s, c.y * s);
-    const double c2 = warp_sum(c.x * c.x + c.y * c.y);
+    const double c = fin[tid].x * s;   // Re <v_i, y>
+    const double c2 = warp_sum(c * c);
     if (MODE == 0) {
-        if (in) ctl->coefA[tid] = cs;
-        if (tid == jj) ctl->alpha[jj] = c.x;
+        if (in) ctl->coefA[tid] = c * s;
+        if (tid == jj) ctl->alpha[jj] = c;
         if (tid != 0) return;
         ctl->c2 = c2;
         ctl->normu2 = fin[SLOT_NRM].x;
@@ -366,8 +370,8 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
     }
     const double nw2 = ctl->wnorm2;
     const bool sub = nw2 > 0.0 && sqrt(c2) > ctl->eta_corr * sqrt(nw2);
-    if (sub && in) ctl->coefC[tid] = cs;
-    if (sub && tid == jj) ctl->alpha[jj] += c.x;
+    if (sub && in) ctl->coefC[tid] = c * s;
+    if (sub && tid == jj) ctl->alpha[jj] += c;
     if (tid != 0) return;
     if (nw2 > 0.0) ctl->max_orth = fmax(ctl->max_orth, sqrt(c2 / nw2));
     ctl->n_c1 += 1;
@@ -395,21 +399,25 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     if (MODE <= 1 && jj >= ctl->m_eff) return;
     if (MODE == 1 && !ctl->corr2) return;
     const int nvec = (MODE == 2) ? ctl->m_eff : ((MODE == 3) ? 0 : jj + 1);
-    __shared__ typename Arith<V>::Coef coef[MMAX + 1];
+    // modes 0 and 1 subtract real multiples (RealAcc), the combine takes complex ones
+    constexpr bool RE = MODE <= 1;
+    using Lin = typename std::conditional<RE, RealLin<V>, CplxLin<V>>::type;
+    __shared__ typename Lin::RCoef coef[MMAX + 1];
     __shared__ double2 red[PSTRIDE];
     __shared__ double2 wtmp[NTHR / 32];
     __shared__ int flag;
     const int tid = threadIdx.x;
     if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
     if (tid < nvec) {
-        const double2 c = (MODE == 0) ? ctl->coefA[tid] : (MODE == 1) ? ctl->coefC[tid] : ctl->coefY[tid];
-        coef[tid] = coef_from<V>(c);
+        if constexpr (RE) coef[tid] = Lin::coef(MODE == 0 ? ctl->coefA[tid] : ctl->coefC[tid]);
+        else coef[tid] = Lin::coef(ctl->coefY[tid]);
     }
     __syncthreads();
     V *out = (MODE >= 2) ? a.W : a.W + (size_t)(jj + 1) * a.ldW;
     const V *src = (MODE == 0) ? a.U : (MODE == 1) ? out : (MODE == 3) ? a.G : nullptr;
     const uint32_t D = a.b.D;
-    DotAcc<V> nrm, gacc;
+    RealAcc<V> nrm;
+    DotAcc<V> gacc;
     const uint32_t ntr = (D + RR * TILE - 1) / (RR * TILE);
     for (uint32_t tile = blockIdx.x; tile < ntr; tile += gridDim.x) {
         const uint32_t r = tile * RR * TILE + tid;
@@ -421,9 +429,9 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
             in[k] = r + k * TILE < D;
             q[k] = in[k] ? r + k * TILE : r;   // past D a row repeats the first, unstored
         }
-        typename Arith<V>::Lin w[RR];
+        Lin w[RR];
 #pragma unroll
-        for (int k = 0; k < RR; ++k) w[k] = lin_init(src ? src[q[k]] : VT<V>::zero());
+        for (int k = 0; k < RR; ++k) w[k] = Lin(src ? src[q[k]] : VT<V>::zero());
         if (MODE == 2) {   // reads W_0 while overwriting it: plain loads
 #pragma unroll 8
             for (int i = 0; i < nvec; ++i) {
@@ -432,7 +440,7 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
 #pragma unroll
                 for (int k = 0; k < RR; ++k) x[k] = wi[q[k]];
 #pragma unroll
-                for (int k = 0; k < RR; ++k) lin_fms(w[k], coef[i], x[k]);
+                for (int k = 0; k < RR; ++k) w[k].fms(coef[i], x[k]);
             }
         } else {
 #pragma unroll 8
@@ -442,15 +450,15 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
 #pragma unroll
                 for (int k = 0; k < RR; ++k) x[k] = ldg(wi + q[k]);
 #pragma unroll
-                for (int k = 0; k < RR; ++k) lin_fms(w[k], coef[i], x[k]);
+                for (int k = 0; k < RR; ++k) w[k].fms(coef[i], x[k]);
             }
         }
 #pragma unroll
         for (int k = 0; k < RR; ++k) {
             if (!in[k]) continue;
-            const V wv = (MODE == 3) ? src[q[k]] : lin_out(w[k]);   // (the load is a plain copy)
+            const V wv = (MODE == 3) ? src[q[k]] : w[k].out();   // (the load is a plain copy)
             out[q[k]] = wv;
-            nrm.add_norm(wv);
+            nrm.add(wv, RealAcc<V>::pre(wv));
             if (a.G && MODE != 3) gacc.add(ldg(a.G + q[k]), wv);
         }
         nrm.renorm();
@@ -459,7 +467,7 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     cta_sum_into(nrm, red, SLOT_NRM, wtmp);
     if (a.G) cta_sum_into(gacc, red, SLOT_G, wtmp);
     double2 *fin = red;
-    if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, 0, true)) return;
+    if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, 0, true, a.G != nullptr)) return;
     if (tid != 0) return;
     const double nw2 = fin[SLOT_NRM].x;
     const double2 gdot = fin[SLOT_G];

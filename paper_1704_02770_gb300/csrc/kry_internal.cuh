@@ -16,8 +16,9 @@ namespace kry {
 // significant bits each, 16 bytes like complex128): the Krylov vectors of dtype KRY_C128E,
 // on which the vector kernels do float-float arithmetic on the FP32 pipe (kry_device.cuh).
 // Inputs and outputs of that dtype stay complex128; they are converted at the boundary.
+// (leading parts first, so that both components of a part are one packed FP32x2 operand)
 struct __align__(16) ffc {
-    float xh, xl, yh, yl;
+    float xh, yh, xl, yl;
 };
 
 // Index of a dtype's launch shape: KRY_C128, KRY_C64, KRY_C128E.
@@ -140,7 +141,8 @@ struct KryHdrB {   // shared scalars (copied to the host when polling)
 struct KryCtlB {
     KryHdrB hd;
     double alpha[MMAX + 1][KBMAX], beta[MMAX + 1][KBMAX], sigma[MMAX + 2][KBMAX];
-    double2 coefA[MMAX + 1][KBMAX], coefC[MMAX + 1][KBMAX], coefY[MMAX + 1][KBMAX];
+    double coefA[MMAX + 1][KBMAX], coefC[MMAX + 1][KBMAX];   // real, as in KryCtl
+    double2 coefY[MMAX + 1][KBMAX];
     double2 g[MMAX + 2][KBMAX];
     double normu2[KBMAX], beta0[KBMAX], tau_ok[KBMAX], err_k[KBMAX], orth[KBMAX];
     int m_eff[KBMAX], corr[KBMAX];
@@ -194,8 +196,8 @@ int launch_exp_b(const ExpArgsB &a, cudaStream_t s);
 // step, time-stepping state and counters.  Written only by single-thread epilogues.
 struct KryCtl {
     double alpha[MMAX + 1], beta[MMAX + 1], sigma[MMAX + 2];
-    double2 coefA[MMAX + 1];   // update coefficients c_i sigma_i of pass B
-    double2 coefC[MMAX + 1];   // correction coefficients of pass C
+    double coefA[MMAX + 1];    // update coefficients c_i sigma_i of pass B (real: see RealAcc)
+    double coefC[MMAX + 1];    // correction coefficients of pass C
     double2 coefY[MMAX + 1];   // combine coefficients -beta0 y_i sigma_i
     double2 g[MMAX + 2];       // readout <psi0, v_i>
     double normu2;             // ||H v_j||^2 of the last pass A

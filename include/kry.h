@@ -237,8 +237,8 @@ int kry_profile_read(kry_ham H, double *ms, double *bytes, int64_t *launches);
  *            first and their loads issued together (else one hop at a time); bit 1 set = the
  *            lower-bit rank table read through the L1 cache instead of staged in shared memory
  *            (at L = 29, 30 that table takes 64 KB of shared memory per CTA);
- *   shape[2] dots of pass A: 0 = the next vector's rows loaded before the current vector's
- *            products are accumulated (complex64), 1 = without that prefetch;
+ *   shape[2] dots of pass A: 0 = two or four units of rows loaded at a time where a thread has
+ *            few vectors, 1 = always one;
  *   shape[3] rows per thread of the update pass: 1, 2 or 4;
  *   shape[4] H.v of batched Hamiltonians (K > 1) in chunks of 8 or 16 realisations, so that
  *            the gathered part of the vector fits in L2 (0 = all K at once).

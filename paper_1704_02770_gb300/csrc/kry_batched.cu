@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots_b(EvArgsB<V> a, int jj)
                         for (int rr = 0; rr < RH; ++rr) dst[rr] = (rr < nr) ? ldg(wi + (size_t)rr * K) : VT<V>::zero();
                     }
                 };
-                // (a prefetch of the next vector's rows, as in the single-realisation dots,
+                // (loading the next vector's rows before this one's products
                 // needs more registers than the eight accumulators of K = 64 leave, and spills)
 #pragma unroll
                 for (int q = 0; q < QD; ++q) {
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
 
 // mode: 0 pass A, 1 pass B, 3 pass C1 (dots of w), 2 pass C2 (correction), 4 combine,
 // 5 load of a general psi0.  One CTA per realisation.  A warp takes a whole slot (lanes over the
-// CTAs' partials, then a shuffle tree) and lane i of warp 0 the scalars of vector i: GB300 issues
+// CTAs' partials) and lane i of warp 0 the scalars of vector i: GB300 issues
 // one FP64 warp instruction per about 77 cycles and SM sub-partition whatever its active lanes, so
 // block-wide trees slot by slot and loops over the vectors in one thread cost tens of us at j = 30.
 __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *__restrict__ part,
@@ -432,13 +432,19 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         const int slot = q < nd ? q : q == nd ? SLOT_NRM : SLOT_G;
         double2 s = make_double2(0.0, 0.0);
         const bool cplx = slot == SLOT_G;   // the others are real
-#pragma unroll 4
-        for (int c = lane; c < grid; c += 32) {
-            const double2 v = __ldg(part + ((size_t)c * PSB + slot) * Kp + k);
-            s.x += v.x;
-            if (cplx) s.y += v.y;
+        for (int c0 = 0; c0 < grid; c0 += 256) {
+            double x[8], y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int c = c0 + 32 * i + lane;
+                double2 v = make_double2(0.0, 0.0);
+                if (c < grid) v = __ldg(part + ((size_t)c * PSB + slot) * Kp + k);
+                x[i] = v.x;
+                y[i] = v.y;
+            }
+            s.x += warp_sum_int<8>(x);
+            if (cplx) s.y += warp_sum_int<8>(y);
         }
-        s = cplx ? warp_sum(s) : make_double2(warp_sum(s.x), 0.0);
         if (lane == 0) fin[slot] = s;
     }
     __syncthreads();
@@ -507,7 +513,7 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
             H.vp_kind[KIND_PASSC] += jj + 2;
         }
         if (!ctl->dots[k] || jj >= ctl->m_eff[k]) return;
-        const double nd2 = warp_sum(c * c);
+        const double cc = c * c, nd2 = warp_sum_int<1>(&cc);
         const bool sub = nw2 > 0.0 && sqrt(nd2) > H.eta_corr * sqrt(nw2);
         if (sub && lane <= jj) ctl->coefC[lane][k] = cs;
         if (sub && lane == jj) ctl->alpha[jj][k] += c;

@@ -106,6 +106,16 @@ __device__ __forceinline__ ffc ldg(const ffc *p)
 __device__ __forceinline__ float2 ldg(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ double2 ldg(const double2 *p) { return __ldg(p); }
 
+// the 16 bytes at p (16-byte aligned): one element, or two of complex64
+__device__ __forceinline__ void ldg_chunk(const float2 *p, float2 *dst)
+{
+    const float4 v = __ldg((const float4 *)p);
+    dst[0] = make_float2(v.x, v.y);
+    dst[1] = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ldg_chunk(const double2 *p, double2 *dst) { dst[0] = __ldg(p); }
+__device__ __forceinline__ void ldg_chunk(const ffc *p, ffc *dst) { dst[0] = ldg(p); }
+
 // Per element type, the accumulator of a neighbour sum: the element itself, or two float-float
 // numbers.
 struct FF4 {   // two float-float numbers (real, imaginary)
@@ -322,6 +332,63 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// ---------------------------------------------------------------- sums without the FP64 pipe
+// GB300 issues one FP64 warp instruction per about 77 cycles and SM sub-partition, so the trees and
+// gathers that end a reduction cost more in FP64 adds than the loads before them.  These sums align
+// the mantissas to the largest exponent of the warp as 64-bit integers, add those exactly (in 26-bit
+// limbs, one redux each) and round once: the terms lose less than 2^-54 of the largest each, which
+// is no more than the roundings of an FP64 sum of as many, and the order does not matter.
+
+// Integer sum over the warp of CNT values per lane (CNT <= 8): every lane gets S and k with the total
+// = S 2^k.  False (uniform) when a value is infinite or NaN, or the largest below 2^-895; subnormal
+// values count as zero.
+template <int CNT>
+__device__ __forceinline__ bool warp_isum(const double *v, long long &S, int &k)
+{
+    unsigned em = 0;
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) em = max(em, ((unsigned)__double2hiint(v[i]) >> 20) & 0x7ffu);
+    em = __reduce_max_sync(0xffffffffu, em);
+    S = 0;
+    k = 0;
+    if (em == 0u) return true;
+    if (em == 0x7ffu || em < 128u) return false;
+    constexpr int SH = CNT == 1 ? 5 : 2;   // 53 bits + SH + log2(32 CNT) <= 63
+    long long q = 0;
+#pragma unroll
+    for (int i = 0; i < CNT; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(v[i]), lo = (unsigned)__double2loint(v[i]), e = (hi >> 20) & 0x7ffu;
+        unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << SH;
+        const unsigned d = em - e;
+        m = e == 0u || d > 63u ? 0ull : m >> d;
+        q += (int)hi < 0 ? -(long long)m : (long long)m;
+    }
+    const unsigned mask = (1u << 26) - 1u;
+    const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)q & mask);
+    const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 26) & mask);
+    const int l2 = __reduce_add_sync(0xffffffffu, (int)(q >> 52));
+    S = (long long)l0 + ((long long)l1 << 26) + ((long long)l2 << 52);
+    k = (int)em - 1075 - SH;
+    return true;
+}
+// S 2^k (k >= -1000), rounded once
+__device__ __forceinline__ double from_isum(long long S, int k)
+{
+    return (double)S * __hiloint2double((k + 1023) << 20, 0);
+}
+// Sum over the warp of CNT values per lane, in every lane.
+template <int CNT>
+__device__ __forceinline__ double warp_sum_int(const double *v)
+{
+    long long S;
+    int k;
+    if (warp_isum<CNT>(v, S, k)) return from_isum(S, k);
+    double t = v[0];
+#pragma unroll
+    for (int i = 1; i < CNT; ++i) t += v[i];
+    return warp_sum(t);
+}
+
 // ---------------------------------------------------------------- real inner products
 // The Hamiltonian is real and symmetric, so the Lanczos process of a complex vector is that of
 // H (+) H on its real and imaginary parts: a vector of 2D reals with the inner product
@@ -338,26 +405,43 @@ __device__ __forceinline__ double warp_sum(double v)
 struct FF {   // a float-float number
     float s, c;
 };
-__device__ __forceinline__ double add2(double a, double b) { return a + b; }
 __device__ __forceinline__ FF add2(FF a, FF b)
 {
     ff_combine(a.s, a.c, b.s, b.c);
     return a;
 }
-__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ FF shfl_xor(FF v, int o)
 {
     return FF{__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o)};
 }
-__device__ __forceinline__ double pick(bool p, double a, double b)
-{
-    // (as integers: a select of doubles occupies the FP64 pipe)
-    return __longlong_as_double(p ? __double_as_longlong(a) : __double_as_longlong(b));
-}
 __device__ __forceinline__ FF pick(bool p, FF a, FF b) { return FF{p ? a.s : b.s, p ? a.c : b.c}; }
 
-// Totals over the warp of N values per lane (N a power of two up to 32), N - 1 + log2(32 / N) adds
-// per lane instead of 5 N: lane l returns the total of value l / (32 / N).
+// Totals over the warp of N values per lane (N a power of two up to 32): lane l returns the total of
+// value l / (32 / N).  Doubles as integers; float-float numbers by exchange, N - 1 + log2(32 / N)
+// adds per lane instead of 5 N.
+template <int N>
+__device__ __forceinline__ double warp_totals(double *v)
+{
+    const int lane = threadIdx.x & 31;
+    long long S = 0;
+    int k = 0;
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        long long Si = 0;
+        int ki = 0;
+        ok &= warp_isum<1>(v + i, Si, ki);
+        if (lane / (32 / N) == i) { S = Si; k = ki; }
+    }
+    if (ok) return from_isum(S, k);
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const double w = warp_sum(v[i]);
+        if (lane / (32 / N) == i) t = w;
+    }
+    return t;
+}
 template <int N, class T>
 __device__ __forceinline__ T warp_totals(T *v)
 {

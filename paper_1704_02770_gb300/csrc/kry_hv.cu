@@ -17,6 +17,8 @@
 
 namespace kry {
 
+constexpr int DOTS_NTHR = 512;   // threads of a large CTA of the dots
+
 struct SmemHead {
     uint32_t koff[20];
     uint32_t bsz[20];
@@ -50,59 +52,47 @@ __global__ void __launch_bounds__(NTHR) k_apply(DevBasis b, DevHam hm, const V *
 
 // Write this CTA's partials, then let the last CTA to finish sum all partials into
 // fin[0..PSTRIDE).  Returns true in the last CTA (all its threads).  Only the slots [0, nlead)
-// and, with tail set, SLOT_NRM and SLOT_G are summed (the others of fin are zero), and all
-// NTHR threads share the work: each of the ns needed slots gets TPS = NTHR / ns threads
-// (rounded down to a power of two), thread t of a slot adds the partials of CTAs t, t + TPS,
-// ..., and the TPS sums are added by a pairwise tree.  With few slots (the updates need two)
-// this keeps the serial tail of the last CTA to a few loads per thread.  The summation order
-// depends only on the grid and the slot count, so results are bitwise reproducible.  With cplx
-// unset the imaginary parts are zero and not summed.
+// and, with tail set, SLOT_NRM and SLOT_G are summed (the others of fin are zero): a warp takes a
+// slot, lane l the partials of CTAs l, l + 32, ..., eight loads at a time.  With cplx unset the imaginary parts are zero and not summed.  The order depends only on the grid,
+// the block and the slot count, so results are bitwise reproducible.
 __device__ __forceinline__ bool finish_partials(const double2 *red, double2 *part, KryCtl *ctl,
                                                 double2 *fin, int *flag, unsigned *counter = nullptr,
                                                 int nlead = PSTRIDE, bool tail = true, bool cplx = true)
 {
-    __shared__ double2 tsum[NTHR];
-    __shared__ int slots[PSTRIDE];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     if (!counter) counter = &ctl->counter;
     if (tid < PSTRIDE) part[(size_t)blockIdx.x * PSTRIDE + tid] = red[tid];
-    __threadfence();
     __syncthreads();
-    if (tid == 0) *flag = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1 : 0;
+    if (tid == 0) {   // (one fence for the CTA: the barrier orders the others' writes before it)
+        __threadfence();
+        *flag = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1 : 0;
+        __threadfence();
+    }
     __syncthreads();
     if (!*flag) return false;
-    __threadfence();
-    int ns = 0;
-    for (int sl = 0; sl < PSTRIDE; ++sl)
-        if (sl < nlead || (tail && (sl == SLOT_NRM || sl == SLOT_G))) {
-            if (tid == 0) slots[ns] = sl;
-            ++ns;
-        }
-    int tps = 1;
-    while (tps * 2 * ns <= NTHR && tps < 128) tps *= 2;
+    // slots 0 .. nlead - 1, then NRM and G unless they are among those
+    const int nt = tail ? (nlead <= SLOT_NRM ? 2 : 0) : 0, ns = nlead + nt;
     if (tid < PSTRIDE) fin[tid] = make_double2(0.0, 0.0);
     __syncthreads();
-    const int si = tid / tps, t = tid - si * tps;
-    if (si < ns) {
-        const int slot = slots[si];
+    for (int q = warp; q < ns; q += nw) {
+        const int slot = q < nlead ? q : SLOT_NRM + (q - nlead);
+        if (!cplx && slot == SLOT_G) continue;
         double2 sum = make_double2(0.0, 0.0);
-#pragma unroll 4
-        for (unsigned c = t; c < gridDim.x; c += tps) {
-            const double2 v = __ldcg(part + (size_t)c * PSTRIDE + slot);
-            sum.x += v.x;
-            if (cplx) sum.y += v.y;
+        for (unsigned c0 = 0; c0 < gridDim.x; c0 += 256) {
+            double x[8], y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned c = c0 + 32 * i + lane;
+                double2 v = make_double2(0.0, 0.0);
+                if (c < gridDim.x) v = __ldcg(part + (size_t)c * PSTRIDE + slot);
+                x[i] = v.x;
+                y[i] = v.y;
+            }
+            sum.x += warp_sum_int<8>(x);
+            if (cplx) sum.y += warp_sum_int<8>(y);
         }
-        tsum[tid] = sum;
+        if (lane == 0) fin[slot] = sum;
     }
-    __syncthreads();
-    for (int w = tps / 2; w > 0; w >>= 1) {
-        if (si < ns && t < w) {
-            tsum[tid].x += tsum[tid + w].x;
-            if (cplx) tsum[tid].y += tsum[tid + w].y;
-        }
-        __syncthreads();
-    }
-    if (si < ns && t == 0) fin[slots[si]] = tsum[tid];
     __syncthreads();
     return true;
 }
@@ -111,7 +101,7 @@ __device__ __forceinline__ bool finish_partials(const double2 *red, double2 *par
 __device__ __forceinline__ void cta_sum_into(double2 v, double2 *red, int slot, double2 *wtmp)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum(v);
+    v = make_double2(warp_sum_int<1>(&v.x), warp_sum_int<1>(&v.y));
     if (lane == 0) wtmp[warp] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -201,148 +191,146 @@ __global__ void __launch_bounds__(NTHR) k_hv(EvArgs<V> a, int jj)
     }
 }
 
+// The row loop of k_dots for one group of 64 threads: NQ vectors from Wg, NU units of rows at a time
+// (all their loads issued before the products), and with NORM also ||y||^2.  NQ is a template
+// parameter because a predicated-off multiply-add takes the FP64 pipe like any other: with a loop
+// over eight vectors and a test in it, the dots with 1 to 8 vectors all took 91 us at L = 24.
+template <class V, int NQ, int NU, bool NORM>
+__device__ __forceinline__ void dots_rows(const V *y, const V *Wg, size_t ldW, uint32_t u0, uint32_t du,
+                                          uint32_t nu, uint32_t D, RealAcc<V> *acc, RealAcc<V> &nrm)
+{
+    constexpr int RPC = 16 / sizeof(V);
+    // units between two foldings of the float-float compensations (8 rows of complex64, 4 else)
+    constexpr uint32_t FOLD = 4;
+    const uint32_t col = threadIdx.x & 63;
+    uint32_t it = 0;
+    for (uint32_t u = u0; u < nu; u += NU * du) {
+        V x[NU][NQ][RPC], yy[NU][RPC];
+#pragma unroll
+        for (int n = 0; n < NU; ++n) {
+            const uint32_t r = ((u + n * du) * 64 + col) * RPC;
+            // zero past D; the second row of a complex64 pair may be the first past D, where the
+            // vectors are padded (ldW is a multiple of 64) and the value is dropped
+#pragma unroll
+            for (int e = 0; e < RPC; ++e) {
+                yy[n][e] = VT<V>::zero();
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) x[n][q][e] = VT<V>::zero();
+            }
+            if (r < D) {
+                ldg_chunk(y + r, yy[n]);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) ldg_chunk(Wg + q * ldW + r, x[n][q]);
+            }
+            if (RPC == 2 && r + 1 == D) {
+                yy[n][RPC - 1] = VT<V>::zero();
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) x[n][q][RPC - 1] = VT<V>::zero();
+            }
+        }
+#pragma unroll
+        for (int n = 0; n < NU; ++n) {
+            if (NU == 1 || u + n * du < nu) {
+#pragma unroll
+                for (int e = 0; e < RPC; ++e) {
+                    const typename RealAcc<V>::Pre p = RealAcc<V>::pre(yy[n][e]);
+                    if (NORM) nrm.add(yy[n][e], p);
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) acc[q].add(x[n][q][e], p);
+                }
+                if (++it % FOLD == 0) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) acc[q].renorm();
+                    nrm.renorm();
+                }
+            }
+        }
+    }
+}
+
 // Dots Re <W_i, y>, i <= j, of a right-hand vector y with the Krylov vectors: a tall-skinny
-// GEMV with plain loads.  The vectors are read as KC interleaved columns of rows (thread k
-// takes rows r0 + k + KC e, so a warp loads 32 consecutive rows), and thread (k, g) takes
-// the vectors i = g, g + NG, ... with one accumulator per vector, so the accumulations of
-// different vectors overlap.  The rows of the next vector are loaded before the current
-// vector's products are accumulated (software prefetch), so the loads of one vector are in
-// flight during the arithmetic of the one before: the complex64 accumulation is error-free
-// float-float arithmetic, about as much FP32 work per byte as the HBM stream supplies, and
-// without the overlap the kernel alternates between waiting on loads and on the FP32 pipe.
-// complex64: KC = 32 (a warp per group of vectors), two CTAs per SM (the prefetch buffer
-// needs the registers); complex128 (FP64-bound, no prefetch): KC = 64, two.  The sums over
-// the columns are taken in a fixed order at the end.  PFT = 0 turns the prefetch off (a
-// launch-shape choice of kry_autotune; the bits are the same).
+// GEMV with plain loads, bound by HBM (complex64, float-float) or the FP64 pipe (complex128).
+// 64 threads (two warps) read 16 bytes each of consecutive rows -- one row, or two of complex64 --
+// of up to QV = 8 vectors, all loads issued before the products are accumulated (one real
+// accumulator per vector and thread); with few vectors they take two or four units of rows at a time
+// (MU = 0: always one, a launch-shape choice of kry_autotune; the bits are the same).  The 64-thread
+// groups of a CTA split the vectors into NVG = 1, 2 or 4 nearly equal shares of at most eight, and
+// the groups left over take other rows, so every warp has the same work at every j.  One CTA of 512
+// threads per SM keeps up to 64 KB of loads in flight per SM (45 bytes per ns and SM at the HBM rate
+// and about 0.8 us of latency need 36 KB) and leaves 152 partial sums per slot to add at the end.
 //   MODE 0 (pass A): y = U = sigma_j H W_j; fills coefA[0..j], alpha_j and ||u||^2.
 //   MODE 1 (pass C1, when pass B flagged it): y = W_{j+1}; measures the loss of
 //          orthogonality and sets up the subtraction of pass C2 when it exceeds eta_corr.
-template <class V, int MODE, int PFT>
-__global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
+template <class V, int MODE, int MU>
+__global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
 {
     pdl_begin();
     KryCtl *ctl = a.ctl;
     if (ctl->done || jj >= ctl->m_eff) return;
     if (MODE == 1 && !ctl->corr) return;
-    constexpr bool DD = std::is_same<V, ffc>::value;   // float-float vectors
-    constexpr bool F32 = std::is_same<V, float2>::value;
-    constexpr int KC = (F32 || DD) ? 32 : 64;          // columns (rows in flight per vector)
-    constexpr int RT = DD ? 4 : 8;                      // rows per column and tile
-    constexpr int NG = NTHR / KC, QD = (MMAX + NG - 1) / NG, TR = KC * RT;
-    constexpr bool PF = PFT && (F32 || DD);   // prefetch (complex128 is FP64-bound: no gain)
+    constexpr int RPC = 16 / sizeof(V);                 // rows of a thread's 16 bytes
+    constexpr int QV = 8;                               // vectors of a group, at most
     __shared__ double2 red[PSTRIDE];
-    __shared__ double wred[NTHR / 32][QD + 1];
+    __shared__ double wred[DOTS_NTHR / 32][QV + 1];
     __shared__ int flag;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int k = tid % KC, g = tid / KC;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ngrp = blockDim.x >> 6, g = tid >> 6;
     if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
     const V *y = (MODE == 0) ? a.U : a.W + (size_t)(jj + 1) * a.ldW;
     const int nv = jj + 1;   // vectors W_0 .. W_j
-    const uint32_t D = a.b.D, ntiles = (D + TR - 1) / TR;
-    // Work split: with nv = NG A + B, every group takes A whole vectors (g, g + NG, ...) over
-    // all the CTA's tiles, and the B remaining vectors are shared by all groups: RX = NG / B
-    // groups per remaining vector (group g: vector NG A + g mod B, every RX-th tile of the
-    // CTA from g / B), so every warp streams about the same number of rows at every j; the
-    // partial sums of the groups that share a vector are added at the end.
-    const int A = nv / NG, Bn = nv % NG;
-    const int RX = Bn > 0 ? NG / Bn : 1;
-    const bool hasx = Bn > 0 && g < Bn * RX;
-    const int xv = NG * A + (Bn > 0 ? g % Bn : 0), xs = Bn > 0 ? g / Bn : 0;
-    const int nslot = A + (hasx ? 1 : 0);   // accumulators this group uses
-    RealAcc<V> acc[QD], nrm;
-    // the norm of y: group 0 over all tiles when A > 0, else the groups of vector 0
-    const bool own_norm = MODE == 0 && (A > 0 ? g == 0 : (hasx && xv == 0));
-    uint32_t tl = 0;   // local index of the tile within this CTA
-    for (uint32_t tile = blockIdx.x; nslot > 0 && tile < ntiles; tile += gridDim.x, ++tl) {
-        const bool xt = hasx && (int)(tl % (uint32_t)RX) == xs;
-        const int nq = A + (xt ? 1 : 0);   // vectors of this tile: A whole ones, then the shared one
-        if (nq == 0) continue;
-        const uint32_t r0 = tile * TR + k;
-        const bool full = tile * TR + TR <= D;
-        // rows r0 + KC e of vector p (zero past D; one test per tile when the tile is full)
-        auto load = [&](const V *p, V *dst) {
-            if (full) {
-#pragma unroll
-                for (int e = 0; e < RT; ++e) dst[e] = ldg(p + r0 + KC * e);
-            } else {
-#pragma unroll
-                for (int e = 0; e < RT; ++e) dst[e] = (r0 + KC * e < D) ? ldg(p + r0 + KC * e) : VT<V>::zero();
-            }
-        };
-        auto vec = [&](int q) { return a.W + (size_t)(q < A ? g + NG * q : xv) * a.ldW; };
-        V uu[RT], cur[RT];
-        load(y, uu);
-        typename RealAcc<V>::Pre up[RT];   // y's rows prepared once for every vector of the tile
-#pragma unroll
-        for (int e = 0; e < RT; ++e) up[e] = RealAcc<V>::pre(uu[e]);
-        if (own_norm && (A > 0 || xt)) {
-#pragma unroll
-            for (int e = 0; e < RT; ++e) nrm.add(uu[e], up[e]);
-        }
-        if (PF) {
-            V nxt[RT];
-            load(vec(0), cur);
-#pragma unroll
-            for (int q = 0; q < QD; ++q) {
-                if (q < nq) {
-                    if (q + 1 < nq) load(vec(q + 1), nxt);
-#pragma unroll
-                    for (int e = 0; e < RT; ++e) acc[q].add(cur[e], up[e]);
-#pragma unroll
-                    for (int e = 0; e < RT; ++e) cur[e] = nxt[e];
-                }
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < QD; ++q) {
-                if (q < nq) {
-                    load(vec(q), cur);
-#pragma unroll
-                    for (int e = 0; e < RT; ++e) acc[q].add(cur[e], up[e]);
-                }
-            }
-        }
-        // fold the float-float compensations back once per tile
-#pragma unroll
-        for (int q = 0; q < QD; ++q)
-            if (q < nq) acc[q].renorm();
-        nrm.renorm();
+    const int nvg = nv <= QV ? 1 : nv <= 2 * QV ? 2 : 4, nrp = ngrp / nvg;   // shares of the vectors, of the rows
+    const int rp = g / nvg, vg = (g + rp) % nvg;   // (rotated: the shares differ by one vector)
+    const int i0 = (nv * vg) / nvg, nq = (nv * (vg + 1)) / nvg - i0;   // this group's vectors i0 .. i0 + nq - 1
+    const uint32_t D = a.b.D, nu = (D + 64 * RPC - 1) / (64 * RPC);   // units of 64 threads' rows
+    RealAcc<V> acc[QV], nrm;
+    const V *Wg = a.W + (size_t)i0 * a.ldW;
+    const uint32_t u0 = blockIdx.x * nrp + rp, du = gridDim.x * nrp;
+#define KRY_DOTS_ROWS(NQ, NU)                                                                          \
+    case NQ:                                                                                           \
+        if (MODE == 0 && vg == 0) dots_rows<V, NQ, MU ? NU : 1, MODE == 0>(y, Wg, a.ldW, u0, du, nu, D, acc, nrm); \
+        else dots_rows<V, NQ, MU ? NU : 1, false>(y, Wg, a.ldW, u0, du, nu, D, acc, nrm);              \
+        break;
+    switch (nq) {
+        KRY_DOTS_ROWS(1, 4)
+        KRY_DOTS_ROWS(2, 4)
+        KRY_DOTS_ROWS(3, 2)
+        KRY_DOTS_ROWS(4, 2)
+        KRY_DOTS_ROWS(5, 2)
+        KRY_DOTS_ROWS(6, 2)
+        KRY_DOTS_ROWS(7, 1)
+        KRY_DOTS_ROWS(8, 1)
+    default: break;
     }
-    // per warp: the sum over its 32 columns; then the warps of a vector's groups, in order
-    // (accumulators that were not used are zero)
+#undef KRY_DOTS_ROWS
+    // per warp: the totals of its vectors (accumulators that were not used are zero); then the
+    // warps of a vector's groups, in order
     {
-        typename RealAcc<V>::Sum v[QD];
+        typename RealAcc<V>::Sum v[QV];
 #pragma unroll
-        for (int q = 0; q < QD; ++q) v[q] = acc[q].sum();
-        const double t = to_double(warp_totals<QD>(v));
-        if (lane % (32 / QD) == 0) wred[warp][lane / (32 / QD)] = t;
+        for (int q = 0; q < QV; ++q) {
+            acc[q].renorm();
+            v[q] = acc[q].sum();
+        }
+        const double t = to_double(warp_totals<QV>(v));
+        if (lane % (32 / QV) == 0) wred[warp][lane / (32 / QV)] = t;
     }
     if (MODE == 0) {
+        nrm.renorm();
         typename RealAcc<V>::Sum v[1] = {nrm.sum()};
         const double t = to_double(warp_totals<1>(v));
-        if (lane == 0) wred[warp][QD] = t;
+        if (lane == 0) wred[warp][QV] = t;
     }
     __syncthreads();
-    constexpr int WG = KC / 32;   // warps per group
-    if (tid < nv) {
-        // vector tid: group tid mod NG at slot tid / NG, or the RX groups sharing it at slot A
+    if (tid < nv || (MODE == 0 && tid == SLOT_NRM)) {
+        const bool isn = tid == SLOT_NRM;
+        int s = 0;   // the share that holds vector tid
+        while (!isn && tid >= (nv * (s + 1)) / nvg) ++s;
+        const int q = isn ? QV : tid - (nv * s) / nvg;
         double t = 0.0;
-        const bool whole = tid < NG * A;
-        for (int sv = 0; sv < (whole ? 1 : RX); ++sv) {
-            const int gg = whole ? tid % NG : (tid - NG * A) + Bn * sv, q = whole ? tid / NG : A;
-#pragma unroll
-            for (int w = 0; w < WG; ++w) t += wred[WG * gg + w][q];
+        for (int p = 0; p < nrp; ++p) {
+            const int w = 2 * (p * nvg + (s + (nvg - 1) * p) % nvg);   // the group of share s in row part p
+            t += wred[w][q] + wred[w + 1][q];
         }
         red[tid] = make_double2(t, 0.0);
-    }
-    if (MODE == 0 && tid == 0) {
-        double t = 0.0;
-        for (int sv = 0; sv < (A > 0 ? 1 : RX); ++sv) {
-            const int gg = A > 0 ? 0 : Bn * sv;
-#pragma unroll
-            for (int w = 0; w < WG; ++w) t += wred[WG * gg + w][QD];
-        }
-        red[SLOT_NRM] = make_double2(t, 0.0);
     }
     __syncthreads();
     double2 *fin = red;
@@ -354,7 +342,7 @@ __global__ void __launch_bounds__(NTHR, 2) k_dots(EvArgs<V> a, int jj)
     const bool in = tid <= jj;
     const double s = in ? ctl->sigma[tid] : 0.0;
     const double c = fin[tid].x * s;   // Re <v_i, y>
-    const double c2 = warp_sum(c * c);
+    const double cc = c * c, c2 = warp_sum_int<1>(&cc);
     if (MODE == 0) {
         if (in) ctl->coefA[tid] = c * s;
         if (tid == jj) ctl->alpha[jj] = c;
@@ -660,6 +648,18 @@ __global__ void __launch_bounds__(NTHR) k_grad_acc(DevBasis b, DevHam hm, double
 
 // ---------------------------------------------------------------- launchers
 
+static int sm_count()
+{
+    static int n = 0;
+    if (!n) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (n <= 0) n = 1;
+    }
+    return n;
+}
+
 size_t apply_smem(const DevBasis &b, int rl_smem, int)
 {
     return sizeof(SmemHead) + (rl_smem ? (sizeof(uint16_t) << b.Llo) : 0);
@@ -671,18 +671,6 @@ static int prep_smem(K kernel, size_t smem)
 {
     if (smem > 48 * 1024) KRY_CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return KRY_OK;
-}
-
-static int sm_count()
-{
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 1;
-    }
-    return n;
 }
 
 int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y, int rl_smem,
@@ -716,8 +704,7 @@ int vector_grid(const DevBasis &b, int rl_smem, int hv_form, int *gridH, int *gr
     const size_t smH = apply_smem(b, rlH, es == sizeof(float2));
     if (int rc = prep_smem(k_hv<V, 0>, smH)) return -rc;
     if (int rc = prep_smem(k_hv<V, 1>, smH)) return -rc;
-    int occA = 0, occB = 0, occH = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occA, k_dots<V, 0, 1>, NTHR, 0);
+    int occB = 0, occH = 0;
     if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1>, NTHR, smH);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0>, NTHR, smH);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occB, k_lincomb<V, 0, 2>, NTHR, 0);
@@ -730,7 +717,9 @@ int vector_grid(const DevBasis &b, int rl_smem, int hv_form, int *gridH, int *gr
         if (int rc = list_hv_grid<V>(b, gridH)) return -rc;
     }
     *gridB = fit(occB);
-    return fit(occA);
+    // the dots: one CTA per SM, fewer when there are not two units of 64 threads' rows for each
+    const uint32_t nu = (b.D + 64 * (16 / es) - 1) / (64 * (16 / es));
+    return (int)std::max<uint32_t>(1u, std::min<uint32_t>((nu + 1) / 2, (uint32_t)sm_count()));
 }
 
 template <class V>
@@ -846,9 +835,9 @@ template int launch_ckpt<float2>(const float2 *, float2 *, size_t, KryCtl *, uin
 template <class V>
 int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, int pdl)
 {
-    const int pf = a.dots_form == 0;
-    if (mode == 0) KRY_CU(launch_ex(pdl, pf ? k_dots<V, 0, 1> : k_dots<V, 0, 0>, grid, NTHR, 0, s, a, jj));
-    else KRY_CU(launch_ex(pdl, pf ? k_dots<V, 1, 1> : k_dots<V, 1, 0>, grid, NTHR, 0, s, a, jj));
+    const int mu = a.dots_form == 0;
+    if (mode == 0) KRY_CU(launch_ex(pdl, mu ? k_dots<V, 0, 1> : k_dots<V, 0, 0>, grid, DOTS_NTHR, 0, s, a, jj));
+    else KRY_CU(launch_ex(pdl, mu ? k_dots<V, 1, 1> : k_dots<V, 1, 0>, grid, DOTS_NTHR, 0, s, a, jj));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }

@@ -343,7 +343,7 @@ struct kry_ham_s {
     size_t g_ldo, g_ldc;
     // per precision, the launch shape of the vector kernels (kry_set_shape, kry_autotune):
     // [0] CTAs of the streaming kernels (0 = occupancy rule), [1] H.v form (bit 0: chunks of
-    // eight gathers; bit 1: rank table through L1), [2] dots form (0 prefetch, 1 none), [3]
+    // eight gathers; bit 1: rank table through L1), [2] dots form (0 several units of rows at a time, 1 one), [3]
     // update rows per thread,
     // [4] batched H.v in chunks of this many realisations (0 = all K)
     int shape[3][5];
@@ -358,7 +358,7 @@ struct kry_ham_s {
     int64_t prof_launches[kry::NKIND];
 };
 
-// Launch shape of a new Hamiltonian: the occupancy-rule grid, prefetching dots, two update
+// Launch shape of a new Hamiltonian: the occupancy-rule grid, two update
 // rows per thread, all realisations at once, and the H.v one hop at a time with the
 // lower-bit rank table in shared memory -- except for lower parts of 14 bits or more (L >=
 // 28), whose table (32-64 KB) would cap the H.v at three or four CTAs per SM: there the

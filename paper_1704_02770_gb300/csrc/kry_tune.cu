@@ -5,7 +5,7 @@
 //   [0] CTAs of the streaming kernels: the occupancy rule (0) or 1..4 times the SM count;
 //   [1] H.v form: bit 0 = rounds of four gathers in flight (else one hop at a time), bit 1 =
 //       the lower-bit rank table read through L1 (else staged in shared memory);
-//   [2] dots: prefetching the next vector's rows (0) or not (1);
+//   [2] dots: several units of rows at a time where the vectors are few (0) or one (1);
 //   [3] rows per thread of the update pass: 1, 2 or 4;
 //   [4] batched H.v in chunks of 8 or 16 realisations (0 = all K at once).
 // Parts [1], [2] and [4] change only the order in which independent loads are issued (the

@@ -579,6 +579,40 @@ template <> struct RealLin<ffc> {
     }
 };
 
+// The update's terms i < j - 1.  In exact arithmetic only c_j and c_{j-1} differ from zero; the others
+// are the rounding of the process (about 2^-50 ||u|| in complex128, 2^-45 in float-float) and the
+// subtraction of their multiples keeps the basis orthogonal.  Where sum_{i<j-1} c_i^2 <=
+// (ETA ||u||)^2 they are summed in FP32 and taken off w once: FP32 loses 2^-23 of each term, so
+// at most 2^-23 sqrt(30) ETA ||u|| in all, 2^-60 (complex128) or 2^-56 (float-float) of ||u||, below
+// the rounding of w itself (2^-53, 2^-48); larger coefficients take the full arithmetic.  This moves
+// all but two of the j + 1 terms off the FP64 pipe (two cycles of it per SM, 77 per warp, a
+// multiply-add) and off the 12-instruction float-float products.  Scales 2^-40 <= sigma_i <= 2^40 keep
+// the elements and coefficients inside the FP32 range.
+template <class V> struct MinorSum {
+    static constexpr bool use = false;   // complex64: the full arithmetic is FP32 already
+    static constexpr double eta = 0.0;
+};
+template <> struct MinorSum<double2> {
+    static constexpr bool use = true;
+    static constexpr double eta = 9.094947017729282e-13;   // 2^-40
+    // the leading 24 bits of a double (|x| < 2^128; below 2^-126 gives 0), by integer operations: the
+    // conversion instruction runs at the FP64 rate
+    __device__ __forceinline__ static float lead(double x)
+    {
+        const int hi = __double2hiint(x), v = (hi & 0x7fffffff) - 0x38000000;
+        const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)v, 3);
+        return __uint_as_float((v > 0 ? b : 0u) | ((unsigned)hi & 0x80000000u));
+    }
+    __device__ __forceinline__ static float2 lead(double2 x) { return make_float2(lead(x.x), lead(x.y)); }
+    __device__ __forceinline__ static void add(RealLin<double2> &l, float2 f) { l.w.x += f2d(f.x); l.w.y += f2d(f.y); }
+};
+template <> struct MinorSum<ffc> {
+    static constexpr bool use = true;
+    static constexpr double eta = 1.4551915228366852e-11;   // 2^-36
+    __device__ __forceinline__ static float2 lead(ffc x) { return make_float2(x.xh, x.yh); }
+    __device__ __forceinline__ static void add(RealLin<ffc> &l, float2 f) { l.c = __fadd2_rn(l.c, f); }
+};
+
 // Linear combinations with complex coefficients (the combine psi = beta V y): w -= c x.
 template <class V> struct CplxLin {
     using RCoef = V;

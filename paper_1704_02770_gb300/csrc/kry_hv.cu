@@ -17,7 +17,7 @@
 
 namespace kry {
 
-constexpr int DOTS_NTHR = 512;   // threads of a large CTA of the dots
+constexpr int DOTS_NTHR = 512;   // threads of a CTA of the dots
 
 struct SmemHead {
     uint32_t koff[20];
@@ -106,7 +106,7 @@ __device__ __forceinline__ void cta_sum_into(double2 v, double2 *red, int slot, 
     __syncthreads();
     if (threadIdx.x == 0) {
         double2 s = make_double2(0.0, 0.0);
-        for (int w = 0; w < NTHR / 32; ++w) { s.x += wtmp[w].x; s.y += wtmp[w].y; }
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) { s.x += wtmp[w].x; s.y += wtmp[w].y; }
         red[slot] = s;
     }
     __syncthreads();
@@ -131,7 +131,7 @@ __device__ __forceinline__ void cta_sum_into(const Acc &acc, double2 *red, int s
     __syncthreads();
     if (threadIdx.x == 0) {
         double2 s = make_double2(0.0, 0.0);
-        for (int w = 0; w < NTHR / 32; ++w) { s.x += wtmp[w].x; s.y += wtmp[w].y; }
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) { s.x += wtmp[w].x; s.y += wtmp[w].y; }
         red[slot] = s;
     }
     __syncthreads();
@@ -346,7 +346,16 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
     if (MODE == 0) {
         if (in) ctl->coefA[tid] = c * s;
         if (tid == jj) ctl->alpha[jj] = c;
+        bool minor = false;
+        if (MinorSum<V>::use) {
+            // rounding level: sum_{i<j-1} c_i^2 <= (eta ||u||)^2, with scales inside the FP32 range
+            const bool small = tid + 1 < jj;
+            const double cm = small ? c * c : 0.0, m2 = warp_sum_int<1>(&cm);
+            minor = __all_sync(0xffffffffu, !small || (s >= 0x1p-40 && s <= 0x1p40)) &&
+                    m2 <= MinorSum<V>::eta * MinorSum<V>::eta * fin[SLOT_NRM].x;
+        }
         if (tid != 0) return;
+        ctl->minor = minor ? 1 : 0;
         ctl->c2 = c2;
         ctl->normu2 = fin[SLOT_NRM].x;
         ctl->n_hv += 1;
@@ -393,10 +402,15 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     __shared__ typename Lin::RCoef coef[MMAX + 1];
     __shared__ double2 red[PSTRIDE];
     __shared__ double2 wtmp[NTHR / 32];
+    __shared__ float mcoef[MMAX + 1];
     __shared__ int flag;
     const int tid = threadIdx.x;
+    const uint32_t nt = blockDim.x;
+    // pass B: the first nminor terms are summed in FP32 (MinorSum)
+    const int nminor = MODE == 0 && MinorSum<V>::use && ctl->minor ? max(jj - 1, 0) : 0;
     if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
     if (tid < nvec) {
+        if (MODE == 0) mcoef[tid] = -(float)ctl->coefA[tid];
         if constexpr (RE) coef[tid] = Lin::coef(MODE == 0 ? ctl->coefA[tid] : ctl->coefC[tid]);
         else coef[tid] = Lin::coef(ctl->coefY[tid]);
     }
@@ -406,16 +420,16 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     const uint32_t D = a.b.D;
     RealAcc<V> nrm;
     DotAcc<V> gacc;
-    const uint32_t ntr = (D + RR * TILE - 1) / (RR * TILE);
+    const uint32_t ntr = (D + RR * nt - 1) / (RR * nt);
     for (uint32_t tile = blockIdx.x; tile < ntr; tile += gridDim.x) {
-        const uint32_t r = tile * RR * TILE + tid;
+        const uint32_t r = tile * RR * nt + tid;
         if (r >= D) continue;
         uint32_t q[RR];
         bool in[RR];
 #pragma unroll
         for (int k = 0; k < RR; ++k) {
-            in[k] = r + k * TILE < D;
-            q[k] = in[k] ? r + k * TILE : r;   // past D a row repeats the first, unstored
+            in[k] = r + k * nt < D;
+            q[k] = in[k] ? r + k * nt : r;   // past D a row repeats the first, unstored
         }
         Lin w[RR];
 #pragma unroll
@@ -431,8 +445,27 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
                 for (int k = 0; k < RR; ++k) w[k].fms(coef[i], x[k]);
             }
         } else {
+            if constexpr (MODE == 0 && MinorSum<V>::use) {
+                if (nminor > 0) {
+                    float2 f[RR];
+#pragma unroll
+                    for (int k = 0; k < RR; ++k) f[k] = make_float2(0.f, 0.f);
 #pragma unroll 8
-            for (int i = 0; i < nvec; ++i) {
+                    for (int i = 0; i < nminor; ++i) {
+                        const V *wi = a.W + (size_t)i * a.ldW;
+                        V x[RR];
+#pragma unroll
+                        for (int k = 0; k < RR; ++k) x[k] = ldg(wi + q[k]);
+#pragma unroll
+                        for (int k = 0; k < RR; ++k)
+                            f[k] = __ffma2_rn(make_float2(mcoef[i], mcoef[i]), MinorSum<V>::lead(x[k]), f[k]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < RR; ++k) MinorSum<V>::add(w[k], f[k]);
+                }
+            }
+#pragma unroll 8
+            for (int i = nminor; i < nvec; ++i) {
                 const V *wi = a.W + (size_t)i * a.ldW;
                 V x[RR];
 #pragma unroll
@@ -660,6 +693,10 @@ static int sm_count()
     return n;
 }
 
+// Threads of a CTA of the updates: 64 in sectors whose rows, at two per thread, would not give every SM
+// two CTAs of 256 (D < 155,648 on 152 SMs), so that more SMs share them.
+static int lincomb_threads(uint32_t D) { return D < (uint32_t)sm_count() * 4u * NTHR ? 64 : NTHR; }
+
 size_t apply_smem(const DevBasis &b, int rl_smem, int)
 {
     return sizeof(SmemHead) + (rl_smem ? (sizeof(uint16_t) << b.Llo) : 0);
@@ -716,7 +753,8 @@ int vector_grid(const DevBasis &b, int rl_smem, int hv_form, int *gridH, int *gr
     if (b.list) {
         if (int rc = list_hv_grid<V>(b, gridH)) return -rc;
     }
-    *gridB = fit(occB);
+    // (the updates of small sectors: CTAs of 64 threads, two rows each)
+    *gridB = lincomb_threads(b.D) == NTHR ? fit(occB) : (int)std::max<uint32_t>(1u, std::min<uint32_t>((b.D + 127) / 128, (uint32_t)sm_count() * 4u));
     // the dots: one CTA per SM, fewer when there are not two units of 64 threads' rows for each
     const uint32_t nu = (b.D + 64 * (16 / es) - 1) / (64 * (16 / es));
     return (int)std::max<uint32_t>(1u, std::min<uint32_t>((nu + 1) / 2, (uint32_t)sm_count()));
@@ -737,10 +775,11 @@ int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 template <class V, int MODE, int COND>
 static cudaError_t launch_lincomb_rr(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
+    const int nt = lincomb_threads(a.b.D);
     switch (a.upd_rows) {
-    case 1: return launch_ex(pdl, k_lincomb<V, MODE, 1, COND>, grid, NTHR, 0, s, a, jj);
-    case 4: return launch_ex(pdl, k_lincomb<V, MODE, 4, COND>, grid, NTHR, 0, s, a, jj);
-    default: return launch_ex(pdl, k_lincomb<V, MODE, 2, COND>, grid, NTHR, 0, s, a, jj);
+    case 1: return launch_ex(pdl, k_lincomb<V, MODE, 1, COND>, grid, nt, 0, s, a, jj);
+    case 4: return launch_ex(pdl, k_lincomb<V, MODE, 4, COND>, grid, nt, 0, s, a, jj);
+    default: return launch_ex(pdl, k_lincomb<V, MODE, 2, COND>, grid, nt, 0, s, a, jj);
     }
 }
 
@@ -753,8 +792,8 @@ int launch_lincomb(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t 
         else KRY_CU((launch_lincomb_rr<V, 0, 0>(a, jj, grid, s, pdl)));
         break;
     case 1: KRY_CU((launch_lincomb_rr<V, 1, 0>(a, jj, grid, s, pdl))); break;
-    case 2: KRY_CU(launch_ex(pdl, k_lincomb<V, 2, 2>, grid, NTHR, 0, s, a, jj)); break;
-    default: KRY_CU(launch_ex(pdl, k_lincomb<V, 3, 2>, grid, NTHR, 0, s, a, jj)); break;
+    case 2: KRY_CU(launch_ex(pdl, k_lincomb<V, 2, 2>, grid, lincomb_threads(a.b.D), 0, s, a, jj)); break;
+    default: KRY_CU(launch_ex(pdl, k_lincomb<V, 3, 2>, grid, lincomb_threads(a.b.D), 0, s, a, jj)); break;
     }
     KRY_CU(cudaGetLastError());
     return KRY_OK;

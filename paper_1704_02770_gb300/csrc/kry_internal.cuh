@@ -202,6 +202,7 @@ struct KryCtl {
     double2 g[MMAX + 2];       // readout <psi0, v_i>
     double normu2;             // ||H v_j||^2 of the last pass A
     double c2;                 // ||V^H H v_j||^2 of the last pass A (Pythagoras test of pass B)
+    int minor;                 // coefA[0 .. j - 2] are at rounding level (MinorSum)
     double beta0;              // ||psi|| at the start of the Krylov step
     double t_now, t_end, tol, tau_prev;
     double eta_corr, eta_bd;   // second-pass and breakdown thresholds (relative)

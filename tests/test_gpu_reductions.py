@@ -53,17 +53,19 @@ def test_general_state_against_eigh(kry, L, N, emulated):
         assert np.linalg.norm(out64.cpu().numpy() - exact) <= 1e-5
 
 
-@pytest.mark.parametrize("scale", [1e-30, 1e-4, 1.0, 1e4])
-def test_sums_scale_with_the_state(kry, scale):
-    """The integer sums align to the largest value, so an unnormalised state loses nothing: P scales
-    with the fourth power of the norm."""
+@pytest.mark.parametrize("emulated,scale", [(False, 1e-30), (False, 1e-4), (False, 1.0), (False, 1e4),
+                                             (True, 1e-8), (True, 1e4)])
+def test_sums_scale_with_the_state(kry, emulated, scale):
+    """The integer sums align to the largest value, and the update sums its rounding-level terms in FP32
+    only where the vectors' scales fit (2^-40 to 2^40), so an unnormalised state loses nothing: P
+    scales with the fourth power of the norm.  (A float-float value below 2^-80 is zero.)"""
     L, N = 11, 5
     h, Hc, psi0 = _case(L, N)
     H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.8, h)
     x = torch.from_numpy(psi0).cuda()
-    P1, _ = H.evolve(x, [0.5, 2.0], tol=1e-10)
+    P1, _ = H.evolve(x, [0.5, 2.0], tol=1e-10, emulated=emulated)
     # (the budget is absolute: 1e-10 of the unit state is 1e-10 s of one with norm s, and P is its square)
-    P, _ = H.evolve(x * scale, [0.5, 2.0], tol=max(1e-10 * scale, 1e-200))
+    P, _ = H.evolve(x * scale, [0.5, 2.0], tol=1e-10 * scale, emulated=emulated)
     assert np.max(np.abs(P / scale**4 - P1)) <= 1e-9
 
 

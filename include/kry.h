@@ -233,10 +233,9 @@ int kry_profile_read(kry_ham H, double *ms, double *bytes, int64_t *launches);
  * dtype, five ints:
  *   shape[0] CTAs of the streaming kernels: 0 = the occupancy rule (whole SMs times the
  *            resident CTAs of each kernel), else that many CTAs;
- *   shape[1] form of the H.v, two bits: bit 0 set = the targets of up to four hops computed
- *            first and their loads issued together (else one hop at a time); bit 1 set = the
- *            lower-bit rank table read through the L1 cache instead of staged in shared memory
- *            (at L = 29, 30 that table takes 64 KB of shared memory per CTA);
+ *   shape[1] form of the H.v, two bits: bit 0 set = the loads of eight hops issued together
+ *            (16-byte elements: of two), else of four; bit 1 set = twice as many blocks of upper
+ *            bits share the work on one lower part;
  *   shape[2] dots of pass A: 0 = two or four units of rows loaded at a time where a thread has
  *            few vectors, 1 = always one;
  *   shape[3] rows per thread of the update pass: 1, 2 or 4;
@@ -246,7 +245,7 @@ int kry_profile_read(kry_ham H, double *ms, double *bytes, int64_t *launches);
  * same); parts 0 and 3 change which rows a thread or CTA sums into its partial norms and dots
  * (the results agree to rounding).  Single-realisation evolutions use parts 0-3, batched ones
  * parts 0 and 4.  New Hamiltonians start at {0, 0, 0, 2, 0}, or {0, 3, 0, 2, 0} for L >= 28
- * (split-table bases), where the rank table of the lower bits is 32-64 KB.
+ * (split-table bases).
  * kry_set_shape returns KRY_EINVAL for values outside those lists; kry_set_grid sets part 0. */
 int kry_set_shape(kry_ham H, int dtype, const int *shape);
 int kry_get_shape(kry_ham H, int dtype, int *shape);

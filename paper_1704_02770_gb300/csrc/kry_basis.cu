@@ -194,6 +194,13 @@ extern "C" int kry_basis_create(int L, int n_up, kry_basis *out)
             lolist[fill[k]++] = (uint16_t)lo;
         }
     }
+    // upper-bit patterns by popcount, ascending within (Lhi <= 16)
+    std::vector<uint16_t> hilist(nhi);
+    {
+        std::vector<uint32_t> fill(Lhi + 2, 0);
+        for (int k = 0; k <= Lhi; ++k) fill[k + 1] = fill[k] + (uint32_t)binom64(Lhi, k);
+        for (uint32_t hi = 0; hi < nhi; ++hi) hilist[fill[__builtin_popcount(hi)]++] = (uint16_t)hi;
+    }
     // block starts: valid blocks in increasing hi are contiguous in rank order
     const uint32_t INV = 0xFFFFFFFFu;
     uint64_t expect = 0;
@@ -234,7 +241,8 @@ extern "C" int kry_basis_create(int L, int n_up, kry_basis *out)
     // device upload: one allocation holding every table and the error flag
     size_t o_blk = 0, o_rl = o_blk + sizeof(uint32_t) * nhi;
     size_t o_ll = o_rl + sizeof(uint16_t) * nlo;
-    size_t o_ko = (o_ll + sizeof(uint16_t) * nlo + 15) & ~(size_t)15;
+    size_t o_hl = o_ll + sizeof(uint16_t) * nlo;
+    size_t o_ko = (o_hl + sizeof(uint16_t) * nhi + 15) & ~(size_t)15;
     size_t o_bs = o_ko + sizeof(uint32_t) * (Llo + 2);
     size_t o_er = (o_bs + sizeof(uint32_t) * (Llo + 1) + 15) & ~(size_t)15;
     size_t o_ts = o_er + 16;
@@ -250,6 +258,7 @@ extern "C" int kry_basis_create(int L, int n_up, kry_basis *out)
         {o_blk, blk.data(), sizeof(uint32_t) * nhi},
         {o_rl, ranklo.data(), sizeof(uint16_t) * nlo},
         {o_ll, lolist.data(), sizeof(uint16_t) * nlo},
+        {o_hl, hilist.data(), sizeof(uint16_t) * nhi},
         {o_ko, koff.data(), sizeof(uint32_t) * (Llo + 2)},
         {o_bs, bsz.data(), sizeof(uint32_t) * (Llo + 1)},
         {o_ts, tstart.data(), sizeof(uint32_t) * tstart.size()},
@@ -263,6 +272,7 @@ extern "C" int kry_basis_create(int L, int n_up, kry_basis *out)
     d.tstart = (const uint32_t *)(base + o_ts);
     d.ranklo = (const uint16_t *)(base + o_rl);
     d.lolist = (const uint16_t *)(base + o_ll);
+    d.hilist = (const uint16_t *)(base + o_hl);
     d.koff = (const uint32_t *)(base + o_ko);
     d.bsz = (const uint32_t *)(base + o_bs);
     d.err = (int *)(base + o_er);

@@ -2,6 +2,8 @@
 // complex arithmetic and dot-product accumulators.
 #pragma once
 
+#include <type_traits>
+
 #include "kry_internal.cuh"
 
 namespace kry {
@@ -106,6 +108,30 @@ __device__ __forceinline__ ffc ldg(const ffc *p)
 __device__ __forceinline__ float2 ldg(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ double2 ldg(const double2 *p) { return __ldg(p); }
 
+// *a where p holds, else zero, as one predicated load (a branch around a load costs more than the load)
+__device__ __forceinline__ float2 ldg_if(bool p, const float2 *a)
+{
+    float2 v;
+    asm("{.reg .pred q; setp.ne.s32 q, %3, 0; mov.b32 %0, 0; mov.b32 %1, 0; @q ld.global.nc.v2.f32 {%0, %1}, [%2];}"
+        : "=&f"(v.x), "=&f"(v.y) : "l"(a), "r"((int)p));
+    return v;
+}
+__device__ __forceinline__ double2 ldg_if(bool p, const double2 *a)
+{
+    double2 v;
+    asm("{.reg .pred q; setp.ne.s32 q, %3, 0; mov.b64 %0, 0; mov.b64 %1, 0; @q ld.global.nc.v2.f64 {%0, %1}, [%2];}"
+        : "=&d"(v.x), "=&d"(v.y) : "l"(a), "r"((int)p));
+    return v;
+}
+__device__ __forceinline__ ffc ldg_if(bool p, const ffc *a)
+{
+    ffc v;
+    asm("{.reg .pred q; setp.ne.s32 q, %5, 0; mov.b32 %0, 0; mov.b32 %1, 0; mov.b32 %2, 0; mov.b32 %3, 0; "
+        "@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];}"
+        : "=&f"(v.xh), "=&f"(v.yh), "=&f"(v.xl), "=&f"(v.yl) : "l"(a), "r"((int)p));
+    return v;
+}
+
 // the 16 bytes at p (16-byte aligned): one element, or two of complex64
 __device__ __forceinline__ void ldg_chunk(const float2 *p, float2 *dst)
 {
@@ -151,15 +177,71 @@ __device__ __forceinline__ float2 axpby(float d, float2 x, float s, float2 a)
     return make_float2(fmaf(d, x.x, s * a.x), fmaf(d, x.y, s * a.y));
 }
 // neighbour sums of the H.v row: acc += v, then y = sd x + shj acc
-template <class V> __device__ __forceinline__ void hv_add(V &acc, V v) { acc = acc + v; }
+__device__ __forceinline__ void hv_add(double2 &acc, double2 v) { acc = acc + v; }
+__device__ __forceinline__ void hv_add(float2 &acc, float2 v) { acc = __fadd2_rn(acc, v); }
 __device__ __forceinline__ void hv_add(FF4 &acc, ffc v)
 {
     ff_combine(acc.sr, acc.cr, v.xh, v.xl);
     ff_combine(acc.si, acc.ci, v.yh, v.yl);
 }
-__device__ __forceinline__ double2 axpby(double d, double2 x, double s, double2 a);
-__device__ __forceinline__ float2 axpby(float d, float2 x, float s, float2 a);
+// acc += v[0] + ... + v[N - 1]
+template <int N, class S, class V> __device__ __forceinline__ void hv_add_n(S &acc, const V *v)
+{
+#pragma unroll
+    for (int u = 0; u < N; ++u) hv_add(acc, v[u]);
+}
+// Neighbour sums of complex128 on 64-bit integers: the mantissas are aligned to the largest exponent
+// seen so far (the sums so far shifted along when it grows), with 5 bits of fraction below and room
+// for 32 terms above.  Each term loses less than 2^-57 of the largest, an FP64 sum 2^-53 of the running
+// one, and a term takes about 14 integer instructions per component where an FP64 add takes the pipe
+// for 77 issue cycles (L = 24: 213 us with FP64 adds, the kernel's bound).
+struct ISum2 {
+    long long re = 0, im = 0;
+    unsigned em = 0;
+    __device__ __forceinline__ static unsigned ex(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu; }
+    __device__ __forceinline__ static long long align(double x, unsigned em)
+    {
+        const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), e = (hi >> 20) & 0x7ffu;
+        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 5;
+        const unsigned d = em - e;
+        const long long q = e == 0u || d > 63u ? 0ll : (long long)(m >> d);
+        return (int)hi < 0 ? -q : q;
+    }
+    // exponents the scale cannot hold, infinities and NaN: the caller sums the row in FP64
+    __device__ __forceinline__ bool special() const { return em == 0x7ffu || (em != 0u && em < 128u); }
+    __device__ __forceinline__ double2 value() const
+    {
+        if (em == 0u) return make_double2(0.0, 0.0);
+        const double f = __hiloint2double((int)(em - 1080u + 1023u) << 20, 0);   // 2^(em - 1075 - 5)
+        return make_double2((double)re * f, (double)im * f);
+    }
+};
+// (two terms at a time whatever N, so that the bits do not depend on how many are loaded together)
+template <int N> __device__ __forceinline__ void hv_add_n(ISum2 &acc, const double2 *v)
+{
+#pragma unroll
+    for (int u0 = 0; u0 < N; u0 += 2) {
+        constexpr int M = N < 2 ? 1 : 2;
+        unsigned em = acc.em;
+#pragma unroll
+        for (int u = u0; u < u0 + M; ++u) em = max(em, max(ISum2::ex(v[u].x), ISum2::ex(v[u].y)));
+        const unsigned d = min(em - acc.em, 63u);
+        acc.re >>= d;
+        acc.im >>= d;
+        acc.em = em;
+#pragma unroll
+        for (int u = u0; u < u0 + M; ++u) {
+            acc.re += ISum2::align(v[u].x, em);
+            acc.im += ISum2::align(v[u].y, em);
+        }
+    }
+}
+__device__ __forceinline__ void hv_add(ISum2 &acc, double2 v) { hv_add_n<1>(acc, &v); }
 template <class V, class R> __device__ __forceinline__ V hv_finish(R sd, V x, R shj, V acc) { return axpby(sd, x, shj, acc); }
+__device__ __forceinline__ double2 hv_finish(double sd, double2 x, double shj, const ISum2 &acc)
+{
+    return axpby(sd, x, shj, acc.value());
+}
 __device__ __forceinline__ ffc hv_finish(double sd, ffc x, double shj, const FF4 &acc)
 {
     const float2 d = dsplit(sd), h = dsplit(shj);
@@ -676,177 +758,138 @@ __device__ __forceinline__ void stage_tables(const DevBasis &b, uint32_t *koff_s
 }
 
 // ---------------------------------------------------------------- matrix-free H.v
-// Row r of H x for the state s = (hi << Llo) | lo (Eq. 1, XXZ form):
+// Row r of sigma H x for the state s = (hi << Llo) | lo (Eq. 1, XXZ form):
 //   (H x)[r] = d(s) x[r] + (J/2) sum_{antiparallel bonds b} x[rank(s ^ bondmask_b)],
-//   d(s) = (J Delta / 4)(nbonds - 2 n_anti(s)) + sum_i h_i (n_i - 1/2).
-// Pull form (one writer per row, no atomics).  The re-rank of a hopped state takes two
-// table lookups; a hop inside the upper part keeps the lower bits, so its target is
-// blk[hi'] + off and the lanes of one block read consecutive elements.
-template <class V>
-__device__ __forceinline__ V hv_row(const DevBasis &b, const DevHam &hm, const V *__restrict__ x,
-                                    uint32_t hi, uint32_t off, int klo, const uint32_t *koff_s,
-                                    const uint16_t *rl)
-{
-    using R = typename VT<V>::R;
-    const int Llo = b.Llo, L = b.L;
-    const uint32_t pos = koff_s[klo] + off;
-    const uint32_t lo = __ldg(b.lolist + pos);
-    const uint32_t s = (hi << Llo) | lo;
-    const uint32_t base = __ldg(b.blk + hi);
-    const uint32_t lomask = (1u << Llo) - 1u;
-    const uint32_t obc = (L >= 2) ? ((1u << (L - 1)) - 1u) : 0u;
-    const uint32_t anti = (s ^ (s >> 1)) & obc;
-    const uint32_t wrap = hm.pbc ? ((s ^ (s >> (L - 1))) & 1u) : 0u;
-    const int nanti = __popc(anti) + (int)wrap;
-    const R d = (R)hm.cz * (R)(hm.nbonds - 2 * nanti) + VT<V>::ehlo(hm, pos) + VT<V>::ehhi(hm, hi);
-    V acc = VT<V>::zero();
-    uint32_t a = anti & ((1u << (Llo - 1)) - 1u);          // bonds inside the lower part
-    while (a) {
-        const int p = __ffs(a) - 1;
-        a &= a - 1u;
-        acc = acc + __ldg(x + base + rl[lo ^ (3u << p)]);
-    }
-    if (b.Lhi > 0 && ((anti >> (Llo - 1)) & 1u)) {         // bond joining the two parts
-        const uint32_t s2 = s ^ (3u << (Llo - 1));
-        acc = acc + __ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]);
-    }
-    uint32_t ah = anti >> Llo;                              // bonds inside the upper part
-    while (ah) {
-        const int q = __ffs(ah) - 1;
-        ah &= ah - 1u;
-        acc = acc + __ldg(x + __ldg(b.blk + (hi ^ (3u << q))) + off);
-    }
-    if (wrap) {                                             // ring bond (L-1, 0)
-        const uint32_t s2 = s ^ ((1u << (L - 1)) | 1u);
-        acc = acc + __ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]);
-    }
-    return axpby(d, __ldg(x + base + off), (R)hm.halfJ, acc);
-}
+//   d(s) = (J Delta / 4)(nbonds - 2 n_anti(s)) + sum_i h_i (n_i - 1/2),
+// with sigma folded into the two factors and the bond energy read from a table dz[n_anti].
+// Pull form, one writer per row, no atomics.  Rows of upper parts hi with the same particle number
+// have the same list of lower parts, so a warp takes an item: 32 consecutive lower parts (one per
+// lane) of NH such blocks.  What depends on lo alone -- the ranks of its hops, rl[lo ^ (3 << p)] --
+// is found once per item and serves NH rows; what depends on hi alone -- the block starts of its hops
+// -- is found once per item by one lane per (block, bond) and shared.  A row then costs about four
+// instructions a hop (a predicated load at block start + rank, and the add) and no unranking.
+// A per-row form (unrank, then a loop over the row's hops) took 404 instructions per row at L = 24
+// and 533 at L = 28, was bound by their issue (59% active) and took 51 us (L = 24 c64).
+// The terms of a row are added in bond order, the ring bond last.
+constexpr int HV_NH = 8;        // blocks of an item, at most
+constexpr int HV_NTHR = 256;    // threads of a CTA of the H.v
 
-// sigma (H x)[r] for the row of hv_row, with the bond energy read from a table
-// dz[n] = (J Delta / 4)(nbonds - 2 n) and sigma folded into the two factors:
-//   sigma (d x_r + (J/2) acc) = (sigma d) x_r + (sigma J/2) acc.
-template <class V>
-__device__ __forceinline__ V hv_row_scaled(const DevBasis &b, const DevHam &hm, const V *__restrict__ x,
-                                           uint32_t hi, uint32_t off, int klo, const uint32_t *koff_s,
-                                           const uint16_t *rl, const typename VT<V>::R *dz,
-                                           typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ)
-{
-    using R = typename VT<V>::R;
-    const int Llo = b.Llo, L = b.L;
-    const uint32_t pos = koff_s[klo] + off;
-    const uint32_t lo = __ldg(b.lolist + pos);
-    const uint32_t s = (hi << Llo) | lo;
-    const uint32_t base = __ldg(b.blk + hi);
-    const uint32_t lomask = (1u << Llo) - 1u;
-    const uint32_t obc = (L >= 2) ? ((1u << (L - 1)) - 1u) : 0u;
-    const uint32_t anti = (s ^ (s >> 1)) & obc;
-    const uint32_t wrap = hm.pbc ? ((s ^ (s >> (L - 1))) & 1u) : 0u;
-    const R d = dz[__popc(anti) + (int)wrap] + VT<V>::ehlo(hm, pos) + VT<V>::ehhi(hm, hi);
-    typename Arith<V>::HvSum acc{};
-    uint32_t a = anti & ((1u << (Llo - 1)) - 1u);          // bonds inside the lower part
-    while (a) {
-        const int p = __ffs(a) - 1;
-        a &= a - 1u;
-        hv_add(acc, ldg(x + base + rl[lo ^ (3u << p)]));
-    }
-    if (b.Lhi > 0 && ((anti >> (Llo - 1)) & 1u)) {         // bond joining the two parts
-        const uint32_t s2 = s ^ (3u << (Llo - 1));
-        hv_add(acc, ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]));
-    }
-    uint32_t ah = anti >> Llo;                              // bonds inside the upper part
-    while (ah) {
-        const int q = __ffs(ah) - 1;
-        ah &= ah - 1u;
-        hv_add(acc, ldg(x + __ldg(b.blk + (hi ^ (3u << q))) + off));
-    }
-    if (wrap) {                                             // ring bond (L-1, 0)
-        const uint32_t s2 = s ^ ((1u << (L - 1)) | 1u);
-        hv_add(acc, ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]));
-    }
-    return hv_finish(sigma * d, ldg(x + base + off), sigma_halfJ, acc);
-}
+// Items by the particle number c of the upper part (its lower part has N - c).
+struct HvPlan {
+    uint32_t first[18];   // first item of class c
+    uint32_t hoff[18];    // first entry of class c in hilist
+    uint32_t nlo[17];     // lower parts of class c
+    uint32_t koff[17];    // their first position in lolist
+    int nh;               // blocks per item
+};
+struct HvWarp {   // shared memory of a warp
+    int steps[HV_NH][16];   // per block: block-start steps of its antiparallel upper bonds, packed
+    uint32_t hi[HV_NH], base[HV_NH], cross[HV_NH], ring[HV_NH];
+    int n[HV_NH];
+};
 
-// The same row as hv_row_scaled with the gathers issued in rounds: the targets of up to
-// RND hops are computed first (taking the antiparallel bonds in ascending order) and
-// their loads issued together, so a thread has up to RND gathers in flight instead of one
-// (a warp issues in order, and the loop of hv_row_scaled waits for each gathered value
-// before it computes the next target).  The terms are added in the same order as in
-// hv_row_scaled, so the result is bitwise the same.
-template <class V, int RND = 4>
-__device__ __forceinline__ V hv_row_chunked(const DevBasis &b, const DevHam &hm, const V *__restrict__ x,
-                                            uint32_t hi, uint32_t off, int klo, const uint32_t *koff_s,
-                                            const uint16_t *rl, const typename VT<V>::R *dz,
-                                            typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ)
+template <class V, int RND>
+__device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, const HvPlan &pl, const V *__restrict__ x,
+                                         V *__restrict__ y, HvWarp &w, const typename VT<V>::R *dz,
+                                         typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ)
 {
     using R = typename VT<V>::R;
-    const int Llo = b.Llo, L = b.L;
-    const uint32_t pos = koff_s[klo] + off;
-    const uint32_t lo = __ldg(b.lolist + pos);
-    const uint32_t s = (hi << Llo) | lo;
-    const uint32_t base = __ldg(b.blk + hi);
-    const uint32_t lomask = (1u << Llo) - 1u;
-    const uint32_t obc = (L >= 2) ? ((1u << (L - 1)) - 1u) : 0u;
-    const uint32_t anti = (s ^ (s >> 1)) & obc;
-    const uint32_t wrap = hm.pbc ? ((s ^ (s >> (L - 1))) & 1u) : 0u;
-    const R d = dz[__popc(anti) + (int)wrap] + VT<V>::ehlo(hm, pos) + VT<V>::ehhi(hm, hi);
-    const V xr = ldg(x + base + off);
-    typename Arith<V>::HvSum acc{};
-    uint32_t a = anti & ((1u << (Llo - 1)) - 1u);          // bonds inside the lower part
-    while (a) {
-        uint32_t t[RND];
-        int n = 0;
+    const int Llo = b.Llo, Lhi = b.Lhi, nlb = Llo - 1, lane = threadIdx.x & 31;
+    const uint32_t total = pl.first[Lhi + 1], nw = blockDim.x >> 5;
+    int c = 0;
+    for (uint32_t item = blockIdx.x * nw + (threadIdx.x >> 5); item < total; item += gridDim.x * nw) {
+        while (item >= pl.first[c + 1]) ++c;
+        const uint32_t nlo = pl.nlo[c], nch = (nlo + 31u) >> 5, rem = item - pl.first[c], g = rem / nch;
+        const uint32_t i = (rem - g * nch) * 32u + lane;   // this lane's lower part
+        const uint32_t h0 = pl.hoff[c] + g * pl.nh;
+        const int nh = min((uint32_t)pl.nh, pl.hoff[c + 1] - h0);
+        // lower part
+        const bool valid = i < nlo;
+        const uint32_t pos = pl.koff[c] + (valid ? i : 0u), lo = __ldg(b.lolist + pos);
+        // upper parts: half a warp per block, lane q for bond q
+        __syncwarp();
+        for (int j = 0; j < nh; j += 2) {
+            const int hh = j + (lane >> 4), q = lane & 15;
+            const bool on = hh < nh;
+            const uint32_t hi = on ? __ldg(b.hilist + h0 + hh) : 0u;
+            const bool aq = on && q < Lhi - 1 && (((hi ^ (hi >> 1)) >> q) & 1u);
+            const uint32_t base = __ldg(b.blk + hi);
+            const uint32_t to = aq ? __ldg(b.blk + (hi ^ (3u << q))) : 0u;
+            const unsigned am = (__ballot_sync(0xffffffffu, aq) >> (lane & 16)) & 0xffffu;
+            if (aq) w.steps[hh][__popc(am & ((1u << q) - 1u))] = (int)(to - base);
+            if (on && q == 0) {
+                w.hi[hh] = hi;
+                w.base[hh] = base;
+                w.n[hh] = __popc(am);
+            }
+            if (on && q == 1 && Lhi > 0) w.cross[hh] = __ldg(b.blk + (hi ^ 1u));
+            if (on && q == 2 && Lhi > 0) w.ring[hh] = __ldg(b.blk + (hi ^ (1u << (Lhi - 1))));
+        }
+        const R eh = VT<V>::ehlo(hm, pos);
+        const uint32_t anti = valid ? (lo ^ (lo >> 1)) & ((1u << nlb) - 1u) : 0u;
+        const uint32_t lomask = (1u << Llo) - 1u;
+        uint32_t t[16];   // ranks of the lower part's hops (any pattern has one)
 #pragma unroll
-        for (int u = 0; u < RND; ++u) {
-            if (a) {
-                const int p = __ffs(a) - 1;
-                a &= a - 1u;
-                t[u] = base + rl[lo ^ (3u << p)];
-                n = u + 1;
+        for (int p0 = 0; p0 < 16; p0 += 4) {
+            if (p0 < nlb) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) t[p0 + u] = __ldg(b.ranklo + ((lo ^ (3u << (p0 + u))) & lomask));
             }
         }
-        V v[RND];
+        const uint32_t tc = __ldg(b.ranklo + (lo ^ (1u << nlb))), tr = __ldg(b.ranklo + (lo ^ 1u));
+        __syncwarp();
+#pragma unroll 1
+        for (int h = 0; h < nh; ++h) {
+            const uint32_t hi = w.hi[h], base = w.base[h];
+            const int n = w.n[h];
+            const V *xb = x + base, *xr = xb + i;
+            const bool pc = valid && Lhi > 0 && (((lo >> nlb) ^ hi) & 1u);                         // joining bond
+            const bool pr = valid && hm.pbc && Lhi > 0 && (((hi >> (Lhi - 1)) ^ lo) & 1u);         // ring bond
+            const V x0 = ldg_if(valid, xr);
+            auto neighbours = [&](auto &acc) {
+                const V vc = ldg_if(pc, x + w.cross[h] + tc), vr = ldg_if(pr, x + w.ring[h] + tr);
 #pragma unroll
-        for (int u = 0; u < RND; ++u)
-            if (u < n) v[u] = ldg(x + t[u]);
+                for (int p0 = 0; p0 < 16; p0 += RND) {
+                    if (p0 < nlb) {
+                        V v[RND];
 #pragma unroll
-        for (int u = 0; u < RND; ++u)
-            if (u < n) hv_add(acc, v[u]);
-    }
-    const bool cross = b.Lhi > 0 && ((anti >> (Llo - 1)) & 1u);   // bond joining the two parts
-    V vc = VT<V>::zero(), vr = VT<V>::zero();
-    if (cross) {
-        const uint32_t s2 = s ^ (3u << (Llo - 1));
-        vc = ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]);
-    }
-    if (wrap) {                                                    // ring bond (L-1, 0)
-        const uint32_t s2 = s ^ ((1u << (L - 1)) | 1u);
-        vr = ldg(x + __ldg(b.blk + (s2 >> Llo)) + rl[s2 & lomask]);
-    }
-    if (cross) hv_add(acc, vc);
-    uint32_t ah = anti >> Llo;                                     // bonds inside the upper part
-    while (ah) {
-        uint32_t t[RND];
-        int n = 0;
-#pragma unroll
-        for (int u = 0; u < RND; ++u) {
-            if (ah) {
-                const int q = __ffs(ah) - 1;
-                ah &= ah - 1u;
-                t[u] = __ldg(b.blk + (hi ^ (3u << q)));
-                n = u + 1;
+                        for (int u = 0; u < RND; ++u) v[u] = ldg_if(anti & (1u << (p0 + u)), xb + t[p0 + u]);
+                        hv_add_n<RND>(acc, v);
+                    }
+                }
+                hv_add(acc, vc);
+#pragma unroll 1
+                for (int i0 = 0; i0 < n; i0 += 4) {
+                    const int4 d = *(const int4 *)(w.steps[h] + i0);   // (entries past n are not used)
+                    V v[4];
+                    v[0] = ldg_if(valid, xr + d.x);
+                    v[1] = ldg_if(valid && i0 + 1 < n, xr + d.y);
+                    v[2] = ldg_if(valid && i0 + 2 < n, xr + d.z);
+                    v[3] = ldg_if(valid && i0 + 3 < n, xr + d.w);
+                    hv_add_n<4>(acc, v);
+                }
+                hv_add(acc, vr);
+            };
+            const R d = dz[__popc(anti) + n + (int)pc + (int)pr] + eh + VT<V>::ehhi(hm, hi);
+            V out;
+            if constexpr (std::is_same<V, double2>::value) {   // on aligned integers, in FP64 where they cannot
+                ISum2 acc{};
+                neighbours(acc);
+                if (__any_sync(0xffffffffu, acc.special())) {
+                    double2 a2 = VT<V>::zero();
+                    neighbours(a2);
+                    out = hv_finish(sigma * d, x0, sigma_halfJ, a2);
+                } else {
+                    out = hv_finish(sigma * d, x0, sigma_halfJ, acc);
+                }
+            } else {
+                typename Arith<V>::HvSum acc{};
+                neighbours(acc);
+                out = hv_finish(sigma * d, x0, sigma_halfJ, acc);
             }
+            if (valid) y[base + i] = out;
         }
-        V v[RND];
-#pragma unroll
-        for (int u = 0; u < RND; ++u)
-            if (u < n) v[u] = ldg(x + t[u] + off);
-#pragma unroll
-        for (int u = 0; u < RND; ++u)
-            if (u < n) hv_add(acc, v[u]);
     }
-    if (wrap) hv_add(acc, vr);
-    return hv_finish(sigma * d, xr, sigma_halfJ, acc);
 }
 
 }  // namespace kry

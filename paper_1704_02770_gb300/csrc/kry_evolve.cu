@@ -128,14 +128,13 @@ struct EvOpts {
 int grid_for(const kry_ham_s *H, int dtype, int *gridH, int *gridB)
 {
     const DevBasis &b = H->b->dev;
-    const int rl = rl_in_smem(b);
     const int hvf = H->shape[dtype_slot(dtype)][1];
-    const int g = dtype == KRY_C64    ? vector_grid<float2>(b, rl, hvf, gridH, gridB)
-                  : dtype == KRY_C128E ? vector_grid<ffc>(b, rl, hvf, gridH, gridB)
-                                       : vector_grid<double2>(b, rl, hvf, gridH, gridB);
+    const int g = dtype == KRY_C64    ? vector_grid<float2>(b, hvf, gridH, gridB)
+                  : dtype == KRY_C128E ? vector_grid<ffc>(b, hvf, gridH, gridB)
+                                       : vector_grid<double2>(b, hvf, gridH, gridB);
     const int ov = H->shape[dtype_slot(dtype)][0];
     if (g > 0 && ov > 0) *gridB = ov;
-    return (g > 0 && ov > 0) ? ov : g;   // vector_grid also sets the kernels' smem limits
+    return (g > 0 && ov > 0) ? ov : g;
 }
 
 void drop_graph(kry_ham_s *H)
@@ -299,7 +298,6 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
     a.G = general ? (const V *)(base + l.oG) : nullptr;
     a.part = (double2 *)(base + l.oPart);
     a.ctl = (KryCtl *)(base + l.oCtl);
-    a.rl_smem = rl_in_smem(b);
     const int *shp = H->shape[dtype_slot(dtype)];
     a.hv_form = shp[1];
     a.dots_form = shp[2];
@@ -842,7 +840,7 @@ extern "C" int kry_apply(kry_ham H, int dtype, const void *d_x, void *d_y, void 
     const DevBasis &b = H->b->dev;
     if (H->K > 1)
         return launch_apply_b(b, H->dev, dtype == KRY_C64, H->K, d_x, d_y, rl_in_smem(b), (cudaStream_t)stream);
-    return launch_apply(b, H->dev, dtype == KRY_C64, d_x, d_y, rl_in_smem(b), (cudaStream_t)stream);
+    return launch_apply(b, H->dev, dtype == KRY_C64, d_x, d_y, (cudaStream_t)stream);
 }
 
 extern "C" int kry_evolve(kry_ham H, int dtype, const void *d_psi0, const double *times, int n_times,

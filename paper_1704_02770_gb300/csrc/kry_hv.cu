@@ -18,34 +18,28 @@
 namespace kry {
 
 constexpr int DOTS_NTHR = 512;   // threads of a CTA of the dots
-
-struct SmemHead {
-    uint32_t koff[20];
-    uint32_t bsz[20];
-};
+// Loads of hops issued together in the two forms of the H.v (eight of 16 bytes would spill)
+template <class V, int FORM> constexpr int HV_RND = FORM == 0 ? 4 : sizeof(V) == 8 ? 8 : 2;
 
 // ---------------------------------------------------------------- y = H x
 
-template <class V>
-__global__ void __launch_bounds__(NTHR) k_apply(DevBasis b, DevHam hm, const V *__restrict__ x,
-                                                V *__restrict__ y, int rl_smem)
+// Bond energies (J Delta / 4)(nbonds - 2 n) for n antiparallel bonds.
+template <class R>
+__device__ __forceinline__ void stage_dz(const DevBasis &b, const DevHam &hm, R *dz)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    SmemHead *hd = (SmemHead *)smem;
-    uint16_t *rl_s = (uint16_t *)(smem + sizeof(SmemHead));
-    stage_tables(b, hd->koff, hd->bsz, rl_s, rl_smem);
+    if (threadIdx.x <= (unsigned)b.L) dz[threadIdx.x] = (R)(hm.cz * (double)(hm.nbonds - 2 * (int)threadIdx.x));
+}
+
+template <class V, int FORM>
+__global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_apply(DevBasis b, DevHam hm, HvPlan pl,
+                                                                          const V *__restrict__ x, V *__restrict__ y)
+{
+    using R = typename VT<V>::R;
+    __shared__ R dz[64];
+    __shared__ __align__(16) HvWarp w[HV_NTHR / 32];
+    stage_dz(b, hm, dz);
     __syncthreads();
-    const uint16_t *rl = rl_smem ? rl_s : b.ranklo;
-    const uint32_t ntiles = (b.D + TILE - 1) / TILE;
-    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint32_t r0 = tile * TILE, t = threadIdx.x;
-        if (r0 + t < b.D) {
-            uint32_t hi, off;
-            int klo;
-            tile_unrank(b, hd->bsz, r0, t, hi, off, klo);
-            y[r0 + t] = hv_row<V>(b, hm, x, hi, off, klo, hd->koff, rl);
-        }
-    }
+    hv_items<V, HV_RND<V, FORM>>(b, hm, pl, x, y, w[threadIdx.x >> 5], dz, (R)1, (R)hm.halfJ);
 }
 
 // ---------------------------------------------------------------- reductions
@@ -154,41 +148,24 @@ __device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, d
 
 // ---------------------------------------------------------------- pass A
 
-// u = sigma_j H W_j, written to U (pass A, part 1).  One thread per row at full occupancy
-// and nothing else: the gathers of the hops are latency-bound, so as many rows as possible
-// are kept in flight.  alpha_j, ||u||^2 and the dots with the earlier vectors are taken by
-// the streaming pass that follows (k_dots, mode 0).  FORM 0 gathers the hops one by one
-// (hv_row_scaled), FORM 1 in rounds of four loads in flight (hv_row_chunked); both give the
-// same bits, the launch shape picks the faster (kry_autotune).
+// u = sigma_j H W_j, written to U (pass A, part 1): the gathers of hv_items at full occupancy and
+// nothing else.  alpha_j, ||u||^2 and the dots with the earlier vectors are taken by the streaming
+// pass that follows (k_dots, mode 0).  FORM 0 issues the loads of four hops together, FORM 1 of
+// eight (16-byte elements: of two); both give the same bits, the launch shape picks the faster (kry_autotune).
 template <class V, int FORM>
-__global__ void __launch_bounds__(NTHR) k_hv(EvArgs<V> a, int jj)
+__global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V> a, HvPlan pl, int jj)
 {
+    using R = typename VT<V>::R;
+    __shared__ R dz[64];
+    __shared__ __align__(16) HvWarp w[HV_NTHR / 32];
+    stage_dz(a.b, a.h, dz);   // (does not depend on the kernels before this one)
+    __syncthreads();
     pdl_begin();
     KryCtl *ctl = a.ctl;
     if (ctl->done || jj >= ctl->m_eff) return;
-    using R = typename VT<V>::R;
-    extern __shared__ __align__(16) unsigned char smem[];
-    SmemHead *hd = (SmemHead *)smem;
-    uint16_t *rl_s = (uint16_t *)(smem + sizeof(SmemHead));
-    __shared__ R dz[64];
-    if (threadIdx.x <= (unsigned)a.b.L) dz[threadIdx.x] = (R)(a.h.cz * (double)(a.h.nbonds - 2 * (int)threadIdx.x));
-    stage_tables(a.b, hd->koff, hd->bsz, rl_s, a.rl_smem);
-    __syncthreads();
-    const uint16_t *rl = a.rl_smem ? rl_s : a.b.ranklo;
     const double s = ctl->sigma[jj];
-    const R sj = (R)s, shj = (R)(s * a.h.halfJ);
-    const V *x = a.W + (size_t)jj * a.ldW;
-    const uint32_t D = a.b.D, ntiles = (D + TILE - 1) / TILE;
-    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint32_t r0 = tile * TILE, r = r0 + threadIdx.x;
-        if (r < D) {
-            uint32_t hi, off;
-            int klo;
-            tile_unrank(a.b, hd->bsz, r0, threadIdx.x, hi, off, klo);
-            a.U[r] = FORM == 1 ? hv_row_chunked<V>(a.b, a.h, x, hi, off, klo, hd->koff, rl, dz, sj, shj)
-                               : hv_row_scaled<V>(a.b, a.h, x, hi, off, klo, hd->koff, rl, dz, sj, shj);
-        }
-    }
+    hv_items<V, HV_RND<V, FORM>>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
+                              (R)(s * a.h.halfJ));
 }
 
 // The row loop of k_dots for one group of 64 threads: NQ vectors from Wg, NU units of rows at a time
@@ -697,64 +674,69 @@ static int sm_count()
 // two CTAs of 256 (D < 155,648 on 152 SMs), so that more SMs share them.
 static int lincomb_threads(uint32_t D) { return D < (uint32_t)sm_count() * 4u * NTHR ? 64 : NTHR; }
 
-size_t apply_smem(const DevBasis &b, int rl_smem, int)
+// Blocks per item of the H.v: more share the lower part's ranks, fewer give more items.  Four from
+// 32 warps per SM and four waves on, then two and one; twice that with bit 1 of the form.
+static HvPlan hv_plan(const DevBasis &b, int hv_form)
 {
-    return sizeof(SmemHead) + (rl_smem ? (sizeof(uint16_t) << b.Llo) : 0);
+    HvPlan p{};
+    const uint64_t warps = (uint64_t)b.D / 32u, full = (uint64_t)sm_count() * 32u;
+    p.nh = (warps >= 16u * full ? 4 : warps >= 4u * full ? 2 : 1) * ((hv_form & 2) ? 2 : 1);
+    auto binom = [](int n, int k) {
+        if (k < 0 || k > n) return (uint32_t)0;
+        uint64_t r = 1;
+        for (int i = 1; i <= k; ++i) r = r * (uint64_t)(n - k + i) / (uint64_t)i;
+        return (uint32_t)r;
+    };
+    uint32_t kofs[18] = {0};   // group offsets of lolist
+    for (int k = 0; k <= b.Llo; ++k) kofs[k + 1] = kofs[k] + binom(b.Llo, k);
+    for (int c = 0; c <= b.Lhi; ++c) {
+        const uint32_t nhi = binom(b.Lhi, c);
+        const int kl = b.N - c;
+        p.hoff[c + 1] = p.hoff[c] + nhi;
+        p.first[c + 1] = p.first[c];
+        if (kl < 0 || kl > b.Llo) continue;
+        p.nlo[c] = kofs[kl + 1] - kofs[kl];
+        p.koff[c] = kofs[kl];
+        p.first[c + 1] += ((p.nlo[c] + 31u) / 32u) * ((nhi + p.nh - 1) / p.nh);
+    }
+    return p;
 }
 
-
-template <class K>
-static int prep_smem(K kernel, size_t smem)
-{
-    if (smem > 48 * 1024) KRY_CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    return KRY_OK;
-}
-
-int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y, int rl_smem,
-                 cudaStream_t s)
+int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y, cudaStream_t s)
 {
     if (b.list) return launch_list_apply(b, h, c64, 1, x, y, s);
-    const size_t smem = apply_smem(b, rl_smem, c64);
-    const uint32_t ntiles = (b.D + TILE - 1) / TILE;
-    int grid = (int)std::min<uint32_t>(ntiles, (uint32_t)sm_count() * 8u);
-    if (c64) {
-        if (int rc = prep_smem(k_apply<float2>, smem)) return rc;
-        k_apply<float2><<<grid, NTHR, smem, s>>>(b, h, (const float2 *)x, (float2 *)y, rl_smem);
-    } else {
-        if (int rc = prep_smem(k_apply<double2>, smem)) return rc;
-        k_apply<double2><<<grid, NTHR, smem, s>>>(b, h, (const double2 *)x, (double2 *)y, rl_smem);
-    }
+    const HvPlan pl = hv_plan(b, 0);
+    const uint32_t ctas = (pl.first[b.Lhi + 1] + HV_NTHR / 32 - 1) / (HV_NTHR / 32);
+    const int grid = (int)std::min<uint32_t>(ctas, (uint32_t)sm_count() * (c64 ? 4u : 3u));
+    if (c64) k_apply<float2, 0><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const float2 *)x, (float2 *)y);
+    else k_apply<double2, 0><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const double2 *)x, (double2 *)y);
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
 
 // CTAs of the vector kernels, whole SMs times their resident CTAs: the streaming dots
 // (returned; also pass C1), the H.v of pass A (*gridH) and the updates, combine and
-// outputs (*gridB).  Also sets the kernels' shared-memory limits.  hv_form is part 1 of the
-// launch shape: bit 0 chunked gathers, bit 1 the lower-bit rank table read through L1
-// instead of staged in shared memory (more CTAs per SM when that table is large).
+// outputs (*gridB).  hv_form is part 1 of the launch shape (hv_plan, k_hv).
 template <class V>
-int vector_grid(const DevBasis &b, int rl_smem, int hv_form, int *gridH, int *gridB)
+int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB)
 {
     const uint32_t es = sizeof(V);
-    const int rlH = rl_smem && !(hv_form & 2);
-    const size_t smH = apply_smem(b, rlH, es == sizeof(float2));
-    if (int rc = prep_smem(k_hv<V, 0>, smH)) return -rc;
-    if (int rc = prep_smem(k_hv<V, 1>, smH)) return -rc;
     int occB = 0, occH = 0;
-    if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1>, NTHR, smH);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0>, NTHR, smH);
+    if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1>, HV_NTHR, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0>, HV_NTHR, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occB, k_lincomb<V, 0, 2>, NTHR, 0);
     const uint32_t ntiles = (b.D + TILE - 1) / TILE;
-    auto fit = [&](int occ) {
-        return (int)std::max<uint32_t>(1u, std::min<uint32_t>(ntiles, (uint32_t)(sm_count() * std::max(1, occ))));
+    auto fit = [&](int occ, uint32_t most) {
+        return (int)std::max<uint32_t>(1u, std::min<uint32_t>(most, (uint32_t)(sm_count() * std::max(1, occ))));
     };
-    *gridH = fit(occH);
     if (b.list) {
+        *gridH = fit(occH, ntiles);
         if (int rc = list_hv_grid<V>(b, gridH)) return -rc;
+    } else {
+        *gridH = fit(occH, (hv_plan(b, hv_form).first[b.Lhi + 1] + HV_NTHR / 32 - 1) / (HV_NTHR / 32));
     }
     // (the updates of small sectors: CTAs of 64 threads, two rows each)
-    *gridB = lincomb_threads(b.D) == NTHR ? fit(occB) : (int)std::max<uint32_t>(1u, std::min<uint32_t>((b.D + 127) / 128, (uint32_t)sm_count() * 4u));
+    *gridB = lincomb_threads(b.D) == NTHR ? fit(occB, ntiles) : (int)std::max<uint32_t>(1u, std::min<uint32_t>((b.D + 127) / 128, (uint32_t)sm_count() * 4u));
     // the dots: one CTA per SM, fewer when there are not two units of 64 threads' rows for each
     const uint32_t nu = (b.D + 64 * (16 / es) - 1) / (64 * (16 / es));
     return (int)std::max<uint32_t>(1u, std::min<uint32_t>((nu + 1) / 2, (uint32_t)sm_count()));
@@ -764,10 +746,8 @@ template <class V>
 int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
     if (a.b.list) return launch_list_hv<V>(a, jj, grid, s, pdl);
-    EvArgs<V> ah = a;
-    ah.rl_smem = a.rl_smem && !(a.hv_form & 2);
-    const size_t smem = apply_smem(a.b, ah.rl_smem, sizeof(V) == sizeof(float2));
-    KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1> : k_hv<V, 0>, grid, NTHR, smem, s, ah, jj));
+    const HvPlan pl = hv_plan(a.b, a.hv_form);
+    KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1> : k_hv<V, 0>, grid, HV_NTHR, 0, s, a, pl, jj));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
@@ -884,9 +864,9 @@ int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, 
 template int launch_dots<double2>(const EvArgs<double2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<float2>(const EvArgs<float2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<ffc>(const EvArgs<ffc> &, int, int, int, cudaStream_t, int);
-template int vector_grid<double2>(const DevBasis &, int, int, int *, int *);
-template int vector_grid<float2>(const DevBasis &, int, int, int *, int *);
-template int vector_grid<ffc>(const DevBasis &, int, int, int *, int *);
+template int vector_grid<double2>(const DevBasis &, int, int *, int *);
+template int vector_grid<float2>(const DevBasis &, int, int *, int *);
+template int vector_grid<ffc>(const DevBasis &, int, int *, int *);
 template int launch_hv<double2>(const EvArgs<double2> &, int, int, cudaStream_t, int);
 template int launch_hv<float2>(const EvArgs<float2> &, int, int, cudaStream_t, int);
 template int launch_hv<ffc>(const EvArgs<ffc> &, int, int, cudaStream_t, int);

@@ -85,6 +85,7 @@ struct DevBasis {
     const uint32_t *tstart;   // [ceil(D / TILE)]
     const uint16_t *ranklo;
     const uint16_t *lolist;
+    const uint16_t *hilist; // upper-bit patterns grouped by popcount, each group ascending [2^Lhi]
     const uint32_t *koff;   // [Llo + 2]
     const uint32_t *bsz;    // [Llo + 1], C(Llo, k)
     int *err;               // device error flag of rank/unrank
@@ -256,7 +257,6 @@ struct EvArgs {
     const V *G;      // readout vector psi0 (general initial state) or nullptr
     double2 *part;   // per-CTA partial sums [grid][PSTRIDE]
     KryCtl *ctl;
-    int rl_smem;     // stage ranklo in shared memory
     // pass B sets this conditional node of the step graph to whether the second
     // Gram-Schmidt pass (pass C) runs (use_cond = 0: no node, pass C kernels always launched)
     cudaGraphConditionalHandle cond;
@@ -279,8 +279,6 @@ struct ExpArgs {
 };
 constexpr int NGL = 64;   // Gauss-Legendre nodes of the per-step integral of P
 
-size_t apply_smem(const DevBasis &b, int rl_smem, int c64);
-
 // sorted-list basis (kry_list.cu)
 int list_build(DevBasis &b, cudaStream_t s);
 int launch_list_rank(const DevBasis &b, const uint64_t *st, uint32_t *rk, int64_t n, cudaStream_t s);
@@ -292,13 +290,12 @@ template <class V> int list_hv_grid(const DevBasis &b, int *grid);
 size_t list_smem(const DevBasis &b);
 
 // kernel launchers (kry_hv.cu)
-int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y,
-                 int rl_smem, cudaStream_t s);
+int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y, cudaStream_t s);
 template <class V> int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl = 1);
 template <class V> int launch_lincomb(const EvArgs<V> &a, int mode, int jj, int grid,
                                       cudaStream_t s, int pdl = 1);
 template <class V> int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, int pdl = 1);
-template <class V> int vector_grid(const DevBasis &b, int rl_smem, int hv_form, int *gridH, int *gridB);
+template <class V> int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB);
 int launch_set_basis_state(void *W0, int c64, uint32_t r0, cudaStream_t s, int ff = 0);
 // complex128 <-> float-float vectors of n elements (the boundary of KRY_C128E)
 int launch_c128_to_ffc(const void *src, void *dst, size_t n, cudaStream_t s);
@@ -343,8 +340,8 @@ struct kry_ham_s {
     int g_C;                    // the graph integrates P for C(t)
     size_t g_ldo, g_ldc;
     // per precision, the launch shape of the vector kernels (kry_set_shape, kry_autotune):
-    // [0] CTAs of the streaming kernels (0 = occupancy rule), [1] H.v form (bit 0: chunks of
-    // eight gathers; bit 1: rank table through L1), [2] dots form (0 several units of rows at a time, 1 one), [3]
+    // [0] CTAs of the streaming kernels (0 = occupancy rule), [1] H.v form (bit 0: other
+    // number of loads at a time; bit 1: twice the blocks per item), [2] dots form (0 several units of rows at a time, 1 one), [3]
     // update rows per thread,
     // [4] batched H.v in chunks of this many realisations (0 = all K)
     int shape[3][5];
@@ -360,10 +357,8 @@ struct kry_ham_s {
 };
 
 // Launch shape of a new Hamiltonian: the occupancy-rule grid, two update
-// rows per thread, all realisations at once, and the H.v one hop at a time with the
-// lower-bit rank table in shared memory -- except for lower parts of 14 bits or more (L >=
-// 28), whose table (32-64 KB) would cap the H.v at three or four CTAs per SM: there the
-// gathers go in rounds and the table is read through L1 (form 3; 2.9x faster at L = 30).
+// rows per thread, all realisations at once, and the H.v with four loads at a time -- from lower
+// parts of 14 bits on (L >= 28) eight (complex64) and twice the blocks per item (3% faster at L = 30).
 inline void default_shape(kry_ham_s *H, int Llo)
 {
     const int v[5] = {0, Llo >= 14 ? 3 : 0, 0, 2, 0};

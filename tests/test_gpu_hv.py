@@ -82,3 +82,45 @@ def test_apply_rejects_bad_arguments(kry):
     with pytest.raises(ValueError):
         H.apply(x[:-1])
     assert kry.load().kry_apply(H._h, 0, x.data_ptr(), x.data_ptr(), None) == kry.KRY_EINVAL
+
+
+@pytest.mark.parametrize("L,N", [(2, 1), (3, 1), (5, 2), (8, 4), (9, 1), (9, 8), (11, 6), (13, 6), (16, 3), (17, 8)])
+@pytest.mark.parametrize("pbc", [True, False])
+def test_apply_edges_of_items(kry, L, N, pbc):
+    """Items of 32 lower parts and up to eight upper parts: sectors whose groups are smaller than a warp,
+    not a multiple of it, or leave an item's blocks unfilled, on open and closed chains.  The complex128
+    sum on aligned integers is at least as close as FP64 adds: 4 ulp of the largest term per row."""
+    h = workloads.quasiperiodic_field(L, 1.7, 0.9)
+    Hc = ob.CSR(L, N, 1.0, 0.6, h, pbc)
+    rng = np.random.default_rng(L * 31 + N)
+    # values over 60 binary orders, some zero
+    x = (rng.normal(size=Hc.D) + 1j * rng.normal(size=Hc.D)) * 2.0 ** rng.integers(-60, 1, size=Hc.D)
+    x[rng.random(Hc.D) < 0.1] = 0.0
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.6, h, pbc=pbc)
+    y = H.apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    yo = Hc.matvec(x)
+    # a row's rounding is relative to its largest hop term, and that of its diagonal to the terms that add
+    # up to it (fields and bonds, which may cancel), not to their sum
+    dmax = 0.5 * np.sum(np.abs(h)) + 0.25 * 0.6 * L
+    big = np.maximum(np.maximum.reduceat(np.abs(Hc.val) * np.abs(x[Hc.col]), Hc.rowptr[:-1]), dmax * np.abs(x))
+    assert np.all(np.abs(y - yo) <= (L + 4) * 2.0**-52 * big + 1e-300)
+    y32 = H.apply(torch.from_numpy(x.astype(np.complex64)).cuda()).cpu().numpy()
+    assert np.all(np.abs(y32 - yo) <= (L + 6) * 2.0**-22 * big + 1e-30)
+
+
+@pytest.mark.parametrize("special", [float("inf"), float("-inf"), float("nan"), 1e-300])
+def test_apply_special_values(kry, special):
+    """Rows whose neighbours hold values the integer sum cannot (infinities, NaN, below 2^-895) are summed
+    in FP64: the same result as the oracle's, and the other rows are untouched."""
+    L, N = 10, 5
+    h = workloads.quasiperiodic_field(L, 1.0, 0.2)
+    Hc = ob.CSR(L, N, 1.0, 1.0, h, True)
+    x = np.zeros(Hc.D, np.complex128) if special == 1e-300 else np.ones(Hc.D, np.complex128)
+    x[17] = complex(special, 2.0 * special if special == 1e-300 else 1.0)
+    y = kry.Hamiltonian(kry.Basis(L, N), 1.0, 1.0, h).apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        yo = Hc.matvec(x)
+    for a, b in ((y.real, yo.real), (y.imag, yo.imag)):
+        assert np.array_equal(np.isfinite(a), np.isfinite(b))
+        ok = np.isfinite(b)
+        assert np.allclose(a[ok], b[ok], rtol=1e-14, atol=0.0)

@@ -624,6 +624,7 @@ template <> struct RealLin<double2> {
     RealLin() = default;
     __device__ __forceinline__ RealLin(double2 src) : w(src) {}
     __device__ __forceinline__ void fms(RCoef nc, double2 x) { w.x = fma(nc, x.x, w.x); w.y = fma(nc, x.y, w.y); }
+    __device__ __forceinline__ void add(double2 p) { w.x += p.x; w.y += p.y; }
     __device__ __forceinline__ double2 out() const { return w; }
 };
 template <> struct RealLin<float2> {
@@ -633,6 +634,7 @@ template <> struct RealLin<float2> {
     RealLin() = default;
     __device__ __forceinline__ RealLin(float2 src) : w(src) {}
     __device__ __forceinline__ void fms(RCoef nc, float2 x) { w = __ffma2_rn(make_float2(nc, nc), x, w); }
+    __device__ __forceinline__ void add(float2 p) { w = __fadd2_rn(w, p); }
     __device__ __forceinline__ float2 out() const { return w; }
 };
 template <> struct RealLin<ffc> {
@@ -653,6 +655,10 @@ template <> struct RealLin<ffc> {
         e = __ffma2_rn(make_float2(nc.x, nc.x), l, e);
         e = __ffma2_rn(make_float2(nc.y, nc.y), h, e);
         ff2_add_neg(s, c, n, e);
+    }
+    __device__ __forceinline__ void add(ffc p)
+    {
+        ff2_add_neg(s, c, make_float2(-p.xh, -p.yh), make_float2(p.xl, p.yl));
     }
     __device__ __forceinline__ ffc out()
     {
@@ -724,6 +730,133 @@ template <> struct CplxLin<ffc> {
     __device__ __forceinline__ ffc out() { return w.out(); }
 };
 
+// ---------------------------------------------------------------- reductions over the CTAs
+
+// Write this CTA's partials, then let the last CTA to finish sum all partials into
+// fin[0..PSTRIDE).  Returns true in the last CTA (all its threads).  Only the slots [0, nlead)
+// and, with tail set, SLOT_NRM and SLOT_G are summed (the others of fin are zero): a warp takes a
+// slot, lane l the partials of CTAs l, l + 32, ..., eight loads at a time.  With cplx unset the imaginary parts are zero and not summed.  The order depends only on the grid,
+// the block and the slot count, so results are bitwise reproducible.
+__device__ __forceinline__ bool finish_partials(const double2 *red, double2 *part, KryCtl *ctl,
+                                                double2 *fin, int *flag, unsigned *counter = nullptr,
+                                                int nlead = PSTRIDE, bool tail = true, bool cplx = true)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    if (!counter) counter = &ctl->counter;
+    if (tid < PSTRIDE) part[(size_t)blockIdx.x * PSTRIDE + tid] = red[tid];
+    __syncthreads();
+    if (tid == 0) {   // (one fence for the CTA: the barrier orders the others' writes before it)
+        __threadfence();
+        *flag = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1 : 0;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!*flag) return false;
+    // slots 0 .. nlead - 1, then NRM and G unless they are among those
+    const int nt = tail ? (nlead <= SLOT_NRM ? 2 : 0) : 0, ns = nlead + nt;
+    if (tid < PSTRIDE) fin[tid] = make_double2(0.0, 0.0);
+    __syncthreads();
+    for (int q = warp; q < ns; q += nw) {
+        const int slot = q < nlead ? q : SLOT_NRM + (q - nlead);
+        if (!cplx && slot == SLOT_G) continue;
+        double2 sum = make_double2(0.0, 0.0);
+        for (unsigned c0 = 0; c0 < gridDim.x; c0 += 256) {
+            double x[8], y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const unsigned c = c0 + 32 * i + lane;
+                double2 v = make_double2(0.0, 0.0);
+                if (c < gridDim.x) v = __ldcg(part + (size_t)c * PSTRIDE + slot);
+                x[i] = v.x;
+                y[i] = v.y;
+            }
+            sum.x += warp_sum_int<8>(x);
+            if (cplx) sum.y += warp_sum_int<8>(y);
+        }
+        if (lane == 0) fin[slot] = sum;
+    }
+    __syncthreads();
+    return true;
+}
+
+// beta_j = ||w|| and the scale of the next vector, or the end of the Krylov space
+__device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, double2 gdot)
+{
+    const double bt = sqrt(nw2);
+    ctl->beta[jj] = bt;
+    if (!(nw2 > ctl->eta_bd * ctl->eta_bd * ctl->normu2)) {   // invariant subspace (or zero vector)
+        ctl->m_eff = jj + 1;
+        ctl->n_bd += 1;
+    } else {
+        const double s = 1.0 / bt;
+        ctl->sigma[jj + 1] = s;
+        ctl->g[jj + 1] = make_double2(gdot.x * s, gdot.y * s);
+    }
+}
+
+// ---------------------------------------------------------------- the H.v's end in the one-read form
+
+// alpha_j = sigma_j Re <W_j, u> from the threads' sums, and in the last CTA the update's coefficients (see
+// k_ortho).  The terms C_ki d_k are at the level of the dots d, so FP32 holds them: it loses 2^-24 of each.
+template <class V>
+__device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, KryCtl *ctl, int jj)
+{
+    __shared__ double2 red[PSTRIDE];
+    __shared__ double wsum[32];
+    __shared__ float Cs[MMAX * MMAX], ds[MMAX + 1];
+    __shared__ int flag;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    al.renorm();
+    typename RealAcc<V>::Sum v[1] = {al.sum()};
+    const double t = to_double(warp_totals<1>(v));
+    if (lane == 0) wsum[warp] = t;
+    if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
+    __syncthreads();
+    if (tid == 0) {
+        double s = 0.0;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) s += wsum[w];
+        red[0].x = s;
+    }
+    __syncthreads();
+    if (!finish_partials(red, part, ctl, red, &flag, nullptr, 1, false, false)) return;
+    for (int e = tid; e < MMAX * MMAX; e += blockDim.x) Cs[e] = ctl->C[e / MMAX][e % MMAX];
+    if (tid <= MMAX) ds[tid] = tid < jj ? ctl->d[tid] : 0.f;   // (d_j = 1 stands apart)
+    __syncthreads();
+    if (tid >= 32) return;
+    const bool inv = lane <= jj;
+    const double s = inv ? ctl->sigma[lane] : 0.0, alpha = red[0].x * ctl->sigma[jj];
+    double c = 0.0;
+    if (lane < jj) {
+        float f = 0.f;
+        for (int k = 0; k <= lane; ++k) f = fmaf(Cs[k * MMAX + lane], ds[k], f);
+        const double b = ctl->beta[lane];
+        c = lane == jj - 1 ? b + (double)f : (double)fmaf((float)b, ds[lane + 1], f);
+    } else if (lane == jj) {
+        c = alpha;
+    }
+    const double cc = c * c, c2 = warp_sum_int<1>(&cc);
+    bool minor = false;
+    if (MinorSum<V>::use) {
+        // rounding level (MinorSum), against ||u||^2 >= alpha_j^2 + beta_{j-1}^2
+        const bool small = lane + 1 < jj;
+        const double cm = small ? cc : 0.0, m2 = warp_sum_int<1>(&cm), big = small ? 0.0 : cc, b2 = warp_sum_int<1>(&big);
+        minor = __all_sync(0xffffffffu, !small || (s >= 0x1p-40 && s <= 0x1p40)) &&
+                m2 <= MinorSum<V>::eta * MinorSum<V>::eta * b2;
+    }
+    if (inv) {
+        ctl->coefA[lane] = c * s;
+        ctl->C[lane][jj] = (float)c;
+    }
+    if (lane != 0) return;
+    ctl->alpha[jj] = alpha;
+    ctl->c2 = c2;
+    ctl->minor = minor ? 1 : 0;
+    ctl->n_hv += 1;
+    ctl->vec_passes += 2;
+    ctl->vp_kind[KIND_HV] += 2;   // the H.v: v_j read, u written
+    ctl->counter = 0;
+}
+
 // ---------------------------------------------------------------- rank tables
 
 // Locate rank r0 + t (< D) as (block hi, offset in block, particles in the lower part):
@@ -788,10 +921,11 @@ struct HvWarp {   // shared memory of a warp
     int n[HV_NH];
 };
 
-template <class V, int RND>
+// With ALPHA *al also sums Re <x, y> over the rows.
+template <class V, int RND, bool ALPHA>
 __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, const HvPlan &pl, const V *__restrict__ x,
                                          V *__restrict__ y, HvWarp &w, const typename VT<V>::R *dz,
-                                         typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ)
+                                         typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ, RealAcc<V> *al)
 {
     using R = typename VT<V>::R;
     const int Llo = b.Llo, Lhi = b.Lhi, nlb = Llo - 1, lane = threadIdx.x & 31;
@@ -888,7 +1022,9 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
                 out = hv_finish(sigma * d, x0, sigma_halfJ, acc);
             }
             if (valid) y[base + i] = out;
+            if (ALPHA) al->add(x0, RealAcc<V>::pre(valid ? out : VT<V>::zero()));
         }
+        if (ALPHA) al->renorm();   // (once per item, at most eight rows)
     }
 }
 

@@ -148,6 +148,11 @@ void drop_graph(kry_ham_s *H)
 // pass C launched in every Lanczos index (true) or as a conditional node
 bool plain_step_graph(const kry_ham_s *H) { return H->plain_graph || !H->cond_pass_c; }
 
+// Update and dots in one pass over the Krylov vectors (k_ortho), from 65,536 rows on: there the vectors'
+// reads cost more than the pass's longer rows (L = 19 c128e: 45.7 -> 43.6 us per Lanczos index, L = 24 c64
+// 188 -> 152, L = 30 c64 10.1 -> 8.2 ms); below, both forms are bound by latency and tie (L = 16 c128).
+int one_read_form(uint32_t D) { return D >= 65536u ? 1 : 0; }
+
 // Profile intervals of the captured step: four per Lanczos index (the H.v, pass A's dots,
 // pass B, pass C), then the small exponential and the combine; kind of the k-th interval.
 int n_intervals(int m) { return 4 * m + 2; }
@@ -195,12 +200,12 @@ int capture_step(kry_ham_s *H, const EvArgs<V> &a, const ExpArgs &ea, int m, int
         mark();
         rc = launch_hv<V>(a, jj, gridH, cs, after_cond ? 0 : 1);
         mark();
-        if (rc == KRY_OK) rc = launch_dots<V>(a, 0, jj, grid, cs);
+        if (rc == KRY_OK && !a.one_read) rc = launch_dots<V>(a, 0, jj, grid, cs);
         mark();
         if (plain) {
-            if (rc == KRY_OK) rc = launch_lincomb<V>(a, 0, jj, gridB, cs);
+            if (rc == KRY_OK) rc = a.one_read ? launch_ortho<V>(a, jj, grid, cs) : launch_lincomb<V>(a, 0, jj, gridB, cs);
             mark();
-            if (rc == KRY_OK) rc = launch_dots<V>(a, 1, jj, grid, cs);
+            if (rc == KRY_OK && !a.one_read) rc = launch_dots<V>(a, 1, jj, grid, cs);
             if (rc == KRY_OK) rc = launch_lincomb<V>(a, 1, jj, gridB, cs);
             continue;
         }
@@ -213,7 +218,7 @@ int capture_step(kry_ham_s *H, const EvArgs<V> &a, const ExpArgs &ea, int m, int
             if (e != cudaSuccess) rc = cuda_fail(e, "conditional handle");
             ab.use_cond = 1;
         }
-        if (rc == KRY_OK) rc = launch_lincomb<V>(ab, 0, jj, gridB, cs);
+        if (rc == KRY_OK) rc = a.one_read ? launch_ortho<V>(ab, jj, grid, cs) : launch_lincomb<V>(ab, 0, jj, gridB, cs);
         mark();
         if (rc == KRY_OK) {
             cudaStreamCaptureStatus cst;
@@ -234,7 +239,7 @@ int capture_step(kry_ham_s *H, const EvArgs<V> &a, const ExpArgs &ea, int m, int
                                                   cudaStreamCaptureModeThreadLocal);
             if (e != cudaSuccess) rc = cuda_fail(e, "conditional node");
             if (rc == KRY_OK) {
-                rc = launch_dots<V>(a, 1, jj, grid, cs2, 0);
+                if (!a.one_read) rc = launch_dots<V>(a, 1, jj, grid, cs2, 0);
                 if (rc == KRY_OK) rc = launch_lincomb<V>(a, 1, jj, gridB, cs2, 0);
                 cudaGraph_t body = nullptr;
                 e = cudaStreamEndCapture(cs2, &body);
@@ -302,6 +307,7 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
     a.hv_form = shp[1];
     a.dots_form = shp[2];
     a.upd_rows = shp[3];
+    a.one_read = one_read_form(b.D);
     ExpArgs ea{};
     ea.ctl = a.ctl;
     ea.times = (const double *)(base + l.oTimes);
@@ -397,7 +403,8 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
     long long launched = 0;
     const long long max_launch = 500000;   // Krylov steps before KRY_ETIMEOUT
     int batch = 1;
-    const int nk = 3 * m + 2;   // kernels of the step graph (pass C not counted)
+    // kernels of the step graph, pass C not counted, and of pass C
+    const int nk = (a.one_read ? 2 : 3) * m + 2, ncc = a.one_read ? 1 : 2;
     for (;;) {
         if (H->prof_on) batch = 1;   // events are read after every step
         for (int i = 0; i < batch; ++i) KRY_CU(cudaGraphLaunch(H->gexec, s));
@@ -408,6 +415,7 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
             for (int k = 0; k < n_intervals(m); ++k) {
                 float ms = 0.f;
                 KRY_CU(cudaEventElapsedTime(&ms, H->prof_ev[k], H->prof_ev[k + 1]));
+                if (a.one_read && kind_of(k, m) == KIND_PASSA) continue;   // (no kernel there)
                 H->prof_ms[kind_of(k, m)] += ms;
                 H->prof_launches[kind_of(k, m)] += 1;
             }
@@ -451,8 +459,8 @@ int evolve_t(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool g
         st->time_ms = ms;
         st->algo_bytes = (double)hp->vec_passes * (double)nvec * (double)es;
         const bool plain = plain_step_graph(H);
-        st->n_launches = launched * (nk + (plain ? 2 * m : 0) + (ea.Yout ? 1 : 0) + ((opt && opt->ckpt) ? 1 : 0)) +
-                         (plain ? 0 : 2 * hp->n_c1) + 1 + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
+        st->n_launches = launched * (nk + (plain ? ncc * m : 0) + (ea.Yout ? 1 : 0) + ((opt && opt->ckpt) ? 1 : 0)) +
+                         (plain ? 0 : a.one_read ? hp->n_corr : 2 * hp->n_c1) + 1 + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
         st->n_second_dots = hp->n_c1;
     }
     if (opt && opt->ckpt) {

@@ -39,57 +39,11 @@ __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_apply(DevBa
     __shared__ __align__(16) HvWarp w[HV_NTHR / 32];
     stage_dz(b, hm, dz);
     __syncthreads();
-    hv_items<V, HV_RND<V, FORM>>(b, hm, pl, x, y, w[threadIdx.x >> 5], dz, (R)1, (R)hm.halfJ);
+    hv_items<V, HV_RND<V, FORM>, false>(b, hm, pl, x, y, w[threadIdx.x >> 5], dz, (R)1, (R)hm.halfJ,
+                                               (RealAcc<V> *)nullptr);
 }
 
 // ---------------------------------------------------------------- reductions
-
-// Write this CTA's partials, then let the last CTA to finish sum all partials into
-// fin[0..PSTRIDE).  Returns true in the last CTA (all its threads).  Only the slots [0, nlead)
-// and, with tail set, SLOT_NRM and SLOT_G are summed (the others of fin are zero): a warp takes a
-// slot, lane l the partials of CTAs l, l + 32, ..., eight loads at a time.  With cplx unset the imaginary parts are zero and not summed.  The order depends only on the grid,
-// the block and the slot count, so results are bitwise reproducible.
-__device__ __forceinline__ bool finish_partials(const double2 *red, double2 *part, KryCtl *ctl,
-                                                double2 *fin, int *flag, unsigned *counter = nullptr,
-                                                int nlead = PSTRIDE, bool tail = true, bool cplx = true)
-{
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    if (!counter) counter = &ctl->counter;
-    if (tid < PSTRIDE) part[(size_t)blockIdx.x * PSTRIDE + tid] = red[tid];
-    __syncthreads();
-    if (tid == 0) {   // (one fence for the CTA: the barrier orders the others' writes before it)
-        __threadfence();
-        *flag = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1 : 0;
-        __threadfence();
-    }
-    __syncthreads();
-    if (!*flag) return false;
-    // slots 0 .. nlead - 1, then NRM and G unless they are among those
-    const int nt = tail ? (nlead <= SLOT_NRM ? 2 : 0) : 0, ns = nlead + nt;
-    if (tid < PSTRIDE) fin[tid] = make_double2(0.0, 0.0);
-    __syncthreads();
-    for (int q = warp; q < ns; q += nw) {
-        const int slot = q < nlead ? q : SLOT_NRM + (q - nlead);
-        if (!cplx && slot == SLOT_G) continue;
-        double2 sum = make_double2(0.0, 0.0);
-        for (unsigned c0 = 0; c0 < gridDim.x; c0 += 256) {
-            double x[8], y[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const unsigned c = c0 + 32 * i + lane;
-                double2 v = make_double2(0.0, 0.0);
-                if (c < gridDim.x) v = __ldcg(part + (size_t)c * PSTRIDE + slot);
-                x[i] = v.x;
-                y[i] = v.y;
-            }
-            sum.x += warp_sum_int<8>(x);
-            if (cplx) sum.y += warp_sum_int<8>(y);
-        }
-        if (lane == 0) fin[slot] = sum;
-    }
-    __syncthreads();
-    return true;
-}
 
 // Sum per-thread values over the CTA (warp shuffles, then warps in order) into red[slot].
 __device__ __forceinline__ void cta_sum_into(double2 v, double2 *red, int slot, double2 *wtmp)
@@ -131,28 +85,14 @@ __device__ __forceinline__ void cta_sum_into(const Acc &acc, double2 *red, int s
     __syncthreads();
 }
 
-// beta_j = ||w|| and the scale of the next vector, or the end of the Krylov space
-__device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, double2 gdot)
-{
-    const double bt = sqrt(nw2);
-    ctl->beta[jj] = bt;
-    if (!(nw2 > ctl->eta_bd * ctl->eta_bd * ctl->normu2)) {   // invariant subspace (or zero vector)
-        ctl->m_eff = jj + 1;
-        ctl->n_bd += 1;
-    } else {
-        const double s = 1.0 / bt;
-        ctl->sigma[jj + 1] = s;
-        ctl->g[jj + 1] = make_double2(gdot.x * s, gdot.y * s);
-    }
-}
-
 // ---------------------------------------------------------------- pass A
 
 // u = sigma_j H W_j, written to U (pass A, part 1): the gathers of hv_items at full occupancy and
 // nothing else.  alpha_j, ||u||^2 and the dots with the earlier vectors are taken by the streaming
 // pass that follows (k_dots, mode 0).  FORM 0 issues the loads of four hops together, FORM 1 of
 // eight (16-byte elements: of two); both give the same bits, the launch shape picks the faster (kry_autotune).
-template <class V, int FORM>
+// ALPHA (the one-read form, k_ortho): the pass also takes alpha_j and sets up the update's coefficients.
+template <class V, int FORM, bool ALPHA>
 __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V> a, HvPlan pl, int jj)
 {
     using R = typename VT<V>::R;
@@ -164,8 +104,10 @@ __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V
     KryCtl *ctl = a.ctl;
     if (ctl->done || jj >= ctl->m_eff) return;
     const double s = ctl->sigma[jj];
-    hv_items<V, HV_RND<V, FORM>>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
-                              (R)(s * a.h.halfJ));
+    RealAcc<V> al;
+    hv_items<V, HV_RND<V, FORM>, ALPHA>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
+                                        (R)(s * a.h.halfJ), &al);
+    if constexpr (ALPHA) alpha_epilogue<V>(al, a.part, ctl, jj);
 }
 
 // The row loop of k_dots for one group of 64 threads: NQ vectors from Wg, NU units of rows at a time
@@ -354,6 +296,275 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
     ctl->corr = 0;
     ctl->corr2 = sub ? 1 : 0;
     if (!sub) finalize_beta(ctl, jj, nw2, ctl->wg);
+    ctl->counter = 0;
+}
+
+// ---------------------------------------------------------------- the one-read pass
+
+// Threads of k_ortho's CTA (one per SM): 16 vectors' rows and accumulators take 96 to 128 registers.
+template <class V> constexpr int ORTHO_NTHR = std::is_same<V, ffc>::value ? 384 : 512;
+constexpr int ORTHO_QV = 16;   // vectors of a group, at most
+constexpr int ORTHO_XU = 2;    // units of a team between two barriers, at most
+
+// The loop is instantiated for 1, 2, 3, 4, 6, 8, 10, 12, 14, 15 and 16 vectors: empty slots of a group of n.
+__device__ __forceinline__ int ortho_pad(int n) { return n <= 4 || n == 15 ? 0 : n & 1; }
+
+// What a 64-thread group of k_ortho does besides its own vectors' terms and dots: FIRST stores w and
+// takes ||w||^2 and <psi0, w>, LAST holds u and the terms j - 1 and j.
+enum { ORTHO_FIRST = 1, ORTHO_LAST = 2, ORTHO_ONLY = 3 };
+
+// The row loop of k_ortho for one group: the nq = NQ or NQ - 1 vectors from i0 on (the first of NQ slots
+// is empty in the latter case), NU units of 64 rows at a time.  The vectors' rows are read once, kept in
+// registers, and used for the update and for the dots with its result; with two groups to a team their
+// partial updates meet in shared memory (two buffers, one barrier per NU units).
+template <class V, int NQ, int NU, int KIND>
+__device__ __forceinline__ void ortho_rows(const EvArgs<V> &a, V *out, int i0, int nq, int jj, bool minor, int rp,
+                                           uint32_t du, uint32_t nu, bool back,
+                                           const typename RealLin<V>::RCoef *coef, const float *mcoef, V *xch,
+                                           RealAcc<V> *acc, RealAcc<V> &nrm, DotAcc<V> &gacc)
+{
+    constexpr uint32_t FOLD = 8;   // rows between two foldings of the float-float compensations
+    constexpr bool LAST = KIND & ORTHO_LAST, FIRST = KIND & ORTHO_FIRST;
+    constexpr int NMAJ = NQ < 2 ? 1 : 2;   // (LAST) terms j - 1 and j
+    const uint32_t D = a.b.D, col = threadIdx.x & 63;
+    const int pad = NQ - nq;
+    const V *Wg = a.W + (ptrdiff_t)(i0 - pad) * (ptrdiff_t)a.ldW;   // (slot 0 is not read where pad is 1)
+    coef += i0;
+    mcoef += i0;
+    uint32_t it = 0;
+    for (uint32_t u0 = blockIdx.x * (du / gridDim.x) + rp; u0 < nu; u0 += NU * du) {
+        uint32_t r[NU];
+        V x[NU][NQ], uu[NU];
+#pragma unroll
+        for (int n = 0; n < NU; ++n) {
+            const uint32_t u = u0 + n * du;
+            r[n] = u < nu ? (back ? nu - 1 - u : u) * 64 + col : D;
+            const bool in = r[n] < D;
+            uu[n] = VT<V>::zero();
+            if (LAST) uu[n] = ldg_if(in, a.U + r[n]);
+            x[n][0] = ldg_if(in && pad == 0, Wg + r[n]);
+#pragma unroll
+            for (int q = 1; q < NQ; ++q) x[n][q] = ldg_if(in, Wg + (size_t)q * a.ldW + r[n]);
+        }
+        // this group's share of w = u - sum c_i W_i; terms at rounding level in FP32
+        RealLin<V> l[NU];
+        float2 f[NU];
+#pragma unroll
+        for (int n = 0; n < NU; ++n) {
+            l[n] = RealLin<V>(uu[n]);
+            f[n] = make_float2(0.f, 0.f);
+        }
+        if (MinorSum<V>::use && minor) {
+            if constexpr (MinorSum<V>::use) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int i = q == 0 ? 0 : q - pad;   // (an empty slot's x is zero)
+#pragma unroll
+                    for (int n = 0; n < NU; ++n) {
+                        if (LAST && q >= NQ - NMAJ) l[n].fms(coef[i], x[n][q]);
+                        else f[n] = __ffma2_rn(make_float2(mcoef[i], mcoef[i]), MinorSum<V>::lead(x[n][q]), f[n]);
+                    }
+                }
+#pragma unroll
+                for (int n = 0; n < NU; ++n)
+                    if (LAST) MinorSum<V>::add(l[n], f[n]);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                for (int n = 0; n < NU; ++n) l[n].fms(coef[q == 0 ? 0 : q - pad], x[n][q]);
+        }
+        if (KIND != ORTHO_ONLY) {
+            // publish this share, meet, take the team's other one: w = LAST's + FIRST's
+            V *buf = xch + ((size_t)(it & 1) * (ORTHO_NTHR<V> / 64) + 2 * rp) * 64 * ORTHO_XU + col;
+#pragma unroll
+            for (int n = 0; n < NU; ++n) {
+                if (LAST) buf[64 * n] = l[n].out();
+                else if (MinorSum<V>::use && minor) *(float2 *)(buf + 64 * (ORTHO_XU + n)) = f[n];
+                else buf[64 * (ORTHO_XU + n)] = l[n].out();
+            }
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + rp) : "memory");
+#pragma unroll
+            for (int n = 0; n < NU; ++n) {
+                if (!LAST) l[n] = RealLin<V>(buf[64 * n]);
+                if (MinorSum<V>::use && minor) {
+                    if constexpr (MinorSum<V>::use)
+                        MinorSum<V>::add(l[n], LAST ? *(const float2 *)(buf + 64 * (ORTHO_XU + n)) : f[n]);
+                } else {
+                    l[n].add(buf[64 * (ORTHO_XU + n)]);
+                }
+            }
+        }
+#pragma unroll
+        for (int n = 0; n < NU; ++n) {
+            if (NU > 1 && KIND == ORTHO_ONLY && u0 + n * du >= nu) break;
+            const V w = l[n].out();
+            const typename RealAcc<V>::Pre p = RealAcc<V>::pre(w);
+            if (FIRST) nrm.add(w, p);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) acc[q].add(x[n][q], p);
+            if (FIRST && r[n] < D) {
+                out[r[n]] = w;
+                if (a.G) gacc.add(ldg(a.G + r[n]), w);
+            }
+        }
+        it += 1;
+        if (it % (FOLD / NU) == 0) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) acc[q].renorm();
+            nrm.renorm();
+            gacc.renorm();
+        }
+    }
+}
+
+// Pass B and pass A's dots in one read of the Krylov vectors: w = u - sum_i c_i W_i, written as W_{j+1},
+// ||w||^2 and the dots Re <W_i, w>, i <= j.  Every vector is orthogonalised against all the earlier ones,
+// with coefficients c_i = Re <v_i, u>, u = (H - s) v_j, that need no pass of their own: H is symmetric, so
+// c_i = Re <(H - s) v_i, v_j>, and the update that made v_{i+1} says what (H - s) v_i is,
+//     (H - s) v_i = sum_{k<=i} C_ki v_k + beta_i v_{i+1}   (C_ki its coefficients c_k),
+// up to the rounding of that update.  With the dots d_k = Re <v_k, v_j> that this kernel measured when it
+// made v_j (d_j = 1), c_i = sum_{k<=i} C_ki d_k + beta_i d_{i+1}: beta_{j-1} for i = j - 1, rounding level
+// below, and c_j = alpha_j comes from the H.v pass.  An error of c_i is the same rounding that a dot product
+// of u has, it leaves the new vector that much off, and the next dots see it.  The Krylov vectors, whose
+// reads bound the step, are read once per Lanczos index instead of twice.
+// 64 threads take one row each of up to 16 vectors at a time; from 17 vectors on two such groups share a
+// row.  (Eight vectors per group, with teams of up to four, took
+// 98.7 us where this takes 90.4, L = 24 c64, and 107.5 against 93.2, L = 23 c128e.)
+// Odd indices run backwards, so that the rows a pass ends with are still in L2 for the next.  When the
+// dots exceed eta_corr, pass C2 (k_lincomb, mode 1) takes them off.
+template <class V, int COND>
+__global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
+{
+    pdl_begin();
+    KryCtl *ctl = a.ctl;
+    if (ctl->done || jj >= ctl->m_eff) return;
+    constexpr int QV = ORTHO_QV, NW = ORTHO_NTHR<V> / 32, NGRP = ORTHO_NTHR<V> / 64;
+    __shared__ double2 red[PSTRIDE];
+    __shared__ double wred[NW][QV + 3];
+    __shared__ typename RealLin<V>::RCoef coef[MMAX + 1];
+    __shared__ float mcoef[MMAX + 1];
+    __shared__ __align__(16) V xch[2 * ORTHO_NTHR<V> * ORTHO_XU];
+    __shared__ int flag;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = tid >> 6;
+    if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
+    if (tid <= jj) {
+        const double c = ctl->coefA[tid];
+        coef[tid] = RealLin<V>::coef(c);
+        mcoef[tid] = -(float)c;
+    }
+    __syncthreads();
+    const bool minor = MinorSum<V>::use && ctl->minor;
+    const int nv = jj + 1;
+    const int nvg = nv <= QV ? 1 : 2, nrp = NGRP / nvg;
+    const int rp = g / nvg, vg = (g + rp) % nvg;   // (rotated: the shares differ by one vector)
+    const int i0 = (nv * vg) / nvg, nq = (nv * (vg + 1)) / nvg - i0;
+    const uint32_t D = a.b.D, nu = (D + 63) / 64, du = gridDim.x * nrp;
+    RealAcc<V> acc[QV], nrm;
+    DotAcc<V> gacc;
+    V *out = a.W + (size_t)(jj + 1) * a.ldW;
+    const int pad = ortho_pad(nq);
+#define KRY_ORTHO(NQ, NU, KIND) \
+    ortho_rows<V, NQ, NU, KIND>(a, out, i0, nq, jj, minor, rp, du, nu, jj & 1, coef, mcoef, xch, acc, nrm, gacc)
+#define KRY_ORTHO_N(NQ, NU) \
+    case NQ: KRY_ORTHO(NQ, NU, ORTHO_ONLY); break;
+#define KRY_ORTHO_3(NQ, NU)                                       \
+    case NQ:                                                      \
+        if (nvg == 1) KRY_ORTHO(NQ, NU, ORTHO_ONLY);              \
+        else if (vg == 0) KRY_ORTHO(NQ, NU, ORTHO_FIRST);         \
+        else KRY_ORTHO(NQ, NU, ORTHO_LAST);                       \
+        break;
+    switch (nq + pad) {
+        KRY_ORTHO_N(1, 8)
+        KRY_ORTHO_N(2, 4)
+        KRY_ORTHO_N(3, 4)
+        KRY_ORTHO_N(4, 4)
+        KRY_ORTHO_N(6, 2)
+        case 8:
+            if (nvg == 1) KRY_ORTHO(8, 2, ORTHO_ONLY);
+            else if (vg == 0) KRY_ORTHO(8, 1, ORTHO_FIRST);
+            else KRY_ORTHO(8, 1, ORTHO_LAST);
+            break;
+        KRY_ORTHO_3(10, 1)
+        KRY_ORTHO_3(12, 1)
+        KRY_ORTHO_3(14, 1)
+        KRY_ORTHO_3(15, 1)
+        KRY_ORTHO_3(16, 1)
+    default: break;
+    }
+#undef KRY_ORTHO_3
+#undef KRY_ORTHO_N
+#undef KRY_ORTHO
+    {
+        typename RealAcc<V>::Sum v[QV];
+#pragma unroll
+        for (int q = 0; q < QV; ++q) {
+            acc[q].renorm();
+            v[q] = acc[q].sum();
+        }
+        const double t = to_double(warp_totals<QV>(v));
+        if (lane % (32 / QV) == 0) wred[warp][lane / (32 / QV)] = t;
+        nrm.renorm();
+        typename RealAcc<V>::Sum n1[1] = {nrm.sum()};
+        const double tn = to_double(warp_totals<1>(n1));
+        if (lane == 0) wred[warp][QV] = tn;
+        if (a.G) {
+            gacc.renorm();
+            const double2 tg = gacc.warp_value();
+            if (lane == 0) { wred[warp][QV + 1] = tg.x; wred[warp][QV + 2] = tg.y; }
+        }
+    }
+    __syncthreads();
+    if (tid < nv) {
+        const int s = nvg == 1 || tid < nv / 2 ? 0 : 1;   // the share that holds vector tid
+        const int f = nvg == 1 ? 0 : s ? nv / 2 : 0, n = nvg == 1 ? nv : s ? nv - nv / 2 : nv / 2;
+        const int q = tid - f + ortho_pad(n);
+        double t = 0.0;
+        for (int p = 0; p < nrp; ++p) {
+            const int w = 2 * (p * nvg + (nvg == 1 ? 0 : (s + p) & 1));   // the group of share s in row part p
+            t += wred[w][q] + wred[w + 1][q];
+        }
+        red[tid] = make_double2(t, 0.0);
+    } else if (tid >= 64 && tid < 67) {   // ||w||^2 and the two parts of <psi0, w>, from the groups of share 0
+        double t = 0.0;
+        if (tid == 64 || a.G)
+            for (int w = 0; w < NW; ++w)
+                if (((w >> 1) + (w >> 1) / nvg) % nvg == 0) t += wred[w][QV + tid - 64];
+        if (tid == 64) red[SLOT_NRM] = make_double2(t, 0.0);
+        else if (tid == 65) red[SLOT_G].x = t;
+        else red[SLOT_G].y = t;
+    }
+    __syncthreads();
+    double2 *fin = red;
+    if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, nv, true, a.G != nullptr)) return;
+    if (tid >= 32) return;
+    const bool inv = tid <= jj;
+    const double s = inv ? ctl->sigma[tid] : 0.0, dd = fin[tid].x * s;   // Re <v_i, w>
+    const double d2 = dd * dd, nd2 = warp_sum_int<1>(&d2), nw2 = fin[SLOT_NRM].x;
+    const double normu2 = ctl->c2 + nw2;   // ||u||^2 = ||c||^2 + ||w||^2 for orthonormal v_i
+    const bool dead = !(nw2 > ctl->eta_bd * ctl->eta_bd * normu2);   // an invariant subspace: nothing to correct
+    const bool sub = !dead && nd2 > ctl->eta_corr * ctl->eta_corr * nw2;
+    if (inv) {
+        if (sub) {
+            ctl->coefC[tid] = dd * s;
+            ctl->C[tid][jj] += (float)dd;
+        }
+        // d of the new vector; after pass C2 it is at rounding level and taken as zero
+        ctl->d[tid] = sub || dead ? 0.f : (float)(dd * rsqrt(nw2));
+    }
+    if (sub && tid == jj) ctl->alpha[jj] += dd;
+    if (tid != 0) return;
+    ctl->normu2 = normu2;
+    ctl->vec_passes += jj + 3 + (a.G ? 1 : 0);
+    ctl->vp_kind[KIND_PASSB] += jj + 3 + (a.G ? 1 : 0);
+    if (ctl->verify || sub) {
+        ctl->n_c1 += 1;
+        if (nw2 > 0.0) ctl->max_orth = fmax(ctl->max_orth, sqrt(nd2 / nw2));
+    }
+    ctl->corr2 = sub ? 1 : 0;
+    if (!sub) finalize_beta(ctl, jj, nw2, fin[SLOT_G]);
+    if (COND && a.use_cond) cudaGraphSetConditional(a.cond, sub ? 1u : 0u);
     ctl->counter = 0;
 }
 
@@ -722,8 +933,8 @@ int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB)
 {
     const uint32_t es = sizeof(V);
     int occB = 0, occH = 0;
-    if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1>, HV_NTHR, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0>, HV_NTHR, 0);
+    if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1, false>, HV_NTHR, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0, false>, HV_NTHR, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occB, k_lincomb<V, 0, 2>, NTHR, 0);
     const uint32_t ntiles = (b.D + TILE - 1) / TILE;
     auto fit = [&](int occ, uint32_t most) {
@@ -747,7 +958,10 @@ int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
     if (a.b.list) return launch_list_hv<V>(a, jj, grid, s, pdl);
     const HvPlan pl = hv_plan(a.b, a.hv_form);
-    KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1> : k_hv<V, 0>, grid, HV_NTHR, 0, s, a, pl, jj));
+    if (a.one_read)
+        KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1, true> : k_hv<V, 0, true>, grid, HV_NTHR, 0, s, a, pl, jj));
+    else
+        KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1, false> : k_hv<V, 0, false>, grid, HV_NTHR, 0, s, a, pl, jj));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
@@ -861,6 +1075,17 @@ int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, 
     return KRY_OK;
 }
 
+template <class V>
+int launch_ortho(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
+{
+    KRY_CU(launch_ex(pdl, a.use_cond ? k_ortho<V, 1> : k_ortho<V, 0>, grid, ORTHO_NTHR<V>, 0, s, a, jj));
+    KRY_CU(cudaGetLastError());
+    return KRY_OK;
+}
+
+template int launch_ortho<double2>(const EvArgs<double2> &, int, int, cudaStream_t, int);
+template int launch_ortho<float2>(const EvArgs<float2> &, int, int, cudaStream_t, int);
+template int launch_ortho<ffc>(const EvArgs<ffc> &, int, int, cudaStream_t, int);
 template int launch_dots<double2>(const EvArgs<double2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<float2>(const EvArgs<float2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<ffc>(const EvArgs<ffc> &, int, int, int, cudaStream_t, int);

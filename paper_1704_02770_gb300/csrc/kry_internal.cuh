@@ -204,6 +204,8 @@ struct KryCtl {
     double normu2;             // ||H v_j||^2 of the last pass A
     double c2;                 // ||V^H H v_j||^2 of the last pass A (Pythagoras test of pass B)
     int minor;                 // coefA[0 .. j - 2] are at rounding level (MinorSum)
+    float C[MMAX][MMAX];       // one-read form: C[k][i], the coefficient of v_k in the update that made v_{i+1}
+    float d[MMAX];             // and Re <v_k, v_j>, k < j, of the last vector
     double beta0;              // ||psi|| at the start of the Krylov step
     double t_now, t_end, tol, tau_prev;
     double eta_corr, eta_bd;   // second-pass and breakdown thresholds (relative)
@@ -263,6 +265,7 @@ struct EvArgs {
     int use_cond;
     // launch shape (host side only): H.v gather form, dots form, update rows per thread
     int hv_form, dots_form, upd_rows;
+    int one_read;    // update and dots in one pass over the Krylov vectors (k_ortho)
 };
 
 struct ExpArgs {
@@ -295,6 +298,7 @@ template <class V> int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStrea
 template <class V> int launch_lincomb(const EvArgs<V> &a, int mode, int jj, int grid,
                                       cudaStream_t s, int pdl = 1);
 template <class V> int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, int pdl = 1);
+template <class V> int launch_ortho(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl = 1);
 template <class V> int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB);
 int launch_set_basis_state(void *W0, int c64, uint32_t r0, cudaStream_t s, int ff = 0);
 // complex128 <-> float-float vectors of n elements (the boundary of KRY_C128E)
@@ -331,6 +335,7 @@ struct kry_ham_s {
     int ws_user;                // ws belongs to the caller (kry_set_workspace): never freed here
     // cached CUDA graph of one Krylov step
     cudaGraphExec_t gexec;
+    int g_one_read;             // the step graph is that of the one-read form
     int g_dtype, g_m, g_general, g_grid, g_gridB, g_gridH, g_shape, g_plain;
     int plain_graph;            // forced plain step graph (kry_profile_enable(H, 2))
     int cond_pass_c;            // pass C as a conditional node (kry_set_second_pass_node)

@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(NTHR) k_list_apply(DevBasis b, DevHam hm, int 
 }
 
 // pass A, part 1, one realisation: U = sigma_j H W_j
-template <class V>
+// (ALPHA as in k_hv)
+template <class V, bool ALPHA>
 __global__ void __launch_bounds__(NTHR) k_list_hv(EvArgs<V> a, int jj)
 {
     pdl_begin();
@@ -181,11 +182,19 @@ __global__ void __launch_bounds__(NTHR) k_list_hv(EvArgs<V> a, int jj)
     const double sd = ctl->sigma[jj];
     const R sj = (R)sd, shj = (R)(sd * a.h.halfJ);
     const V *x = a.W + (size_t)jj * a.ldW;
+    RealAcc<V> al;
+    int it = 0;
     for (uint32_t r = blockIdx.x * NTHR + threadIdx.x; r < a.b.D; r += gridDim.x * NTHR) {
         R d;
         const auto acc = list_row<V>(a.b, a.h, x, r, __ldg(a.b.states + r), 0, 1, cb, &d);
-        a.U[r] = hv_finish(sj * d, ldg(x + r), shj, acc);
+        const V x0 = ldg(x + r), u = hv_finish(sj * d, x0, shj, acc);
+        a.U[r] = u;
+        if (ALPHA) {
+            al.add(x0, RealAcc<V>::pre(u));
+            if ((++it & 3) == 0) al.renorm();
+        }
     }
+    if constexpr (ALPHA) alpha_epilogue<V>(al, a.part, ctl, jj);
 }
 
 // pass A, part 1, K realisations: U[:, k] = sigma_j[k] H_k W_j[:, k]
@@ -280,15 +289,16 @@ template <class V>
 int list_hv_grid(const DevBasis &b, int *grid)
 {
     const size_t sm = list_smem(b);
-    if (int rc = list_prep(k_list_hv<V>, sm)) return rc;
-    *grid = list_grid_of(k_list_hv<V>, sm, b.D);
+    if (int rc = list_prep(k_list_hv<V, false>, sm)) return rc;
+    if (int rc = list_prep(k_list_hv<V, true>, sm)) return rc;
+    *grid = list_grid_of(k_list_hv<V, true>, sm, b.D);
     return KRY_OK;
 }
 
 template <class V>
 int launch_list_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
-    KRY_CU(launch_ex(pdl, k_list_hv<V>, grid, NTHR, list_smem(a.b), s, a, jj));
+    KRY_CU(launch_ex(pdl, a.one_read ? k_list_hv<V, true> : k_list_hv<V, false>, grid, NTHR, list_smem(a.b), s, a, jj));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }

@@ -1,0 +1,145 @@
+"""The one-read form (sectors of 65,536 states and more): the update and the dots of its result in one pass
+over the Krylov vectors, with coefficients from the recurrence instead of dots of u.
+
+Sectors just above the line (D = 77,520 and 92,378: neither a multiple of the 64 rows of a unit) and a
+sorted-list one; m runs over every split of the vectors (1 to 16 in a group, two groups from 17 on)."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from oracle import basis as ob
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def kry():
+    import paper_1704_02770_gb300 as k
+    k.load()
+    return k
+
+
+def _setup(kry, L, N, lst=False, hh=1.3):
+    h = workloads.quasiperiodic_field(L, hh, 0.7)
+    return h, kry.Hamiltonian(kry.Basis(L, N, list=lst), 1.0, 0.8, h)
+
+
+@pytest.fixture(scope="module")
+def reference():
+    """psi(0.6) of a fixed dense state in the (20, 7) sector from the oracle's Krylov evolution."""
+    L, N = 20, 7
+    h = workloads.quasiperiodic_field(L, 1.3, 0.7)
+    H = ob.CSR(L, N, 1.0, 0.8, h, True)
+    rng = np.random.default_rng(8)
+    psi0 = rng.normal(size=H.D) + 1j * rng.normal(size=H.D)
+    psi0 /= np.linalg.norm(psi0)
+    P, psi, _ = _oracle(H, psi0, [0.3, 0.6])
+    return psi0, P, psi
+
+
+def _oracle(H, psi0, times):
+    # power series of exp(-iHt) in steps of 0.05: 30 terms of a norm below 0.05 * 20 = 1, to rounding
+    P, psi, t = [], psi0.copy(), 0.0
+    for tt in times:
+        while t < tt - 1e-12:
+            dt = min(0.05, tt - t)
+            term = psi.copy()
+            for n in range(1, 31):
+                term = H.matvec(term) * (-1j * dt / n)
+                psi = psi + term
+            t += dt
+        P.append(abs(np.vdot(psi0, psi)) ** 2)
+    return np.array(P), psi, None
+
+
+# each m ends its step in another split: one group of 1 to 16 vectors with and without an empty slot, then two
+@pytest.mark.parametrize("m", [5, 7, 9, 12, 15, 16, 17, 18, 23, 29, 31, 32])
+@pytest.mark.parametrize("form", ["c128", "c128e", "c64"])
+def test_every_split_against_the_power_series(kry, reference, m, form):
+    psi0, P0, psi1 = reference
+    _, H = _setup(kry, 20, 7)
+    x = torch.from_numpy(psi0).cuda()
+    if form == "c64":
+        x = x.to(torch.complex64)
+    out = torch.empty_like(x)
+    tol = 1e-6 if form == "c64" else 1e-10
+    P, st = H.evolve(x, [0.3, 0.6], m=m, tol=tol, psi_out=out, emulated=form == "c128e")
+    err = np.linalg.norm(out.cpu().numpy() - psi1)
+    # the budget, and for complex64 the rounding of the stored vectors, 2^-24 per step and operation
+    assert err <= (1e-5 if form == "c64" else tol), err
+    assert np.max(np.abs(P - P0)) <= (1e-5 if form == "c64" else tol)
+    assert st["n_second_pass"] == 0
+
+
+@pytest.mark.parametrize("form,bound", [("c128", 5e-14), ("c128e", 2e-12), ("c64", 2e-6)])
+def test_orthogonality_and_forced_second_pass(kry, form, bound):
+    """The coefficients of the recurrence keep every new vector as orthogonal as dots of u do (the bounds are
+    about 1e2 units of roundoff of the vector storage), the check and the forced subtraction change nothing
+    beyond it, and the conditional node gives the same bits."""
+    L, N = 19, 9
+    _, H = _setup(kry, L, N)
+    s, times, tol = 0, [0.5, 3.0], 1e-6 if form == "c64" else 1e-10
+    s = sum(1 << (2 * i) for i in range(N))
+    P0, st0 = H.return_probability(s, times, tol=tol, dtype=form)
+    H.orth_check(True)
+    P1, st1 = H.return_probability(s, times, tol=tol, dtype=form)
+    H.orth_check(2)
+    P2, st2 = H.return_probability(s, times, tol=tol, dtype=form)
+    H.orth_check(False)
+    H.second_pass_node(True)
+    P3, st3 = H.return_probability(s, times, tol=tol, dtype=form)
+    H.second_pass_node(False)
+    print(f"[one-read] {form}: max |<v_i, w>|/||w|| = {st1['max_orth_loss']:.2e}")
+    assert 0.0 < st1["max_orth_loss"] <= bound and st0["n_second_pass"] == 0
+    # (all but those whose dots are exactly zero, as those of a basis state's first vector, are subtracted)
+    assert st2["n_second_dots"] == st2["n_hv"] and st2["n_second_pass"] >= st2["n_hv"] - st2["n_krylov_steps"]
+    bar = 1e-6 if form == "c64" else 1e-12
+    assert np.max(np.abs(P1 - P0)) <= bar and np.max(np.abs(P2 - P0)) <= bar
+    assert np.array_equal(P3, P0)
+    m = 30
+    assert (st0["n_launches"] - 1) % (3 * m + 2) == 0
+
+
+@pytest.mark.parametrize("form", ["c128", "c128e", "c64"])
+def test_invariant_subspaces(kry, form):
+    """Sparse fields: a Krylov space that ends early (no hopping: every basis state is an eigenvector; a
+    single bond's worth of weight) is found and P stays exact."""
+    L, N = 20, 7
+    H = kry.Hamiltonian(kry.Basis(L, N), 0.0, 1.0, workloads.quasiperiodic_field(L, 1.0, 0.1))
+    s = (1 << N) - 1
+    P, st = H.return_probability(s, [1.0, 10.0], tol=1e-6, dtype=form)
+    assert np.max(np.abs(P - 1.0)) <= 1e-6 and st["n_breakdowns"] >= 1
+
+
+def test_list_basis_agrees_with_the_split_tables(kry):
+    L, N = 20, 7
+    h, H = _setup(kry, L, N)
+    _, Hl = _setup(kry, L, N, lst=True)
+    s = sum(1 << (2 * i) for i in range(N))
+    for form, tol, bar in (("c128", 1e-10, 1e-12), ("c128e", 1e-10, 1e-12), ("c64", 1e-7, 1e-6)):
+        P, _ = H.return_probability(s, [0.5, 4.0], tol=tol, dtype=form)
+        Pl, _ = Hl.return_probability(s, [0.5, 4.0], tol=tol, dtype=form)
+        assert np.max(np.abs(P - Pl)) <= bar
+
+
+def test_profile_and_shapes(kry):
+    """Kind 0 (pass A's dots) stays empty and the update's bytes are one read; shapes give equal results."""
+    L, N, m = 20, 7, 30
+    _, H = _setup(kry, L, N)
+    s = sum(1 << (2 * i) for i in range(N))
+    P0, _ = H.return_probability(s, [2.0], m=m)
+    H.profile(True)
+    P1, st = H.return_probability(s, [2.0], m=m)
+    pr = H.profile_read()
+    H.profile(False)
+    vec = H.basis.dim * 16 * st["n_krylov_steps"]
+    assert np.array_equal(P0, P1)
+    assert pr["dots"]["launches"] == 0 and pr["update"]["launches"] == m * pr["smallexp"]["launches"]
+    assert pr["update"]["bytes"] == pytest.approx(vec * sum(j + 3 for j in range(m)), rel=1e-12)
+    assert pr["hv"]["bytes"] == pytest.approx(vec * 2 * m, rel=1e-12)
+    for shape in ([0, 1, 0, 2, 0], [0, 2, 0, 2, 0], [0, 3, 1, 4, 0], [77, 0, 0, 1, 0]):
+        H.set_shape(shape)
+        P, _ = H.return_probability(s, [2.0], m=m)
+        assert np.max(np.abs(P - P0)) <= 1e-12
+

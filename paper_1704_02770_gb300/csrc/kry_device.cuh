@@ -916,13 +916,13 @@ struct HvPlan {
     int nh;               // blocks per item
 };
 struct HvWarp {   // shared memory of a warp
-    int steps[HV_NH][16];   // per block: block-start steps of its antiparallel upper bonds, packed
+    int steps[HV_NH][24];   // per block: block-start steps of its antiparallel upper bonds (at most 15), packed
     uint32_t hi[HV_NH], base[HV_NH], cross[HV_NH], ring[HV_NH];
     int n[HV_NH];
 };
 
 // With ALPHA *al also sums Re <x, y> over the rows.
-template <class V, int RND, bool ALPHA>
+template <class V, int RND, int URND, bool ALPHA>
 __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, const HvPlan &pl, const V *__restrict__ x,
                                          V *__restrict__ y, HvWarp &w, const typename VT<V>::R *dz,
                                          typename VT<V>::R sigma, typename VT<V>::R sigma_halfJ, RealAcc<V> *al)
@@ -993,14 +993,14 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
                 }
                 hv_add(acc, vc);
 #pragma unroll 1
-                for (int i0 = 0; i0 < n; i0 += 4) {
-                    const int4 d = *(const int4 *)(w.steps[h] + i0);   // (entries past n are not used)
-                    V v[4];
-                    v[0] = ldg_if(valid, xr + d.x);
-                    v[1] = ldg_if(valid && i0 + 1 < n, xr + d.y);
-                    v[2] = ldg_if(valid && i0 + 2 < n, xr + d.z);
-                    v[3] = ldg_if(valid && i0 + 3 < n, xr + d.w);
-                    hv_add_n<4>(acc, v);
+                for (int i0 = 0; i0 < n; i0 += URND) {
+                    V v[URND];
+#pragma unroll
+                    for (int u = 0; u < URND; ++u) {   // (entries past n are not used)
+                        const bool on = valid && (u == 0 || i0 + u < n);
+                        v[u] = ldg_if(on, xr + w.steps[h][i0 + u]);
+                    }
+                    hv_add_n<URND>(acc, v);
                 }
                 hv_add(acc, vr);
             };

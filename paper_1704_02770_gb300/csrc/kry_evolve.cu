@@ -128,10 +128,9 @@ struct EvOpts {
 int grid_for(const kry_ham_s *H, int dtype, int *gridH, int *gridB)
 {
     const DevBasis &b = H->b->dev;
-    const int hvf = H->shape[dtype_slot(dtype)][1];
-    const int g = dtype == KRY_C64    ? vector_grid<float2>(b, hvf, gridH, gridB)
-                  : dtype == KRY_C128E ? vector_grid<ffc>(b, hvf, gridH, gridB)
-                                       : vector_grid<double2>(b, hvf, gridH, gridB);
+    const int g = dtype == KRY_C64    ? vector_grid<float2>(b, gridH, gridB)
+                  : dtype == KRY_C128E ? vector_grid<ffc>(b, gridH, gridB)
+                                       : vector_grid<double2>(b, gridH, gridB);
     const int ov = H->shape[dtype_slot(dtype)][0];
     if (g > 0 && ov > 0) *gridB = ov;
     return (g > 0 && ov > 0) ? ov : g;

@@ -18,8 +18,9 @@
 namespace kry {
 
 constexpr int DOTS_NTHR = 512;   // threads of a CTA of the dots
-// Loads of hops issued together in the two forms of the H.v (eight of 16 bytes would spill)
-template <class V, int FORM> constexpr int HV_RND = FORM == 0 ? 4 : sizeof(V) == 8 ? 8 : 2;
+// Loads of hops issued together in the forms of the H.v: inside the lower bits (bit 0 of the form) and
+// inside the upper bits (bit 1); eight of 16 bytes would spill
+template <class V, int BIT> constexpr int HV_RND = BIT == 0 ? 4 : sizeof(V) == 8 ? 8 : 2;
 
 // ---------------------------------------------------------------- y = H x
 
@@ -30,7 +31,7 @@ __device__ __forceinline__ void stage_dz(const DevBasis &b, const DevHam &hm, R 
     if (threadIdx.x <= (unsigned)b.L) dz[threadIdx.x] = (R)(hm.cz * (double)(hm.nbonds - 2 * (int)threadIdx.x));
 }
 
-template <class V, int FORM>
+template <class V>
 __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_apply(DevBasis b, DevHam hm, HvPlan pl,
                                                                           const V *__restrict__ x, V *__restrict__ y)
 {
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_apply(DevBa
     __shared__ __align__(16) HvWarp w[HV_NTHR / 32];
     stage_dz(b, hm, dz);
     __syncthreads();
-    hv_items<V, HV_RND<V, FORM>, false>(b, hm, pl, x, y, w[threadIdx.x >> 5], dz, (R)1, (R)hm.halfJ,
+    hv_items<V, 4, 4, false>(b, hm, pl, x, y, w[threadIdx.x >> 5], dz, (R)1, (R)hm.halfJ,
                                                (RealAcc<V> *)nullptr);
 }
 
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V
     if (ctl->done || jj >= ctl->m_eff) return;
     const double s = ctl->sigma[jj];
     RealAcc<V> al;
-    hv_items<V, HV_RND<V, FORM>, ALPHA>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
+    hv_items<V, HV_RND<V, (FORM & 1)>, HV_RND<V, (FORM >> 1)>, ALPHA>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
                                         (R)(s * a.h.halfJ), &al);
     if constexpr (ALPHA) alpha_epilogue<V>(al, a.part, ctl, jj);
 }
@@ -885,13 +886,14 @@ static int sm_count()
 // two CTAs of 256 (D < 155,648 on 152 SMs), so that more SMs share them.
 static int lincomb_threads(uint32_t D) { return D < (uint32_t)sm_count() * 4u * NTHR ? 64 : NTHR; }
 
-// Blocks per item of the H.v: more share the lower part's ranks, fewer give more items.  Four from
-// 32 warps per SM and four waves on, then two and one; twice that with bit 1 of the form.
-static HvPlan hv_plan(const DevBasis &b, int hv_form)
+// Blocks per item of the H.v: more share the lower part's ranks, fewer give more items.  One below four
+// items of 32 rows per warp slot, two below 16, four below 200 (L = 24 c64: 40.5 us with four, 47 with one)
+// and eight from there on (3% faster than four at L = 30).
+static HvPlan hv_plan(const DevBasis &b)
 {
     HvPlan p{};
     const uint64_t warps = (uint64_t)b.D / 32u, full = (uint64_t)sm_count() * 32u;
-    p.nh = (warps >= 16u * full ? 4 : warps >= 4u * full ? 2 : 1) * ((hv_form & 2) ? 2 : 1);
+    p.nh = warps >= 200u * full ? 8 : warps >= 16u * full ? 4 : warps >= 4u * full ? 2 : 1;
     auto binom = [](int n, int k) {
         if (k < 0 || k > n) return (uint32_t)0;
         uint64_t r = 1;
@@ -916,25 +918,24 @@ static HvPlan hv_plan(const DevBasis &b, int hv_form)
 int launch_apply(const DevBasis &b, const DevHam &h, int c64, const void *x, void *y, cudaStream_t s)
 {
     if (b.list) return launch_list_apply(b, h, c64, 1, x, y, s);
-    const HvPlan pl = hv_plan(b, 0);
+    const HvPlan pl = hv_plan(b);
     const uint32_t ctas = (pl.first[b.Lhi + 1] + HV_NTHR / 32 - 1) / (HV_NTHR / 32);
     const int grid = (int)std::min<uint32_t>(ctas, (uint32_t)sm_count() * (c64 ? 4u : 3u));
-    if (c64) k_apply<float2, 0><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const float2 *)x, (float2 *)y);
-    else k_apply<double2, 0><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const double2 *)x, (double2 *)y);
+    if (c64) k_apply<float2><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const float2 *)x, (float2 *)y);
+    else k_apply<double2><<<grid, HV_NTHR, 0, s>>>(b, h, pl, (const double2 *)x, (double2 *)y);
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
 
 // CTAs of the vector kernels, whole SMs times their resident CTAs: the streaming dots
 // (returned; also pass C1), the H.v of pass A (*gridH) and the updates, combine and
-// outputs (*gridB).  hv_form is part 1 of the launch shape (hv_plan, k_hv).
+// outputs (*gridB).
 template <class V>
-int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB)
+int vector_grid(const DevBasis &b, int *gridH, int *gridB)
 {
     const uint32_t es = sizeof(V);
     int occB = 0, occH = 0;
-    if (hv_form & 1) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 1, false>, HV_NTHR, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0, false>, HV_NTHR, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0, true>, HV_NTHR, 0);   // (the same for every form)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occB, k_lincomb<V, 0, 2>, NTHR, 0);
     const uint32_t ntiles = (b.D + TILE - 1) / TILE;
     auto fit = [&](int occ, uint32_t most) {
@@ -944,7 +945,7 @@ int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB)
         *gridH = fit(occH, ntiles);
         if (int rc = list_hv_grid<V>(b, gridH)) return -rc;
     } else {
-        *gridH = fit(occH, (hv_plan(b, hv_form).first[b.Lhi + 1] + HV_NTHR / 32 - 1) / (HV_NTHR / 32));
+        *gridH = fit(occH, (hv_plan(b).first[b.Lhi + 1] + HV_NTHR / 32 - 1) / (HV_NTHR / 32));
     }
     // (the updates of small sectors: CTAs of 64 threads, two rows each)
     *gridB = lincomb_threads(b.D) == NTHR ? fit(occB, ntiles) : (int)std::max<uint32_t>(1u, std::min<uint32_t>((b.D + 127) / 128, (uint32_t)sm_count() * 4u));
@@ -957,11 +958,12 @@ template <class V>
 int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
     if (a.b.list) return launch_list_hv<V>(a, jj, grid, s, pdl);
-    const HvPlan pl = hv_plan(a.b, a.hv_form);
-    if (a.one_read)
-        KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1, true> : k_hv<V, 0, true>, grid, HV_NTHR, 0, s, a, pl, jj));
-    else
-        KRY_CU(launch_ex(pdl, (a.hv_form & 1) ? k_hv<V, 1, false> : k_hv<V, 0, false>, grid, HV_NTHR, 0, s, a, pl, jj));
+    const HvPlan pl = hv_plan(a.b);
+    auto go = [&](auto k0, auto k1, auto k2, auto k3) {
+        return launch_ex(pdl, a.hv_form == 0 ? k0 : a.hv_form == 1 ? k1 : a.hv_form == 2 ? k2 : k3, grid, HV_NTHR, 0, s, a, pl, jj);
+    };
+    if (a.one_read) KRY_CU(go(k_hv<V, 0, true>, k_hv<V, 1, true>, k_hv<V, 2, true>, k_hv<V, 3, true>));
+    else KRY_CU(go(k_hv<V, 0, false>, k_hv<V, 1, false>, k_hv<V, 2, false>, k_hv<V, 3, false>));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
@@ -1089,9 +1091,9 @@ template int launch_ortho<ffc>(const EvArgs<ffc> &, int, int, cudaStream_t, int)
 template int launch_dots<double2>(const EvArgs<double2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<float2>(const EvArgs<float2> &, int, int, int, cudaStream_t, int);
 template int launch_dots<ffc>(const EvArgs<ffc> &, int, int, int, cudaStream_t, int);
-template int vector_grid<double2>(const DevBasis &, int, int *, int *);
-template int vector_grid<float2>(const DevBasis &, int, int *, int *);
-template int vector_grid<ffc>(const DevBasis &, int, int *, int *);
+template int vector_grid<double2>(const DevBasis &, int *, int *);
+template int vector_grid<float2>(const DevBasis &, int *, int *);
+template int vector_grid<ffc>(const DevBasis &, int *, int *);
 template int launch_hv<double2>(const EvArgs<double2> &, int, int, cudaStream_t, int);
 template int launch_hv<float2>(const EvArgs<float2> &, int, int, cudaStream_t, int);
 template int launch_hv<ffc>(const EvArgs<ffc> &, int, int, cudaStream_t, int);

@@ -299,7 +299,7 @@ template <class V> int launch_lincomb(const EvArgs<V> &a, int mode, int jj, int 
                                       cudaStream_t s, int pdl = 1);
 template <class V> int launch_dots(const EvArgs<V> &a, int mode, int jj, int grid, cudaStream_t s, int pdl = 1);
 template <class V> int launch_ortho(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl = 1);
-template <class V> int vector_grid(const DevBasis &b, int hv_form, int *gridH, int *gridB);
+template <class V> int vector_grid(const DevBasis &b, int *gridH, int *gridB);
 int launch_set_basis_state(void *W0, int c64, uint32_t r0, cudaStream_t s, int ff = 0);
 // complex128 <-> float-float vectors of n elements (the boundary of KRY_C128E)
 int launch_c128_to_ffc(const void *src, void *dst, size_t n, cudaStream_t s);
@@ -345,8 +345,8 @@ struct kry_ham_s {
     int g_C;                    // the graph integrates P for C(t)
     size_t g_ldo, g_ldc;
     // per precision, the launch shape of the vector kernels (kry_set_shape, kry_autotune):
-    // [0] CTAs of the streaming kernels (0 = occupancy rule), [1] H.v form (bit 0: other
-    // number of loads at a time; bit 1: twice the blocks per item), [2] dots form (0 several units of rows at a time, 1 one), [3]
+    // [0] CTAs of the streaming kernels (0 = occupancy rule), [1] H.v form (number of
+    // loads at a time; bit 0: lower bits, bit 1: upper bits), [2] dots form (0 several units of rows at a time, 1 one), [3]
     // update rows per thread,
     // [4] batched H.v in chunks of this many realisations (0 = all K)
     int shape[3][5];
@@ -363,7 +363,7 @@ struct kry_ham_s {
 
 // Launch shape of a new Hamiltonian: the occupancy-rule grid, two update
 // rows per thread, all realisations at once, and the H.v with four loads at a time -- from lower
-// parts of 14 bits on (L >= 28) eight (complex64) and twice the blocks per item (3% faster at L = 30).
+// parts of 14 bits on (L >= 28) eight (complex64; two of 16 bytes).
 inline void default_shape(kry_ham_s *H, int Llo)
 {
     const int v[5] = {0, Llo >= 14 ? 3 : 0, 0, 2, 0};

@@ -3,8 +3,8 @@
 // parts, tuned one after another (coordinate descent, each part over its candidates with the
 // others at their best so far):
 //   [0] CTAs of the streaming kernels: the occupancy rule (0) or 1..4 times the SM count;
-//   [1] H.v form: bit 0 = eight gathers at a time (16-byte elements: two), else four, bit 1 = twice
-//       the blocks of upper bits per item;
+//   [1] H.v form: eight gathers at a time (16-byte elements: two) instead of four, bit 0 inside the
+//       lower bits, bit 1 inside the upper bits;
 //   [2] dots: several units of rows at a time where the vectors are few (0) or one (1);
 //   [3] rows per thread of the update pass: 1, 2 or 4;
 //   [4] batched H.v in chunks of 8 or 16 realisations (0 = all K at once).

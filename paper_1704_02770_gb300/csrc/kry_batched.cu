@@ -135,8 +135,9 @@ __global__ void __launch_bounds__(NTHR) k_apply_b(DevBasis b, DevHam hm, int K, 
 // ---------------------------------------------------------------- pass A (batched)
 
 // Part 1: U[:, k] = sigma_j[k] H_k W_j[:, k] for every realisation (warp per state, lanes over
-// k), at full occupancy: nothing but the gathers.
-template <class V, int KQ>
+// k), at full occupancy: nothing but the gathers.  FLAT (K <= 16): a thread per element instead, its
+// realisation fixed, because a warp per state would leave half its lanes and more idle.
+template <class V, int KQ, bool FLAT>
 __global__ void __launch_bounds__(NTHR) k_hv_b(EvArgsB<V> a, int jj)
 {
     using R = typename VT<V>::R;
@@ -149,27 +150,45 @@ __global__ void __launch_bounds__(NTHR) k_hv_b(EvArgsB<V> a, int jj)
     __syncthreads();
     const uint16_t *rl = a.rl_smem ? rl_s : a.b.ranklo;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = a.K;
-    R sg[KQ];
-#pragma unroll
-    for (int q = 0; q < KQ; ++q) {
-        const int k = lane + 32 * q;
-        sg[q] = (k < K) ? (R)ctl->sigma[jj][k] : (R)0;
-    }
     const V *x = a.W + (size_t)jj * a.ldW;
-    const uint32_t D = a.b.D, ntiles = (D + TROWS - 1) / TROWS;
-    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint32_t r0 = tile * TROWS;
-        for (int rr = warp; rr < TROWS; rr += NTHR / 32) {
-            if (r0 + rr >= D) break;
+    const uint32_t D = a.b.D;
+    if constexpr (FLAT) {
+        const uint32_t per = NTHR / K * K;   // elements of a CTA's unit: whole states
+        const int k = threadIdx.x % K;
+        const R sg = (R)ctl->sigma[jj][k];
+        const uint32_t rows = per / K, ntiles = (D + rows - 1) / rows;
+        for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+            const uint32_t r = tile * rows + threadIdx.x / K;
+            if (threadIdx.x >= per || r >= D) break;
             uint32_t hi, off;
             int klo;
-            tile_unrank(a.b, hd->bsz, r0, rr, hi, off, klo);
-            V u[KQ];
-            hv_row_b<V, KQ>(a.b, a.h, x, K, hi, off, klo, hd->koff, rl, u, lane);
+            tile_unrank(a.b, hd->bsz, r & ~(uint32_t)(TILE - 1), r & (uint32_t)(TILE - 1), hi, off, klo);
+            V u[1];
+            hv_row_b<V, 1>(a.b, a.h, x, K, hi, off, klo, hd->koff, rl, u, k);
+            a.U[(size_t)r * K + k] = scale(u[0], sg);
+        }
+    } else {
+        R sg[KQ];
 #pragma unroll
-            for (int q = 0; q < KQ; ++q) {
-                const int k = lane + 32 * q;
-                if (k < K) a.U[(size_t)(r0 + rr) * K + k] = scale(u[q], sg[q]);
+        for (int q = 0; q < KQ; ++q) {
+            const int k = lane + 32 * q;
+            sg[q] = (k < K) ? (R)ctl->sigma[jj][k] : (R)0;
+        }
+        const uint32_t ntiles = (D + TROWS - 1) / TROWS;
+        for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+            const uint32_t r0 = tile * TROWS;
+            for (int rr = warp; rr < TROWS; rr += NTHR / 32) {
+                if (r0 + rr >= D) break;
+                uint32_t hi, off;
+                int klo;
+                tile_unrank(a.b, hd->bsz, r0, rr, hi, off, klo);
+                V u[KQ];
+                hv_row_b<V, KQ>(a.b, a.h, x, K, hi, off, klo, hd->koff, rl, u, lane);
+#pragma unroll
+                for (int q = 0; q < KQ; ++q) {
+                    const int k = lane + 32 * q;
+                    if (k < K) a.U[(size_t)(r0 + rr) * K + k] = scale(u[q], sg[q]);
+                }
             }
         }
     }
@@ -409,25 +428,204 @@ __global__ void __launch_bounds__(NTHR, 1) k_lincomb_b(EvArgsB<V> a, int jj)
     }
 }
 
+// ---------------------------------------------------------------- the one-read pass (batched)
+
+// Threads of a group: the elements of whole states that fit 64 threads, or 128 where that leaves fewer idle.
+static __host__ __device__ int ortho_group(int K) { return K > 64 || (K > 32 && K < 64) ? 128 : 64; }
+// Threads of a CTA: an even number of groups
+// (the 64-bit indices and the coefficients per lane need more registers than k_ortho's)
+template <class V, int T> constexpr int ORTHO_B_NTHR = T == 64 && !std::is_same<V, ffc>::value ? 384 : 256;
+
+constexpr int ALPHA_NTHR = 512;
+
+// Re <W_j[:, k], U[:, k]> of every realisation, on k_ortho_b's split of the elements: the CTAs' shares go to
+// part[CTA][Kp] (doubles).  A pass of its own, because the H.v's forms split the states in different ways
+// and alpha_j's bits must not depend on them; two of the step's j + 5 vector reads.
+template <class V, int T>
+__global__ void __launch_bounds__(ALPHA_NTHR) k_alpha_b(EvArgsB<V> a, int jj)
+{
+    KryCtlB *ctl = a.ctl;
+    if (ctl->hd.done || jj >= ctl->hd.m_run) return;
+    constexpr int NGRP = ALPHA_NTHR / T, NU = 4;
+    using Sum = typename RealAcc<V>::Sum;
+    __shared__ Sum sums[ALPHA_NTHR];
+    const int K = a.K, tid = threadIdx.x, g = tid / T, t = tid % T;
+    const uint32_t unit = T / K * K;
+    const size_t n = (size_t)a.b.D * K;
+    const uint32_t nu = (uint32_t)((n + unit - 1) / unit), du = gridDim.x * NGRP;
+    const V *x = a.W + (size_t)jj * a.ldW;
+    RealAcc<V> al;
+    for (uint32_t u0 = blockIdx.x * NGRP + g; u0 < nu; u0 += NU * du) {
+        V xv[NU], uv[NU];
+#pragma unroll
+        for (int q = 0; q < NU; ++q) {
+            const size_t r = (size_t)(u0 + q * du) * unit + t;
+            const bool in = t < (int)unit && u0 + q * du < nu && r < n;
+            xv[q] = ldg_if(in, x + r);
+            uv[q] = ldg_if(in, a.U + r);
+        }
+#pragma unroll
+        for (int q = 0; q < NU; ++q) al.add(xv[q], RealAcc<V>::pre(uv[q]));
+        al.renorm();
+    }
+    sums[tid] = al.sum();
+    __syncthreads();
+    if (tid < a.Kp) {
+        Sum tot{};
+        if (tid < K)
+            for (int gg = 0; gg < NGRP; ++gg)
+                for (uint32_t r = tid; r < unit; r += K) tot = add2(tot, sums[gg * T + r]);
+        ((double *)a.part)[(size_t)blockIdx.x * a.Kp + tid] = to_double(tot);
+    }
+}
+
+// k_ortho for K realisations: thread t of a group takes the element of state t / K and realisation t % K of
+// its unit of T / K states, so that its accumulators belong to one realisation; the coefficients are kept
+// per realisation in shared memory.  At the end the sums of a realisation's threads go to part[CTA][slot].
+// The two-pass form pads K to 32, 64 or 128 lanes and reads the vectors twice.
+template <class V, int T>
+__global__ void __launch_bounds__(ORTHO_B_NTHR<V, T>, 1) k_ortho_b(EvArgsB<V> a, int jj)
+{
+    KryCtlB *ctl = a.ctl;
+    if (ctl->hd.done || jj >= ctl->hd.m_run) return;
+    constexpr int QV = ORTHO_QV, NT = ORTHO_B_NTHR<V, T>, NGRP = NT / T;
+    using RCoef = typename RealLin<V>::RCoef;
+    using Sum = typename RealAcc<V>::Sum;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int K = a.K, tid = threadIdx.x, g = tid / T, t = tid % T;
+    const uint32_t unit = T / K * K;
+    const int k = t % K;   // (threads past the unit sum zeros)
+    RCoef *coef = (RCoef *)smem;                              // [MMAX + 1][K]
+    float *mcoef = (float *)(coef + (MMAX + 1) * K);          // [MMAX + 1][K]
+    const size_t off = ((sizeof(RCoef) + sizeof(float)) * (MMAX + 1) * K + 15) & ~(size_t)15;
+    V *xch = (V *)(smem + off);                               // [2][NGRP][T][XU]
+    Sum *sums = (Sum *)(smem + off);                          // afterwards [QV + 3][NT]
+    bool mine = true;
+    for (int e = tid; e < (jj + 1) * K; e += NT) {
+        const double c = ctl->coefA[e / K][e % K];
+        coef[e] = RealLin<V>::coef(c);
+        mcoef[e] = -(float)c;
+    }
+    if (MinorSum<V>::use && tid < K) mine = ctl->minor[tid] != 0;
+    const bool minor = __syncthreads_and(mine) && MinorSum<V>::use;
+    const int nv = jj + 1;
+    const int nvg = nv <= QV ? 1 : 2, nrp = NGRP / nvg;
+    const int rp = g / nvg, vg = (g + rp) % nvg;
+    const int i0 = (nv * vg) / nvg, nq = (nv * (vg + 1)) / nvg - i0, pad = ortho_pad(nq);
+    const size_t n = (size_t)a.b.D * K;
+    const uint32_t nu = (uint32_t)((n + unit - 1) / unit), du = gridDim.x * nrp;
+    RealAcc<V> acc[QV], nrm;
+    DotAcc<V> gacc;
+    V *out = a.W + (size_t)(jj + 1) * a.ldW;
+#define KRY_ORTHO(NQ, NU, KIND)                                                                                      \
+    ortho_rows<V, NQ, NU, KIND, T, NGRP, 2>(a.W, a.ldW, a.U, a.G, out, n, unit, t, i0, nq, minor, rp, blockIdx.x * nrp + rp, \
+                                      du, nu, jj & 1, coef + k, mcoef + k, K, xch, acc, nrm, gacc)
+#define KRY_ORTHO_N(NQ, NU) \
+    case NQ: KRY_ORTHO(NQ, NU, ORTHO_ONLY); break;
+#define KRY_ORTHO_3(NQ)                                           \
+    case NQ:                                                      \
+        if (nvg == 1) KRY_ORTHO(NQ, 1, ORTHO_ONLY);               \
+        else if (vg == 0) KRY_ORTHO(NQ, 1, ORTHO_FIRST);          \
+        else KRY_ORTHO(NQ, 1, ORTHO_LAST);                        \
+        break;
+    if (rp < nrp) {
+        switch (nq + pad) {
+            KRY_ORTHO_N(1, 8)
+            KRY_ORTHO_N(2, 4)
+            KRY_ORTHO_N(3, 4)
+            KRY_ORTHO_N(4, 4)
+            KRY_ORTHO_N(6, 2)
+            KRY_ORTHO_3(8)
+            KRY_ORTHO_3(10)
+            KRY_ORTHO_3(12)
+            KRY_ORTHO_3(14)
+            KRY_ORTHO_3(15)
+            KRY_ORTHO_3(16)
+        default: break;
+        }
+    }
+#undef KRY_ORTHO_3
+#undef KRY_ORTHO_N
+#undef KRY_ORTHO
+    __syncthreads();   // (the exchange buffers become the sums)
+#pragma unroll
+    for (int q = 0; q < QV; ++q) {
+        acc[q].renorm();
+        sums[q * NT + tid] = acc[q].sum();
+    }
+    nrm.renorm();
+    sums[QV * NT + tid] = nrm.sum();
+    if (a.G) {
+        gacc.renorm();
+        const double2 gv = gacc.value();
+        sums[(QV + 1) * NT + tid] = from_double<Sum>(gv.x);
+        sums[(QV + 2) * NT + tid] = from_double<Sum>(gv.y);
+    }
+    __syncthreads();
+    double2 *pc = a.part + (size_t)blockIdx.x * PSB * a.Kp;
+    const int nslot = nv + 1 + (a.G ? 2 : 0);
+    for (int e = tid; e < nslot * K; e += NT) {
+        const int i = e / K, kk = e % K;
+        int s = 0, q;   // the share and slot that hold sum i
+        if (i < nv) {
+            s = nvg == 1 || i < nv / 2 ? 0 : 1;
+            const int f = s ? nv / 2 : 0, ns = nvg == 1 ? nv : s ? nv - nv / 2 : nv / 2;
+            q = i - f + ortho_pad(ns);
+        } else {
+            q = QV + (i - nv);
+        }
+        Sum tot{};
+        for (int p = 0; p < nrp; ++p) {
+            const int gg = p * nvg + (nvg == 1 ? 0 : (s + p) & 1);   // the group of share s in part p
+            for (uint32_t r = kk; r < unit; r += K) tot = add2(tot, sums[q * NT + gg * T + r]);
+        }
+        const double v = to_double(tot);
+        if (i < nv) pc[(size_t)i * a.Kp + kk] = make_double2(v, 0.0);
+        else if (i == nv) pc[(size_t)SLOT_NRM * a.Kp + kk] = make_double2(v, 0.0);
+        else if (i == nv + 1) pc[(size_t)SLOT_G * a.Kp + kk].x = v;
+        else pc[(size_t)SLOT_G * a.Kp + kk].y = v;
+    }
+}
+
 // ---------------------------------------------------------------- per-realisation reductions
 
 // mode: 0 pass A, 1 pass B, 3 pass C1 (dots of w), 2 pass C2 (correction), 4 combine,
-// 5 load of a general psi0.  One CTA per realisation.  A warp takes a whole slot (lanes over the
+// 5 load of a general psi0; one-read form: 6 alpha_j and the update's coefficients (partials [CTA][Kp]
+// of k_alpha_b), 7 the dots and the norm of the update (see k_ortho).  One CTA per realisation.  A warp takes a whole slot (lanes over the
 // CTAs' partials) and lane i of warp 0 the scalars of vector i: GB300 issues
 // one FP64 warp instruction per about 77 cycles and SM sub-partition whatever its active lanes, so
 // block-wide trees slot by slot and loops over the vectors in one thread cost tens of us at j = 30.
 __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *__restrict__ part,
-                                                  int grid, int Kp, int mode, int jj, int general)
+                                                  int grid, int Kp, int mode, int jj, int general, float *Cb,
+                                                  float *db)
 {
     KryHdrB &H = ctl->hd;
     if (H.done) return;
-    if (mode <= 3 && jj >= H.m_run) return;
+    if ((mode <= 3 || mode >= 6) && jj >= H.m_run) return;
     const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (mode == 2 && !H.corr_any) return;   // pass C2 did not run
     if (mode == 3 && !H.dots_any) return;   // pass C1 did not run
     __shared__ double2 fin[PSB];
-    const int nd = (mode == 0 || mode == 3) ? jj + 1 : 0;
-    const int ns = nd + (mode != 3 ? 1 : 0) + (general && mode != 0 && mode != 3 ? 1 : 0);
+    __shared__ float Cs[MMAX * MMAX], ds[MMAX + 1];
+    const int nd = (mode == 0 || mode == 3 || mode == 7) ? jj + 1 : 0;
+    const int ns = mode == 6 ? 0 : nd + (mode != 3 ? 1 : 0) + (general && mode != 0 && mode != 3 ? 1 : 0);
+    if (mode == 6) {
+        for (int e = tid; e < MMAX * MMAX; e += 256) Cs[e] = Cb[(size_t)k * MMAX * MMAX + e];
+        if (tid <= MMAX) ds[tid] = tid < jj ? db[(size_t)k * MMAX + tid] : 0.f;
+        if (warp == 0) {
+            double s = 0.0;
+            for (int c0 = 0; c0 < grid; c0 += 256) {
+                double x[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int c = c0 + 32 * i + lane;
+                    x[i] = c < grid ? __ldg((const double *)part + (size_t)c * Kp + k) : 0.0;
+                }
+                s += warp_sum_int<8>(x);
+            }
+            if (lane == 0) fin[0].x = s;
+        }
+    }
     for (int q = warp; q < ns; q += 8) {
         const int slot = q < nd ? q : q == nd ? SLOT_NRM : SLOT_G;
         double2 s = make_double2(0.0, 0.0);
@@ -458,6 +656,42 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         const double s = ctl->sigma[lane][k];
         c = fin[lane].x * s;
         cs = c * s;
+    }
+    if (mode == 6) {
+        if (k == 0 && lane == 0) {
+            H.n_hv += 1;
+            H.vec_passes += 2;
+            H.vp_kind[KIND_HV] += 2;
+            H.corr_any = 0;
+            H.dots_any = 0;
+        }
+        const bool run = jj < ctl->m_eff[k], inv = lane <= jj;
+        const double s = inv ? ctl->sigma[lane][k] : 0.0, alpha = fin[0].x * ctl->sigma[jj][k];
+        double cc = 0.0;
+        if (lane < jj) {
+            float f = 0.f;
+            for (int i = 0; i <= lane; ++i) f = fmaf(Cs[i * MMAX + lane], ds[i], f);
+            const double b = ctl->beta[lane][k];
+            cc = lane == jj - 1 ? b + (double)f : (double)fmaf((float)b, ds[lane + 1], f);
+        } else if (lane == jj) {
+            cc = alpha;
+        }
+        if (!run) cc = 0.0;   // (invariant subspace already reached: the next vectors stay zero)
+        const double q2 = cc * cc, c2 = warp_sum_int<1>(&q2);
+        const bool small = lane + 1 < jj;
+        const double cm = small ? q2 : 0.0, m2 = warp_sum_int<1>(&cm), big = small ? 0.0 : q2, b2 = warp_sum_int<1>(&big);
+        // rounding level (MinorSum; its bound for complex128, the smaller one, for both types)
+        const bool minor = __all_sync(0xffffffffu, !small || !run || (s >= 0x1p-40 && s <= 0x1p40)) &&
+                           m2 <= MinorSum<double2>::eta * MinorSum<double2>::eta * b2;
+        if (inv) {
+            ctl->coefA[lane][k] = cc * s;
+            Cb[((size_t)k * MMAX + lane) * MMAX + jj] = (float)cc;
+        }
+        if (lane != 0) return;
+        ctl->c2[k] = c2;
+        ctl->minor[k] = minor ? 1 : 0;
+        if (run) ctl->alpha[jj][k] = alpha;
+        return;
     }
     auto finalize = [&](double w2, double2 gd) {
         const double bt = sqrt(w2);
@@ -507,6 +741,29 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         } else {
             finalize(nw2, gdot);
         }
+    } else if (mode == 7) {
+        if (k == 0 && lane == 0) {
+            H.vec_passes += jj + 3 + (general ? 1 : 0);
+            H.vp_kind[KIND_PASSB] += jj + 3 + (general ? 1 : 0);
+        }
+        const double cc = c * c, nd2 = warp_sum_int<1>(&cc);
+        const bool run = jj < ctl->m_eff[k];
+        const double normu2 = ctl->c2[k] + nw2;   // ||u||^2 = ||c||^2 + ||w||^2
+        const bool dead = !(nw2 > H.eta_bd * H.eta_bd * normu2);
+        const bool sub = run && !dead && nd2 > H.eta_corr * H.eta_corr * nw2;
+        if (lane <= jj) {
+            ctl->coefC[lane][k] = sub ? cs : 0.0;
+            if (sub) Cb[((size_t)k * MMAX + lane) * MMAX + jj] += (float)c;
+            db[(size_t)k * MMAX + lane] = sub || dead || !run ? 0.f : (float)(c * rsqrt(nw2));
+        }
+        if (sub && lane == jj) ctl->alpha[jj][k] += c;
+        if (lane != 0) return;
+        ctl->corr[k] = sub ? 1 : 0;
+        if (!run) return;
+        ctl->normu2[k] = normu2;
+        if ((H.verify || sub) && nw2 > 0.0) ctl->orth[k] = fmax(ctl->orth[k], sqrt(nd2 / nw2));
+        if (sub) H.corr_any = 1;
+        else finalize(nw2, gdot);
     } else if (mode == 3) {
         if (k == 0 && lane == 0) {
             H.vec_passes += jj + 2;
@@ -633,7 +890,7 @@ int batched_grid(const DevBasis &b, int Kp, int rl_smem, int *gridB)
     const size_t es = sizeof(V);
     int o1 = 1, o2 = 1;
     KRY_KQ_SWITCH(Kp, {
-        if (int rc = set_smem(k_hv_b<V, KQ>, hv_b_smem(b, rl_smem))) return -rc;
+        if (int rc = set_smem(k_hv_b<V, KQ, false>, hv_b_smem(b, rl_smem))) return -rc;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_dots_b<V, KQ>, NTHR, 0);
         const size_t sL = lincomb_b_smem(Kp, es);
         if (int rc = set_smem(k_lincomb_b<V, 0, KQ>, sL)) return -rc;
@@ -645,6 +902,54 @@ int batched_grid(const DevBasis &b, int Kp, int rl_smem, int *gridB)
     };
     *gridB = fit(o2);
     return fit(o1);
+}
+
+// The H.v at full occupancy, its own grid
+template <class V>
+static int launch_hv_b(const EvArgsB<V> &a, int jj, cudaStream_t s)
+{
+    const size_t sH = hv_b_smem(a.b, a.rl_smem);
+    auto go = [&](auto kernel, uint32_t items) {
+        int oh = 0;
+        if (int rc = set_smem(kernel, sH)) return rc;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&oh, kernel, NTHR, sH);
+        const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(items, (uint32_t)(sm_count_b() * std::max(1, oh))));
+        kernel<<<grid, NTHR, sH, s>>>(a, jj);
+        KRY_CU(cudaGetLastError());
+        return (int)KRY_OK;
+    };
+    if (a.K <= 16) {
+        const uint32_t rows = (uint32_t)(NTHR / a.K);
+        return go(k_hv_b<V, 1, true>, (a.b.D + rows - 1) / rows);
+    }
+    KRY_KQ_SWITCH(a.Kp, { return go(k_hv_b<V, KQ, false>, (a.b.D + TROWS - 1) / TROWS); });
+    return KRY_OK;
+}
+
+// alpha_j's partial sums; returns the CTAs (the reduction's grid), or minus a status
+template <class V>
+int launch_alpha_b(const EvArgsB<V> &a, int jj, cudaStream_t s)
+{
+    const size_t units = ((size_t)a.b.D * a.K + ALPHA_NTHR - 1) / ALPHA_NTHR;
+    const int grid = (int)std::max<size_t>(1, std::min<size_t>((units + 3) / 4, (size_t)sm_count_b() * 2));
+    if (ortho_group(a.K) == 64) k_alpha_b<V, 64><<<grid, ALPHA_NTHR, 0, s>>>(a, jj);
+    else k_alpha_b<V, 128><<<grid, ALPHA_NTHR, 0, s>>>(a, jj);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? grid : -cuda_fail(e, "k_alpha_b");
+}
+
+template <class V>
+int launch_ortho_b(const EvArgsB<V> &a, int jj, int grid, cudaStream_t s)
+{
+    auto go = [&](auto kernel, int nt) {
+        const size_t off = ((sizeof(typename RealLin<V>::RCoef) + sizeof(float)) * (MMAX + 1) * a.K + 15) & ~(size_t)15;
+        const size_t sm = off + std::max(sizeof(V) * 2 * nt * ORTHO_XU, sizeof(typename RealAcc<V>::Sum) * (ORTHO_QV + 3) * nt);
+        if (int rc = set_smem(kernel, sm)) return rc;
+        kernel<<<grid, nt, sm, s>>>(a, jj);
+        KRY_CU(cudaGetLastError());
+        return (int)KRY_OK;
+    };
+    return ortho_group(a.K) == 64 ? go(k_ortho_b<V, 64>, ORTHO_B_NTHR<V, 64>) : go(k_ortho_b<V, 128>, ORTHO_B_NTHR<V, 128>);
 }
 
 // pass A: the H.v at full occupancy (its own grid), then the dots on the common grid
@@ -682,8 +987,7 @@ int launch_passA_b(const EvArgsB<V> &a, int jj, int grid, cudaStream_t s, int pa
         }
         KRY_CU(cudaGetLastError());
     } else {
-        KRY_KQ_SWITCH(a.Kp, { k_hv_b<V, KQ><<<hv_grid(k_hv_b<V, KQ>, ntiles), NTHR, sH, s>>>(a, jj); });
-        KRY_CU(cudaGetLastError());
+        if (int rc = launch_hv_b<V>(a, jj, s)) return rc;
     }
     if (part == 1) return KRY_OK;
     KRY_KQ_SWITCH(a.Kp, { k_dots_b<V, KQ><<<grid, NTHR, 0, s>>>(a, jj); });
@@ -711,9 +1015,9 @@ int launch_lincomb_b(const EvArgsB<V> &a, int mode, int jj, int grid, cudaStream
 // mode 0, 1 follow passes A, B; 3 and 2 passes C1 and C2; 4 the combine (then the shared
 // step bookkeeping); 5 the load of a general psi0.
 int launch_reduce_b(KryCtlB *ctl, const double2 *part, int grid, int K, int Kp, int mode, int jj,
-                    int general, double, cudaStream_t s)
+                    int general, cudaStream_t s, float *C, float *d)
 {
-    k_reduce_b<<<K, 256, 0, s>>>(ctl, part, grid, Kp, mode, jj, general);
+    k_reduce_b<<<K, 256, 0, s>>>(ctl, part, grid, Kp, mode, jj, general, C, d);
     KRY_CU(cudaGetLastError());
     if (mode == 2) {
         k_mrun_b<<<1, 1, 0, s>>>(ctl);
@@ -757,10 +1061,16 @@ int launch_set_basis_state_b(void *W0, int c64, int K, const KryCtlB *ctl, cudaS
     return KRY_OK;
 }
 
+template int launch_alpha_b<ffc>(const EvArgsB<ffc> &, int, cudaStream_t);
+template int launch_ortho_b<ffc>(const EvArgsB<ffc> &, int, int, cudaStream_t);
 template int batched_grid<ffc>(const DevBasis &, int, int, int *);
 template int launch_passA_b<ffc>(const EvArgsB<ffc> &, int, int, cudaStream_t, int);
 template int launch_lincomb_b<ffc>(const EvArgsB<ffc> &, int, int, int, cudaStream_t);
+template int launch_alpha_b<double2>(const EvArgsB<double2> &, int, cudaStream_t);
+template int launch_ortho_b<double2>(const EvArgsB<double2> &, int, int, cudaStream_t);
 template int batched_grid<double2>(const DevBasis &, int, int, int *);
+template int launch_alpha_b<float2>(const EvArgsB<float2> &, int, cudaStream_t);
+template int launch_ortho_b<float2>(const EvArgsB<float2> &, int, int, cudaStream_t);
 template int batched_grid<float2>(const DevBasis &, int, int, int *);
 template int launch_passA_b<double2>(const EvArgsB<double2> &, int, int, cudaStream_t, int);
 template int launch_passA_b<float2>(const EvArgsB<float2> &, int, int, cudaStream_t, int);

@@ -542,6 +542,14 @@ __device__ __forceinline__ T warp_totals(T *v)
     for (; o >= 1; o >>= 1) v[0] = add2(v[0], shfl_xor(v[0], o));
     return v[0];
 }
+__device__ __forceinline__ double add2(double a, double b) { return a + b; }
+template <class S> __device__ __forceinline__ S from_double(double v);
+template <> __device__ __forceinline__ double from_double<double>(double v) { return v; }
+template <> __device__ __forceinline__ FF from_double<FF>(double v)
+{
+    const float2 f = dsplit(v);
+    return FF{f.x, f.y};
+}
 __device__ __forceinline__ double to_double(double v) { return v; }
 __device__ __forceinline__ double to_double(FF v) { return (double)v.s + (double)v.c; }
 
@@ -855,6 +863,131 @@ __device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, Kr
     ctl->vec_passes += 2;
     ctl->vp_kind[KIND_HV] += 2;   // the H.v: v_j read, u written
     ctl->counter = 0;
+}
+
+// ---------------------------------------------------------------- the one-read pass: rows
+// (k_ortho, k_ortho_b)
+
+// Threads of a CTA (one per SM): 16 vectors' rows and accumulators take 96 to 128 registers.
+template <class V> constexpr int ORTHO_NTHR = std::is_same<V, ffc>::value ? 384 : 512;
+constexpr int ORTHO_QV = 16;   // vectors of a group, at most
+constexpr int ORTHO_XU = 2;    // units of a team between two barriers, at most
+
+// The loop is instantiated for 1, 2, 3, 4, 6, 8, 10, 12, 14, 15 and 16 vectors: empty slots of a group of n.
+__device__ __forceinline__ int ortho_pad(int n) { return n <= 4 || n == 15 ? 0 : n & 1; }
+
+// What a group of T threads does besides its own vectors' terms and dots: FIRST stores w and takes ||w||^2
+// and <psi0, w>, LAST holds u and the terms j - 1 and j.
+enum { ORTHO_FIRST = 1, ORTHO_LAST = 2, ORTHO_ONLY = 3 };
+
+// The row loop for one of the CTA's NG groups: the nq = NQ or NQ - 1 vectors from i0 on (the first of NQ slots is empty in
+// the latter case), NU units of `unit` elements at a time (thread t of the group takes element t of a unit).
+// The vectors' elements are read once, kept in registers, and used for the update and for the dots with its
+// result; with two groups to a team their partial updates meet in shared memory (two buffers, one barrier
+// per NU units).  The coefficient of vector i is coef[i * cs], its FP32 form mcoef[i * cs].
+template <class V, int NQ, int NU, int KIND, int T, int NG, int B>
+__device__ __forceinline__ void ortho_rows(const V *W, size_t ldW, const V *U, const V *G, V *out, size_t n, uint32_t unit,
+                                           uint32_t t, int i0, int nq, bool minor, int rp, uint32_t first, uint32_t du,
+                                           uint32_t nu, bool back, const typename RealLin<V>::RCoef *coef,
+                                           const float *mcoef, int cs, V *xch, RealAcc<V> *acc, RealAcc<V> &nrm,
+                                           DotAcc<V> &gacc)
+{
+    // (single realisations index rows by 32 bits, batched ones elements of [D][K] by 64)
+    using idx_t = typename std::conditional<B == 1, uint32_t, size_t>::type;
+    constexpr uint32_t FOLD = 8;   // elements between two foldings of the float-float compensations
+    constexpr bool LAST = KIND & ORTHO_LAST, FIRST = KIND & ORTHO_FIRST;
+    constexpr int NMAJ = NQ < 2 ? 1 : 2;   // (LAST) terms j - 1 and j
+    const int pad = NQ - nq;
+    const V *Wg = W + (ptrdiff_t)(i0 - pad) * (ptrdiff_t)ldW;   // (slot 0 is not read where pad is 1)
+    const int step = B == 1 ? 1 : cs;
+    coef += i0 * step;
+    mcoef += i0 * step;
+    uint32_t it = 0;
+    for (uint32_t u0 = first; u0 < nu; u0 += NU * du) {
+        idx_t r[NU];
+        V x[NU][NQ], uu[NU];
+#pragma unroll
+        for (int k = 0; k < NU; ++k) {
+            const uint32_t u = u0 + k * du;
+            r[k] = u < nu && t < unit ? (idx_t)(back ? nu - 1 - u : u) * unit + t : (idx_t)n;
+            const bool in = r[k] < (idx_t)n;
+            uu[k] = VT<V>::zero();
+            if (LAST) uu[k] = ldg_if(in, U + r[k]);
+            x[k][0] = ldg_if(in && pad == 0, Wg + r[k]);
+#pragma unroll
+            for (int q = 1; q < NQ; ++q) x[k][q] = ldg_if(in, Wg + (size_t)q * ldW + r[k]);
+        }
+        // this group's share of w = u - sum c_i W_i; terms at rounding level in FP32
+        RealLin<V> l[NU];
+        float2 f[NU];
+#pragma unroll
+        for (int k = 0; k < NU; ++k) {
+            l[k] = RealLin<V>(uu[k]);
+            f[k] = make_float2(0.f, 0.f);
+        }
+        if (MinorSum<V>::use && minor) {
+            if constexpr (MinorSum<V>::use) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    const int i = (q == 0 ? 0 : q - pad) * step;   // (an empty slot's x is zero)
+#pragma unroll
+                    for (int k = 0; k < NU; ++k) {
+                        if (LAST && q >= NQ - NMAJ) l[k].fms(coef[i], x[k][q]);
+                        else f[k] = __ffma2_rn(make_float2(mcoef[i], mcoef[i]), MinorSum<V>::lead(x[k][q]), f[k]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < NU; ++k)
+                    if (LAST) MinorSum<V>::add(l[k], f[k]);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                for (int k = 0; k < NU; ++k) l[k].fms(coef[(q == 0 ? 0 : q - pad) * step], x[k][q]);
+        }
+        if (KIND != ORTHO_ONLY) {
+            // publish this share, meet, take the team's other one: w = LAST's + FIRST's
+            V *buf = xch + ((it & 1) * NG + 2 * rp) * T * ORTHO_XU + t;
+#pragma unroll
+            for (int k = 0; k < NU; ++k) {
+                if (LAST) buf[T * k] = l[k].out();
+                else if (MinorSum<V>::use && minor) *(float2 *)(buf + T * (ORTHO_XU + k)) = f[k];
+                else buf[T * (ORTHO_XU + k)] = l[k].out();
+            }
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + rp), "n"(2 * T) : "memory");
+#pragma unroll
+            for (int k = 0; k < NU; ++k) {
+                if (!LAST) l[k] = RealLin<V>(buf[T * k]);
+                if (MinorSum<V>::use && minor) {
+                    if constexpr (MinorSum<V>::use)
+                        MinorSum<V>::add(l[k], LAST ? *(const float2 *)(buf + T * (ORTHO_XU + k)) : f[k]);
+                } else {
+                    l[k].add(buf[T * (ORTHO_XU + k)]);
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NU; ++k) {
+            if (NU > 1 && KIND == ORTHO_ONLY && u0 + k * du >= nu) break;
+            const V w = l[k].out();
+            const typename RealAcc<V>::Pre p = RealAcc<V>::pre(w);
+            if (FIRST) nrm.add(w, p);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) acc[q].add(x[k][q], p);
+            if (FIRST && r[k] < (idx_t)n) {
+                out[r[k]] = w;
+                if (G) gacc.add(ldg(G + r[k]), w);
+            }
+        }
+        it += 1;
+        if (it % (FOLD / NU) == 0) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) acc[q].renorm();
+            nrm.renorm();
+            gacc.renorm();
+        }
+    }
 }
 
 // ---------------------------------------------------------------- rank tables

@@ -70,7 +70,7 @@ int ensure_workspace(kry_ham_s *H, size_t bytes)
 }
 
 struct Layout {
-    size_t ldW, oW, oU, oG, oPart, oCtl, oTimes, oP, oY, oC, oGL, bytes;
+    size_t ldW, oW, oU, oG, oPart, oCtl, oTimes, oP, oY, oC, oGL, oCd, bytes;
 };
 
 void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w);   // (adjoint section)
@@ -499,9 +499,14 @@ Layout layout_b(const kry_ham_s *H, int dtype, int m, int grid, int n_times)
     l.oP = round_up(l.oTimes + sizeof(double) * (size_t)n_times, 256);
     l.oC = round_up(l.oP + sizeof(double) * (size_t)n_times * H->K, 256);
     l.oGL = round_up(l.oC + sizeof(double) * (size_t)n_times * H->K, 256);
-    l.bytes = round_up(l.oGL + sizeof(double) * 2 * NGL, 256);
+    l.oCd = round_up(l.oGL + sizeof(double) * 2 * NGL, 256);
+    l.bytes = round_up(l.oCd + sizeof(float) * (MMAX + 1) * MMAX * (size_t)H->K, 256);
     return l;
 }
+
+// The batched one-read form (k_ortho_b), from 32,768 elements on (L = 15 K = 9 c128, 57,915 elements: 88 ->
+// 50 us per Lanczos index; L = 20 K = 64 c64: 819 -> 581).
+int one_read_form_b(const kry_ham_s *H) { return (size_t)H->b->D * (size_t)H->K >= 32768u ? 1 : 0; }
 
 // CTAs of the batched dots of pass A (returned) and of the update, second pass and combine
 // (*gridB), both by the occupancy rule; an autotuned override sets *gridB.
@@ -509,6 +514,20 @@ int grid_for_b(const kry_ham_s *H, int dtype, int *gridB)
 {
     const DevBasis &b = H->b->dev;
     const int Kp = padded_k(H->K);
+    if (one_read_form_b(H)) {
+        // k_ortho_b: one CTA per SM, each at least a unit of states for every group
+        int dev = 0, sms = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const size_t units = ((size_t)b.D * (size_t)H->K + 511) / 512;
+        const int og = (int)std::max<size_t>(1, std::min<size_t>(units, (size_t)sms));
+        const int g0 = dtype == KRY_C64     ? batched_grid<float2>(b, Kp, rl_in_smem(b), gridB)
+                       : dtype == KRY_C128E ? batched_grid<ffc>(b, Kp, rl_in_smem(b), gridB)
+                                            : batched_grid<double2>(b, Kp, rl_in_smem(b), gridB);
+        if (g0 <= 0) return g0;
+        if (H->shape[dtype_slot(dtype)][0] > 0) *gridB = H->shape[dtype_slot(dtype)][0];
+        return og;
+    }
     const int g = dtype == KRY_C64     ? batched_grid<float2>(b, Kp, rl_in_smem(b), gridB)
                   : dtype == KRY_C128E ? batched_grid<ffc>(b, Kp, rl_in_smem(b), gridB)
                                        : batched_grid<double2>(b, Kp, rl_in_smem(b), gridB);
@@ -542,24 +561,42 @@ int capture_step_b(kry_ham_s *H, const EvArgsB<V> &a, const ExpArgsB &ea, int m,
     const double2 *part = a.part;
     for (int jj = 0; jj < m && rc == KRY_OK; ++jj) {
         mark();
+        if (a.one_read) {
+            // the H.v, alpha_j and its reduction; update and dots, their reduction; C2, its reduction, m_run
+            rc = launch_passA_b<V>(a, jj, grid, cs, 1);
+            int ga = 0;
+            if (rc == KRY_OK) {
+                ga = launch_alpha_b<V>(a, jj, cs);
+                if (ga <= 0) rc = -ga;
+            }
+            if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, ga, a.K, a.Kp, 6, jj, general, cs, a.C, a.d);
+            mark();
+            mark();
+            if (rc == KRY_OK) rc = launch_ortho_b<V>(a, jj, grid, cs);
+            if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, grid, a.K, a.Kp, 7, jj, general, cs, a.C, a.d);
+            mark();
+            if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 1, jj, gridB, cs);
+            if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 2, jj, general, cs);
+            continue;
+        }
         rc = launch_passA_b<V>(a, jj, grid, cs, 1);
         mark();
         if (rc == KRY_OK) rc = launch_passA_b<V>(a, jj, grid, cs, 2);
-        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, grid, a.K, a.Kp, 0, jj, general, 0, cs);
+        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, grid, a.K, a.Kp, 0, jj, general, cs);
         mark();
         if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 0, jj, gridB, cs);
-        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 1, jj, general, 0, cs);
+        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 1, jj, general, cs);
         mark();
         if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 4, jj, gridB, cs);
-        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 3, jj, general, 0, cs);
+        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 3, jj, general, cs);
         if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 1, jj, gridB, cs);
-        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 2, jj, general, 0, cs);
+        if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 2, jj, general, cs);
     }
     mark();
     if (rc == KRY_OK) rc = launch_exp_b(ea, cs);
     mark();
     if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 2, 0, gridB, cs);
-    if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 4, 0, general, 0, cs);
+    if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 4, 0, general, cs);
     mark();
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     if (rc != KRY_OK) { if (g) cudaGraphDestroy(g); return rc; }
@@ -598,6 +635,9 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
     a.Kp = Kp;
     a.rl_smem = rl_in_smem(b);
     a.kch = H->shape[dtype_slot(dtype)][4];
+    a.one_read = one_read_form_b(H);
+    a.C = (float *)(base + l.oCd);
+    a.d = a.C + (size_t)MMAX * MMAX * K;
     ExpArgsB ea{};
     ea.ctl = a.ctl;
     ea.times = (const double *)(base + l.oTimes);
@@ -681,7 +721,7 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
             KRY_CU(cudaMemcpyAsync((void *)a.G, d_psi0, nvec * es, cudaMemcpyDeviceToDevice, s));
         }
         if (int rc = launch_lincomb_b<V>(a, 3, 0, gridB, s)) return rc;
-        if (int rc = launch_reduce_b(a.ctl, a.part, gridB, K, Kp, 5, 0, 1, 0, s)) return rc;
+        if (int rc = launch_reduce_b(a.ctl, a.part, gridB, K, Kp, 5, 0, 1, s)) return rc;
     } else {
         KRY_CU(cudaMemsetAsync(a.W, 0, nvec * es, s));
         if (int rc = launch_set_basis_state_b(a.W, dtype == KRY_C64, K, a.ctl, s, FF)) return rc;
@@ -700,6 +740,7 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
             for (int k = 0; k < n_intervals(m); ++k) {
                 float ms = 0.f;
                 KRY_CU(cudaEventElapsedTime(&ms, H->prof_ev[k], H->prof_ev[k + 1]));
+                if (a.one_read && kind_of(k, m) == KIND_PASSA) continue;   // (no kernel there)
                 H->prof_ms[kind_of(k, m)] += ms;
                 H->prof_launches[kind_of(k, m)] += 1;
             }
@@ -743,7 +784,7 @@ int evolve_bt(kry_ham_s *H, int dtype, const void *d_psi0, uint64_t state, bool 
         st->max_orth_loss = *std::max_element(orth.begin(), orth.end());
         st->time_ms = ms;
         st->algo_bytes = (double)hp->vec_passes * (double)nvec * (double)es;
-        st->n_launches = launched * (10 * m + 5) + (general ? 2 : 1) + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
+        st->n_launches = launched * ((a.one_read ? 8 : 10) * m + 5) + (general ? 2 : 1) + (FF && general ? 1 : 0) + (FF && d_psi_out ? 1 : 0);
         st->n_second_dots = 0;
     }
     return KRY_OK;

@@ -302,124 +302,6 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
 
 // ---------------------------------------------------------------- the one-read pass
 
-// Threads of k_ortho's CTA (one per SM): 16 vectors' rows and accumulators take 96 to 128 registers.
-template <class V> constexpr int ORTHO_NTHR = std::is_same<V, ffc>::value ? 384 : 512;
-constexpr int ORTHO_QV = 16;   // vectors of a group, at most
-constexpr int ORTHO_XU = 2;    // units of a team between two barriers, at most
-
-// The loop is instantiated for 1, 2, 3, 4, 6, 8, 10, 12, 14, 15 and 16 vectors: empty slots of a group of n.
-__device__ __forceinline__ int ortho_pad(int n) { return n <= 4 || n == 15 ? 0 : n & 1; }
-
-// What a 64-thread group of k_ortho does besides its own vectors' terms and dots: FIRST stores w and
-// takes ||w||^2 and <psi0, w>, LAST holds u and the terms j - 1 and j.
-enum { ORTHO_FIRST = 1, ORTHO_LAST = 2, ORTHO_ONLY = 3 };
-
-// The row loop of k_ortho for one group: the nq = NQ or NQ - 1 vectors from i0 on (the first of NQ slots
-// is empty in the latter case), NU units of 64 rows at a time.  The vectors' rows are read once, kept in
-// registers, and used for the update and for the dots with its result; with two groups to a team their
-// partial updates meet in shared memory (two buffers, one barrier per NU units).
-template <class V, int NQ, int NU, int KIND>
-__device__ __forceinline__ void ortho_rows(const EvArgs<V> &a, V *out, int i0, int nq, int jj, bool minor, int rp,
-                                           uint32_t du, uint32_t nu, bool back,
-                                           const typename RealLin<V>::RCoef *coef, const float *mcoef, V *xch,
-                                           RealAcc<V> *acc, RealAcc<V> &nrm, DotAcc<V> &gacc)
-{
-    constexpr uint32_t FOLD = 8;   // rows between two foldings of the float-float compensations
-    constexpr bool LAST = KIND & ORTHO_LAST, FIRST = KIND & ORTHO_FIRST;
-    constexpr int NMAJ = NQ < 2 ? 1 : 2;   // (LAST) terms j - 1 and j
-    const uint32_t D = a.b.D, col = threadIdx.x & 63;
-    const int pad = NQ - nq;
-    const V *Wg = a.W + (ptrdiff_t)(i0 - pad) * (ptrdiff_t)a.ldW;   // (slot 0 is not read where pad is 1)
-    coef += i0;
-    mcoef += i0;
-    uint32_t it = 0;
-    for (uint32_t u0 = blockIdx.x * (du / gridDim.x) + rp; u0 < nu; u0 += NU * du) {
-        uint32_t r[NU];
-        V x[NU][NQ], uu[NU];
-#pragma unroll
-        for (int n = 0; n < NU; ++n) {
-            const uint32_t u = u0 + n * du;
-            r[n] = u < nu ? (back ? nu - 1 - u : u) * 64 + col : D;
-            const bool in = r[n] < D;
-            uu[n] = VT<V>::zero();
-            if (LAST) uu[n] = ldg_if(in, a.U + r[n]);
-            x[n][0] = ldg_if(in && pad == 0, Wg + r[n]);
-#pragma unroll
-            for (int q = 1; q < NQ; ++q) x[n][q] = ldg_if(in, Wg + (size_t)q * a.ldW + r[n]);
-        }
-        // this group's share of w = u - sum c_i W_i; terms at rounding level in FP32
-        RealLin<V> l[NU];
-        float2 f[NU];
-#pragma unroll
-        for (int n = 0; n < NU; ++n) {
-            l[n] = RealLin<V>(uu[n]);
-            f[n] = make_float2(0.f, 0.f);
-        }
-        if (MinorSum<V>::use && minor) {
-            if constexpr (MinorSum<V>::use) {
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const int i = q == 0 ? 0 : q - pad;   // (an empty slot's x is zero)
-#pragma unroll
-                    for (int n = 0; n < NU; ++n) {
-                        if (LAST && q >= NQ - NMAJ) l[n].fms(coef[i], x[n][q]);
-                        else f[n] = __ffma2_rn(make_float2(mcoef[i], mcoef[i]), MinorSum<V>::lead(x[n][q]), f[n]);
-                    }
-                }
-#pragma unroll
-                for (int n = 0; n < NU; ++n)
-                    if (LAST) MinorSum<V>::add(l[n], f[n]);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q)
-#pragma unroll
-                for (int n = 0; n < NU; ++n) l[n].fms(coef[q == 0 ? 0 : q - pad], x[n][q]);
-        }
-        if (KIND != ORTHO_ONLY) {
-            // publish this share, meet, take the team's other one: w = LAST's + FIRST's
-            V *buf = xch + ((size_t)(it & 1) * (ORTHO_NTHR<V> / 64) + 2 * rp) * 64 * ORTHO_XU + col;
-#pragma unroll
-            for (int n = 0; n < NU; ++n) {
-                if (LAST) buf[64 * n] = l[n].out();
-                else if (MinorSum<V>::use && minor) *(float2 *)(buf + 64 * (ORTHO_XU + n)) = f[n];
-                else buf[64 * (ORTHO_XU + n)] = l[n].out();
-            }
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + rp) : "memory");
-#pragma unroll
-            for (int n = 0; n < NU; ++n) {
-                if (!LAST) l[n] = RealLin<V>(buf[64 * n]);
-                if (MinorSum<V>::use && minor) {
-                    if constexpr (MinorSum<V>::use)
-                        MinorSum<V>::add(l[n], LAST ? *(const float2 *)(buf + 64 * (ORTHO_XU + n)) : f[n]);
-                } else {
-                    l[n].add(buf[64 * (ORTHO_XU + n)]);
-                }
-            }
-        }
-#pragma unroll
-        for (int n = 0; n < NU; ++n) {
-            if (NU > 1 && KIND == ORTHO_ONLY && u0 + n * du >= nu) break;
-            const V w = l[n].out();
-            const typename RealAcc<V>::Pre p = RealAcc<V>::pre(w);
-            if (FIRST) nrm.add(w, p);
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) acc[q].add(x[n][q], p);
-            if (FIRST && r[n] < D) {
-                out[r[n]] = w;
-                if (a.G) gacc.add(ldg(a.G + r[n]), w);
-            }
-        }
-        it += 1;
-        if (it % (FOLD / NU) == 0) {
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) acc[q].renorm();
-            nrm.renorm();
-            gacc.renorm();
-        }
-    }
-}
-
 // Pass B and pass A's dots in one read of the Krylov vectors: w = u - sum_i c_i W_i, written as W_{j+1},
 // ||w||^2 and the dots Re <W_i, w>, i <= j.  Every vector is orthogonalised against all the earlier ones,
 // with coefficients c_i = Re <v_i, u>, u = (H - s) v_j, that need no pass of their own: H is symmetric, so
@@ -467,7 +349,8 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     V *out = a.W + (size_t)(jj + 1) * a.ldW;
     const int pad = ortho_pad(nq);
 #define KRY_ORTHO(NQ, NU, KIND) \
-    ortho_rows<V, NQ, NU, KIND>(a, out, i0, nq, jj, minor, rp, du, nu, jj & 1, coef, mcoef, xch, acc, nrm, gacc)
+    ortho_rows<V, NQ, NU, KIND, 64, NGRP, 1>(a.W, a.ldW, a.U, a.G, out, a.b.D, 64u, tid & 63, i0, nq, minor, rp, \
+                                       blockIdx.x * nrp + rp, du, nu, jj & 1, coef, mcoef, 1, xch, acc, nrm, gacc)
 #define KRY_ORTHO_N(NQ, NU) \
     case NQ: KRY_ORTHO(NQ, NU, ORTHO_ONLY); break;
 #define KRY_ORTHO_3(NQ, NU)                                       \

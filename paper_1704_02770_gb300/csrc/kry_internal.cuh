@@ -153,6 +153,8 @@ struct KryCtlB {
     int r0k[KBMAX];         // basis index of each realisation's initial state (hd.r0 >= 0)
     double pint[KBMAX];     // int_0^t_now P_k(t') dt' (temporal autocorrelation)
     double shift[KBMAX];    // s_k of the Lanczos operator H_k - s_k I
+    double c2[KBMAX];       // one-read form: ||c||^2 of the update's coefficients
+    int minor[KBMAX];       // and whether all but the last two are at rounding level (MinorSum)
 };
 
 template <class V>
@@ -168,6 +170,10 @@ struct EvArgsB {
     int K, Kp;       // realisations; Kp = K rounded up to a power of two >= 32
     int rl_smem;
     int kch;         // H.v in chunks of kch realisations (8 or 16; 0 = all K at once)
+    int one_read;    // update and dots in one pass over the Krylov vectors (k_ortho_b)
+    // one-read form, per realisation: C[k][i][i'] the coefficient of v_i in the update that made v_{i'+1},
+    // d[k][i] = Re <v_i, v_j> of the last vector
+    float *C, *d;
 };
 
 struct ExpArgsB {
@@ -185,8 +191,12 @@ struct ExpArgsB {
 // pass A of the batched path: part 0 = the H.v and the dots, 1 = the H.v only, 2 = the dots only
 template <class V> int launch_passA_b(const EvArgsB<V> &a, int jj, int grid, cudaStream_t s, int part = 0);
 template <class V> int launch_lincomb_b(const EvArgsB<V> &a, int mode, int jj, int grid, cudaStream_t s);
+// (C, d: of the one-read form, modes 6 and 7)
 int launch_reduce_b(KryCtlB *ctl, const double2 *part, int grid, int K, int Kp, int mode, int jj,
-                    int general, double es_bytes_per_vec, cudaStream_t s);
+                    int general, cudaStream_t s, float *C = nullptr, float *d = nullptr);
+// one-read form: alpha_j's partial sums (returns the CTAs, or minus a status) and the update with its dots
+template <class V> int launch_alpha_b(const EvArgsB<V> &a, int jj, cudaStream_t s);
+template <class V> int launch_ortho_b(const EvArgsB<V> &a, int jj, int grid, cudaStream_t s);
 template <class V> int batched_grid(const DevBasis &b, int Kp, int rl_smem, int *gridB);
 int launch_apply_b(const DevBasis &b, const DevHam &h, int c64, int K, const void *x, void *y,
                    int rl_smem, cudaStream_t s);

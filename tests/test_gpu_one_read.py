@@ -143,3 +143,60 @@ def test_profile_and_shapes(kry):
         P, _ = H.return_probability(s, [2.0], m=m)
         assert np.max(np.abs(P - P0)) <= 1e-12
 
+
+# 32,768 elements and more: groups of 64 threads with one to many states (K = 10, 16, 31, 64), of 128 (33,
+# 100, 128), units that do not divide the elements, a thread per element in the H.v up to K = 16
+@pytest.mark.parametrize("K", [10, 16, 17, 31, 33, 64, 100, 128])
+@pytest.mark.parametrize("form", ["c128", "c128e", "c64"])
+def test_batched_against_single_realisations(kry, K, form):
+    L, N = 14, 7
+    h = np.array([workloads.quasiperiodic_field(L, 1.3, p) for p in workloads.phases(9, K)])
+    B = kry.Basis(L, N)
+    H = kry.Hamiltonian(B, 1.0, 0.8, h)
+    states = workloads.random_basis_states(L, N, 5, K)
+    times, tol = [0.4, 1.5, 4.0], 1e-7 if form == "c64" else 1e-10
+    # (the common step is the smallest of the realisations', so the errors differ within the budgets)
+    bar = 2e-6 if form == "c64" else 1e-11
+    P, C, st = H.return_probability_states(states, times, m=30, tol=tol, dtype=form, autocorrelation=True)
+    P18, _ = H.return_probability_states(states, times, m=18, tol=tol, dtype=form)
+    assert np.max(np.abs(P18 - P)) <= 10 * bar
+    H.orth_check(True)
+    P2, st2 = H.return_probability_states(states, times, m=30, tol=tol, dtype=form)
+    H.orth_check(False)
+    assert st["n_second_pass"] == 0 and np.max(np.abs(P2 - P)) <= bar
+    assert 0.0 < st2["max_orth_loss"] <= (2e-6 if form == "c64" else 2e-12)
+    for k in (0, K // 2, K - 1):
+        Hk = kry.Hamiltonian(B, 1.0, 0.8, h[k])
+        Ck, Pk, _ = Hk.autocorrelation(states[k], times, m=30, tol=tol, dtype=form)
+        assert np.max(np.abs(P[:, k] - Pk)) <= bar and np.max(np.abs(C[:, k] - Ck)) <= bar
+
+
+@pytest.mark.parametrize("K", [12, 40])
+@pytest.mark.parametrize("form", ["c128", "c128e", "c64"])
+def test_batched_general_state_and_idle_realisations(kry, K, form):
+    """Dense initial states with psi_out, and realisations whose Krylov space ends at once beside others that
+    run on (their vectors stay zero)."""
+    L, N = 14, 7
+    h = np.array([workloads.quasiperiodic_field(L, 1.3, p) for p in workloads.phases(9, K)])
+    B = kry.Basis(L, N)
+    H = kry.Hamiltonian(B, 1.0, 0.8, h)
+    D = B.dim
+    rng = np.random.default_rng(2)
+    x = rng.normal(size=(D, K)) + 1j * rng.normal(size=(D, K))
+    x /= np.linalg.norm(x, axis=0)
+    dt = torch.complex64 if form == "c64" else torch.complex128
+    tol = 1e-6 if form == "c64" else 1e-10
+    xs = torch.from_numpy(x.reshape(-1)).cuda().to(dt)
+    out = torch.empty_like(xs)
+    P, _ = H.evolve(xs, [0.5, 1.0], tol=tol, psi_out=out, emulated=form == "c128e")
+    got = out.cpu().numpy().reshape(D, K)
+    for k in (0, K - 1):
+        Hk = kry.Hamiltonian(B, 1.0, 0.8, h[k])
+        o1 = torch.empty(D, dtype=dt, device="cuda")
+        P1, _ = Hk.evolve(xs.view(D, K)[:, k].contiguous(), [0.5, 1.0], tol=tol, psi_out=o1, emulated=form == "c128e")
+        assert np.linalg.norm(got[:, k] - o1.cpu().numpy()) <= (1e-5 if form == "c64" else tol)
+        assert np.max(np.abs(P[:, k] - P1)) <= (1e-5 if form == "c64" else tol)
+    # the ferromagnetic state of N = L is an eigenstate; in this sector a state of one domain with J = 0
+    H0 = kry.Hamiltonian(B, 0.0, 1.0, h)
+    P0, st0 = H0.return_probability((1 << N) - 1, [1.0, 5.0], tol=1e-6, dtype=form)
+    assert np.max(np.abs(P0 - 1.0)) <= 1e-6 and st0["n_breakdowns"] >= K

@@ -259,7 +259,7 @@ int capture_step(kry_ham_s *H, const EvArgs<V> &a, const ExpArgs &ea, int m, int
         va.ldOut = opt->ldOut;
         va.ctl = a.ctl;
         va.D = a.b.D;
-        rc = launch_vecout<V>(va, gridB, cs);
+        rc = launch_vecout<V>(va, cs);
     }
     }   // (the vector outputs of the adjoint are complex128 or complex64 only)
     mark();

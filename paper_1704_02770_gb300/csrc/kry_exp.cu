@@ -488,7 +488,15 @@ __global__ void __launch_bounds__(32 * EXPW) k_smallexp(ExpArgs ea)
             __syncthreads();
             for (int o = ob + warp; o < min(next, ob + 32); o += EXPW) {
                 if (lane >= me) continue;
-                const double2 s = jacobi_anger_sum(sm.jb + (o - ob) * (KMAX + 2), sm.tch + lane, 32, K);
+                // sum_k w_k J_k T_kj, the degrees by k mod 4 (phases 1, -i, -1, i): one multiply-add each
+                const double *J = sm.jb + (o - ob) * (KMAX + 2);
+                double part[4] = {0.0, 0.0, 0.0, 0.0};
+                for (int k0 = 0; k0 <= K; k0 += 4) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (k0 + q <= K) part[q] = fma(J[k0 + q], sm.tch[(k0 + q) * 32 + lane], part[q]);
+                }
+                const double2 s = make_double2(2.0 * (part[0] - part[2]) - J[0] * sm.tch[lane], 2.0 * (part[3] - part[1]));
                 double sn, cs;
                 sincos(fmax(ea.times[o] - t_now, 0.0) * c, &sn, &cs);
                 const double2 y = cmul(make_double2(cs, -sn), s);

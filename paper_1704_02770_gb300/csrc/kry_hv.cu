@@ -629,32 +629,51 @@ __global__ void k_set_basis_state_ff(ffc *W0, uint32_t r0) { W0[r0] = ffc{1.f, 0
 
 // ---------------------------------------------------------------- dense vector output
 
+constexpr int VECOUT_NTHR = 128;
+
 // psi(t_o) = sum_j Yout[o][j] W_j for every output time o inside the current step (the
 // small exponential fills Yout and [out_begin, out_end)); runs before the combine
-// overwrites W_0.
+// overwrites W_0.  Bound by the multiply-adds (FP64: 4 per element, vector and output): eight outputs
+// share a vector's load (one output at a time re-read all vectors, 819 us for 20 outputs at L = 18).
 template <class V>
-__global__ void __launch_bounds__(NTHR) k_vecout(VecOutArgs<V> a)
+__global__ void __launch_bounds__(VECOUT_NTHR) k_vecout(VecOutArgs<V> a)
 {
     pdl_begin();
     KryCtl *ctl = a.ctl;
     if (ctl->done) return;
     const int ob = ctl->out_begin, oe = ctl->out_end, me = ctl->m_eff;
     if (ob >= oe) return;
-    __shared__ V cf[MMAX];
-    for (int o = ob; o < oe; ++o) {
+    constexpr int NO = 8;
+    __shared__ V cf[MMAX][NO];
+    for (int o0 = ob; o0 < oe; o0 += NO) {
+        const int no = min(NO, oe - o0);
         __syncthreads();
-        if (threadIdx.x < me) cf[threadIdx.x] = VT<V>::from(a.Yout[(size_t)o * MMAX + threadIdx.x]);
+        for (int e = threadIdx.x; e < me * NO; e += VECOUT_NTHR) {
+            const int j = e / NO, q = e % NO;
+            cf[j][q] = q < no ? VT<V>::from(a.Yout[(size_t)(o0 + q) * MMAX + j]) : VT<V>::zero();
+        }
         __syncthreads();
-        V *out = a.out + (size_t)o * a.ldOut;
-        for (size_t r = (size_t)blockIdx.x * NTHR + threadIdx.x; r < a.D; r += (size_t)gridDim.x * NTHR) {
-            V w = VT<V>::zero();
+        for (size_t r = (size_t)blockIdx.x * VECOUT_NTHR + threadIdx.x; r < a.D; r += (size_t)gridDim.x * VECOUT_NTHR) {
+            V w[NO];
+#pragma unroll
+            for (int q = 0; q < NO; ++q) w[q] = VT<V>::zero();
+            V next = a.W[r];
+#pragma unroll 2
             for (int j = 0; j < me; ++j) {
-                const V v = a.W[(size_t)j * a.ldW + r];
-                const V c = cf[j];
-                w.x += c.x * v.x - c.y * v.y;
-                w.y += c.x * v.y + c.y * v.x;
+                const V v = next;
+                if (j + 1 < me) next = a.W[(size_t)(j + 1) * a.ldW + r];
+#pragma unroll
+                for (int q = 0; q < NO; ++q) {
+                    if (q < 4 || no > 4) {   // (a full or a half block: a predicated-off FP64 multiply-add costs as much)
+                        const V c = cf[j][q];
+                        w[q].x = fma(c.x, v.x, fma(-c.y, v.y, w[q].x));
+                        w[q].y = fma(c.x, v.y, fma(c.y, v.x, w[q].y));
+                    }
+                }
             }
-            out[r] = w;
+#pragma unroll
+            for (int q = 0; q < NO; ++q)
+                if (q < no) a.out[(size_t)(o0 + q) * a.ldOut + r] = w[q];
         }
     }
 }
@@ -920,9 +939,10 @@ int launch_ffc_to_c128(const void *src, void *dst, size_t n, cudaStream_t s)
 }
 
 template <class V>
-int launch_vecout(const VecOutArgs<V> &a, int grid, cudaStream_t s)
+int launch_vecout(const VecOutArgs<V> &a, cudaStream_t s)
 {
-    KRY_CU(launch_pdl(k_vecout<V>, grid, NTHR, 0, s, a));
+    const int g = (int)std::max<uint32_t>(1u, std::min<uint32_t>((a.D + VECOUT_NTHR - 1) / VECOUT_NTHR, (uint32_t)sm_count() * 4u));
+    KRY_CU(launch_pdl(k_vecout<V>, g, VECOUT_NTHR, 0, s, a));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }
@@ -946,8 +966,8 @@ int launch_grad_acc(const DevBasis &b, const DevHam &h, double J, const double2 
     return KRY_OK;
 }
 
-template int launch_vecout<double2>(const VecOutArgs<double2> &, int, cudaStream_t);
-template int launch_vecout<float2>(const VecOutArgs<float2> &, int, cudaStream_t);
+template int launch_vecout<double2>(const VecOutArgs<double2> &, cudaStream_t);
+template int launch_vecout<float2>(const VecOutArgs<float2> &, cudaStream_t);
 template int launch_ckpt<double2>(const double2 *, double2 *, size_t, KryCtl *, uint32_t, int, cudaStream_t);
 template int launch_ckpt<float2>(const float2 *, float2 *, size_t, KryCtl *, uint32_t, int, cudaStream_t);
 template <class V>

@@ -250,7 +250,7 @@ struct VecOutArgs {
     KryCtl *ctl;
     uint32_t D;
 };
-template <class V> int launch_vecout(const VecOutArgs<V> &a, int grid, cudaStream_t s);
+template <class V> int launch_vecout(const VecOutArgs<V> &a, cudaStream_t s);
 template <class V> int launch_ckpt(const V *W0, V *ckpt, size_t ldC, KryCtl *ctl, uint32_t D, int grid,
                                    cudaStream_t s);
 // Gradient integrand: acc[i] += sum_q w_q sum_r conj(lam_{nq-1-q}[r]) psi_q[r] dH_i[r] over the L

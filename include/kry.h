@@ -235,9 +235,9 @@ int kry_profile_read(kry_ham H, double *ms, double *bytes, int64_t *launches);
  * dtype, five ints:
  *   shape[0] CTAs of the streaming kernels: 0 = the occupancy rule (whole SMs times the
  *            resident CTAs of each kernel), else that many CTAs;
- *   shape[1] form of the H.v, two bits: the loads of eight hops issued together (16-byte
- *            elements: of two) instead of four, bit 0 inside the lower bits, bit 1 inside the
- *            upper bits;
+ *   shape[1] form of the H.v, two bits: the loads of eight hops issued together instead of
+ *            four (complex128: four instead of two, float-float: two instead of four), bit 0
+ *            inside the lower bits, bit 1 inside the upper bits;
  *   shape[2] dots of pass A: 0 = two or four units of rows loaded at a time where a thread has
  *            few vectors, 1 = always one;
  *   shape[3] rows per thread of the update pass: 1, 2 or 4;

@@ -1052,6 +1052,7 @@ struct HvWarp {   // shared memory of a warp
     int steps[HV_NH][24];   // per block: block-start steps of its antiparallel upper bonds (at most 15), packed
     uint32_t hi[HV_NH], base[HV_NH], cross[HV_NH], ring[HV_NH];
     int n[HV_NH];
+    uint16_t lower[16][32];   // per lane: ranks of its lower part's hops, packed (complex128 with ALPHA)
 };
 
 // With ALPHA *al also sums Re <x, y> over the rows.
@@ -1095,13 +1096,24 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
         const R eh = VT<V>::ehlo(hm, pos);
         const uint32_t anti = valid ? (lo ^ (lo >> 1)) & ((1u << nlb) - 1u) : 0u;
         const uint32_t lomask = (1u << Llo) - 1u;
-        uint32_t t[16];   // ranks of the lower part's hops (any pattern has one)
+        // Ranks of the lower part's hops (any pattern has one), in registers; for complex128 with ALPHA packed
+        // per lane in shared memory: the rows' loops then run to the longest list of the warp (about nine hops
+        // at L = 24) instead of over all Llo - 1 bonds, and its sum costs 40 instructions a term (189 -> 163
+        // us).  The other types lose what it takes to pack (L = 26 c64 138 -> 153 us).
+        constexpr bool PACK = ALPHA && std::is_same<V, double2>::value;
+        uint32_t t[16];
+        const int cnt = __popc(anti), most = PACK ? __reduce_max_sync(0xffffffffu, cnt) : nlb;
 #pragma unroll
         for (int p0 = 0; p0 < 16; p0 += 4) {
             if (p0 < nlb) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) t[p0 + u] = __ldg(b.ranklo + ((lo ^ (3u << (p0 + u))) & lomask));
             }
+        }
+        if (PACK) {
+#pragma unroll
+            for (int p = 0; p < 16; ++p)
+                if ((anti >> p) & 1u) w.lower[__popc(anti & ((1u << p) - 1u))][lane] = (uint16_t)t[p];
         }
         const uint32_t tc = __ldg(b.ranklo + (lo ^ (1u << nlb))), tr = __ldg(b.ranklo + (lo ^ 1u));
         __syncwarp();
@@ -1115,13 +1127,23 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
             const V x0 = ldg_if(valid, xr);
             auto neighbours = [&](auto &acc) {
                 const V vc = ldg_if(pc, x + w.cross[h] + tc), vr = ldg_if(pr, x + w.ring[h] + tr);
-#pragma unroll
-                for (int p0 = 0; p0 < 16; p0 += RND) {
-                    if (p0 < nlb) {
+                if (PACK) {
+#pragma unroll 1
+                    for (int k0 = 0; k0 < most; k0 += RND) {   // (entries past a lane's own are not used)
                         V v[RND];
 #pragma unroll
-                        for (int u = 0; u < RND; ++u) v[u] = ldg_if(anti & (1u << (p0 + u)), xb + t[p0 + u]);
+                        for (int u = 0; u < RND; ++u) v[u] = ldg_if(k0 + u < cnt, xb + w.lower[(k0 + u) & 15][lane]);
                         hv_add_n<RND>(acc, v);
+                    }
+                } else {
+#pragma unroll
+                    for (int p0 = 0; p0 < 16; p0 += RND) {
+                        if (p0 < nlb) {
+                            V v[RND];
+#pragma unroll
+                            for (int u = 0; u < RND; ++u) v[u] = ldg_if(anti & (1u << (p0 + u)), xb + t[p0 + u]);
+                            hv_add_n<RND>(acc, v);
+                        }
                     }
                 }
                 hv_add(acc, vc);

@@ -20,7 +20,8 @@ namespace kry {
 constexpr int DOTS_NTHR = 512;   // threads of a CTA of the dots
 // Loads of hops issued together in the forms of the H.v: inside the lower bits (bit 0 of the form) and
 // inside the upper bits (bit 1); eight of 16 bytes would spill
-template <class V, int BIT> constexpr int HV_RND = BIT == 0 ? 4 : sizeof(V) == 8 ? 8 : 2;
+template <class V, int BIT> constexpr int HV_RND =
+    sizeof(V) == 8 ? (BIT == 0 ? 4 : 8) : (BIT == 0) == std::is_same<V, double2>::value ? 2 : 4;
 
 // ---------------------------------------------------------------- y = H x
 

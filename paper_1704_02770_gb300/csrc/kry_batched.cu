@@ -7,11 +7,13 @@
 //
 //   k_apply_b      y = H x for all K (warp per state, lanes over k)
 //   k_hv_b         u = H v_j for all K (pass A, part 1)
-//   k_dots_b       all dots <v_i, u> and ||u||^2 per realisation (pass A, part 2)
-//   k_lincomb_b    update / correction / combine / load with per-realisation coefficients,
-//                  and the dots of the new vector with the earlier ones (pass C1)
-//   k_reduce_b     per-realisation sum of the per-CTA partials (CTA order, deterministic)
-//                  and the scalar epilogue of each pass
+//   k_alpha_b      alpha_j per realisation (one-read form, from 32,768 elements on)
+//   k_ortho_b      update and the dots of the new vector in one read (one-read form)
+//   k_dots_b       all dots <v_i, u> and ||u||^2 per realisation (two-pass form: pass A, part 2)
+//   k_lincomb_b    update (two-pass form) / correction / combine / load with per-realisation
+//                  coefficients, and the dots of the new vector with the earlier ones (pass C1)
+//   k_reduce_b     per-realisation sum of the per-CTA partials (deterministic) and the
+//                  scalar epilogue of each pass
 #include <cuda_runtime.h>
 
 #include <algorithm>

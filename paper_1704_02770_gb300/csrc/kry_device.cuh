@@ -286,7 +286,7 @@ __device__ __forceinline__ void pdl_begin()
 // product is split exactly (p = a*b rounded, e = fma(a, b, -p)) and summed with Knuth's
 // TwoSum into a float pair (s, c): the rounding errors of s are kept exactly, and c gathers
 // them in plain float.  c is folded back into s (renorm, a TwoSum) after every few terms --
-// the callers do it once per tile -- so that its own rounding stays at 2^-48 of |s|: left to
+// the callers do it every few rows -- so that its own rounding stays at 2^-48 of |s|: left to
 // grow over the N terms of a thread, c's rounding errors add up to about N 2^-48 of the sum
 // (5e-11 relative at N = 16K, the rows per thread of an L = 30 sector).
 
@@ -1033,7 +1033,8 @@ __device__ __forceinline__ void stage_tables(const DevBasis &b, uint32_t *koff_s
 // lane) of NH such blocks.  What depends on lo alone -- the ranks of its hops, rl[lo ^ (3 << p)] --
 // is found once per item and serves NH rows; what depends on hi alone -- the block starts of its hops
 // -- is found once per item by one lane per (block, bond) and shared.  A row then costs about four
-// instructions a hop (a predicated load at block start + rank, and the add) and no unranking.
+// instructions a hop (a predicated load at block start + rank, and the add) and no unranking (L = 24
+// c64: 40 us, L = 26 138).
 // A per-row form (unrank, then a loop over the row's hops) took 404 instructions per row at L = 24
 // and 533 at L = 28, was bound by their issue (59% active) and took 51 us (L = 24 c64).
 // The terms of a row are added in bond order, the ring bond last.

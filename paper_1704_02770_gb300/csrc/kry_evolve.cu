@@ -3,8 +3,11 @@
 // kry_apply / kry_evolve / kry_return_probability.
 //
 // One Krylov step, captured once per (precision, m) and replayed:
-//   for j = 0..m-1:  pass A (u = H v_j, then the dots <v_i, u>)  ->  pass B (update)
-//                    ->  pass C (second Gram-Schmidt pass, runs only when flagged)
+//   for j = 0..m-1:  one-read form: H.v with alpha_j  ->  update and dots of w in one pass
+//                    ->  pass C2 (subtracts the dots, only when flagged)
+//                    two-pass form (below 65,536 states): pass A (u = H v_j, then the dots
+//                    <v_i, u>)  ->  pass B (update)  ->  pass C (second Gram-Schmidt pass,
+//                    only when flagged)
 //   small exponential + step control + dense output of P  ->  combine psi = beta V y.
 // Device flags end the Lanczos loop early on an invariant subspace and turn every kernel
 // into a no-op once the last output time is reached; the host only polls that flag.

@@ -1,13 +1,16 @@
 // Vector kernels of the Krylov step (Sec. 2, "Krylov subspace methods"):
 //   k_apply     y = H x (matrix-free, Eq. 1)
-//   k_hv        u = sigma_j H v_j with alpha_j = <v_j, u> and ||u||^2 (pass A, part 1)
-//   k_dots      <v_i, y> for the Krylov vectors, a tall-skinny GEMV with plain loads
-//               (pass A part 2 with y = u; pass C1 with y = w)
-//   k_lincomb   w = src - sum_i c_i W_i (MODE 0: Lanczos update, pass B; 1: the second
-//               Gram-Schmidt subtraction, pass C2; 2: combine psi = beta V y; 3: load the
+//   k_hv        u = sigma_j H v_j (pass A, part 1); in the one-read form also alpha_j = Re <v_j, u>
+//   k_dots      Re <v_i, y> for the Krylov vectors, a tall-skinny GEMV with plain loads (two-pass
+//               form: pass A part 2 with y = u, alpha_j and ||u||^2 included; pass C1 with y = w)
+//   k_ortho     the one-read form: the update w, written as W_{j+1}, ||w||^2 and the dots of w with
+//               every Krylov vector, which give the next update's coefficients
+//   k_lincomb   w = src - sum_i c_i W_i (MODE 0: Lanczos update, pass B of the two-pass form; 1: the
+//               second Gram-Schmidt subtraction, pass C2; 2: combine psi = beta V y; 3: load the
 //               initial vector)
-// Every reduction ends in the last CTA to finish (ticket counter), which sums the
-// per-CTA partials in CTA order: results are bitwise reproducible for a fixed grid.
+//   k_vecout    psi at output times inside the step (adjoint)
+// Every reduction ends in the last CTA to finish (ticket counter), which sums the per-CTA
+// partials as integers of one exponent: results are bitwise reproducible for a fixed grid.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -89,11 +92,12 @@ __device__ __forceinline__ void cta_sum_into(const Acc &acc, double2 *red, int s
 
 // ---------------------------------------------------------------- pass A
 
-// u = sigma_j H W_j, written to U (pass A, part 1): the gathers of hv_items at full occupancy and
-// nothing else.  alpha_j, ||u||^2 and the dots with the earlier vectors are taken by the streaming
-// pass that follows (k_dots, mode 0).  FORM 0 issues the loads of four hops together, FORM 1 of
-// eight (16-byte elements: of two); both give the same bits, the launch shape picks the faster (kry_autotune).
-// ALPHA (the one-read form, k_ortho): the pass also takes alpha_j and sets up the update's coefficients.
+// u = sigma_j H W_j, written to U (pass A, part 1): the gathers of hv_items at full occupancy.  Without
+// ALPHA (two-pass form) nothing else: alpha_j, ||u||^2 and the dots with the earlier vectors are taken
+// by the streaming pass that follows (k_dots, mode 0).  With ALPHA (one-read form, k_ortho) the pass
+// also takes alpha_j and sets up the update's coefficients (L = 24 c64: 40 us without, 50 with).
+// FORM: how many loads are issued together inside the lower and the upper bits (HV_RND); every form
+// gives the same bits, the launch shape picks the fastest (kry_autotune).
 template <class V, int FORM, bool ALPHA>
 __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V> a, HvPlan pl, int jj)
 {

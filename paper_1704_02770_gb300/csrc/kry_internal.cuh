@@ -372,8 +372,8 @@ struct kry_ham_s {
 };
 
 // Launch shape of a new Hamiltonian: the occupancy-rule grid, two update
-// rows per thread, all realisations at once, and the H.v with four loads at a time -- from lower
-// parts of 14 bits on (L >= 28) eight (complex64; two of 16 bytes).
+// rows per thread, all realisations at once, and the H.v with four loads at a time (complex128 two) -- from lower
+// parts of 14 bits on (L >= 28) the other form (complex64 eight, float-float two, complex128 four).
 inline void default_shape(kry_ham_s *H, int Llo)
 {
     const int v[5] = {0, Llo >= 14 ? 3 : 0, 0, 2, 0};

@@ -29,7 +29,9 @@ METRIC = "Krylov H.v state-updates/s (+ % HBM roofline), FP64 vs FP32/batched at
 WORKLOAD = "L24_mixed"
 HBM_PEAK_FALLBACK = 6800.0
 # profiled kernel kinds: pass A's H.v (k_hv) and dots (k_dots<.,0>), pass B's update
-# (k_lincomb<.,0>), pass C (the second Gram-Schmidt pass), the small exponential, the combine
+# (k_lincomb<.,0>), pass C (the second Gram-Schmidt pass), the small exponential, the combine.
+# In the one-read form (sectors of 65,536 states and more, ensembles of 32,768 elements and more) the
+# dots are taken by the update's kernel (k_ortho, k_ortho_b) and their kind stays empty.
 KIND_NAMES = ("hv", "dots", "update", "passC", "smallexp", "combine")
 KERNEL_OF = {"hv": "k_hv", "dots": "k_dots<.,0>", "update": "k_lincomb<.,0>",
              "passC": "k_dots<.,1> + k_lincomb<.,1>", "smallexp": "k_smallexp", "combine": "k_lincomb<.,2>"}
@@ -216,6 +218,22 @@ def fp64_pipe_ops(kind, D, m, krylov_steps, L, N, pbc):
     return per * D * krylov_steps
 
 
+def fp64_one_read(kind, D, m, krylov_steps):
+    """(flops, FP64 pipe instructions) of all launches of `kind` in the one-read form.  Per element at index
+    j: k_ortho two multiply-adds for each of the j + 1 real dots, two for each of the last two terms of the
+    update (the others are at rounding level and summed in FP32) and two for ||w||^2; the H.v, whose
+    neighbours are summed on integers, two for alpha_j and eleven instructions (16 flops) for the diagonal
+    term, the scales and the conversion of the sum."""
+    if kind == "hv":
+        fl, ops = m * 20.0, m * 13.0
+    elif kind == "update":
+        ops = sum(2.0 * (j + 1) + 2.0 * min(2, j + 1) + 2.0 for j in range(m))
+        fl = 2.0 * ops
+    else:
+        return 0.0, 0.0
+    return fl * D * krylov_steps, ops * D * krylov_steps
+
+
 MEASURED_FP64 = {}   # filled by run_ours from kry_measure_peaks on this GPU
 
 
@@ -229,6 +247,8 @@ def roofline(prof, form, D, c, L, N, clocks, traffic_key=None):
     peaks = measured_peaks()
     peak = peaks["hbm_gbs"] if peaks and "hbm_gbs" in peaks else HBM_PEAK_FALLBACK
     dom = max(("hv", "dots", "update"), key=lambda k: prof[k]["ms"])   # the dominant kernel
+    one_read = prof["dots"]["launches"] == 0
+    kernel = "k_ortho" if one_read and dom == "update" else KERNEL_OF[dom]
     per = {k: {"ms": round(prof[k]["ms"], 3),
                "GBps": (prof[k]["bytes"] / (prof[k]["ms"] * 1e6)) if prof[k]["ms"] else None,
                "launches": prof[k]["launches"]} for k in KIND_NAMES}
@@ -245,7 +265,8 @@ def roofline(prof, form, D, c, L, N, clocks, traffic_key=None):
         # recovered from the kernel's algorithmic bytes, PASSES[dom](j) vectors at index j
         per_step = sum(PASSES[dom](j) for j in range(c["m"])) * D * 16
         steps = prof[dom]["bytes"] / per_step
-        fl = fp64_flops(dom, D, c["m"], steps, L, N, c["pbc"])
+        fl, ops = (fp64_one_read(dom, D, c["m"], steps) if one_read else
+                   (fp64_flops(dom, D, c["m"], steps, L, N, c["pbc"]), fp64_pipe_ops(dom, D, c["m"], steps, L, N, c["pbc"])))
         mhz = clocks["sm_mhz"] or 2070.0
         if MEASURED_FP64.get("tflops"):
             fp64_peak = MEASURED_FP64["tflops"]
@@ -256,20 +277,19 @@ def roofline(prof, form, D, c, L, N, clocks, traffic_key=None):
             fp64_peak = 152 * 4 * mhz * 1e6 / 1e12
             src = "nominal: 152 SMs x 4 flop/clk x median SM clock (no measurement)"
         ach_fl = fl / (prof[dom]["ms"] * 1e-3) / 1e12
-        ops = fp64_pipe_ops(dom, D, c["m"], steps, L, N, c["pbc"])
         ach_ops = ops / (prof[dom]["ms"] * 1e-3) / 1e12
         ops_peak = fp64_peak / 2.0
         pipe = {"achieved": ach_ops, "peak": ops_peak, "unit": "T FP64 instr/s", "frac": ach_ops / ops_peak,
                 "peak_source": "the measured multiply-add rate, one instruction each",
-                "note": "adds occupy the pipe like multiply-adds; the H.v is add-heavy"}
-        return {"bound": "alu", "kernel": KERNEL_OF[dom], "kind": dom, "achieved": ach_fl, "peak": fp64_peak,
+                "note": "adds occupy the pipe like multiply-adds"}
+        return {"bound": "alu", "kernel": kernel, "kind": dom, "achieved": ach_fl, "peak": fp64_peak,
                 "unit": "TFLOP/s", "frac": ach_fl / fp64_peak,
                 "peak_source": src,
                 "traffic": tr, "algo_bytes_per_launch": prof[dom]["bytes"] / nl,
                 "fp64_pipe_view": pipe,
                 "hbm_view": hbm, "per_kind": per, "kernel_time_share": share,
                 "profiled_region_s": prof.get("_sec"), "timing": TIMING_NOTE}
-    return dict(bound="hbm", kernel=KERNEL_OF[dom], kind=dom, traffic=tr, algo_bytes_per_launch=prof[dom]["bytes"] / nl,
+    return dict(bound="hbm", kernel=kernel, kind=dom, traffic=tr, algo_bytes_per_launch=prof[dom]["bytes"] / nl,
                 per_kind=per, kernel_time_share=share, profiled_region_s=prof.get("_sec"),
                 timing=TIMING_NOTE, **hbm)
 
@@ -795,8 +815,8 @@ def run_reference(args):
 def run_ncu_case(args):
     """One Krylov step of the workload in the given precision, with no autotuning and no
     warm-up, so that a kernel's launch index is known: per Lanczos index j the launches
-    are k_hv, k_dots (pass A), k_lincomb (pass B), k_dots, k_lincomb (pass C, no-ops unless
-    flagged), then the small exponential and the combine.  c64b: the batched K = 64
+    are k_hv, k_ortho (update and dots), k_lincomb (pass C2, a no-op unless flagged), then the small
+    exponential and the combine.  c64b: the batched K = 64
     ensemble of L = 22 in complex64.  c64l: the L = 55, N = 5 ring (sorted-list basis)."""
     import numpy as np
     import torch

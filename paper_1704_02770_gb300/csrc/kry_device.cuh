@@ -190,50 +190,62 @@ template <int N, class S, class V> __device__ __forceinline__ void hv_add_n(S &a
 #pragma unroll
     for (int u = 0; u < N; ++u) hv_add(acc, v[u]);
 }
-// Neighbour sums of complex128 on 64-bit integers: the mantissas are aligned to the largest exponent
-// seen so far (the sums so far shifted along when it grows), with 5 bits of fraction below and room
-// for 32 terms above.  Each term loses less than 2^-57 of the largest, an FP64 sum 2^-53 of the running
-// one, and a term takes about 14 integer instructions per component where an FP64 add takes the pipe
-// for 77 issue cycles (L = 24: 213 us with FP64 adds, the kernel's bound).
-struct ISum2 {
-    long long re = 0, im = 0;
-    unsigned em = 0;
-    __device__ __forceinline__ static unsigned ex(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7ffu; }
+// Neighbour sums of complex128 on 64-bit integers, the real and the imaginary parts each on a scale of their
+// own (H is real, so neither part may cost the other accuracy): the mantissas of a part are aligned to its
+// largest exponent so far (the sum so far shifted along when it grows), with 5 bits of fraction below and room
+// for 32 terms above.  Each term loses less than 2^-56 of the largest of its part (the bits shifted out, and
+// one unit for a negative term), an FP64 sum 2^-53 of the running one; a single term is exact.  A term takes
+// about 16 integer instructions per part where an FP64 add takes the pipe for 77 issue cycles (L = 24: 213 us
+// with FP64 adds, the kernel's bound).
+struct ISum {
+    long long s = 0;
+    unsigned top = 0, low = 0;   // largest high word without its sign, and the low words' bits
+    __device__ __forceinline__ static unsigned mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+    // mantissa of x in units of 2^(em - 1080), em >= its exponent; x, or for a negative x its complement.  The
+    // shift is clamped to 64 by the instruction.  (A zero or subnormal x counts as 2^-1023 here: from em = 128 on
+    // that is shifted out, and below that value() and special() do not use the sum.)
     __device__ __forceinline__ static long long align(double x, unsigned em)
     {
-        const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), e = (hi >> 20) & 0x7ffu;
-        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 5;
-        const unsigned d = em - e;
-        const long long q = e == 0u || d > 63u ? 0ll : (long long)(m >> d);
-        return (int)hi < 0 ? -q : q;
+        const unsigned lo = (unsigned)__double2loint(x);
+        const unsigned h5 = (__funnelshift_l(lo, (unsigned)__double2hiint(x), 5) & 0x1ffffffu) | 0x2000000u;
+        unsigned long long q;
+        asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"((unsigned long long)h5 << 32 | (unsigned long long)(lo << 5)), "r"(em - (mag(x) >> 20)));
+        return (long long)q ^ (long long)(__double2hiint(x) >> 31);
     }
-    // exponents the scale cannot hold, infinities and NaN: the caller sums the row in FP64
-    __device__ __forceinline__ bool special() const { return em == 0x7ffu || (em != 0u && em < 128u); }
-    __device__ __forceinline__ double2 value() const
+    // a and, with PAIR, b
+    template <bool PAIR> __device__ __forceinline__ void add(double a, double b)
     {
-        if (em == 0u) return make_double2(0.0, 0.0);
-        const double f = __hiloint2double((int)(em - 1080u + 1023u) << 20, 0);   // 2^(em - 1075 - 5)
-        return make_double2((double)re * f, (double)im * f);
+        const unsigned t = max(top, PAIR ? max(mag(a), mag(b)) : mag(a)), em = t >> 20;
+        low |= PAIR ? (unsigned)__double2loint(a) | (unsigned)__double2loint(b) : (unsigned)__double2loint(a);
+        asm("shr.s64 %0, %0, %1;" : "+l"(s) : "r"(em - (top >> 20)));
+        top = t;
+        s += align(a, em);
+        if (PAIR) s += align(b, em);
     }
+    // infinities, NaN and exponents the scale cannot hold, down to subnormal values: the caller sums the row in
+    // FP64
+    __device__ __forceinline__ bool special() const
+    {
+        return top >= 0x7ff00000u || (top < (128u << 20) && (top | low) != 0u);
+    }
+    __device__ __forceinline__ double value() const
+    {
+        if (top == 0u) return 0.0;
+        return (double)s * __hiloint2double((int)((top >> 20) - 1080u + 1023u) << 20, 0);   // 2^(em - 1075 - 5)
+    }
+};
+struct ISum2 {
+    ISum re, im;
+    __device__ __forceinline__ bool special() const { return re.special() || im.special(); }
+    __device__ __forceinline__ double2 value() const { return make_double2(re.value(), im.value()); }
 };
 // (two terms at a time whatever N, so that the bits do not depend on how many are loaded together)
 template <int N> __device__ __forceinline__ void hv_add_n(ISum2 &acc, const double2 *v)
 {
 #pragma unroll
-    for (int u0 = 0; u0 < N; u0 += 2) {
-        constexpr int M = N < 2 ? 1 : 2;
-        unsigned em = acc.em;
-#pragma unroll
-        for (int u = u0; u < u0 + M; ++u) em = max(em, max(ISum2::ex(v[u].x), ISum2::ex(v[u].y)));
-        const unsigned d = min(em - acc.em, 63u);
-        acc.re >>= d;
-        acc.im >>= d;
-        acc.em = em;
-#pragma unroll
-        for (int u = u0; u < u0 + M; ++u) {
-            acc.re += ISum2::align(v[u].x, em);
-            acc.im += ISum2::align(v[u].y, em);
-        }
+    for (int u = 0; u < N; u += 2) {
+        acc.re.add<(N > 1)>(v[u].x, v[N > 1 ? u + 1 : u].x);
+        acc.im.add<(N > 1)>(v[u].y, v[N > 1 ? u + 1 : u].y);
     }
 }
 __device__ __forceinline__ void hv_add(ISum2 &acc, double2 v) { hv_add_n<1>(acc, &v); }
@@ -1182,7 +1194,7 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
             if constexpr (std::is_same<V, double2>::value) {   // on aligned integers, in FP64 where they cannot
                 ISum2 acc{};
                 neighbours(acc);
-                if (__any_sync(0xffffffffu, acc.special())) {
+                if (acc.special()) {   // (a row's own decision: its bits do not depend on the warp's other rows)
                     double2 a2 = VT<V>::zero();
                     neighbours(a2);
                     out = hv_finish(sigma * d, x0, sigma_halfJ, a2);

@@ -84,12 +84,20 @@ def test_apply_rejects_bad_arguments(kry):
     assert kry.load().kry_apply(H._h, 0, x.data_ptr(), x.data_ptr(), None) == kry.KRY_EINVAL
 
 
+def _largest(Hc, h, x):
+    """Per row, the scale of the rounding of H x for a real x: its largest hop term, and the terms that add up
+    to its diagonal (fields and bonds, which may cancel)."""
+    dmax = 0.5 * np.sum(np.abs(h)) + 0.25 * 0.6 * len(h)
+    return np.maximum(np.maximum.reduceat(np.abs(Hc.val) * np.abs(x[Hc.col]), Hc.rowptr[:-1]), dmax * np.abs(x))
+
+
 @pytest.mark.parametrize("L,N", [(2, 1), (3, 1), (5, 2), (8, 4), (9, 1), (9, 8), (11, 6), (13, 6), (16, 3), (17, 8)])
 @pytest.mark.parametrize("pbc", [True, False])
 def test_apply_edges_of_items(kry, L, N, pbc):
     """Items of 32 lower parts and up to eight upper parts: sectors whose groups are smaller than a warp,
     not a multiple of it, or leave an item's blocks unfilled, on open and closed chains.  The complex128
-    sum on aligned integers is at least as close as FP64 adds: 4 ulp of the largest term per row."""
+    sum on aligned integers is bounded as FP64 adds are, the real and the imaginary part each by its own
+    largest term."""
     h = workloads.quasiperiodic_field(L, 1.7, 0.9)
     Hc = ob.CSR(L, N, 1.0, 0.6, h, pbc)
     rng = np.random.default_rng(L * 31 + N)
@@ -99,11 +107,10 @@ def test_apply_edges_of_items(kry, L, N, pbc):
     H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.6, h, pbc=pbc)
     y = H.apply(torch.from_numpy(x).cuda()).cpu().numpy()
     yo = Hc.matvec(x)
-    # a row's rounding is relative to its largest hop term, and that of its diagonal to the terms that add
-    # up to it (fields and bonds, which may cancel), not to their sum
-    dmax = 0.5 * np.sum(np.abs(h)) + 0.25 * 0.6 * L
-    big = np.maximum(np.maximum.reduceat(np.abs(Hc.val) * np.abs(x[Hc.col]), Hc.rowptr[:-1]), dmax * np.abs(x))
-    assert np.all(np.abs(y - yo) <= (L + 4) * 2.0**-52 * big + 1e-300)
+    big = _largest(Hc, h, x.real), _largest(Hc, h, x.imag)
+    assert np.all(np.abs(y.real - yo.real) <= (L + 4) * 2.0**-52 * big[0] + 1e-300)
+    assert np.all(np.abs(y.imag - yo.imag) <= (L + 4) * 2.0**-52 * big[1] + 1e-300)
+    big = np.maximum(*big)
     y32 = H.apply(torch.from_numpy(x.astype(np.complex64)).cuda()).cpu().numpy()
     assert np.all(np.abs(y32 - yo) <= (L + 6) * 2.0**-22 * big + 1e-30)
 
@@ -124,3 +131,40 @@ def test_apply_special_values(kry, special):
         assert np.array_equal(np.isfinite(a), np.isfinite(b))
         ok = np.isfinite(b)
         assert np.allclose(a[ok], b[ok], rtol=1e-14, atol=0.0)
+
+
+@pytest.mark.parametrize("scale", [1e-4, 1e-8, 1e-12, 1e-20, 1e-120, 1e-290, 1e-318])
+@pytest.mark.parametrize("L,N", [(6, 3), (13, 6), (16, 8)])
+def test_apply_keeps_the_smaller_part(kry, L, N, scale):
+    """H is real: a real or imaginary part far below the other (a complex-step derivative, two real vectors in
+    one complex one), down to subnormal values, keeps its own accuracy.  (1e-290 and below: the spacing of the
+    subnormal numbers, 2^-1074 per term, is added to the bound.)"""
+    h = workloads.quasiperiodic_field(L, 1.7, 0.9)
+    Hc = ob.CSR(L, N, 1.0, 0.6, h, True)
+    rng = np.random.default_rng(L)
+    a, b = rng.normal(size=Hc.D), rng.normal(size=Hc.D) * scale
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.6, h)
+    for re, im in ((a, b), (b, a)):
+        y = H.apply(torch.from_numpy(re + 1j * im).cuda()).cpu().numpy()
+        for got, part in ((y.real, re), (y.imag, im)):
+            want = Hc.matvec(part.astype(np.complex128)).real
+            assert np.all(np.abs(got - want) <= (L + 4) * (2.0**-52 * _largest(Hc, h, part) + 2.0**-1074))
+
+
+@pytest.mark.parametrize("value", [float("inf"), 1e-300, 5e-324])
+def test_apply_rows_do_not_depend_on_others(kry, value):
+    """A value outside the integer sum's range changes the rows it is a neighbour of and no bit of the others."""
+    L, N = 13, 6
+    h = workloads.quasiperiodic_field(L, 1.7, 0.9)
+    Hc = ob.CSR(L, N, 1.0, 0.6, h, True)
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.6, h)
+    rng = np.random.default_rng(3)
+    x = rng.normal(size=Hc.D) + 1j * rng.normal(size=Hc.D)
+    y = H.apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    touched = np.zeros(Hc.D, bool)
+    for r in (5, 700, 1300):
+        x[r] = complex(value, -value)
+        touched |= np.logical_or.reduceat(Hc.col == r, Hc.rowptr[:-1])
+        touched[r] = True
+    y2 = H.apply(torch.from_numpy(x).cuda()).cpu().numpy()
+    assert touched.sum() < 60 and np.array_equal(y[~touched], y2[~touched])

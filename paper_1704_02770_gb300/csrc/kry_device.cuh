@@ -434,18 +434,20 @@ __device__ __forceinline__ double warp_sum(double v)
 // is no more than the roundings of an FP64 sum of as many, and the order does not matter.
 
 // Integer sum over the warp of CNT values per lane (CNT <= 8): every lane gets S and k with the total
-// = S 2^k.  False (uniform) when a value is infinite or NaN, or the largest below 2^-895; subnormal
-// values count as zero.
+// = S 2^k.  False (uniform) when a value is infinite or NaN, or the largest below 2^-895 and not zero
+// (beside larger ones, subnormal values count as zero).
 template <int CNT>
 __device__ __forceinline__ bool warp_isum(const double *v, long long &S, int &k)
 {
-    unsigned em = 0;
+    unsigned top = 0;   // largest high word without its sign, not zero for a value that is not
 #pragma unroll
-    for (int i = 0; i < CNT; ++i) em = max(em, ((unsigned)__double2hiint(v[i]) >> 20) & 0x7ffu);
-    em = __reduce_max_sync(0xffffffffu, em);
+    for (int i = 0; i < CNT; ++i)
+        top = max(top, ((unsigned)__double2hiint(v[i]) & 0x7fffffffu) | min((unsigned)__double2loint(v[i]), 1u));
+    top = __reduce_max_sync(0xffffffffu, top);
     S = 0;
     k = 0;
-    if (em == 0u) return true;
+    if (top == 0u) return true;
+    const unsigned em = top >> 20;
     if (em == 0x7ffu || em < 128u) return false;
     constexpr int SH = CNT == 1 ? 5 : 2;   // 53 bits + SH + log2(32 CNT) <= 63
     long long q = 0;

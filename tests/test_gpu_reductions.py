@@ -78,3 +78,23 @@ def test_non_finite_states_are_refused(kry, bad):
     x[7] = bad
     with pytest.raises(kry.KryError):
         H.evolve(x, [0.5], tol=1e-10)
+
+
+@pytest.mark.parametrize("L,N,K", [(11, 5, 1), (11, 5, 3), (20, 7, 1), (14, 7, 10)])
+def test_norms_whose_squares_are_subnormal(kry, L, N, K):
+    """A state of norm 1e-155 has a squared norm of 1e-310, summed from subnormal squares: it is not zero and the
+    evolution runs.  (Both forms of the pass, single and batched.)  The D squares are off by up to half the
+    spacing 5e-324 of the subnormal numbers each, so the squared norm by less than D 5e-324 / 1e-310, and psi
+    by that times the spectral half-width (below 20) and t."""
+    s = 1e-155
+    h = np.array([workloads.quasiperiodic_field(L, 1.2, p) for p in workloads.phases(4, K)])
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.8, h if K > 1 else h[0])
+    D = H.basis.dim
+    rng = np.random.default_rng(5)
+    x = rng.normal(size=(D, K)) + 1j * rng.normal(size=(D, K))
+    x = torch.from_numpy((x / np.linalg.norm(x, axis=0)).reshape(-1)).cuda()
+    out1, out = torch.empty_like(x), torch.empty_like(x)
+    H.evolve(x, [0.5], tol=1e-8, psi_out=out1)
+    H.evolve(x * s, [0.5], tol=1e-8 * s, psi_out=out)
+    err = torch.linalg.vector_norm((out / s - out1).view(D, K), dim=0).max().item()
+    assert err <= 1e-8 + 20.0 * 0.5 * D * 5e-324 / s**2

@@ -609,6 +609,11 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
     if (mode == 3 && !H.dots_any) return;   // pass C1 did not run
     __shared__ double2 fin[PSB];
     __shared__ float Cs[MMAX * MMAX], ds[MMAX + 1];
+    // one-read form: lane i's coefficient c_i, after pass C2 with its correction (1 / sigma_i is the norm that
+    // made v_i)
+    double ci = 0.0;
+    if (Cb && (mode == 7 || mode == 2) && tid <= jj)
+        ci = (ctl->coefA[tid][k] + (mode == 2 ? ctl->coefC[tid][k] : 0.0)) * (tid ? ctl->beta[tid - 1][k] : ctl->beta0[k]);
     const int nd = (mode == 0 || mode == 3 || mode == 7) ? jj + 1 : 0;
     const int ns = mode == 6 ? 0 : nd + (mode != 3 ? 1 : 0) + (general && mode != 0 && mode != 3 ? 1 : 0);
     if (mode == 6) {
@@ -674,7 +679,8 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
             float f = 0.f;
             for (int i = 0; i <= lane; ++i) f = fmaf(Cs[i * MMAX + lane], ds[i], f);
             const double b = ctl->beta[lane][k];
-            cc = lane == jj - 1 ? b + (double)f : (double)fmaf((float)b, ds[lane + 1], f);
+            const bool sub = lane == jj - 1;   // d_j = 1
+            cc = fma(b, (double)(sub ? f : f + ds[lane + 1]), sub ? b : 0.0);
         } else if (lane == jj) {
             cc = alpha;
         }
@@ -685,10 +691,7 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         // rounding level (MinorSum; its bound for complex128, the smaller one, for both types)
         const bool minor = __all_sync(0xffffffffu, !small || !run || (s >= 0x1p-40 && s <= 0x1p40)) &&
                            m2 <= MinorSum<double2>::eta * MinorSum<double2>::eta * b2;
-        if (inv) {
-            ctl->coefA[lane][k] = cc * s;
-            Cb[((size_t)k * MMAX + lane) * MMAX + jj] = (float)cc;
-        }
+        if (inv) ctl->coefA[lane][k] = cc * s;
         if (lane != 0) return;
         ctl->c2[k] = c2;
         ctl->minor[k] = minor ? 1 : 0;
@@ -754,9 +757,11 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         const bool dead = !(nw2 > H.eta_bd * H.eta_bd * normu2);
         const bool sub = run && !dead && nd2 > H.eta_corr * H.eta_corr * nw2;
         if (lane <= jj) {
+            const double rb = rsqrt(nw2);
+            const bool off = sub || dead || !run;   // (after a subtraction mode 2 sets C)
             ctl->coefC[lane][k] = sub ? cs : 0.0;
-            if (sub) Cb[((size_t)k * MMAX + lane) * MMAX + jj] += (float)c;
-            db[(size_t)k * MMAX + lane] = sub || dead || !run ? 0.f : (float)(c * rsqrt(nw2));
+            Cb[((size_t)k * MMAX + lane) * MMAX + jj] = off ? 0.f : (float)(ci * rb);
+            db[(size_t)k * MMAX + lane] = off ? 0.f : (float)(c * rb);
         }
         if (sub && lane == jj) ctl->alpha[jj][k] += c;
         if (lane != 0) return;
@@ -784,10 +789,11 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         } else {
             finalize(nw2, gdot);
         }
-    } else if (lane != 0) {
-        return;
     } else if (mode == 2) {
-        if (k == 0 && lane == 0) {
+        if (Cb && lane <= jj && jj < ctl->m_eff[k] && ctl->corr[k])
+            Cb[((size_t)k * MMAX + lane) * MMAX + jj] = (float)(ci * rsqrt(nw2));
+        if (lane != 0) return;
+        if (k == 0) {
             H.vec_passes += jj + 3 + (general ? 1 : 0);
             H.vp_kind[KIND_PASSC] += jj + 3 + (general ? 1 : 0);
         }
@@ -795,7 +801,7 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
             atomicAdd(&H.n_corr, 1ull);
             finalize(nw2, gdot);
         }
-    } else {   // 4 combine, 5 load of psi0
+    } else if (lane == 0) {   // 4 combine, 5 load of psi0
         const double b0 = sqrt(nw2);
         if (!(b0 > 0.0)) {
             H.err = KRY_EINVAL;

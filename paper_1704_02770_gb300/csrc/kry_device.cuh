@@ -820,6 +820,7 @@ __device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, d
 
 // alpha_j = sigma_j Re <W_j, u> from the threads' sums, and in the last CTA the update's coefficients (see
 // k_ortho).  The terms C_ki d_k are at the level of the dots d, so FP32 holds them: it loses 2^-24 of each.
+// Both are free of H's scale (C_ki is kept over beta_i), so that FP32 holds them for any of it.
 template <class V>
 __device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, KryCtl *ctl, int jj)
 {
@@ -852,7 +853,8 @@ __device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, Kr
         float f = 0.f;
         for (int k = 0; k <= lane; ++k) f = fmaf(Cs[k * MMAX + lane], ds[k], f);
         const double b = ctl->beta[lane];
-        c = lane == jj - 1 ? b + (double)f : (double)fmaf((float)b, ds[lane + 1], f);
+        const bool sub = lane == jj - 1;   // d_j = 1
+        c = fma(b, (double)(sub ? f : f + ds[lane + 1]), sub ? b : 0.0);
     } else if (lane == jj) {
         c = alpha;
     }
@@ -865,10 +867,7 @@ __device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, Kr
         minor = __all_sync(0xffffffffu, !small || (s >= 0x1p-40 && s <= 0x1p40)) &&
                 m2 <= MinorSum<V>::eta * MinorSum<V>::eta * b2;
     }
-    if (inv) {
-        ctl->coefA[lane] = c * s;
-        ctl->C[lane][jj] = (float)c;
-    }
+    if (inv) ctl->coefA[lane] = c * s;
     if (lane != 0) return;
     ctl->alpha[jj] = alpha;
     ctl->c2 = c2;

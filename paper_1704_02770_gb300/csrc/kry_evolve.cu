@@ -579,7 +579,7 @@ int capture_step_b(kry_ham_s *H, const EvArgsB<V> &a, const ExpArgsB &ea, int m,
             if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, grid, a.K, a.Kp, 7, jj, general, cs, a.C, a.d);
             mark();
             if (rc == KRY_OK) rc = launch_lincomb_b<V>(a, 1, jj, gridB, cs);
-            if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 2, jj, general, cs);
+            if (rc == KRY_OK) rc = launch_reduce_b(a.ctl, part, gridB, a.K, a.Kp, 2, jj, general, cs, a.C);
             continue;
         }
         rc = launch_passA_b<V>(a, jj, grid, cs, 1);

@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
 // c_i = Re <(H - s) v_i, v_j>, and the update that made v_{i+1} says what (H - s) v_i is,
 //     (H - s) v_i = sum_{k<=i} C_ki v_k + beta_i v_{i+1}   (C_ki its coefficients c_k),
 // up to the rounding of that update.  With the dots d_k = Re <v_k, v_j> that this kernel measured when it
-// made v_j (d_j = 1), c_i = sum_{k<=i} C_ki d_k + beta_i d_{i+1}: beta_{j-1} for i = j - 1, rounding level
+// made v_j (d_j = 1), c_i = beta_i (sum_{k<=i} (C_ki / beta_i) d_k + d_{i+1}): beta_{j-1} for i = j - 1, rounding level
 // below, and c_j = alpha_j comes from the H.v pass.  An error of c_i is the same rounding that a dot product
 // of u has, it leaves the new vector that much off, and the next dots see it.  The Krylov vectors, whose
 // reads bound the step, are read once per Lanczos index instead of twice.
@@ -333,6 +333,7 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     __shared__ double wred[NW][QV + 3];
     __shared__ typename RealLin<V>::RCoef coef[MMAX + 1];
     __shared__ float mcoef[MMAX + 1];
+    __shared__ double ci[MMAX + 1];   // c_i
     __shared__ __align__(16) V xch[2 * ORTHO_NTHR<V> * ORTHO_XU];
     __shared__ int flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = tid >> 6;
@@ -341,6 +342,7 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
         const double c = ctl->coefA[tid];
         coef[tid] = RealLin<V>::coef(c);
         mcoef[tid] = -(float)c;
+        ci[tid] = c * (tid ? ctl->beta[tid - 1] : ctl->beta0);   // (1 / sigma_i is the norm that made v_i)
     }
     __syncthreads();
     const bool minor = MinorSum<V>::use && ctl->minor;
@@ -435,12 +437,11 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     const bool dead = !(nw2 > ctl->eta_bd * ctl->eta_bd * normu2);   // an invariant subspace: nothing to correct
     const bool sub = !dead && nd2 > ctl->eta_corr * ctl->eta_corr * nw2;
     if (inv) {
-        if (sub) {
-            ctl->coefC[tid] = dd * s;
-            ctl->C[tid][jj] += (float)dd;
-        }
+        const double rb = rsqrt(nw2);
+        if (sub) ctl->coefC[tid] = dd * s;   // (pass C2 sets C)
+        else if (!dead) ctl->C[tid][jj] = (float)(ci[tid] * rb);
         // d of the new vector; after pass C2 it is at rounding level and taken as zero
-        ctl->d[tid] = sub || dead ? 0.f : (float)(dd * rsqrt(nw2));
+        ctl->d[tid] = sub || dead ? 0.f : (float)(dd * rb);
     }
     if (sub && tid == jj) ctl->alpha[jj] += dd;
     if (tid != 0) return;
@@ -566,8 +567,11 @@ __global__ void __launch_bounds__(NTHR, RR == 4 ? 2 : 4) k_lincomb(EvArgs<V> a, 
     if (a.G) cta_sum_into(gacc, red, SLOT_G, wtmp);
     double2 *fin = red;
     if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, 0, true, a.G != nullptr)) return;
-    if (tid != 0) return;
     const double nw2 = fin[SLOT_NRM].x;
+    if (MODE == 1 && a.one_read && tid <= jj)
+        ctl->C[tid][jj] =
+            (float)((ctl->coefA[tid] + ctl->coefC[tid]) * (tid ? ctl->beta[tid - 1] : ctl->beta0) * rsqrt(nw2));
+    if (tid != 0) return;
     const double2 gdot = fin[SLOT_G];
     if (MODE == 0) {
         ctl->vec_passes += jj + 3 + (a.G ? 1 : 0);

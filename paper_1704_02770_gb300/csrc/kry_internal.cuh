@@ -171,8 +171,8 @@ struct EvArgsB {
     int rl_smem;
     int kch;         // H.v in chunks of kch realisations (8 or 16; 0 = all K at once)
     int one_read;    // update and dots in one pass over the Krylov vectors (k_ortho_b)
-    // one-read form, per realisation: C[k][i][i'] the coefficient of v_i in the update that made v_{i'+1},
-    // d[k][i] = Re <v_i, v_j> of the last vector
+    // one-read form, per realisation: C[k][i][i'] the coefficient of v_i in the update that made v_{i'+1} over
+    // beta_i', d[k][i] = Re <v_i, v_j> of the last vector
     float *C, *d;
 };
 
@@ -191,7 +191,7 @@ struct ExpArgsB {
 // pass A of the batched path: part 0 = the H.v and the dots, 1 = the H.v only, 2 = the dots only
 template <class V> int launch_passA_b(const EvArgsB<V> &a, int jj, int grid, cudaStream_t s, int part = 0);
 template <class V> int launch_lincomb_b(const EvArgsB<V> &a, int mode, int jj, int grid, cudaStream_t s);
-// (C, d: of the one-read form, modes 6 and 7)
+// (C, d: of the one-read form, modes 6 and 7; C also in its mode 2)
 int launch_reduce_b(KryCtlB *ctl, const double2 *part, int grid, int K, int Kp, int mode, int jj,
                     int general, cudaStream_t s, float *C = nullptr, float *d = nullptr);
 // one-read form: alpha_j's partial sums (returns the CTAs, or minus a status) and the update with its dots
@@ -214,8 +214,8 @@ struct KryCtl {
     double normu2;             // ||H v_j||^2 of the last pass A
     double c2;                 // ||V^H H v_j||^2 of the last pass A (Pythagoras test of pass B)
     int minor;                 // coefA[0 .. j - 2] are at rounding level (MinorSum)
-    float C[MMAX][MMAX];       // one-read form: C[k][i], the coefficient of v_k in the update that made v_{i+1}
-    float d[MMAX];             // and Re <v_k, v_j>, k < j, of the last vector
+    float C[MMAX][MMAX];       // one-read form: C[k][i], the coefficient of v_k in the update that made v_{i+1},
+    float d[MMAX];             // over beta_i, and Re <v_k, v_j>, k < j, of the last vector
     double beta0;              // ||psi|| at the start of the Krylov step
     double t_now, t_end, tol, tau_prev;
     double eta_corr, eta_bd;   // second-pass and breakdown thresholds (relative)

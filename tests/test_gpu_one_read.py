@@ -200,3 +200,27 @@ def test_batched_general_state_and_idle_realisations(kry, K, form):
     H0 = kry.Hamiltonian(B, 0.0, 1.0, h)
     P0, st0 = H0.return_probability((1 << N) - 1, [1.0, 5.0], tol=1e-6, dtype=form)
     assert np.max(np.abs(P0 - 1.0)) <= 1e-6 and st0["n_breakdowns"] >= K
+
+
+@pytest.mark.parametrize("exponent", [133, 60, -30])
+@pytest.mark.parametrize("K", [1, 10])
+def test_recurrence_is_free_of_the_scale_of_H(kry, K, exponent):
+    """2^e H over times 2^-e t is the same evolution (2^133 is beyond the range of FP32): the coefficients of
+    the recurrence are kept over beta_i, so P, the orthogonality of the vectors and the number of subtractions
+    do not notice.  (Below about 2^-40 the absolute floor of the small exponential's half-width, 1e-12, would
+    shorten the steps.)"""
+    L, N = (20, 7) if K == 1 else (14, 7)
+    s = sum(1 << (2 * i) for i in range(N))
+    h = np.array([workloads.quasiperiodic_field(L, 1.3, p) for p in workloads.phases(9, K)])
+    B = kry.Basis(L, N)
+    f = 2.0**exponent
+    times = np.array([0.5, 2.0])
+    out = []
+    for J, hh, t in ((1.0, h, times), (f, f * h, times / f)):
+        H = kry.Hamiltonian(B, J, 0.8, hh if K > 1 else hh[0])
+        H.orth_check(True)
+        out.append(H.return_probability(s, t, tol=1e-10))
+    (P1, st1), (P2, st2) = out
+    print(f"[scale 2^{exponent}] K={K}: |dP| {np.max(np.abs(P2 - P1)):.1e}, loss {st1['max_orth_loss']:.1e} and {st2['max_orth_loss']:.1e}")
+    assert np.max(np.abs(P2 - P1)) <= 1e-10
+    assert st2["n_second_pass"] == 0 and 0.0 < st2["max_orth_loss"] <= (5e-14 if K == 1 else 2e-12)

@@ -42,74 +42,6 @@ __device__ __forceinline__ int cheb_degree(double x)
     return K < KMAX ? K : KMAX;
 }
 
-// J_k(x) for k = 0..K into out[0..K] (x >= 0).
-__device__ void bessel_seq(double x, int K, double *out)
-{
-    if (x < 1e-6) {
-        for (int k = 0; k <= K; ++k) out[k] = 0.0;
-        out[0] = 1.0 - 0.25 * x * x;
-        if (K >= 1) out[1] = 0.5 * x - x * x * x / 16.0;
-        if (K >= 2) out[2] = x * x / 8.0;
-        if (K >= 3) out[3] = x * x * x / 48.0;
-        return;
-    }
-    int ns = (K > (int)x ? K : (int)x) + 40;
-    ns += ns & 1;
-    const double inv = 2.0 / x;
-    double jp1 = 0.0, jk = 1e-280, sum = 0.0;
-    for (int k = ns; k >= 1; --k) {
-        const double jm1 = (double)k * inv * jk - jp1;
-        jp1 = jk;
-        jk = jm1;
-        const int idx = k - 1;
-        if (idx <= K) out[idx] = jm1;
-        if (idx >= 2 && !(idx & 1)) sum += jm1;
-        if (fabs(jk) > 1e250) {
-            jk *= 1e-250;
-            jp1 *= 1e-250;
-            sum *= 1e-250;
-            for (int t = idx; t <= K; ++t) out[t] *= 1e-250;
-        }
-    }
-    const double invS = 1.0 / (out[0] + 2.0 * sum);
-    for (int k = 0; k <= K; ++k) out[k] *= invS;
-}
-
-// sum_k w_k c_k v_k as a complex number, for real c_k, v_k
-__device__ __forceinline__ double2 jacobi_anger_sum(const double *c, const double *v, int vstride, int K)
-{
-    double re = 0.0, im = 0.0;
-    for (int k = 0; k <= K; ++k) {
-        const double t = c[k] * v[k * vstride] * (k == 0 ? 1.0 : 2.0);
-        switch (k & 3) {
-        case 0: re += t; break;
-        case 1: im -= t; break;
-        case 2: re -= t; break;
-        default: im += t; break;
-        }
-    }
-    return make_double2(re, im);
-}
-
-// Error-estimate sum: sum_k w_k I_k v_k with I_k = int_0^x J_k from the J sequence.
-__device__ __forceinline__ double2 integral_sum(const double *J, const double *v, int vstride, int K)
-{
-    double re = 0.0, im = 0.0, ip1 = 0.0, ip2 = 0.0;   // I_{k+1}, I_{k+2}
-    for (int k = K; k >= 0; --k) {
-        const double Ik = (k + 1 <= K ? 2.0 * J[k + 1] : 0.0) + ip2;
-        ip2 = ip1;
-        ip1 = Ik;
-        const double t = Ik * v[k * vstride] * (k == 0 ? 1.0 : 2.0);
-        switch (k & 3) {
-        case 0: re += t; break;
-        case 1: im -= t; break;
-        case 2: re -= t; break;
-        default: im += t; break;
-        }
-    }
-    return make_double2(re, im);
-}
-
 __device__ __forceinline__ double2 cmul(double2 a, double2 b)
 {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -170,12 +102,15 @@ __device__ double2 chebyshev_basis(ExpSmem &sm, int me, int K)
     return make_double2(c, r);
 }
 
-// ---- the same sums straight from the backward recurrence, without a stored sequence
+// ---- sums over the Bessel functions straight from the backward recurrence
+constexpr int NKD = KMAX + 64;   // table of the doubles k: the recurrence starts at most at KMAX + 41
+
 // Miller's recurrence for J_K(x) .. J_0(x), unnormalised, handed to f from k = K down; the caller's
 // sums are scaled along by f.scale when the values are.  Returns 1 / (J_0 + 2 sum J_2k), the factor
 // that normalises them.  Integer tests of the exponent and a table of the doubles k spare the FP64
-// pipe (77 issue cycles per instruction of a warp): two and a half instructions per index.
-template <class F>
+// pipe (77 issue cycles per instruction of a warp): two and a half instructions per index.  ANY: arguments
+// above the table too, which a Krylov step does not have (x <= XMAX) and kry_tridiag_expv takes.
+template <bool ANY = false, class F>
 __device__ __forceinline__ double bessel_down(double x, int K, const double *kd, F &f)
 {
     if (x < 1e-6) {
@@ -185,10 +120,24 @@ __device__ __forceinline__ double bessel_down(double x, int K, const double *kd,
         f.add(0, 1.0 - 0.25 * x * x);
         return 1.0;
     }
-    int ns = (K > (int)x ? K : (int)x) + 40;
+    const int xi = ANY ? (int)fmin(x, 1048576.0) : (int)x;   // (the expansion holds to about x = 100)
+    int ns = (K > xi ? K : xi) + 40;
     ns += ns & 1;
     const double inv = 2.0 / x;
     double jp1 = 0.0, jk = 1e-280, sum = 0.0, j0 = 0.0;
+    if constexpr (ANY) {
+        for (; ns >= NKD; --ns) {
+            const double jm1 = (double)ns * inv * jk - jp1;
+            jp1 = jk;
+            jk = jm1;
+            if (ns & 1) sum += jm1;
+            if (fabs(jk) > 1e250) {
+                jk *= 1e-250;
+                jp1 *= 1e-250;
+                sum *= 1e-250;
+            }
+        }
+    }
     for (int k = ns; k >= 1; --k) {
         const double jm1 = kd[k] * inv * jk - jp1;
         jp1 = jk;
@@ -253,7 +202,7 @@ struct BesselRead {   // sum_k J_k w_k G_k
 constexpr int EXPW = 4;   // warps of the small exponential, one per SM sub-partition (each has its own FP64 pipe)
 struct ExpSmem4 : ExpSmem {
     double S[KMAX + 2];        // sums of BesselErr
-    double kd[KMAX + 64];      // the doubles 0, 1, 2, ...
+    double kd[NKD];            // the doubles 0, 1, 2, ...
     double2 yp[EXPW][32];      // partial sums of y
     double cr[2], inv[32];     // T's centre and half-width; normalisation of the candidates' sequences
     double tau, err;
@@ -404,7 +353,7 @@ __global__ void __launch_bounds__(32 * EXPW) k_smallexp(ExpArgs ea)
         }
         sm.g[lane] = g;
     }
-    for (int k = threadIdx.x; k < KMAX + 64; k += 32 * EXPW) sm.kd[k] = (double)k;
+    for (int k = threadIdx.x; k < NKD; k += 32 * EXPW) sm.kd[k] = (double)k;
     __syncthreads();
     const double beta0 = ctl->beta0, h = sm.be[me - 1];
     const double t_now = ctl->t_now, t_end = ctl->t_end, tol = ctl->tol;
@@ -524,37 +473,39 @@ __global__ void __launch_bounds__(32 * EXPW) k_smallexp(ExpArgs ea)
     }
 }
 
-// Test hook: y = exp(-i tau T) e_1 and err(tau) for given T, h (beta = 1).
-__global__ void __launch_bounds__(32) k_expv_test(const double *alpha, const double *beta, int me,
-                                                  double h, double tau, double *y, double *err)
+// y = exp(-i tau T) e_1 and err(tau) for given T, h (beta = 1): the step's own functions on one CTA of four warps.
+__global__ void __launch_bounds__(32 * EXPW) k_expv(const double *alpha, const double *beta, int me, double h,
+                                                    double tau, double *y, double *err)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ExpSmem &sm = *(ExpSmem *)smem_raw;
-    const int lane = threadIdx.x;
-    if (lane < me) {
+    ExpSmem4 &sm = *(ExpSmem4 *)smem_raw;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0 && lane < me) {
         sm.al[lane] = alpha[lane];
         sm.be[lane] = (lane + 1 < me) ? beta[lane] : h;
     }
-    __syncwarp();
-    // radius first (with K = 0), then the full basis for the needed degree
-    double2 cr = chebyshev_basis(sm, me, 0);
-    const int K = cheb_degree(tau * cr.y);
-    cr = chebyshev_basis(sm, me, K);
-    double *myJ = sm.jb + lane * (KMAX + 2);
-    bessel_seq(tau * cr.y, K, myJ);
-    __syncwarp();
-    const double *J0 = sm.jb;   // lane 0's sequence (all lanes computed the same)
-    if (lane < me) {
-        const double2 s = jacobi_anger_sum(J0, sm.tch + lane, 32, K);
-        double sn, cs;
-        sincos(tau * cr.x, &sn, &cs);
-        const double2 yy = cmul(make_double2(cs, -sn), s);
-        y[2 * lane] = yy.x;
-        y[2 * lane + 1] = yy.y;
+    for (int k = threadIdx.x; k < NKD; k += 32 * EXPW) sm.kd[k] = (double)k;
+    __syncthreads();
+    const double x = tau * gershgorin(sm, me).y;   // (every warp)
+    const int K = cheb_degree(x);
+    if (warp == 1) exp_basis(sm, me, K, 0.0);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        BesselErrStore f;
+        f.S = sm.S;
+        f.st = BesselStore{sm.jb, K};
+        if (x < 1e-6)
+            for (int k = 4; k <= K; ++k) f.st.out[k] = 0.0;
+        sm.inv[0] = bessel_down<true>(x, K, sm.kd, f);
+        *err = fabs(h) / sm.cr[1] * f.value(sm.inv[0]);
     }
-    if (lane == 0) {
-        const double2 s = integral_sum(J0, sm.tch + (me - 1), 32, K);
-        *err = fabs(h) / cr.y * sqrt(s.x * s.x + s.y * s.y);
+    __syncthreads();
+    exp_parts(sm, sm.jb, me, K);
+    __syncthreads();
+    if (warp == 0 && lane < me) {
+        const double2 v = exp_y(sm, tau * sm.cr[0]);
+        y[2 * lane] = v.x * sm.inv[0];
+        y[2 * lane + 1] = v.y * sm.inv[0];
     }
 }
 
@@ -599,7 +550,7 @@ __global__ void __launch_bounds__(32) k_exp_scan_b(ExpArgsB ea)
     const int k = blockIdx.x, lane = threadIdx.x;
     const int me = ctl->m_eff[k];
     load_tridiag_b(sm, ctl, k, me, ea);
-    for (int q = lane; q < KMAX + 64; q += 32) sm.kd[q] = (double)q;
+    for (int q = lane; q < NKD; q += 32) sm.kd[q] = (double)q;
     __syncwarp();
     const double beta0 = ctl->beta0[k], h = sm.be[me - 1];
     const double remaining = H.t_end - H.t_now;
@@ -650,7 +601,7 @@ __global__ void __launch_bounds__(32 * EXPW) k_exp_apply_b(ExpArgsB ea)
     for (int o = 16; o > 0; o >>= 1) tau = fmin(tau, __shfl_xor_sync(0xffffffffu, tau, o));
     const int me = ctl->m_eff[k];
     if (warp == 0) load_tridiag_b(sm, ctl, k, me, ea);
-    for (int q = threadIdx.x; q < KMAX + 64; q += 32 * EXPW) sm.kd[q] = (double)q;
+    for (int q = threadIdx.x; q < NKD; q += 32 * EXPW) sm.kd[q] = (double)q;
     __syncthreads();
     const double beta0 = ctl->beta0[k], h = sm.be[me - 1];
     const double t_now = H.t_now, t_end = H.t_end, remaining = t_end - t_now;
@@ -755,9 +706,9 @@ extern "C" int kry_tridiag_expv(const double *alpha, const double *beta, int m, 
     if (e == cudaSuccess && m > 1)
         e = cudaMemcpyAsync(db, beta, sizeof(double) * (m - 1), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_expv_test, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ExpSmem));
+        e = cudaFuncSetAttribute(k_expv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ExpSmem4));
     if (e == cudaSuccess) {
-        k_expv_test<<<1, 32, sizeof(ExpSmem), s>>>(da, db, m, h, tau, dy, de);
+        k_expv<<<1, 32 * EXPW, sizeof(ExpSmem4), s>>>(da, db, m, h, tau, dy, de);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(y_out, dy, sizeof(double) * 2 * m, cudaMemcpyDeviceToHost, s);
@@ -876,10 +827,10 @@ extern "C" int kry_tridiag_expv_noalloc(const double *alpha, const double *beta,
     if (e == cudaSuccess && m > 1)
         e = cudaMemcpyAsync(db, beta, sizeof(double) * (m - 1), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_expv_test, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(ExpSmem));
+        e = cudaFuncSetAttribute(k_expv, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(ExpSmem4));
     if (e == cudaSuccess) {
-        k_expv_test<<<1, 32, sizeof(ExpSmem), s>>>(da, db, m, h, tau, dy, de);
+        k_expv<<<1, 32 * EXPW, sizeof(ExpSmem4), s>>>(da, db, m, h, tau, dy, de);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(y_out, dy, sizeof(double) * 2 * m, cudaMemcpyDeviceToHost, s);

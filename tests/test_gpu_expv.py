@@ -1,4 +1,5 @@
-"""Device small exponential (kry_tridiag_expv) against the oracle's Pade exponential.
+"""Device small exponential (kry_tridiag_expv: the functions that the Krylov step's kernels run) against
+the oracle's Pade exponential.
 
 y = exp(-i tau T) e_1 must match to 1e-13; the error estimate err = h |e_m^T tau
 phi_1(-i tau (T - c)) e_1| is checked against the last first-column entry of the Pade
@@ -60,6 +61,24 @@ def test_expv_large_argument(kry):
     assert np.max(np.abs(y - yr)) < 1e-12
     assert abs(err - er) <= 1e-10 * er + 1e-15
     assert abs(np.linalg.norm(y) - 1.0) < 1e-12
+
+
+@pytest.mark.parametrize("x", [0.9e-6, 1.1e-6, 0.02, 20.0, 60.0, 75.0, 90.0, 128.0, 250.0])
+@pytest.mark.parametrize("m", [3, 4, 31])
+def test_expv_over_the_argument(kry, x, m):
+    """tau * half-width on both sides of the short series, through the step's range (to 50), and beyond, where
+    the expansion ends at degree 128 and y misses at most the terms 2 |J_k(x)|, k > 128."""
+    from scipy.special import jv
+    rng = np.random.default_rng(m)
+    a, b = rng.normal(size=m), np.abs(rng.normal(size=m - 1)) + 0.2
+    off = np.r_[0.0, b] + np.r_[b, 0.0]
+    tau = x / (0.5 * (np.max(a + off) - np.min(a - off)))
+    y, err = kry.tridiag_expv(a, b, 0.9, tau)
+    yr, er = _reference(a, np.r_[b, 0.0], 0.9, tau)
+    tail = 2.0 * np.sum(np.abs(jv(np.arange(129, 400), x)))
+    assert np.max(np.abs(y - yr)) < 1e-12 + tail
+    if x <= 60.0:   # (the short series of J_k ends at x^3, its next terms are below 1e-12 of it)
+        assert abs(err - er) <= 1e-10 * er + 1e-20
 
 
 def test_expv_rejects_bad_arguments(kry):

@@ -610,12 +610,11 @@ __global__ void __launch_bounds__(32 * EXPW) k_exp_apply_b(ExpArgsB ea)
     const int Kc = cheb_degree(tau * cr.y);
     if (warp == 1) {
         exp_basis(sm, me, Kc, ctl->shift[k]);   // T holds H_k - s_k I
-    } else if (warp == 0) {
-        BesselStore f{sm.jb, Kc};   // (the lanes write the same values)
+    } else if (threadIdx.x == 0) {   // (one lane: the sequence is rescaled in place)
+        BesselStore f{sm.jb, Kc};
         if (tau * cr.y < 1e-6)
             for (int q = 4; q <= Kc; ++q) f.out[q] = 0.0;
-        const double n = bessel_down(tau * cr.y, Kc, sm.kd, f);
-        if (lane == 0) sm.inv[0] = n;
+        sm.inv[0] = bessel_down(tau * cr.y, Kc, sm.kd, f);
     }
     __syncthreads();
     const double c = sm.cr[0], r = sm.cr[1];

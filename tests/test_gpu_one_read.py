@@ -224,3 +224,73 @@ def test_recurrence_is_free_of_the_scale_of_H(kry, K, exponent):
     print(f"[scale 2^{exponent}] K={K}: |dP| {np.max(np.abs(P2 - P1)):.1e}, loss {st1['max_orth_loss']:.1e} and {st2['max_orth_loss']:.1e}")
     assert np.max(np.abs(P2 - P1)) <= 1e-10
     assert st2["n_second_pass"] == 0 and 0.0 < st2["max_orth_loss"] <= (5e-14 if K == 1 else 2e-12)
+
+
+@pytest.mark.parametrize("K", [10, 40, 64])
+@pytest.mark.parametrize("form,eps,tol", [("c128", 1e-6, 1e-10), ("c128e", 1e-6, 1e-10), ("c64", 1e-4, 2e-5)])
+def test_batched_second_pass_of_some_realisations(kry, K, form, eps, tol):
+    """States within eps of an eigenvector: the first update cancels all but eps of H v, so its dots exceed the
+    threshold and pass C2 subtracts them, in these realisations alone (0, 3 and K - 1); realisation 1 is the
+    eigenvector itself, whose Krylov space ends at once, and the others are random.  Where the corrected
+    coefficients were wrong the part of size eps would be, above the tolerance.  (complex64: the rounding of
+    H v leaves ||w|| = 4e-7 for the eigenvector, and the step's budget, 0.05 tol / t_end, has to be above it.)"""
+    from scipy.sparse import csr_matrix
+    from scipy.sparse.linalg import eigsh
+    L, N = 14, 7
+    h = np.array([workloads.quasiperiodic_field(L, 1.3, p) for p in workloads.phases(9, K)])
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.8, h)
+    D = H.basis.dim
+    rng = np.random.default_rng(6)
+    x = rng.normal(size=(D, K)) + 1j * rng.normal(size=(D, K))
+    x /= np.linalg.norm(x, axis=0)
+    csr, near = {}, (0, 3, K - 1)
+    for k in near + (1,):
+        csr[k] = ob.CSR(L, N, 1.0, 0.8, h[k], True)
+        A = csr_matrix((csr[k].val, csr[k].col, csr[k].rowptr), shape=(D, D))
+        v = eigsh(A, k=1, which="SA", tol=1e-15)[1][:, 0]
+        x[:, k] = v + (eps * x[:, k] if k != 1 else 0.0)
+        x[:, k] /= np.linalg.norm(x[:, k])
+    xs = torch.from_numpy(x.reshape(-1)).cuda()
+    if form == "c64":
+        xs = xs.to(torch.complex64)
+    out = torch.empty_like(xs)
+    P, st = H.evolve(xs, [0.3, 0.6], tol=tol, psi_out=out, emulated=form == "c128e")
+    got = out.cpu().numpy().reshape(D, K)
+    print(f"[second pass] K={K} {form}: {st['n_second_pass']} of {st['n_hv'] * K} updates")
+    assert 3 * st["n_krylov_steps"] <= st["n_second_pass"] < 3 * st["n_hv"] and st["n_breakdowns"] >= st["n_krylov_steps"]
+    csr[2] = ob.CSR(L, N, 1.0, 0.8, h[2], True)
+    x0 = xs.cpu().numpy().reshape(D, K).astype(np.complex128)
+    for k in csr:
+        Pk, psi, _ = _oracle(csr[k], x0[:, k].copy(), [0.3, 0.6])
+        err = np.linalg.norm(got[:, k] - psi)
+        assert err <= tol and np.max(np.abs(P[:, k] - Pk)) <= tol, (k, err)
+
+
+@pytest.mark.parametrize("L,N,hh", [(8, 4, 0.5), (10, 5, 1.5), (20, 7, 1.3)])
+def test_complex64_keeps_psi_over_many_steps(kry, L, N, hh):
+    """The real inner product leaves Im <v_i, v_j> to itself, which rounding lets grow where Ritz values converge
+    (small sectors).  Over many steps in complex64 the norm of psi and psi itself must not notice: the reference
+    is the spectral exponential, in the largest sector the FP64 evolution.  The bar: every step rounds its 31
+    vectors' combination and each product by 2^-24 (an error that turns with the state, so the steps' add up
+    at worst linearly), and the budget tol."""
+    h = workloads.quasiperiodic_field(L, hh, 0.3)
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 1.0, h)
+    D = H.basis.dim
+    rng = np.random.default_rng(3)
+    psi0 = rng.normal(size=D) + 1j * rng.normal(size=D)
+    psi0 /= np.linalg.norm(psi0)
+    x = torch.from_numpy(psi0).cuda()
+    t, out = 200.0 if D < 1000 else 40.0, torch.empty_like(x)
+    if D < 1000:
+        lam, Q = np.linalg.eigh(ob.CSR(L, N, 1.0, 1.0, h, True).dense())
+        exact = Q @ (np.exp(-1j * lam * t) * (Q.T @ psi0))
+    else:
+        H.evolve(x, [t], tol=1e-10, psi_out=out)
+        exact = out.cpu().numpy()
+    o64 = torch.empty_like(x, dtype=torch.complex64)
+    _, st = H.evolve(x.to(torch.complex64), [t], tol=1e-6, psi_out=o64)
+    got = o64.cpu().numpy().astype(np.complex128)
+    err, drift = np.linalg.norm(got - exact), abs(np.linalg.norm(got) - 1.0)
+    print(f"[c64 psi] L={L}: {st['n_krylov_steps']} steps, |dpsi| {err:.2e}, | ||psi|| - 1 | {drift:.2e}")
+    assert st["n_krylov_steps"] >= 10
+    assert err <= 1e-6 + st["n_hv"] * 2.0**-24 and drift <= 1e-6 + st["n_krylov_steps"] * 2.0**-22

@@ -245,8 +245,9 @@ int kry_profile_read(kry_ham H, double *ms, double *bytes, int64_t *launches);
  *            the gathered part of the vector fits in L2 (0 = all K at once).
  * Parts 1, 2 and 4 change only the order of independent loads (the results are bitwise the
  * same); parts 0 and 3 change which rows a thread or CTA sums into its partial norms and dots
- * (the results agree to rounding).  Single-realisation evolutions use parts 0-3, batched ones
- * parts 0 and 4.  New Hamiltonians start at {0, 0, 0, 2, 0}, or {0, 3, 0, 2, 0} for L >= 28
+ * (the results agree to rounding).  Single-realisation evolutions use part 0, part 1 (split-table
+ * bases) and, below 65,536 states, parts 2 and 3 (from there on one pass takes the dots and the update, and
+ * part 3 acts on the second Gram-Schmidt pass alone); batched ones use parts 0 and 4.  New Hamiltonians start at {0, 0, 0, 2, 0}, or {0, 3, 0, 2, 0} for L >= 28
  * (split-table bases).
  * kry_set_shape returns KRY_EINVAL for values outside those lists; kry_set_grid sets part 0. */
 int kry_set_shape(kry_ham H, int dtype, const int *shape);
@@ -257,7 +258,8 @@ int kry_set_grid(kry_ham H, int dtype, int grid);
  * basis state probe_state to t_probe (reps replays after one capture run, best kept) for
  * candidate shapes, one part after another with the other parts at their best so far: part 0
  * over {0, 1, 2, 3, 4 x the SM count}, then part 1 over {0..3}, part 2 over {0, 1}, part 3 over
- * {2, 1, 4} (K > 1: part 0, then part 4 over {0, 16, 8}).  Keeps the fastest for later calls on
+ * {2, 1, 4}, without the parts that H's evolutions do not use (K > 1: part 0, then part 4 over
+ * {0, 16, 8}).  Keeps the fastest for later calls on
  * H with this dtype and returns it in shape_out[5].  cand_out (host, [max_cand][5]) and ms_out
  * ([max_cand]) receive the shapes tried and their times, *n_cand how many were stored. */
 int kry_autotune(kry_ham H, int dtype, int m, uint64_t probe_state, double t_probe, int reps,

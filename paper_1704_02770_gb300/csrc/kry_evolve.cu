@@ -150,11 +150,6 @@ void drop_graph(kry_ham_s *H)
 // pass C launched in every Lanczos index (true) or as a conditional node
 bool plain_step_graph(const kry_ham_s *H) { return H->plain_graph || !H->cond_pass_c; }
 
-// Update and dots in one pass over the Krylov vectors (k_ortho), from 65,536 rows on: there the vectors'
-// reads cost more than the pass's longer rows (L = 19 c128e: 45.7 -> 43.6 us per Lanczos index, L = 24 c64
-// 188 -> 152, L = 30 c64 10.1 -> 8.2 ms); below, both forms are bound by latency and tie (L = 16 c128).
-int one_read_form(uint32_t D) { return D >= 65536u ? 1 : 0; }
-
 // Profile intervals of the captured step: four per Lanczos index (the H.v, pass A's dots,
 // pass B, pass C), then the small exponential and the combine; kind of the k-th interval.
 int n_intervals(int m) { return 4 * m + 2; }

@@ -278,6 +278,11 @@ struct EvArgs {
     int one_read;    // update and dots in one pass over the Krylov vectors (k_ortho)
 };
 
+// Update and dots in one pass over the Krylov vectors (k_ortho), from 65,536 rows on: there the vectors'
+// reads cost more than the pass's longer rows (L = 19 c128e: 45.7 -> 43.6 us per Lanczos index, L = 24 c64
+// 188 -> 152, L = 30 c64 10.1 -> 8.2 ms); below, both forms are bound by latency and tie (L = 16 c128).
+inline bool one_read_form(uint32_t D) { return D >= 65536u; }
+
 struct ExpArgs {
     KryCtl *ctl;
     const double *times;
@@ -345,7 +350,6 @@ struct kry_ham_s {
     int ws_user;                // ws belongs to the caller (kry_set_workspace): never freed here
     // cached CUDA graph of one Krylov step
     cudaGraphExec_t gexec;
-    int g_one_read;             // the step graph is that of the one-read form
     int g_dtype, g_m, g_general, g_grid, g_gridB, g_gridH, g_shape, g_plain;
     int plain_graph;            // forced plain step graph (kry_profile_enable(H, 2))
     int cond_pass_c;            // pass C as a conditional node (kry_set_second_pass_node)

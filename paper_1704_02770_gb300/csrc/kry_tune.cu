@@ -1,5 +1,5 @@
 // Launch-shape autotuner: measures short probe evolutions of the handle's own workload for
-// candidate launch shapes of the vector kernels and keeps the fastest.  A shape has four
+// candidate launch shapes of the vector kernels and keeps the fastest.  A shape has five
 // parts, tuned one after another (coordinate descent, each part over its candidates with the
 // others at their best so far):
 //   [0] CTAs of the streaming kernels: the occupancy rule (0) or 1..4 times the SM count;
@@ -10,8 +10,9 @@
 //   [4] batched H.v in chunks of 8 or 16 realisations (0 = all K at once).
 // Parts [1], [2] and [4] change only the order in which independent loads are issued (the
 // same bits); parts [0] and [3] change which rows a CTA or thread sums into its partial norms
-// and dots (results agree to rounding).  Single-realisation handles tune parts [0]-[3],
-// batched handles (K > 1) parts [0] and [4].
+// and dots (results agree to rounding).  A handle tunes the parts that reach a kernel of its step: batched
+// handles (K > 1) parts [0] and [4], single realisations [0], [1] (split tables only), and in the two-pass
+// form (below 65,536 states) [2] and [3].
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -108,7 +109,13 @@ extern "C" int kry_autotune(kry_ham H, int dtype, int m, uint64_t probe_state, d
         return rc;
     };
     const std::vector<int> cands[NS] = {{0, sms, 2 * sms, 3 * sms, 4 * sms}, {0, 1, 2, 3}, {0, 1}, {2, 1, 4}, {0, 16, 8}};
-    const std::vector<int> parts = H->K > 1 ? std::vector<int>{0, 4} : std::vector<int>{0, 1, 2, 3};
+    std::vector<int> parts = {0};
+    if (H->K > 1) {
+        parts.push_back(4);
+    } else {
+        if (!H->b->dev.list) parts.push_back(1);
+        if (!one_read_form(H->b->dev.D)) parts.insert(parts.end(), {2, 3});
+    }
     double best_ms = 1e300;
     for (int part : parts) {
         for (int v : cands[part]) {

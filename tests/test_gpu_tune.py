@@ -100,6 +100,19 @@ def test_autotune_single(kry, tmp_path):
     assert len(json.load(open(cache))) == 1
 
 
+@pytest.mark.parametrize("lst,fixed", [(False, [2, 3, 4]), (True, [1, 2, 3, 4])])
+def test_autotune_leaves_out_parts_without_a_kernel(kry, lst, fixed):
+    """From 65,536 states on no kernel takes the dots alone and the update's rows per thread reach only the
+    second pass, and the sorted-list H.v has one form: the tuner probes the other parts."""
+    L, N = 20, 7
+    H = kry.Hamiltonian(kry.Basis(L, N, list=lst), 1.0, 1.0, workloads.quasiperiodic_field(L, 1.0, 0.4))
+    s0 = H.get_shape("c64")
+    res = H.autotune(sum(1 << (2 * i) for i in range(N)), 0.3, dtype="c64", reps=1)
+    shapes = [s for s, _ in res["candidates"]]
+    assert len(shapes) == (5 if lst else 8)
+    assert all(s[q] == s0[q] for s in shapes + [res["shape"]] for q in fixed)
+
+
 def test_autotune_batched(kry):
     L, N, K = 14, 7, 8
     h = [workloads.quasiperiodic_field(L, 1.0, p) for p in workloads.phases(11, K)]

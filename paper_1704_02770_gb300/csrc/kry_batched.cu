@@ -442,7 +442,8 @@ constexpr int ALPHA_NTHR = 512;
 
 // Re <W_j[:, k], U[:, k]> of every realisation, on k_ortho_b's split of the elements: the CTAs' shares go to
 // part[CTA][Kp] (doubles).  A pass of its own, because the H.v's forms split the states in different ways
-// and alpha_j's bits must not depend on them; two of the step's j + 5 vector reads.
+// and alpha_j's bits must not depend on them; two of the step's j + 5 vector reads.  In the first Krylov step
+// also c_0 = Re <W_0[:, k], U[:, k]> (see alpha_epilogue), to part[gridDim + CTA][Kp].
 template <class V, int T>
 __global__ void __launch_bounds__(ALPHA_NTHR) k_alpha_b(EvArgsB<V> a, int jj)
 {
@@ -455,30 +456,41 @@ __global__ void __launch_bounds__(ALPHA_NTHR) k_alpha_b(EvArgsB<V> a, int jj)
     const uint32_t unit = T / K * K;
     const size_t n = (size_t)a.b.D * K;
     const uint32_t nu = (uint32_t)((n + unit - 1) / unit), du = gridDim.x * NGRP;
-    const V *x = a.W + (size_t)jj * a.ldW;
-    RealAcc<V> al;
-    for (uint32_t u0 = blockIdx.x * NGRP + g; u0 < nu; u0 += NU * du) {
-        V xv[NU], uv[NU];
+    const bool first = jj > 0 && ctl->hd.n_steps == 0;
+    auto dots = [&](const V *x, double *out) {
+        RealAcc<V> al;
+        for (uint32_t u0 = blockIdx.x * NGRP + g; u0 < nu; u0 += NU * du) {
+            V xv[NU], uv[NU];
 #pragma unroll
-        for (int q = 0; q < NU; ++q) {
-            const size_t r = (size_t)(u0 + q * du) * unit + t;
-            const bool in = t < (int)unit && u0 + q * du < nu && r < n;
-            xv[q] = ldg_if(in, x + r);
-            uv[q] = ldg_if(in, a.U + r);
+            for (int q = 0; q < NU; ++q) {
+                const size_t r = (size_t)(u0 + q * du) * unit + t;
+                const bool in = t < (int)unit && u0 + q * du < nu && r < n;
+                xv[q] = ldg_if(in, x + r);
+                uv[q] = ldg_if(in, a.U + r);
+            }
+#pragma unroll
+            for (int q = 0; q < NU; ++q) al.add(xv[q], RealAcc<V>::pre(uv[q]));
+            al.renorm();
         }
-#pragma unroll
-        for (int q = 0; q < NU; ++q) al.add(xv[q], RealAcc<V>::pre(uv[q]));
-        al.renorm();
-    }
-    sums[tid] = al.sum();
-    __syncthreads();
-    if (tid < a.Kp) {
-        Sum tot{};
-        if (tid < K)
-            for (int gg = 0; gg < NGRP; ++gg)
-                for (uint32_t r = tid; r < unit; r += K) tot = add2(tot, sums[gg * T + r]);
-        ((double *)a.part)[(size_t)blockIdx.x * a.Kp + tid] = to_double(tot);
-    }
+        __syncthreads();
+        sums[tid] = al.sum();
+        __syncthreads();
+        if (tid < a.Kp) {
+            Sum tot{};
+            if (tid < K)
+                for (int gg = 0; gg < NGRP; ++gg)
+                    for (uint32_t r = tid; r < unit; r += K) tot = add2(tot, sums[gg * T + r]);
+            out[(size_t)blockIdx.x * a.Kp + tid] = to_double(tot);
+        }
+    };
+    double *part = (double *)a.part;
+    dots(a.W + (size_t)jj * a.ldW, part);
+    if (!first) return;
+    part += (size_t)gridDim.x * a.Kp;
+    if (a.G) dots(a.W, part);
+    else if (tid < a.Kp)   // basis states: one element
+        part[(size_t)blockIdx.x * a.Kp + tid] =
+            blockIdx.x == 0 && tid < K ? real_part(a.U + (size_t)ctl->r0k[tid] * K + tid) : 0.0;
 }
 
 // k_ortho for K realisations: thread t of a group takes the element of state t / K and realisation t % K of
@@ -592,8 +604,8 @@ __global__ void __launch_bounds__(ORTHO_B_NTHR<V, T>, 1) k_ortho_b(EvArgsB<V> a,
 // ---------------------------------------------------------------- per-realisation reductions
 
 // mode: 0 pass A, 1 pass B, 3 pass C1 (dots of w), 2 pass C2 (correction), 4 combine,
-// 5 load of a general psi0; one-read form: 6 alpha_j and the update's coefficients (partials [CTA][Kp]
-// of k_alpha_b), 7 the dots and the norm of the update (see k_ortho).  One CTA per realisation.  A warp takes a whole slot (lanes over the
+// 5 load of a general psi0; one-read form: 6 alpha_j, c_0 and the update's coefficients (partials of
+// k_alpha_b), 7 the dots and the norm of the update (see k_ortho).  One CTA per realisation.  A warp takes a whole slot (lanes over the
 // CTAs' partials) and lane i of warp 0 the scalars of vector i: GB300 issues
 // one FP64 warp instruction per about 77 cycles and SM sub-partition whatever its active lanes, so
 // block-wide trees slot by slot and loops over the vectors in one thread cost tens of us at j = 30.
@@ -619,18 +631,19 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
     if (mode == 6) {
         for (int e = tid; e < MMAX * MMAX; e += 256) Cs[e] = Cb[(size_t)k * MMAX * MMAX + e];
         if (tid <= MMAX) ds[tid] = tid < jj ? db[(size_t)k * MMAX + tid] : 0.f;
-        if (warp == 0) {
+        if (warp == 0 || (warp == 1 && jj > 0 && H.n_steps == 0)) {   // alpha_j; c_0
+            const double *pa = (const double *)part + (size_t)warp * grid * Kp;
             double s = 0.0;
             for (int c0 = 0; c0 < grid; c0 += 256) {
                 double x[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const int c = c0 + 32 * i + lane;
-                    x[i] = c < grid ? __ldg((const double *)part + (size_t)c * Kp + k) : 0.0;
+                    x[i] = c < grid ? __ldg(pa + (size_t)c * Kp + k) : 0.0;
                 }
                 s += warp_sum_int<8>(x);
             }
-            if (lane == 0) fin[0].x = s;
+            if (lane == 0) fin[warp].x = s;
         }
     }
     for (int q = warp; q < ns; q += 8) {
@@ -684,6 +697,7 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         } else if (lane == jj) {
             cc = alpha;
         }
+        if (lane == 0 && jj > 0 && H.n_steps == 0) cc = fin[1].x * s;
         if (!run) cc = 0.0;   // (invariant subspace already reached: the next vectors stay zero)
         const double q2 = cc * cc, c2 = warp_sum_int<1>(&q2);
         const bool small = lane + 1 < jj;

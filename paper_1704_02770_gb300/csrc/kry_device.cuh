@@ -821,31 +821,54 @@ __device__ __forceinline__ void finalize_beta(KryCtl *ctl, int jj, double nw2, d
 // alpha_j = sigma_j Re <W_j, u> from the threads' sums, and in the last CTA the update's coefficients (see
 // k_ortho).  The terms C_ki d_k are at the level of the dots d, so FP32 holds them: it loses 2^-24 of each.
 // Both are free of H's scale (C_ki is kept over beta_i), so that FP32 holds them for any of it.
-template <class V>
-__device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, KryCtl *ctl, int jj)
+// In the first Krylov step v_0 = psi0 / ||psi0||, and P = |sum_i <psi0, v_i> y_i|^2 sees every other vector's
+// component along it at first order.  There c_0 is the dot with the u that was stored, whose rounding the
+// recurrence does not know, so that the update takes that off along psi0 as well: a basis state's is u's
+// element r0, a general state's the sum a0 (A0).  (With c_0 from the recurrence the rounding of u[r0] stayed in
+// W_2, W_3, ...: L = 20, N = 7 c64, P at t = 0.05 off by 5.5e-10 instead of 7e-13.)
+__device__ __forceinline__ double real_part(const float2 *p) { return (double)__ldcg(p).x; }
+__device__ __forceinline__ double real_part(const double2 *p) { return __ldcg(p).x; }
+__device__ __forceinline__ double real_part(const ffc *p)
+{
+    const float4 v = __ldcg((const float4 *)p);
+    return (double)v.x + (double)v.z;
+}
+// first: c_0 is taken here (not the first index of the first step).
+template <class V, bool A0>
+__device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, RealAcc<V> &a0, bool first, const V *U, double2 *part,
+                                               KryCtl *ctl, int jj)
 {
     __shared__ double2 red[PSTRIDE];
-    __shared__ double wsum[32];
+    __shared__ double wsum[1 + A0][32];
     __shared__ float Cs[MMAX * MMAX], ds[MMAX + 1];
     __shared__ int flag;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, r0 = ctl->r0;
+    const int ns = A0 && first ? 2 : 1;
     al.renorm();
     typename RealAcc<V>::Sum v[1] = {al.sum()};
     const double t = to_double(warp_totals<1>(v));
-    if (lane == 0) wsum[warp] = t;
+    if (lane == 0) wsum[0][warp] = t;
+    if (A0 && first) {
+        a0.renorm();
+        typename RealAcc<V>::Sum v0[1] = {a0.sum()};
+        const double t0 = to_double(warp_totals<1>(v0));
+        if (lane == 0) wsum[A0][warp] = t0;
+    }
     if (tid < PSTRIDE) red[tid] = make_double2(0.0, 0.0);
     __syncthreads();
-    if (tid == 0) {
+    if (tid < ns) {
         double s = 0.0;
-        for (int w = 0; w < (int)blockDim.x / 32; ++w) s += wsum[w];
-        red[0].x = s;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) s += wsum[tid][w];
+        red[tid].x = s;
     }
     __syncthreads();
-    if (!finish_partials(red, part, ctl, red, &flag, nullptr, 1, false, false)) return;
+    if (!finish_partials(red, part, ctl, red, &flag, nullptr, ns, false, false)) return;
+    double c0 = 0.0;
+    if (first && lane == 0) c0 = A0 ? red[A0].x : real_part(U + r0);
     for (int e = tid; e < MMAX * MMAX; e += blockDim.x) Cs[e] = ctl->C[e / MMAX][e % MMAX];
     if (tid <= MMAX) ds[tid] = tid < jj ? ctl->d[tid] : 0.f;   // (d_j = 1 stands apart)
     __syncthreads();
-    if (tid >= 32) return;
+    if (tid >= 64) return;   // lane i for vector i; warp 1 tests the sizes (MinorSum)
     const bool inv = lane <= jj;
     const double s = inv ? ctl->sigma[lane] : 0.0, alpha = red[0].x * ctl->sigma[jj];
     double c = 0.0;
@@ -858,20 +881,25 @@ __device__ __forceinline__ void alpha_epilogue(RealAcc<V> &al, double2 *part, Kr
     } else if (lane == jj) {
         c = alpha;
     }
-    const double cc = c * c, c2 = warp_sum_int<1>(&cc);
-    bool minor = false;
-    if (MinorSum<V>::use) {
-        // rounding level (MinorSum), against ||u||^2 >= alpha_j^2 + beta_{j-1}^2
-        const bool small = lane + 1 < jj;
-        const double cm = small ? cc : 0.0, m2 = warp_sum_int<1>(&cm), big = small ? 0.0 : cc, b2 = warp_sum_int<1>(&big);
-        minor = __all_sync(0xffffffffu, !small || (s >= 0x1p-40 && s <= 0x1p40)) &&
-                m2 <= MinorSum<V>::eta * MinorSum<V>::eta * b2;
+    if (first && lane == 0) c = s * c0;
+    const double cc = c * c;
+    if (warp == 1) {
+        bool minor = false;
+        if (MinorSum<V>::use) {
+            // rounding level, against ||u||^2 >= alpha_j^2 + beta_{j-1}^2
+            const bool small = lane + 1 < jj;
+            const double cm = small ? cc : 0.0, m2 = warp_sum_int<1>(&cm), big = small ? 0.0 : cc, b2 = warp_sum_int<1>(&big);
+            minor = __all_sync(0xffffffffu, !small || (s >= 0x1p-40 && s <= 0x1p40)) &&
+                    m2 <= MinorSum<V>::eta * MinorSum<V>::eta * b2;
+        }
+        if (lane == 0) ctl->minor = minor ? 1 : 0;
+        return;
     }
     if (inv) ctl->coefA[lane] = c * s;
+    const double c2 = warp_sum_int<1>(&cc);
     if (lane != 0) return;
     ctl->alpha[jj] = alpha;
     ctl->c2 = c2;
-    ctl->minor = minor ? 1 : 0;
     ctl->n_hv += 1;
     ctl->vec_passes += 2;
     ctl->vp_kind[KIND_HV] += 2;   // the H.v: v_j read, u written
@@ -1211,6 +1239,30 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
             if (ALPHA) al->add(x0, RealAcc<V>::pre(valid ? out : VT<V>::zero()));
         }
         if (ALPHA) al->renorm();   // (once per item, at most eight rows)
+    }
+}
+
+// *acc sums Re <x, y> over the rows that this thread has written in hv_items.  (A pass of its own: in
+// hv_items' loop its accumulators and loads cost every step 2%, c128e at L = 23, for what the first one needs.)
+template <class V>
+__device__ __forceinline__ void hv_items_dot(const DevBasis &b, const HvPlan &pl, const V *__restrict__ x, const V *y,
+                                             RealAcc<V> *acc)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t total = pl.first[b.Lhi + 1], nw = blockDim.x >> 5;
+    int c = 0;
+    for (uint32_t item = blockIdx.x * nw + (threadIdx.x >> 5); item < total; item += gridDim.x * nw) {
+        while (item >= pl.first[c + 1]) ++c;
+        const uint32_t nlo = pl.nlo[c], nch = (nlo + 31u) >> 5, rem = item - pl.first[c], g = rem / nch;
+        const uint32_t i = (rem - g * nch) * 32u + lane, h0 = pl.hoff[c] + g * pl.nh;
+        const int nh = min((uint32_t)pl.nh, pl.hoff[c + 1] - h0);
+        if (i < nlo) {
+            for (int h = 0; h < nh; ++h) {
+                const uint32_t r = __ldg(b.blk + __ldg(b.hilist + h0 + h)) + i;
+                acc->add(ldg(x + r), RealAcc<V>::pre(y[r]));
+            }
+        }
+        acc->renorm();
     }
 }
 

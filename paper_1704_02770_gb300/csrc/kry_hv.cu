@@ -95,10 +95,11 @@ __device__ __forceinline__ void cta_sum_into(const Acc &acc, double2 *red, int s
 // u = sigma_j H W_j, written to U (pass A, part 1): the gathers of hv_items at full occupancy.  Without
 // ALPHA (two-pass form) nothing else: alpha_j, ||u||^2 and the dots with the earlier vectors are taken
 // by the streaming pass that follows (k_dots, mode 0).  With ALPHA (one-read form, k_ortho) the pass
-// also takes alpha_j and sets up the update's coefficients (L = 24 c64: 40 us without, 50 with).
+// also takes alpha_j and sets up the update's coefficients (L = 24 c64: 40 us without, 50 with), and with A0 (a
+// general psi0) in the first Krylov step c_0 (alpha_epilogue).
 // FORM: how many loads are issued together inside the lower and the upper bits (HV_RND); every form
 // gives the same bits, the launch shape picks the fastest (kry_autotune).
-template <class V, int FORM, bool ALPHA>
+template <class V, int FORM, bool ALPHA, bool A0>
 __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V> a, HvPlan pl, int jj)
 {
     using R = typename VT<V>::R;
@@ -111,9 +112,14 @@ __global__ void __launch_bounds__(HV_NTHR, sizeof(V) == 8 ? 4 : 3) k_hv(EvArgs<V
     if (ctl->done || jj >= ctl->m_eff) return;
     const double s = ctl->sigma[jj];
     RealAcc<V> al;
-    hv_items<V, HV_RND<V, (FORM & 1)>, HV_RND<V, (FORM >> 1)>, ALPHA>(a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s,
-                                        (R)(s * a.h.halfJ), &al);
-    if constexpr (ALPHA) alpha_epilogue<V>(al, a.part, ctl, jj);
+    hv_items<V, HV_RND<V, (FORM & 1)>, HV_RND<V, (FORM >> 1)>, ALPHA>(
+        a.b, a.h, pl, a.W + (size_t)jj * a.ldW, a.U, w[threadIdx.x >> 5], dz, (R)s, (R)(s * a.h.halfJ), &al);
+    if constexpr (ALPHA) {
+        const bool first = jj > 0 && ctl->n_steps == 0;
+        RealAcc<V> a0;
+        if (A0 && first) hv_items_dot<V>(a.b, pl, a.W, a.U, &a0);
+        alpha_epilogue<V, A0>(al, a0, first, a.U, a.part, ctl, jj);
+    }
 }
 
 // The row loop of k_dots for one group of 64 threads: NQ vectors from Wg, NU units of rows at a time
@@ -314,8 +320,10 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
 //     (H - s) v_i = sum_{k<=i} C_ki v_k + beta_i v_{i+1}   (C_ki its coefficients c_k),
 // up to the rounding of that update.  With the dots d_k = Re <v_k, v_j> that this kernel measured when it
 // made v_j (d_j = 1), c_i = beta_i (sum_{k<=i} (C_ki / beta_i) d_k + d_{i+1}): beta_{j-1} for i = j - 1, rounding level
-// below, and c_j = alpha_j comes from the H.v pass.  An error of c_i is the same rounding that a dot product
-// of u has, it leaves the new vector that much off, and the next dots see it.  The Krylov vectors, whose
+// below, and c_j = alpha_j comes from the H.v pass (as c_0 does in the first Krylov step, see alpha_epilogue).
+// What the recurrence leaves out is the rounding of the stored u along v_i, which stays in the new vector, and
+// the next dots see it: of the order of the rounding of w itself, except where v_i is a few elements and P
+// reads it, which is v_0.  The Krylov vectors, whose
 // reads bound the step, are read once per Lanczos index instead of twice.
 // 64 threads take one row each of up to 16 vectors at a time; from 17 vectors on two such groups share a
 // row.  (Eight vectors per group, with teams of up to four, took
@@ -333,7 +341,6 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     __shared__ double wred[NW][QV + 3];
     __shared__ typename RealLin<V>::RCoef coef[MMAX + 1];
     __shared__ float mcoef[MMAX + 1];
-    __shared__ double ci[MMAX + 1];   // c_i
     __shared__ __align__(16) V xch[2 * ORTHO_NTHR<V> * ORTHO_XU];
     __shared__ int flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = tid >> 6;
@@ -342,7 +349,6 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
         const double c = ctl->coefA[tid];
         coef[tid] = RealLin<V>::coef(c);
         mcoef[tid] = -(float)c;
-        ci[tid] = c * (tid ? ctl->beta[tid - 1] : ctl->beta0);   // (1 / sigma_i is the norm that made v_i)
     }
     __syncthreads();
     const bool minor = MinorSum<V>::use && ctl->minor;
@@ -406,6 +412,8 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
             if (lane == 0) { wred[warp][QV + 1] = tg.x; wred[warp][QV + 2] = tg.y; }
         }
     }
+    // c_i (1 / sigma_i is the norm that made v_i) in warp 1; loaded here, its latency passes beside the reduction
+    const double ci = warp == 1 && lane <= jj ? ctl->coefA[lane] * (lane ? ctl->beta[lane - 1] : ctl->beta0) : 0.0;
     __syncthreads();
     if (tid < nv) {
         const int s = nvg == 1 || tid < nv / 2 ? 0 : 1;   // the share that holds vector tid
@@ -429,20 +437,23 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     __syncthreads();
     double2 *fin = red;
     if (!finish_partials(red, a.part, ctl, fin, &flag, nullptr, nv, true, a.G != nullptr)) return;
-    if (tid >= 32) return;
-    const bool inv = tid <= jj;
-    const double s = inv ? ctl->sigma[tid] : 0.0, dd = fin[tid].x * s;   // Re <v_i, w>
+    // Scalar epilogue, lane i for vector i: warp 1 keeps C and d of the new vector while warp 0 ends the index (the
+    // FP64 square roots of both in one warp, and the sums of alpha_epilogue, took 1 us longer: P at L = 24 c64 76.6 -> 76.1 ms).
+    if (tid >= 64) return;
+    const bool inv = lane <= jj;
+    const double s = inv ? ctl->sigma[lane] : 0.0, dd = fin[lane].x * s;   // Re <v_i, w>
     const double d2 = dd * dd, nd2 = warp_sum_int<1>(&d2), nw2 = fin[SLOT_NRM].x;
     const double normu2 = ctl->c2 + nw2;   // ||u||^2 = ||c||^2 + ||w||^2 for orthonormal v_i
     const bool dead = !(nw2 > ctl->eta_bd * ctl->eta_bd * normu2);   // an invariant subspace: nothing to correct
     const bool sub = !dead && nd2 > ctl->eta_corr * ctl->eta_corr * nw2;
-    if (inv) {
+    if (warp == 1) {
         const double rb = rsqrt(nw2);
-        if (sub) ctl->coefC[tid] = dd * s;   // (pass C2 sets C)
-        else if (!dead) ctl->C[tid][jj] = (float)(ci[tid] * rb);
+        if (inv && !sub && !dead) ctl->C[lane][jj] = (float)(ci * rb);   // (after a subtraction pass C2 sets C)
         // d of the new vector; after pass C2 it is at rounding level and taken as zero
-        ctl->d[tid] = sub || dead ? 0.f : (float)(dd * rb);
+        if (inv) ctl->d[lane] = sub || dead ? 0.f : (float)(dd * rb);
+        return;
     }
+    if (inv && sub) ctl->coefC[lane] = dd * s;
     if (sub && tid == jj) ctl->alpha[jj] += dd;
     if (tid != 0) return;
     ctl->normu2 = normu2;
@@ -846,7 +857,7 @@ int vector_grid(const DevBasis &b, int *gridH, int *gridB)
 {
     const uint32_t es = sizeof(V);
     int occB = 0, occH = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0, true>, HV_NTHR, 0);   // (the same for every form)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occH, k_hv<V, 0, true, false>, HV_NTHR, 0);   // (the same for every form)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occB, k_lincomb<V, 0, 2>, NTHR, 0);
     const uint32_t ntiles = (b.D + TILE - 1) / TILE;
     auto fit = [&](int occ, uint32_t most) {
@@ -873,8 +884,9 @@ int launch_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
     auto go = [&](auto k0, auto k1, auto k2, auto k3) {
         return launch_ex(pdl, a.hv_form == 0 ? k0 : a.hv_form == 1 ? k1 : a.hv_form == 2 ? k2 : k3, grid, HV_NTHR, 0, s, a, pl, jj);
     };
-    if (a.one_read) KRY_CU(go(k_hv<V, 0, true>, k_hv<V, 1, true>, k_hv<V, 2, true>, k_hv<V, 3, true>));
-    else KRY_CU(go(k_hv<V, 0, false>, k_hv<V, 1, false>, k_hv<V, 2, false>, k_hv<V, 3, false>));
+    if (a.one_read && a.G) KRY_CU(go(k_hv<V, 0, true, true>, k_hv<V, 1, true, true>, k_hv<V, 2, true, true>, k_hv<V, 3, true, true>));
+    else if (a.one_read) KRY_CU(go(k_hv<V, 0, true, false>, k_hv<V, 1, true, false>, k_hv<V, 2, true, false>, k_hv<V, 3, true, false>));
+    else KRY_CU(go(k_hv<V, 0, false, false>, k_hv<V, 1, false, false>, k_hv<V, 2, false, false>, k_hv<V, 3, false, false>));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }

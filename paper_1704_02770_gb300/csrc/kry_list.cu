@@ -167,9 +167,11 @@ __global__ void __launch_bounds__(NTHR) k_list_apply(DevBasis b, DevHam hm, int 
 }
 
 // pass A, part 1, one realisation: U = sigma_j H W_j
-// (ALPHA as in k_hv)
-template <class V, bool ALPHA>
-__global__ void __launch_bounds__(NTHR) k_list_hv(EvArgs<V> a, int jj)
+// (ALPHA and A0 as in k_hv)
+// Five CTAs per SM: with registers for six the complex64 form with ALPHA takes 17.5 ms instead of 16.7 (P at
+// L = 55, N = 4 to t = 20; 341,055 rows).
+template <class V, bool ALPHA, bool A0>
+__global__ void __launch_bounds__(NTHR, 5) k_list_hv(EvArgs<V> a, int jj)
 {
     pdl_begin();
     KryCtl *ctl = a.ctl;
@@ -182,7 +184,8 @@ __global__ void __launch_bounds__(NTHR) k_list_hv(EvArgs<V> a, int jj)
     const double sd = ctl->sigma[jj];
     const R sj = (R)sd, shj = (R)(sd * a.h.halfJ);
     const V *x = a.W + (size_t)jj * a.ldW;
-    RealAcc<V> al;
+    const bool first = jj > 0 && ctl->n_steps == 0;
+    RealAcc<V> al, a0;
     int it = 0;
     for (uint32_t r = blockIdx.x * NTHR + threadIdx.x; r < a.b.D; r += gridDim.x * NTHR) {
         R d;
@@ -191,10 +194,14 @@ __global__ void __launch_bounds__(NTHR) k_list_hv(EvArgs<V> a, int jj)
         a.U[r] = u;
         if (ALPHA) {
             al.add(x0, RealAcc<V>::pre(u));
-            if ((++it & 3) == 0) al.renorm();
+            if (A0 && first) a0.add(ldg(a.W + r), RealAcc<V>::pre(u));
+            if ((++it & 3) == 0) {
+                al.renorm();
+                a0.renorm();
+            }
         }
     }
-    if constexpr (ALPHA) alpha_epilogue<V>(al, a.part, ctl, jj);
+    if constexpr (ALPHA) alpha_epilogue<V, A0>(al, a0, first, a.U, a.part, ctl, jj);
 }
 
 // pass A, part 1, K realisations: U[:, k] = sigma_j[k] H_k W_j[:, k]
@@ -289,16 +296,17 @@ template <class V>
 int list_hv_grid(const DevBasis &b, int *grid)
 {
     const size_t sm = list_smem(b);
-    if (int rc = list_prep(k_list_hv<V, false>, sm)) return rc;
-    if (int rc = list_prep(k_list_hv<V, true>, sm)) return rc;
-    *grid = list_grid_of(k_list_hv<V, true>, sm, b.D);
+    if (int rc = list_prep(k_list_hv<V, false, false>, sm)) return rc;
+    if (int rc = list_prep(k_list_hv<V, true, false>, sm)) return rc;
+    if (int rc = list_prep(k_list_hv<V, true, true>, sm)) return rc;
+    *grid = list_grid_of(k_list_hv<V, true, false>, sm, b.D);
     return KRY_OK;
 }
 
 template <class V>
 int launch_list_hv(const EvArgs<V> &a, int jj, int grid, cudaStream_t s, int pdl)
 {
-    KRY_CU(launch_ex(pdl, a.one_read ? k_list_hv<V, true> : k_list_hv<V, false>, grid, NTHR, list_smem(a.b), s, a, jj));
+    KRY_CU(launch_ex(pdl, !a.one_read ? k_list_hv<V, false, false> : a.G ? k_list_hv<V, true, true> : k_list_hv<V, true, false>, grid, NTHR, list_smem(a.b), s, a, jj));
     KRY_CU(cudaGetLastError());
     return KRY_OK;
 }

@@ -222,8 +222,9 @@ int kry_tridiag_expv_noalloc(const double *alpha, const double *beta, int m, dou
  *   update w = u - sum c_i v_i and ||w||^2), 2 = pass C (the second Gram-Schmidt pass, when
  *   flagged), 3 = small exponential and step control, 4 = combine psi = beta V y,
  *   5 = pass A's H.v (u = sigma_j (H - s) v_j),
- * (in sectors of 65,536 states and more one pass over the Krylov vectors takes the update and
- * the dots of its result, counted under 1, and kind 0 stays empty),
+ * (in sectors of 65,536 states and more, and in ensembles of 32,768 states times realisations and
+ * more, one pass over the Krylov vectors takes the update and the dots of its result, counted
+ * under 1, and kind 0 stays empty),
  * the summed event time in ms, the algorithmic HBM bytes (vector reads and writes by
  * formula; gathers of H.v beyond one read of v_j are not counted) and the count of
  * profiled intervals, accumulated since the last kry_profile_enable(H, 1).  Arrays have 6
@@ -281,8 +282,9 @@ int kry_autotune(kry_ham H, int dtype, int m, uint64_t probe_state, double t_pro
  * second pass is also taken when the lengths of u = H v_j, of its projections c = V^H u and
  * of w = u - V c disagree with Pythagoras, | ||w||^2 - (||u||^2 - ||c||^2) | > eta ||c|| ||w||
  * plus the storage-precision noise, a sign that V has lost orthogonality.  (In sectors of 65,536
- * states and more the dots of every new vector are measured in any case, by the pass that makes
- * it, and the subtraction is made whenever they exceed eta ||w||.)  Returns
+ * states and more, and in ensembles of 32,768 states times realisations and more, the dots of every
+ * new vector are measured in any case, by the pass that makes it, and the subtraction is made
+ * whenever they exceed eta ||w||.)  Returns
  * KRY_EINVAL for other values of on. */
 int kry_set_orth_check(kry_ham H, int on);
 

@@ -1090,11 +1090,11 @@ __device__ __forceinline__ void stage_tables(const DevBasis &b, uint32_t *koff_s
 // have the same list of lower parts, so a warp takes an item: 32 consecutive lower parts (one per
 // lane) of NH such blocks.  What depends on lo alone -- the ranks of its hops, rl[lo ^ (3 << p)] --
 // is found once per item and serves NH rows; what depends on hi alone -- the block starts of its hops
-// -- is found once per item by one lane per (block, bond) and shared.  A row then costs about four
-// instructions a hop (a predicated load at block start + rank, and the add) and no unranking (L = 24
-// c64: 40 us, L = 26 138).
+// -- is found once per item by one lane per (block, bond) and shared.  A row then needs no unranking: about 350
+// thread instructions in all at L = 24 (c64, 13 hops, alpha_j included; every lower bond is issued for all lanes,
+// with or without a hop), 40 us without alpha_j, 138 at L = 26.
 // A per-row form (unrank, then a loop over the row's hops) took 404 instructions per row at L = 24
-// and 533 at L = 28, was bound by their issue (59% active) and took 51 us (L = 24 c64).
+// and 533 at L = 28 without alpha_j, was bound by their issue (59% active) and took 51 us (L = 24 c64).
 // The terms of a row are added in bond order, the ring bond last.
 constexpr int HV_NH = 8;        // blocks of an item, at most
 constexpr int HV_NTHR = 256;    // threads of a CTA of the H.v
@@ -1157,7 +1157,7 @@ __device__ __forceinline__ void hv_items(const DevBasis &b, const DevHam &hm, co
         const uint32_t lomask = (1u << Llo) - 1u;
         // Ranks of the lower part's hops (any pattern has one), in registers; for complex128 with ALPHA packed
         // per lane in shared memory: the rows' loops then run to the longest list of the warp (about nine hops
-        // at L = 24) instead of over all Llo - 1 bonds, and its sum costs 40 instructions a term (189 -> 163
+        // at L = 24) instead of over all Llo - 1 bonds, and its sum costs 32 instructions a term (189 -> 163
         // us).  The other types lose what it takes to pack (L = 26 c64 138 -> 153 us).
         constexpr bool PACK = ALPHA && std::is_same<V, double2>::value;
         uint32_t t[16];

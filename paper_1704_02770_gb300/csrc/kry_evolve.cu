@@ -502,8 +502,9 @@ Layout layout_b(const kry_ham_s *H, int dtype, int m, int grid, int n_times)
     return l;
 }
 
-// The batched one-read form (k_ortho_b), from 32,768 elements on (L = 15 K = 9 c128, 57,915 elements: 88 ->
-// 50 us per Lanczos index; L = 20 K = 64 c64: 819 -> 581).
+// The batched one-read form (k_ortho_b), from 32,768 elements on.  Two-pass and one-read form, us per Lanczos index
+// in c128, c128e and c64: L = 12 K = 16 (14,784 elements) 46.9/49.8, 40.3/42.9, 39.1/40.6; L = 14 K = 9 (30,888)
+// 53.2/49.2, 40.4/41.3, 38.0/38.6; L = 15 K = 9 (57,915) 72.8/54.1, 50.4/44.4, 45.9/40.8; L = 20 K = 64 c64 819/539.
 int one_read_form_b(const kry_ham_s *H) { return (size_t)H->b->D * (size_t)H->K >= 32768u ? 1 : 0; }
 
 // CTAs of the batched dots of pass A (returned) and of the update, second pass and combine

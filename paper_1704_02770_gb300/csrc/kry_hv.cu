@@ -327,7 +327,9 @@ __global__ void __launch_bounds__(DOTS_NTHR, 1) k_dots(EvArgs<V> a, int jj)
 // reads bound the step, are read once per Lanczos index instead of twice.
 // 64 threads take one row each of up to 16 vectors at a time; from 17 vectors on two such groups share a
 // row.  (Eight vectors per group, with teams of up to four, took
-// 98.7 us where this takes 90.4, L = 24 c64, and 107.5 against 93.2, L = 23 c128e.)
+// 98.7 us where this takes 90.4, L = 24 c64, and 107.5 against 93.2, L = 23 c128e.)  Sixteen vectors' rows and
+// accumulators do not fit the 128 registers of 512 threads: complex64 spills 368 bytes per thread (708 loaded
+// back), complex128 108 (348); c128e has 168 and no spills.
 // Odd indices run backwards, so that the rows a pass ends with are still in L2 for the next.  When the
 // dots exceed eta_corr, pass C2 (k_lincomb, mode 1) takes them off.
 template <class V, int COND>
@@ -809,8 +811,11 @@ static int sm_count()
 static int lincomb_threads(uint32_t D) { return D < (uint32_t)sm_count() * 4u * NTHR ? 64 : NTHR; }
 
 // Blocks per item of the H.v: more share the lower part's ranks, fewer give more items.  One below four
-// items of 32 rows per warp slot, two below 16, four below 200 (L = 24 c64: 40.5 us with four, 47 with one)
-// and eight from there on (3% faster than four at L = 30).
+// items of 32 rows per warp slot, two below 16, four below 200 and eight from there on.  kry_apply with one, two,
+// four and eight, in us (complex64; complex128), by items of 32 rows per slot:
+//   0.3 (L = 18)   9.3 9.3 9.3 12.2; 8.9 10.0 16.4 24.6     17 (L = 24)   53.8 41.5 37.3 37.3; 171 160 158 158
+//   4.5 (L = 22)   18.5 14.4 15.9 16.4; 50.0 47.2 52.8 54.8 67 (L = 26)   200 154 141 130; 694 641 623 618
+//   8.7 (L = 23)   28.8 22.6 22.6 24.6; 88 82 80 81         258 (L = 28)  975 724 655 616; 3450 3215 3121 3050
 static HvPlan hv_plan(const DevBasis &b)
 {
     HvPlan p{};

@@ -279,8 +279,10 @@ struct EvArgs {
 };
 
 // Update and dots in one pass over the Krylov vectors (k_ortho), from 65,536 rows on: there the vectors'
-// reads cost more than the pass's longer rows (L = 19 c128e: 45.7 -> 43.6 us per Lanczos index, L = 24 c64
-// 188 -> 152, L = 30 c64 10.1 -> 8.2 ms); below, both forms are bound by latency and tie (L = 16 c128).
+// reads cost more than the pass's longer rows; below, both forms are bound by latency.  Two-pass and one-read
+// form, us per Lanczos index in c128, c128e and c64: 12,870 rows 30.7/32.3, 28.4/27.2, 26.5/26.3; 48,620
+// 36.1/35.7, 31.5/28.6, 28.1/26.8; 92,378 45.6/43.5, 39.6/33.8, 33.7/30.6; 184,756 63.7/58.8, 45.8/43.1,
+// 36.3/36.9; L = 24 c64 188/152, L = 30 c64 10,100/8,200.
 inline bool one_read_form(uint32_t D) { return D >= 65536u; }
 
 struct ExpArgs {

@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(256) k_reduce_b(KryCtlB *ctl, const double2 *_
         const bool run = jj < ctl->m_eff[k];
         const double normu2 = ctl->c2[k] + nw2;   // ||u||^2 = ||c||^2 + ||w||^2
         const bool dead = !(nw2 > H.eta_bd * H.eta_bd * normu2);
-        const bool sub = run && !dead && nd2 > H.eta_corr * H.eta_corr * nw2;
+        const bool sub = run && nw2 > 0.0 && nd2 > H.eta_corr * H.eta_corr * nw2;   // (as in k_ortho)
         if (lane <= jj) {
             const double rb = rsqrt(nw2);
             const bool off = sub || dead || !run;   // (after a subtraction mode 2 sets C)

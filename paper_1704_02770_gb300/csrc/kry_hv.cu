@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(ORTHO_NTHR<V>, 1) k_ortho(EvArgs<V> a, int jj)
     const double s = inv ? ctl->sigma[lane] : 0.0, dd = fin[lane].x * s;   // Re <v_i, w>
     const double d2 = dd * dd, nd2 = warp_sum_int<1>(&d2), nw2 = fin[SLOT_NRM].x;
     const double normu2 = ctl->c2 + nw2;   // ||u||^2 = ||c||^2 + ||w||^2 for orthonormal v_i
-    const bool dead = !(nw2 > ctl->eta_bd * ctl->eta_bd * normu2);   // an invariant subspace: nothing to correct
-    const bool sub = !dead && nd2 > ctl->eta_corr * ctl->eta_corr * nw2;
+    const bool dead = !(nw2 > ctl->eta_bd * ctl->eta_bd * normu2);   // an invariant subspace
+    // (where the space ends too: w is rounding then, its dots refine alpha_j and its length the error estimate)
+    const bool sub = nw2 > 0.0 && nd2 > ctl->eta_corr * ctl->eta_corr * nw2;
     if (warp == 1) {
         const double rb = rsqrt(nw2);
         if (inv && !sub && !dead) ctl->C[lane][jj] = (float)(ci * rb);   // (after a subtraction pass C2 sets C)

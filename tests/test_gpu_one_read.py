@@ -319,3 +319,28 @@ def test_complex64_early_P_of_a_basis_state(kry, K, lst, general):
         P4, _ = H.return_probability(s, times, tol=1e-8, dtype="c64")
     print(f"[early P] K={K} list={lst} general={general}: {np.max(np.abs(P4 - P8) / (1 - P8)**2) * 2**24:.2f} x 2^-24 (1 - P)^2")
     assert np.all(np.abs(P4 - P8) <= 4.0 * 2.0**-24 * (1.0 - P8)**2 + 1e-13)
+
+
+@pytest.mark.parametrize("K", [1, 10])
+@pytest.mark.parametrize("form,eps", [("c128", 2.0**-53), ("c128e", 2.0**-48)])
+def test_eigenvector_keeps_its_phase(kry, K, form, eps):
+    """From an eigenvector the first update leaves rounding alone.  The Krylov space ends there, and the dots of
+    that rest are still taken off: they refine alpha_0, whose error turns the phase by t times as much.  Bar: one
+    rounding of the energy, eps |E| t, and what the eigenvector itself is off by (its residual, times t)."""
+    from scipy.sparse import csr_matrix
+    from scipy.sparse.linalg import eigsh
+    L, N = (20, 7) if K == 1 else (14, 7)
+    h = workloads.quasiperiodic_field(L, 1.3, 0.7)
+    c = ob.CSR(L, N, 1.0, 0.8, h, True)
+    A = csr_matrix((c.val, c.col, c.rowptr), shape=(c.D, c.D))
+    lam, V = eigsh(A, k=1, which="SA", tol=1e-15, v0=np.ones(c.D))
+    E, v = lam[0], V[:, 0] / np.linalg.norm(V[:, 0])
+    t, res = 3.0, np.linalg.norm(A @ v - E * v)
+    H = kry.Hamiltonian(kry.Basis(L, N), 1.0, 0.8, np.tile(h, (K, 1)) if K > 1 else h)
+    x = torch.from_numpy(np.repeat(v[:, None], K, axis=1).astype(np.complex128).reshape(-1)).cuda()
+    out = torch.empty_like(x)
+    _, st = H.evolve(x, [t], tol=1e-10, psi_out=out, emulated=form == "c128e")
+    err = np.linalg.norm(out.cpu().numpy().reshape(-1, K) - (np.exp(-1j * t * E) * v)[:, None], axis=0).max()
+    print(f"[eigenvector] K={K} {form}: |dpsi| {err:.1e}, eps |E| t {eps * abs(E) * t:.1e}, residual t {res * t:.1e}")
+    assert st["n_breakdowns"] >= K and st["n_second_pass"] >= 1
+    assert err <= eps * abs(E) * t + 2.0 * res * t + 1e-14
